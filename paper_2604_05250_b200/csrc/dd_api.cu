@@ -117,6 +117,7 @@ int dd_release(void)
     DD_CUDA_TRY(cudaDeviceSynchronize());
     if (ctx->verify_ws) DD_CUDA_TRY(cudaFree(ctx->verify_ws));
     if (ctx->verify_cnt) DD_CUDA_TRY(cudaFree(ctx->verify_cnt));
+    if (ctx->head_ws) DD_CUDA_TRY(cudaFree(ctx->head_ws));
     if (ctx->staging) DD_CUDA_TRY(cudaFree(ctx->staging));
     if (ctx->attn_status) DD_CUDA_TRY(cudaFree(ctx->attn_status));
     if (ctx->mirror) DD_CUDA_TRY(cudaFreeHost(const_cast<unsigned int *>(ctx->mirror)));

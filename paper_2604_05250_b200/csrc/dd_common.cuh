@@ -16,6 +16,8 @@ struct DeviceCtx {
     size_t verify_ws_bytes = 0;
     void *verify_cnt = nullptr;     // dd_verify completion counters: all zero between launches
     size_t verify_cnt_bytes = 0;
+    void *head_ws = nullptr;        // dd_lm_head_verify: plan, list of flagged rows, their hidden states
+    size_t head_ws_bytes = 0;
     void *staging = nullptr;        // device copies of host buffers (the *_host calls)
     size_t staging_bytes = 0;
     unsigned int *attn_status = nullptr;  // one word: first expired wait of the attention kernel

@@ -15,9 +15,18 @@
 // every flagged row's partials in fp64 with the streaming kernel's fold and runs dd_verify's
 // decision stage per sequence.
 //
+// Only flagged positions need logits.  A first small kernel (lm_head_rows_kernel) lists the flagged
+// rows and, where that leaves fewer 128-row tiles, copies their hidden states one after the other
+// into scratch; the products then run over those.  How many there are is known on the device only:
+// it picks the width N of the vocabulary tiles too (a tensor map per width travels with the launch).
+// 16 sequences of 256 positions, 62 % of them flagged, K = 4096, V = 126464: 3024 us
+// with every row multiplied, 1961 us so.
+//
 // Tensor memory (512 columns): TRUST/CONF, N <= 256: the verifier's two accumulators at columns 0
 // and 256.  KL, N <= 128: the drafter's at 0 and 128, the verifier's at 256 and 384; a work item
-// runs the k loop over the drafter's operands first, then over the verifier's.
+// runs the k loop over the drafter's operands first, then over the verifier's.  An item with no more
+// than 128 rows (the last row block, or the only one) uses one accumulator and leaves the other to
+// the next such item: its products run while this one is reduced.
 //
 //   warps 0-3   epilogue of rows 0-127 of the item (thread = row = tensor-memory lane)
 //   warps 4-7   epilogue of rows 128-255
@@ -41,31 +50,135 @@ using namespace ddptx;
 constexpr int kThreads = 320;
 constexpr int kEpilogueWarps = 8;
 constexpr int kLoadWarp = 8, kMmaWarp = 9;
-constexpr int kRowsPerItem = 256;          // two accumulators of 128 rows
+constexpr int kTileRows = 128;
+constexpr int kRowsPerItem = 2 * kTileRows; // two accumulators
 constexpr int kBlockK = 64;                // one 128-byte swizzled box per k-step
-constexpr int kStages = 3;
+constexpr int kMaxStages = 6;
 constexpr int kMaxN = 256;
 constexpr uint32_t kTmemCols = 512;        // see the layout above
-constexpr int kATileBytes = 128 * kBlockK * 2;                        // 16 KB: 128 rows x 64 bf16
-constexpr int kStageBytes = 2 * kATileBytes + kMaxN * kBlockK * 2;    // 64 KB
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
+constexpr int kATileBytes = kTileRows * kBlockK * 2;                  // 16 KB: 128 rows x 64 bf16
+constexpr int kRingBytes = 3 * (2 * kATileBytes + kMaxN * kBlockK * 2);   // 192 KB: three stages of the largest kind
+constexpr int kSmemBytes = kRingBytes + 1024 + 256;
 constexpr unsigned kErrLmFull = 0xC00, kErrLmEmpty = 0xD00, kErrLmAcc = 0xE00;
+
+// Widths of the vocabulary tiles: kWidths multiples of 32 downwards from the largest.
+template <bool KL>
+struct Widths {
+    static constexpr int max_n = KL ? kMaxN / 2 : kMaxN;
+    static constexpr int count = max_n / 64 + 1;              // down to half of it
+};
+
+// What the first kernel finds out, for the two behind it.
+struct LmPlan {
+    int n_rows;                // rows to multiply: the flagged ones, or all of them where that costs no more
+    int gathered;              // 1: their hidden states stand one after the other in the scratch
+    int N;                     // vocabulary entries per work item
+    int n_tiles;               // ceil(V / N): the "chunks" of a row
+};
 
 struct LmParams {
     int rows, K, V;            // rows = B * P
-    int N;                     // vocabulary entries per work item (a multiple of 32, <= 256; KL: <= 128)
-    int n_tiles;               // ceil(V / N): the "chunks" of a row
-    int row_blocks;            // ceil(rows / 256)
+    int ctas;                  // CTAs the tile width is chosen for
+    int min_n;                 // the narrowest width the scratch has partials for
+    int can_gather;            // the scratch has room for the hidden states
+    LmPlan *plan;
+    int *row_map;              // [rows]: the row that gathered row i is (not written where nothing is gathered)
 };
+
+// Tensor maps of one launch: hidden states (as passed, and as gathered) and weights (a map per width).
+template <bool KL>
+struct LmMaps {
+    CUtensorMap h, h_gathered, w[Widths<KL>::count];
+    CUtensorMap hd, hd_gathered, wd[KL ? Widths<KL>::count : 1];      // the drafter's, KL only
+};
+
+// Vocabulary entries per work item: the width for which the slowest of `ctas` CTAs finishes first.
+// A work item of n entries takes about (fixed + n) units of time: the hidden-state tiles it loads and
+// the MMAs' shared-memory reads of them do not shrink with n.  Measured at K = 4096 (time per item
+// against n, tile widths forced): fixed = 140 for one product per item, 157 for the KL mode's two.
+// Counting n alone picked tiles of 128 entries at 4096 rows, 25 % slower than 256.
+template <bool KL>
+__host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int min_n)
+{
+    constexpr int fixed = KL ? 157 : 140;
+    int best = Widths<KL>::max_n;
+    long best_cost = -1;
+    for (int i = 0; i < Widths<KL>::count; ++i) {
+        const int n = Widths<KL>::max_n - 32 * i;
+        if (n < min_n) break;
+        const long items = ((V + n - 1) / n) * row_blocks;
+        const long cost = ((items + ctas - 1) / ctas) * (fixed + n);
+        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = n; }
+    }
+    return best;
+}
+
+// First launch of dd_lm_head_verify.  Every block counts all flags (a few KB) and the flags before its
+// own rows; the first one writes the plan.  Gathering pays where it leaves fewer 128-row tiles (at
+// K = 4096, V = 126464 a tile of rows costs 85 us, copying 128 rows less than one); elsewhere nothing is
+// copied.  One warp per row.
+constexpr int kRowsThreads = 256;
+constexpr int kRowsPerBlock = kRowsThreads / 32;
+template <bool KL>
+__global__ void __launch_bounds__(kRowsThreads)
+lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden, uint4 *gathered,
+                    const uint4 *hidden_d, uint4 *gathered_d)
+{
+    __shared__ int s_before, s_all;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int first = blockIdx.x * kRowsPerBlock;
+    if (tid == 0) s_before = s_all = 0;
+    __syncthreads();
+    int before = 0, all = 0;
+    auto count = [&](int i, int n) { all += n; before += i < first ? n : 0; };
+    int done = 0;
+    if ((reinterpret_cast<uintptr_t>(flags) & 7) == 0) {           // eight flags at a time (first is a multiple of eight)
+        done = q.rows & ~7;
+        for (int i = 8 * tid; i < done; i += 8 * kRowsThreads) {
+            const uint2 w = *reinterpret_cast<const uint2 *>(flags + i);
+            count(i, __popc(__vsetne4(w.x, 0u)) + __popc(__vsetne4(w.y, 0u)));
+        }
+    }
+    for (int i = done + tid; i < q.rows; i += kRowsThreads) count(i, flags[i] != 0);
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    all = __reduce_add_sync(0xFFFFFFFFu, all);
+    if (lane == 0) { atomicAdd(&s_before, before); atomicAdd(&s_all, all); }
+    __syncthreads();
+    all = s_all;
+    const bool gather = q.can_gather && (all + kTileRows - 1) / kTileRows < (q.rows + kTileRows - 1) / kTileRows;
+    if (blockIdx.x == 0 && tid == 0) {
+        LmPlan plan;
+        plan.n_rows = gather ? all : q.rows;
+        plan.gathered = gather;
+        plan.N = pick_tile_n<KL>(q.V, (plan.n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n);
+        plan.n_tiles = (q.V + plan.N - 1) / plan.N;
+        *q.plan = plan;
+    }
+    if (!gather) return;
+    const int row = first + warp;
+    if (row >= q.rows || !flags[row]) return;
+    const bool mine = lane < warp && flags[first + lane] != 0;
+    const int at = s_before + __popc(__ballot_sync(0xFFFFFFFFu, mine));
+    if (lane == 0) q.row_map[at] = row;
+    const int vecs = q.K / 8;                                      // 16-byte vectors per row
+    auto copy = [&](uint4 *dst, const uint4 *src) {
+        dst += (size_t)at * vecs;
+        src += (size_t)row * vecs;
+#pragma unroll 8
+        for (int i = lane; i < vecs; i += 32) dst[i] = src[i];
+    };
+    copy(gathered, hidden);
+    if (KL) copy(gathered_d, hidden_d);
+}
 
 // One row's partial of one vocabulary tile into the global table.  Nothing else happens in this
 // kernel: rows are folded and sequences decided by lm_head_fold_kernel, launched behind it on the
 // same stream.  (Folding in here, by whichever warp stores a row's last tile, put every fold of the
 // launch on the one CTA that finishes last: all rows of a row block complete together, with the
 // last tile.  170 of 217 us on a 256-row, 143-tile problem were that CTA folding alone.)
-__device__ __forceinline__ void store_partial(const ddv::VerifyParams &p, const ddv::Partial &c, int row, int tile)
+__device__ __forceinline__ void store_partial(const ddv::VerifyParams &p, const ddv::Partial &c, int row, int tile, int n_tiles)
 {
-    ddv::Partial *dst = p.partials + ddv::checked(p, (long)row * p.nchunks + tile, (long)p.B * p.P * p.nchunks, ddv::kSitePartial);
+    ddv::Partial *dst = p.partials + ddv::checked(p, (long)row * n_tiles + tile, (long)p.B * p.P * n_tiles, ddv::kSitePartial);
     __stcg(reinterpret_cast<float4 *>(dst), make_float4(c.m_v, c.s_v, __int_as_float(c.idx), c.m_d));
     __stcg(reinterpret_cast<float4 *>(dst) + 1, make_float4(c.s_d, c.t, 0.f, 0.f));
 }
@@ -87,14 +200,14 @@ __device__ __forceinline__ void rows_done(const ddv::VerifyParams &p, int b, int
     ddv::decide_sequence(p, b, stage);
 }
 
-// Second launch of dd_lm_head_verify: one warp per row folds the row's tile partials (fp64, tile
+// Last launch of dd_lm_head_verify: one warp per row folds the row's tile partials (fp64, tile
 // order: the streaming kernel's fold) and stores score and argmax; one warp per sequence accounts
 // for the rows that are not flagged; the warp that accounts for a sequence's last row runs the
 // decision stage.  The partials were written by the previous kernel on the stream.
 constexpr int kFoldThreads = 128;
 constexpr int kFoldDecideKeys = 2048;      // keys of one sequence each warp can keep in shared memory
 template <bool KL>
-__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::VerifyParams p, int rows)
+__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::VerifyParams p, int rows, const LmPlan *plan)
 {
     __shared__ uint32_t s_keys[kFoldThreads / 32][kFoldDecideKeys];
     ddv::DecideStage stage;
@@ -105,8 +218,9 @@ __global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::V
         if (!p.flags[w]) return;
         float score;
         int argmax;
-        ddv::fold_partials<KL>(p.partials + ddv::checked_run(p, (long)w * p.nchunks, p.nchunks, (long)rows * p.nchunks, ddv::kSitePartial),
-                               p.nchunks, score, argmax);
+        const int n_tiles = plan->n_tiles;
+        ddv::fold_partials<KL>(p.partials + ddv::checked_run(p, (long)w * n_tiles, n_tiles, (long)rows * n_tiles, ddv::kSitePartial),
+                               n_tiles, score, argmax);
         if ((threadIdx.x & 31) == 0) {
             const size_t row_at = ddv::checked(p, w, (long)p.B * p.P, ddv::kSiteRow);
             __stcg(p.row_score + row_at, score);
@@ -122,33 +236,67 @@ __global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::V
     }
 }
 
+// The work items of a CTA, in order: every role walks the same way.  Items that follow each other share a
+// vocabulary tile (weights from L2).
+struct Walk {
+    int item, n_items, row_blocks, n_rows;
+    int tile, row0;
+    bool two;              // the item has more than 128 rows: both accumulators
+    int one;               // else: the accumulator it uses (such items take turns)
+    __device__ __forceinline__ Walk(const LmPlan &plan)
+    {
+        n_rows = plan.n_rows;
+        row_blocks = (n_rows + kRowsPerItem - 1) / kRowsPerItem;
+        n_items = plan.n_tiles * row_blocks;
+        item = blockIdx.x;
+        one = 1;
+        set();
+    }
+    __device__ __forceinline__ void set()
+    {
+        if (item >= n_items) return;
+        tile = item / row_blocks;
+        row0 = (item - tile * row_blocks) * kRowsPerItem;
+        two = n_rows - row0 > kTileRows;
+        if (!two) one ^= 1;
+    }
+    __device__ __forceinline__ bool valid() const { return item < n_items; }
+    __device__ __forceinline__ void next() { item += gridDim.x; set(); }
+    __device__ __forceinline__ bool uses(int acc) const { return two || one == acc; }
+};
+
 // Epilogue warps: every accumulator row becomes one partial.  Columns are visited in index order
 // with a strict comparison, so the index kept is the lowest index of the maximum.  KL (Eq. 4-5):
 // the drafter's accumulator is read beside the verifier's, and the row also keeps the drafter's
 // running maximum m_d, s_d = sum 2^(d*log2e - M_d) and t = sum 2^(d*log2e - M_d) * (d - v), both
 // rescaled whenever the maximum moves.
 template <bool KL>
-__device__ __forceinline__ void epilogue(const LmParams &q, const ddv::VerifyParams &p, uint32_t tmem,
-                                         uint32_t bar_acc_full, uint32_t bar_acc_empty,
-                                         volatile uint32_t *abort_flag, int n_items)
+__device__ __forceinline__ void epilogue(const LmParams &q, const LmPlan &plan, const ddv::VerifyParams &p, uint32_t tmem,
+                                         uint32_t bars_acc_full, uint32_t bars_acc_empty, volatile uint32_t *abort_flag)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int acc = warp >> 2;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;          // this warp's 32 tensor-memory lanes
     const uint32_t tacc = tmem + lane_off + (KL ? 256u + (uint32_t)acc * 128u : (uint32_t)acc * 256u);   // verifier
     const uint32_t dacc = tmem + lane_off + (uint32_t)acc * 128u;                                          // drafter (KL)
-    uint32_t n_done = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n_done) {
-        const int tile = item / q.row_blocks, rb = item - tile * q.row_blocks;
-        const int row = rb * kRowsPerItem + acc * 128 + (warp & 3) * 32 + lane, col0 = tile * q.N;
+    Walk walk(plan);
+    for (uint32_t n_done = 0; walk.valid(); walk.next()) {
+        if (!walk.uses(acc)) continue;
+        const int tile = walk.tile, col0 = tile * plan.N;
+        int row = walk.row0 + (walk.two ? acc * kTileRows : 0) + (warp & 3) * 32 + lane;
+        // the row of the caller's tensors, or -1: nothing to store
+        if (row >= plan.n_rows) row = -1;
+        else if (plan.gathered) row = q.row_map[row];
+        else if (!p.flags[row]) row = -1;
         bool arrived = false;
         for (uint32_t it = 0; it < (1u << 22); ++it) {
-            if (mbar_try_wait(bar_acc_full, n_done & 1)) { arrived = true; break; }
+            if (mbar_try_wait(bars_acc_full + 8u * acc, n_done & 1)) { arrived = true; break; }
             if (it > 64) {
                 __nanosleep(64);
                 if (*abort_flag) break;
             }
         }
+        ++n_done;
         if (!arrived) {
             if (lane == 0) {
                 *abort_flag = 1u;
@@ -160,7 +308,7 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const ddv::VerifyPar
         float m = -INFINITY, M = -INFINITY, s = 0.f;
         float m_d = -INFINITY, M_d = -INFINITY, s_d = 0.f, t = 0.f;
         int idx = 0x7FFFFFFF;
-        for (int cb = 0; cb < q.N / 32; ++cb) {
+        for (int cb = 0; cb < plan.N / 32; ++cb) {
             uint32_t r[32], rd[32];              // rd: the drafter's logits, KL only
             tmem_ld32(tacc + cb * 32, r);
             if constexpr (KL) tmem_ld32(dacc + cb * 32, rd);
@@ -204,15 +352,15 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const ddv::VerifyPar
                     }
             }
         }
-        // both accumulators may be overwritten once every epilogue warp has read its lanes
+        // the accumulator may be overwritten once its four epilogue warps have read their lanes
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_acc_empty);
+        if (lane == 0) mbar_arrive(bars_acc_empty + 8u * acc);
 
         ddv::Partial c;
         c.m_v = m; c.s_v = s; c.idx = idx;
         c.m_d = KL ? m_d : 0.f; c.s_d = s_d; c.t = t; c.pad0 = c.pad1 = 0.f;
-        if (row < q.rows && p.flags[row]) store_partial(p, c, row, tile);
+        if (row >= 0) store_partial(p, c, row, tile, plan.n_tiles);
     }
 }
 
@@ -222,31 +370,34 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const ddv::VerifyPar
 // accumulators are [0,N) and [256,256+N) (N <= 256).
 template <bool KL>
 __global__ void __launch_bounds__(kThreads, 1)
-lm_head_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
-               const __grid_constant__ CUtensorMap tm_hd, const __grid_constant__ CUtensorMap tm_wd,
-               const LmParams q, const ddv::VerifyParams p)
+lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const ddv::VerifyParams p)
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;     // swizzled tiles: 1024-byte aligned
     unsigned char *smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));
-    const uint32_t bars = smem_base + kStages * kStageBytes;
+    const uint32_t bars = smem_base + kRingBytes;
     auto bar_full = [&](int s) { return bars + 8u * s; };
-    auto bar_empty = [&](int s) { return bars + 8u * (kStages + s); };
-    const uint32_t bar_acc_full = bars + 8u * (2 * kStages), bar_acc_empty = bars + 8u * (2 * kStages + 1);
-    const uint32_t tmem_slot = bars + 8u * (2 * kStages + 2);
-    volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + kStages * kStageBytes + 8 * (2 * kStages + 2));
+    auto bar_empty = [&](int s) { return bars + 8u * (kMaxStages + s); };
+    const uint32_t bars_acc_full = bars + 8u * (2 * kMaxStages), bars_acc_empty = bars_acc_full + 16u;
+    const uint32_t tmem_slot = bars_acc_empty + 16u;
+    volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + (tmem_slot - smem_base));
     volatile uint32_t *abort_flag = tmem_slot_gen + 1;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n_items = q.n_tiles * q.row_blocks;
+    const LmPlan plan = *q.plan;
     const int k_steps = q.K / kBlockK;
+    // a stage: one or two tiles of hidden states (two unless no item has more than 128 rows), one of weights
+    const uint32_t a_bytes = plan.n_rows > kTileRows ? 2 * kATileBytes : kATileBytes;
+    const uint32_t b_bytes = (uint32_t)plan.N * kBlockK * 2;
+    const uint32_t stage_bytes = a_bytes + b_bytes;
+    const uint32_t stages = min((uint32_t)kMaxStages, kRingBytes / stage_bytes);
 
     if (tid == 0) {
-        prefetch_tmap(&tm_h); prefetch_tmap(&tm_w);
-        if (KL) { prefetch_tmap(&tm_hd); prefetch_tmap(&tm_wd); }
-        for (int s = 0; s < kStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        mbar_init(bar_acc_full, 1);
-        mbar_init(bar_acc_empty, kEpilogueWarps);
+        for (int s = 0; s < kMaxStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(bars_acc_full + 8u * a, 1);
+            mbar_init(bars_acc_empty + 8u * a, kEpilogueWarps / 2);
+        }
         fence_mbar_init();
         *abort_flag = 0u;
     }
@@ -274,58 +425,69 @@ lm_head_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__
 
     if (warp == kLoadWarp && lane == 0) {
         // ===================================================================== TMA producer
-        uint32_t step = 0;                                    // k-steps issued over all items
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            const int tile = item / q.row_blocks, rb = item - tile * q.row_blocks;
-            const int row0 = rb * kRowsPerItem, col0 = tile * q.N;
-            bool ok = true;
-            for (int ks2 = 0; ks2 < (KL ? 2 : 1) * k_steps; ++ks2, ++step) {
-                const int s = step % kStages;
-                const uint32_t use = step / kStages;
-                if (use > 0 && !wait(bar_empty(s), (use - 1) & 1)) { give_up(kErrLmEmpty); ok = false; break; }
-                const uint32_t dst = smem_base + s * kStageBytes;
+        const int width = (Widths<KL>::max_n - plan.N) / 32;
+        const CUtensorMap *h = plan.gathered ? &maps.h_gathered : &maps.h, *w = &maps.w[width];
+        const CUtensorMap *hd = plan.gathered ? &maps.hd_gathered : &maps.hd, *wd = &maps.wd[KL ? width : 0];
+        prefetch_tmap(h); prefetch_tmap(w);
+        if (KL) { prefetch_tmap(hd); prefetch_tmap(wd); }
+        uint32_t s = 0, round = 0;                            // stage, and how often the ring has been gone round
+        bool ok = true;
+        for (Walk walk(plan); walk.valid() && ok; walk.next()) {
+            const int col0 = walk.tile * plan.N;
+            const uint32_t bytes = (walk.two ? 2 * kATileBytes : kATileBytes) + b_bytes;
+            for (int ks2 = 0; ks2 < (KL ? 2 : 1) * k_steps; ++ks2) {
+                if (round > 0 && !wait(bar_empty(s), (round - 1) & 1)) { give_up(kErrLmEmpty); ok = false; break; }
+                const uint32_t dst = smem_base + s * stage_bytes;
                 const bool drafter = KL && ks2 < k_steps;                 // the drafter's pass comes first
                 const int ks = ks2 < k_steps ? ks2 : ks2 - k_steps;
-                const CUtensorMap *mh = drafter ? &tm_hd : &tm_h, *mw = drafter ? &tm_wd : &tm_w;
-                mbar_expect_tx(bar_full(s), (uint32_t)(2 * kATileBytes + q.N * kBlockK * 2));
-                tma_load_2d(dst, mh, bar_full(s), ks * kBlockK, row0);
-                tma_load_2d(dst + kATileBytes, mh, bar_full(s), ks * kBlockK, row0 + 128);
-                tma_load_2d(dst + 2 * kATileBytes, mw, bar_full(s), ks * kBlockK, col0);
+                const CUtensorMap *mh = drafter ? hd : h, *mw = drafter ? wd : w;
+                mbar_expect_tx(bar_full(s), bytes);
+                tma_load_2d(dst, mh, bar_full(s), ks * kBlockK, walk.row0);
+                if (walk.two) tma_load_2d(dst + kATileBytes, mh, bar_full(s), ks * kBlockK, walk.row0 + kTileRows);
+                tma_load_2d(dst + a_bytes, mw, bar_full(s), ks * kBlockK, col0);
+                if (++s == stages) { s = 0; ++round; }
             }
-            if (!ok) break;
         }
     } else if (warp == kMmaWarp && lane == 0) {
         // ===================================================================== MMA issuer
-        const uint32_t idesc = idesc_bf16(128, q.N, false);
-        uint32_t step = 0, n_done = 0;                        // k-steps consumed, items finished
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n_done) {
-            // the epilogue of the previous item has read both accumulators
-            if (n_done > 0 && !wait(bar_acc_empty, (n_done - 1) & 1)) { give_up(kErrLmAcc); break; }
+        const uint32_t idesc = idesc_bf16(128, plan.N, false);
+        uint32_t s = 0, round = 0;
+        uint32_t uses[2] = {0, 0};                            // items each accumulator has taken part in
+        bool ok = true;
+        for (Walk walk(plan); walk.valid() && ok; walk.next()) {
+            // the epilogue of the accumulators' previous item has read them
+            for (int a = 0; a < 2 && ok; ++a) {
+                if (!walk.uses(a)) continue;
+                if (uses[a] > 0 && !wait(bars_acc_empty + 8u * a, (uses[a] - 1) & 1)) { give_up(kErrLmAcc); ok = false; }
+                ++uses[a];
+            }
+            if (!ok) break;
             tc_fence_after();
-            bool ok = true;
-            for (int ks2 = 0; ks2 < (KL ? 2 : 1) * k_steps; ++ks2, ++step) {
-                const int s = step % kStages;
-                if (!wait(bar_full(s), (step / kStages) & 1)) { give_up(kErrLmFull); ok = false; break; }
+            for (int ks2 = 0; ks2 < (KL ? 2 : 1) * k_steps; ++ks2) {
+                if (!wait(bar_full(s), round & 1)) { give_up(kErrLmFull); ok = false; break; }
                 tc_fence_after();
                 const int ks = ks2 < k_steps ? ks2 : ks2 - k_steps;
                 // accumulator columns of this pass: see the layout above
-                const uint32_t acc0 = tmem + ((KL && ks2 >= k_steps) ? 256u : 0u), acc1 = acc0 + (KL ? 128u : 256u);
-                const uint32_t base = smem_base + s * kStageBytes;
+                const uint32_t half = (KL && ks2 >= k_steps) ? 256u : 0u, other = KL ? 128u : 256u;
+                const uint32_t acc0 = tmem + half + (!walk.two && walk.one ? other : 0u), acc1 = tmem + half + other;
+                const uint32_t base = smem_base + s * stage_bytes;
                 const uint64_t a0 = smem_desc_sw128(base, 16, 1024), a1 = smem_desc_sw128(base + kATileBytes, 16, 1024);
-                const uint64_t b = smem_desc_sw128(base + 2 * kATileBytes, 16, 1024);
+                const uint64_t b = smem_desc_sw128(base + a_bytes, 16, 1024);
 #pragma unroll
                 for (int kk = 0; kk < kBlockK / 16; ++kk) {
                     const uint32_t off = (uint32_t)(kk * 32) >> 4;            // 16 bf16 = 32 bytes per MMA
                     mma_ss(acc0, a0 + off, b + off, idesc, (ks > 0 || kk > 0));
-                    mma_ss(acc1, a1 + off, b + off, idesc, (ks > 0 || kk > 0));
+                    if (walk.two) mma_ss(acc1, a1 + off, b + off, idesc, (ks > 0 || kk > 0));
                 }
                 mma_commit(bar_empty(s));                                      // the stage is free once these have run
+                if (++s == stages) { s = 0; ++round; }
             }
             if (!ok) break;
-            mma_commit(bar_acc_full);
+            for (int a = 0; a < 2; ++a)
+                if (walk.uses(a)) mma_commit(bars_acc_full + 8u * a);
         }
     } else if (warp < kEpilogueWarps) {
-        epilogue<KL>(q, p, tmem, bar_acc_full, bar_acc_empty, abort_flag, n_items);
+        epilogue<KL>(q, plan, p, tmem, bars_acc_full, bars_acc_empty, abort_flag);
     }
 
     __syncwarp();

@@ -460,22 +460,48 @@ int make_matrix_tmap(CUtensorMap *m, const void *base, long n_rows, int K, int b
     return DD_OK;
 }
 
-// Vocabulary entries per work item: the multiple of 32 (at most `max_n`, at least half of it) for
-// which the slowest CTA of `ctas` finishes first.  A work item of n entries takes about
-// (fixed + n) units of time: the hidden-state tiles it loads and the MMAs' shared-memory reads of
-// them do not shrink with n.  Measured at K = 4096 (time per item against n, tile widths forced):
-// fixed = 140 for one product per item, 157 for the KL mode's two.  Counting n alone picked tiles
-// of 128 entries at 4096 rows, 25 % slower than 256.
-int pick_tile_n(int V, long row_blocks, int ctas, int max_n, int fixed)
+template <bool KL>
+int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void *dw, const void *vh, const void *vw,
+                   char *gathered, size_t gathered_bytes, int ctas, cudaStream_t stream)
 {
-    int best = max_n;
-    long best_cost = -1;
-    for (int n = max_n; n >= max_n / 2; n -= 32) {
-        const long items = ((V + n - 1) / n) * row_blocks;
-        const long cost = ((items + ctas - 1) / ctas) * (fixed + n);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = n; }
+    using namespace ddlm;
+    int rc, dev = 0;
+    DD_CUDA_TRY(cudaGetDevice(&dev));
+    {
+        static bool attr_done[64] = {};
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (!attr_done[dev]) {
+            DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+            attr_done[dev] = true;
+        }
     }
-    return best;
+    LmMaps<KL> m;
+    if ((rc = make_matrix_tmap(&m.h, vh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
+    if ((rc = make_matrix_tmap(&m.h_gathered, gathered, q.rows, q.K, kTileRows)) != DD_OK) return rc;
+    m.hd = m.h; m.hd_gathered = m.h_gathered;          // not read outside the KL mode
+    if (KL) {
+        if ((rc = make_matrix_tmap(&m.hd, dh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
+        if ((rc = make_matrix_tmap(&m.hd_gathered, gathered + (q.can_gather ? gathered_bytes : 0), q.rows, q.K, kTileRows)) != DD_OK) return rc;
+    }
+    for (int i = 0; i < Widths<KL>::count; ++i) {
+        if ((rc = make_matrix_tmap(&m.w[i], vw, q.V, q.K, Widths<KL>::max_n - 32 * i)) != DD_OK) return rc;
+        if (KL && (rc = make_matrix_tmap(&m.wd[i], dw, q.V, q.K, Widths<KL>::max_n - 32 * i)) != DD_OK) return rc;
+    }
+    // One CTA per SM, fewer if even the narrowest tiles of all rows do not make that many items.
+    const long items = (long)((q.V + Widths<KL>::max_n / 2 - 1) / (Widths<KL>::max_n / 2)) * ((q.rows + kRowsPerItem - 1) / kRowsPerItem);
+    const unsigned grid = (unsigned)(items < ctas ? items : ctas);
+    lm_head_rows_kernel<KL><<<(unsigned)((q.rows + kRowsPerBlock - 1) / kRowsPerBlock), kRowsThreads, 0, stream>>>(
+        q, p.flags, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
+        static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
+    DD_CUDA_TRY(cudaGetLastError());
+    lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
+    DD_CUDA_TRY(cudaGetLastError());
+    // one warp per row, then one per sequence
+    const unsigned fold_grid = (unsigned)(((long)q.rows + p.B + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
+    lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q.rows, q.plan);
+    DD_CUDA_TRY(cudaGetLastError());
+    dd::count_launch(3);
+    return DD_OK;
 }
 
 }  // namespace
@@ -503,16 +529,17 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     int cap = g_max_ctas.load(std::memory_order_relaxed);
     const int ctas = cap > 0 && cap < sms ? cap : sms;
 
-    ddlm::LmParams q;
-    q.rows = (int)rows; q.K = K; q.V = V;
-    q.row_blocks = (int)((rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem);
-    q.N = kl ? pick_tile_n(V, q.row_blocks, sms, ddlm::kMaxN / 2, 157) : pick_tile_n(V, q.row_blocks, sms, ddlm::kMaxN, 140);
-    q.n_tiles = (V + q.N - 1) / q.N;
-    if (rows * q.n_tiles >= (1L << 31) - (1L << 24)) return DD_ERR_UNSUPPORTED;
+    // the narrowest tiles that the device may choose bound the partials
+    const int max_n = kl ? ddlm::Widths<true>::max_n : ddlm::Widths<false>::max_n;
+    int min_n = max_n / 2;
+    while (rows * ((V + min_n - 1) / min_n) >= (1L << 31) - (1L << 24)) {
+        if (min_n == max_n) return DD_ERR_UNSUPPORTED;
+        min_n += 32;
+    }
 
     VerifyParams p;
-    p.nchunks = q.n_tiles;
-    p.chunk = q.N;
+    p.nchunks = (V + min_n - 1) / min_n;
+    p.chunk = min_n;
     dd::DeviceCtx *ctx = dd::current_ctx();
     if (!ctx) return DD_ERR_CUDA;
     if ((rc = dd::ensure_mirror(ctx)) != DD_OK) return rc;
@@ -532,45 +559,22 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     p.partials = (Partial *)w;
     fill_params(p, nullptr, nullptr, tokens, mask_flags, mode, tau, k, seed, out_tokens, out_mask, out_score, B, P, V);
 
-    CUtensorMap tm_h, tm_w, tm_hd, tm_wd;
-    if ((rc = make_matrix_tmap(&tm_h, verifier_hidden, rows, K, 128)) != DD_OK) return rc;
-    if ((rc = make_matrix_tmap(&tm_w, verifier_weight, V, K, q.N)) != DD_OK) return rc;
-    tm_hd = tm_h; tm_wd = tm_w;                    // not read outside the KL mode
-    if (kl) {
-        if ((rc = make_matrix_tmap(&tm_hd, drafter_hidden, rows, K, 128)) != DD_OK) return rc;
-        if ((rc = make_matrix_tmap(&tm_wd, drafter_weight, V, K, q.N)) != DD_OK) return rc;
-    }
-
-    int dev = 0;
-    DD_CUDA_TRY(cudaGetDevice(&dev));
-    {
-        static bool attr_done[64] = {};
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (!attr_done[dev]) {
-            DD_CUDA_TRY(cudaFuncSetAttribute(ddlm::lm_head_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             ddlm::kSmemBytes));
-            DD_CUDA_TRY(cudaFuncSetAttribute(ddlm::lm_head_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             ddlm::kSmemBytes));
-            attr_done[dev] = true;
-        }
-    }
-    const long items = (long)q.n_tiles * q.row_blocks;
-    const unsigned grid = (unsigned)(items < ctas ? items : ctas);
-    if (kl)
-        ddlm::lm_head_kernel<true><<<grid, ddlm::kThreads, ddlm::kSmemBytes, (cudaStream_t)stream>>>(tm_h, tm_w, tm_hd, tm_wd, q, p);
-    else
-        ddlm::lm_head_kernel<false><<<grid, ddlm::kThreads, ddlm::kSmemBytes, (cudaStream_t)stream>>>(tm_h, tm_w, tm_hd, tm_wd, q, p);
-    DD_CUDA_TRY(cudaGetLastError());
-    dd::count_launch();
-    // one warp per row, then one per sequence
-    const unsigned fold_grid = (unsigned)((rows + B + ddlm::kFoldThreads / 32 - 1) / (ddlm::kFoldThreads / 32));
-    if (kl)
-        ddlm::lm_head_fold_kernel<true><<<fold_grid, ddlm::kFoldThreads, 0, (cudaStream_t)stream>>>(p, (int)rows);
-    else
-        ddlm::lm_head_fold_kernel<false><<<fold_grid, ddlm::kFoldThreads, 0, (cudaStream_t)stream>>>(p, (int)rows);
-    DD_CUDA_TRY(cudaGetLastError());
-    dd::count_launch();
-    return DD_OK;
+    // scratch of this entry point: the plan, the list of flagged rows, their hidden states
+    const size_t map_bytes = ((size_t)rows * 4 + 255) & ~size_t(255), gathered_bytes = ((size_t)rows * K * 2 + 255) & ~size_t(255);
+    ddlm::LmParams q;
+    q.can_gather = dd::ensure_bytes(&ctx->head_ws, &ctx->head_ws_bytes, 256 + map_bytes + (kl ? 2 : 1) * gathered_bytes) == DD_OK;
+    // no room for a copy of the hidden states: every row is multiplied
+    if (!q.can_gather && (rc = dd::ensure_bytes(&ctx->head_ws, &ctx->head_ws_bytes, 256 + map_bytes)) != DD_OK) return rc;
+    q.rows = (int)rows; q.K = K; q.V = V;
+    q.min_n = min_n;
+    q.ctas = sms;
+    q.plan = (ddlm::LmPlan *)ctx->head_ws;
+    q.row_map = (int *)((char *)ctx->head_ws + 256);
+    char *gathered = (char *)ctx->head_ws + (q.can_gather ? 256 + map_bytes : 0);
+    return kl ? launch_lm_head<true>(q, p, drafter_hidden, drafter_weight, verifier_hidden, verifier_weight, gathered,
+                                     gathered_bytes, ctas, (cudaStream_t)stream)
+              : launch_lm_head<false>(q, p, nullptr, nullptr, verifier_hidden, verifier_weight, gathered, 0, ctas,
+                                      (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------

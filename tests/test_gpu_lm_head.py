@@ -143,6 +143,31 @@ def test_llada_shaped_full_size_kl(dd, oracle_mod):
     assert 20 <= rejected <= 120
 
 
+@pytest.mark.parametrize("n", [0, 1, 127, 128, 129, 256, 257, 384, 385])
+def test_flagged_rows_at_the_edges_of_tiles(dd, oracle_mod, n):
+    """Flagged rows gathered into fewer 128-row tiles (n <= 384 of 400 rows), or left where they are
+    (385); the last item of a vocabulary tile with one or two tiles of rows, the first one with none.
+    Every unflagged hidden state is NaN: none may reach a result."""
+    rng = np.random.default_rng(n)
+    dh, dw, vh, vw, tokens, flags = synth.lm_head_pair_inputs(2, 200, 128, 1500, "all", 0.2, seed=77)
+    flags[:] = 0
+    flags.reshape(-1)[rng.choice(400, size=n, replace=False)] = 1
+    clean_v, clean_d = vh.copy(), dh.copy()
+    vh[flags == 0] = dh[flags == 0] = 0x7FC0
+    for mode, drafter in ((CONF, False), (KL, True)):
+        import torch
+        ref = oracle_mod.lm_head_verify(clean_d if drafter else None, dw if drafter else None, clean_v, vw, tokens, flags, mode, 0.05, 5, 1)
+        on = lambda x: to_torch_bf16(x, "cuda")
+        got = dd.lm_head_verify(on(dh) if drafter else None, on(dw) if drafter else None, on(vh), on(vw),
+                                torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda(), mode, 0.05, 5, 1)
+        torch.cuda.synchronize()
+        assert dd.verify_status() == 0
+        ot, om, osc = (x.cpu().numpy() for x in got)
+        close = (ref["top2_gap"] <= TOP2_GAP) & flags.astype(bool) & (om == 0) & (ref["out_mask"] == 0)
+        ref = dict(ref, out_tokens=np.where(close, ot, ref["out_tokens"]))
+        check_verify(ot, om, osc, ref, flags, tokens, **(dict(score_abs=KL_SCORE_ABS) if drafter else {}))
+
+
 def test_results_do_not_depend_on_the_grid(dd, oracle_mod):
     import torch
     hidden, weight, tokens, flags = synth.lm_head_inputs(2, 150, 128, 3000, 97, seed=12)
