@@ -1,7 +1,8 @@
 // dd_bidir_attention: full-sequence bidirectional attention (Section 2.2; Eq. 3
 // evaluated over the whole key range) for sm_100a, and dd_block_attention: the same
 // equation for a block of Nq queries against Nkv (cached) keys, with a per-sequence
-// number of valid keys and either memory layout.  One kernel serves both.
+// number of valid keys and either memory layout.  One kernel serves both; two persistent forms of
+// it take many short items (see attention_impl).
 //
 // One CTA owns two tiles of 128 query rows of one (batch, head) and walks over
 // the keys in tiles of 128.  The CTA is warp-specialised:
@@ -21,11 +22,21 @@
 // fp32's relative precision; the step only has to leave fp32 its range); only then
 // is O rescaled in tensor memory.  O is normalised by the row sum at the end and
 // rounded to bf16 once.
+//
+// What bounds it.  The chain of one query tile: softmax (some 2000 cycles a key tile) -> P V (512) -> next S
+// (512) -> softmax, plus the hand-overs; the other query tile's chain fills the tensor core meanwhile.  So
+// the weights are handed over in two parts, P V starting on the first three quarters of the keys while the
+// last quarter is computed, and the issuing thread runs under elect_one: N = 8192 1076 -> 920 us, 32 heads
+// of 1024 tokens 23.4 -> 20.4.  Under this load the SM clock sits at 1.6-1.75 GHz (power), which is the
+// other bound.  Built and not faster: scores in two halves of 64 keys with barriers of their own (S products
+// of 128 x 64 are bound by shared memory), two threads per row (sixteen softmax warps), the scores read
+// twice in rolled loops instead of kept in 128 registers.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "dd_common.cuh"
 #include "dd_ptx.cuh"
@@ -43,9 +54,9 @@ constexpr int kSoftmaxWarps = 8;
 constexpr int kLoadWarp = 8, kMmaWarp = 9;
 constexpr uint32_t kTmemCols = 512; // S_0 [0,128)  S_1 [128,256)  O_0 [256,256+D)  O_1 [256+D,256+2D)
 // log2 of the largest P tolerated before the reference point moves.  A move costs the row's warp a
-// wait for the previous P V product, a pass over the accumulator in tensor memory and a second
-// weighting of the tile: with a step of 8, rows whose scores are peaked (a planted low-rank
-// component; trained heads) moved often enough to cost 25-40 % of the throughput.  With 24 the sum
+// pass over the accumulator in tensor memory in front of the tile's weights: with a step of 8, rows whose scores are peaked (a planted low-rank
+// component; trained heads) moved often enough to cost 25-40 % of the throughput (when a move meant a
+// second weighting as well).  With 24 the sum
 // of a row's weights stays below N * 2^24 and fp32 holds O for |v| * N < 2^100.
 constexpr float kRescaleStep = 24.f;
 
@@ -60,6 +71,7 @@ struct AttnParams {
     float scale_log2;          // scale * log2(e)
     unsigned int *status;      // health word of the attention kernel on this device
     unsigned int *mirror;      // its copy in mapped host memory (written only when a wait expires)
+    void *out;                 // where attention_persistent_kernel stores its result (the others through a tensor map)
 };
 
 template <int D>
@@ -68,8 +80,8 @@ struct Smem {
     static constexpr int kQ = 0;                                   // two query tiles
     static constexpr int kRing = kQTiles * kTileBytes;             // kStages K/V tiles
     static constexpr int kBars = kRing + kStages * kTileBytes;
-    // barriers (8 bytes each): q_full[2], kv_full[kStages], kv_empty[kStages], s_full[2], p_full[2], o_full[2]
-    static constexpr int kNumBars = 2 + 2 * kStages + 6;
+    // barriers (8 bytes each): q_full[2], kv_full[kStages], kv_empty[kStages], s_full[2], p_full[2], o_full[2], p_early[2]
+    static constexpr int kNumBars = 2 + 2 * kStages + 8;
     static constexpr int kTmemSlot = kBars + 8 * kNumBars;
     static constexpr int kTotal = kTmemSlot + 16;
     // every tile starts on the 1024-byte boundary the 128-byte swizzle needs, the barriers on 8 bytes,
@@ -87,75 +99,94 @@ __device__ __forceinline__ void report(const AttnParams &p, unsigned code)
     }
 }
 
-// One key tile of the online softmax for one query row; s[] holds the raw scores.
-// Row maximum of the raw scores (keys past the sequence end excluded).
+// One pair of exponentials in this many is computed on the FMA pipe (0: none).  At D = 64 a key tile costs
+// half the tensor time and the same number of exponentials, and the special-function unit (16 per clock)
+// is what both query tiles of a CTA compete for: one in eight gained 8 %, one in four 12 % (3 x 24 heads of
+// 1357 tokens 72.9 -> 66.2 us, 32 heads of 4096 239 -> 208).  At D = 128 the tensor core, and the
+// chip's power, are the bound, and the extra instructions cost 5-10 %.
+template <int D> constexpr int kPolyOneIn = D == 64 ? 4 : 0;
+
+// 2^x of two values on the FMA pipe: x = n + f with n the nearest integer (read off the low bits of
+// x + 1.5 * 2^23), 2^f on [-1/2, 1/2] as a polynomial of degree five (relative error 1.5e-7, fitted
+// by weighted least squares; ex2.approx has 2^-22 = 2.4e-7), n added to the exponent.  Below 2^-125
+// the result is 2^-125 instead of zero.
+__device__ __forceinline__ float2 ex2_poly(float2 x)
+{
+    auto c = [](float v) { return make_float2(v, v); };
+    x.x = max_nan(x.x, -125.f);      // a NaN stays one (and its row becomes NaN, whichever pair it falls into)
+    x.y = max_nan(x.y, -125.f);
+    const float2 t = __fadd2_rn(x, c(12582912.f));
+    const float2 f = __ffma2_rn(__fadd2_rn(t, c(-12582912.f)), c(-1.f), x);
+    float2 y = __ffma2_rn(f, c(0.001327647129073739f), c(0.009675541892647743f));
+    y = __ffma2_rn(y, f, c(0.05550713092088699f));
+    y = __ffma2_rn(y, f, c(0.24022120237350464f));
+    y = __ffma2_rn(y, f, c(0.6931469440460205f));
+    y = __ffma2_rn(y, f, c(1.0000001192092896f));
+    return make_float2(__int_as_float(__float_as_int(y.x) + (__float_as_int(t.x) << 23)),
+                       __int_as_float(__float_as_int(y.y) + (__float_as_int(t.y) << 23)));
+}
+
+// Row maximum of the raw scores of one key tile (keys past the sequence end excluded).
 template <bool kMasked>
 __device__ __forceinline__ float row_max(const float (&s)[kBlockN], int valid)
 {
-    float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int i = 0; i < kBlockN; i += 4) {
-        if (!kMasked || i + 0 < valid) m0 = fmaxf(m0, s[i + 0]);
-        if (!kMasked || i + 1 < valid) m1 = fmaxf(m1, s[i + 1]);
-        if (!kMasked || i + 2 < valid) m2 = fmaxf(m2, s[i + 2]);
-        if (!kMasked || i + 3 < valid) m3 = fmaxf(m3, s[i + 3]);
-    }
-    return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+    for (int i = 0; i < kBlockN; i += 8)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = i + 2 * u;
+            if (!kMasked) {
+                m[u] = max3(m[u], s[e], s[e + 1]);
+            } else {
+                if (e < valid) m[u] = fmaxf(m[u], s[e]);
+                if (e + 1 < valid) m[u] = fmaxf(m[u], s[e + 1]);
+            }
+        }
+    return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
 }
 
-// Weights P = 2^(s*c - m_ref) of the tile as packed bf16 into tensor memory, 32 keys (16
-// columns) at a time; returns the sum of the weights as rounded, and through mx the row
-// maximum of the raw scores seen on the way (so the caller can tell afterwards whether
-// m_ref was still a good reference point).  Two values per instruction where the
-// hardware has a packed form.
-template <bool kMasked>
-__device__ __forceinline__ float weights_to_tmem(const float (&s)[kBlockN], int valid, float c, float m_ref,
-                                                 uint32_t tmem_p, float &mx)
+// Weights P = 2^(s*c - m_ref) of 32 keys (from key q * 32 of the tile) as packed bf16 into tensor memory (16
+// columns); adds the weights as rounded to sum_a + sum_b, so that O / l is an exact convex combination.  Two
+// values per instruction where the hardware has a packed form; one pair in kPoly (0: none) goes to the
+// FMA pipe.
+template <bool kMasked, int kPoly>
+__device__ __forceinline__ void weights_to_tmem(const float (&s)[kBlockN], int q, int valid, float c, float m_ref,
+                                                uint32_t tmem_p, float2 &sum_a, float2 &sum_b)
 {
     const float2 c2 = make_float2(c, c), nm2 = make_float2(-m_ref, -m_ref);
-    float2 sum2 = make_float2(0.f, 0.f);
-    float m0 = -INFINITY, m1 = -INFINITY;
+    uint32_t pk[16];
 #pragma unroll
-    for (int q = 0; q < kBlockN / 32; ++q) {
-        uint32_t pk[16];
-#pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-            const int e = q * 32 + i;
-            const float2 a = __ffma2_rn(make_float2(s[e], s[e + 1]), c2, nm2);
-            float p0 = ex2(a.x), p1 = ex2(a.y);
-            if (kMasked) {
-                // keys past the end of the sequence get weight zero (a select, not -inf arithmetic: scale may be 0)
-                p0 = e < valid ? p0 : 0.f;
-                p1 = e + 1 < valid ? p1 : 0.f;
-                if (e < valid) m0 = fmaxf(m0, s[e]);
-                if (e + 1 < valid) m1 = fmaxf(m1, s[e + 1]);
-            } else {
-                m0 = fmaxf(m0, s[e]);
-                m1 = fmaxf(m1, s[e + 1]);
-            }
-            __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);
-            const uint32_t w = *reinterpret_cast<uint32_t *>(&b);
-            pk[i / 2] = w;
-            // the row sum takes the weights as rounded, so that O / l is an exact convex combination
-            sum2 = __fadd2_rn(sum2, make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)));
+    for (int i = 0; i < 32; i += 2) {
+        const int e = q * 32 + i;
+        const float2 a = __ffma2_rn(make_float2(s[e], s[e + 1]), c2, nm2);
+        float2 p;
+        if (!kMasked && kPoly > 0 && (i / 2) % (kPoly > 0 ? kPoly : 1) == kPoly - 1) p = ex2_poly(a);
+        else p = make_float2(ex2(a.x), ex2(a.y));
+        if (kMasked) {
+            // keys past the end of the sequence get weight zero (a select, not -inf arithmetic: scale may be 0)
+            p.x = e < valid ? p.x : 0.f;
+            p.y = e + 1 < valid ? p.y : 0.f;
         }
-        tmem_st16(tmem_p + q * 16, pk);
+        __nv_bfloat162 b = __floats2bfloat162_rn(p.x, p.y);
+        const uint32_t w = *reinterpret_cast<uint32_t *>(&b);
+        pk[i / 2] = w;
+        float2 &sum = (i & 2) ? sum_a : sum_b;
+        sum = __fadd2_rn(sum, make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)));
     }
-    mx = fmaxf(m0, m1);
-    return sum2.x + sum2.y;
+    tmem_st16(tmem_p + q * 16, pk);
 }
 
-// One key tile of one query row, shared by both attention kernels: reads the row's 128 scores
-// from tensor memory (the S product has completed), weights them against the reference point the
-// row inherits (the first tile of a row takes its own maximum) and writes P over S.  Only a row
-// whose maximum turns out to have grown past the reference point by more than the allowed step
-// moves it, rescales O in tensor memory (which holds the sum over the earlier tiles once the
-// barrier o_full_bar has completed the phase o_parity) and weights the tile again.  Returns 0, or
-// the error code of the wait that expired.  The caller hands P over (wait for the stores, fence,
-// arrive).
-template <int D>
-__device__ __forceinline__ unsigned softmax_tile(uint32_t tS, uint32_t tO, uint32_t o_full_bar, uint32_t o_parity,
-                                                 bool first, int valid, float c, float &m_ref, float &l_run)
+// One key tile of one query row, shared by both attention kernels: reads the row's 128 scores from tensor
+// memory (the S product has completed), moves the row's reference point if the tile's maximum outgrows
+// it by more than the allowed step (the first tile sets it), and writes the weights over S.  They are handed
+// to the issuing thread in two parts: `early` after three quarters of the keys, the rest by the caller
+// (each time: wait for the stores, fence, arrive), so that P V runs while the last quarter is computed.  A
+// row that moves rescales O in tensor memory.  O then holds the sum over the earlier tiles: their P V
+// products were issued before this S product by the same thread, so they had completed when S arrived.
+template <int D, typename Early>
+__device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, bool first, int valid, float c, float &m_ref,
+                                             float &l_run, Early early)
 {
     float s[kBlockN];
 #pragma unroll
@@ -163,33 +194,38 @@ __device__ __forceinline__ unsigned softmax_tile(uint32_t tS, uint32_t tO, uint3
         tmem_ld32(tS + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[cb * 32]));
     tmem_wait_ld();
     const bool masked = valid < kBlockN;
-    if (first) m_ref = (masked ? row_max<true>(s, valid) : row_max<false>(s, valid)) * c;
-    float mx;
-    float sum = masked ? weights_to_tmem<true>(s, valid, c, m_ref, tS, mx)
-                       : weights_to_tmem<false>(s, valid, c, m_ref, tS, mx);
-    const bool move = mx * c > m_ref + kRescaleStep;
-    if (__any_sync(0xffffffffu, move)) {
-        const float m_new = move ? mx * c : m_ref;
+    const float mx = (masked ? row_max<true>(s, valid) : row_max<false>(s, valid)) * c;
+    if (first) {
+        m_ref = mx;
+    } else if (__any_sync(0xffffffffu, mx > m_ref + kRescaleStep)) {
+        const float m_new = mx > m_ref + kRescaleStep ? mx : m_ref;
         const float alpha = ex2(m_ref - m_new);       // 1 where the row does not move
         m_ref = m_new;
         l_run *= alpha;
-        if (!mbar_wait(o_full_bar, o_parity)) return kErrWaitO;
-        tc_fence_after();
 #pragma unroll
         for (int cb = 0; cb < D / 32; ++cb) {
             uint32_t r[32];
             tmem_ld32(tO + cb * 32, r);
-            tmem_wait_ld();
+            tmem_wait_ld(r);
 #pragma unroll
             for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
             tmem_st32(tO + cb * 32, r);
         }
-        tmem_wait_st();                               // the first weights are overwritten next
-        sum = masked ? weights_to_tmem<true>(s, valid, c, m_ref, tS, mx)
-                     : weights_to_tmem<false>(s, valid, c, m_ref, tS, mx);
     }
-    l_run += sum;
-    return 0;
+    float2 sum_a = make_float2(0.f, 0.f), sum_b = sum_a;
+    auto weights = [&](auto is_masked, auto poly) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (q == 3) early();
+            weights_to_tmem<decltype(is_masked)::value, decltype(poly)::value>(s, q, valid, c, m_ref, tS, sum_a, sum_b);
+        }
+    };
+    // One branch for the whole tile and not one per 32 keys: every basic block ends with its exponentials
+    // drained (N = 8192: 962 -> 920 us).
+    if (masked) weights(std::true_type(), std::integral_constant<int, 0>());
+    else weights(std::false_type(), std::integral_constant<int, kPolyOneIn<D>>());
+    sum_a = __fadd2_rn(sum_a, sum_b);
+    l_run += sum_a.x + sum_a.y;
 }
 
 // 32 columns of one output row, scaled, rounded to bf16 and written to the staging tile in the
@@ -233,10 +269,11 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     auto bar_s_full = [&](int g) { return bars + 8u * (2 + 2 * kStages + g); };
     auto bar_p_full = [&](int g) { return bars + 8u * (4 + 2 * kStages + g); };
     auto bar_o_full = [&](int g) { return bars + 8u * (6 + 2 * kStages + g); };
+    auto bar_p_early = [&](int g) { return bars + 8u * (8 + 2 * kStages + g); };
     const uint32_t tmem_slot = smem_base + Smem<D>::kTmemSlot;
     volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + Smem<D>::kTmemSlot);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int bh = blockIdx.x / p.m_blocks;
     const int mb = blockIdx.x - bh * p.m_blocks;
     const int row0 = mb * (kQTiles * kBlockM);
@@ -265,9 +302,8 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // zeros) before the CTA's first barrier: they travel while tensor memory is allocated and the
     // other barriers are set up (cfg1: 22.9 -> 22.0 us).  Nothing else in the CTA touches those
     // buffers or barriers before the __syncthreads below.
-    const bool early = warp == kLoadWarp && lane == 0 && (!kBlock || nkv > 0);
-    bool early_sent = false;
-    if (warp == kLoadWarp && lane == 0) {
+    const bool early = !kBlock || nkv > 0;
+    if (warp == kLoadWarp && elect_one()) {
         prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
         mbar_init(bar_q(0), 1); mbar_init(bar_q(1), 1);
         for (int s = 0; s < kStages; ++s) mbar_init(bar_kv_full(s), 1);
@@ -281,7 +317,6 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             mbar_expect_tx(bar_kv_full(0), kTileBytes);
 #pragma unroll
             for (int cx = 0; cx < kBoxes; ++cx) load_box(sRing + cx * kBoxBytes, &tm_k, bar_kv_full(0), cx * 64, 0);
-            early_sent = true;
         }
     }
     if (tid == 0) {
@@ -290,6 +325,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         for (int g = 0; g < kQTiles; ++g) {
             mbar_init(bar_s_full(g), 1);
             mbar_init(bar_p_full(g), kBlockM);
+            mbar_init(bar_p_early(g), kBlockM);
             mbar_init(bar_o_full(g), 1);
         }
         fence_mbar_init();
@@ -300,7 +336,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot_gen;
+    const uint32_t tmem = warp_uniform(*tmem_slot_gen);
     const bool healthy = tmem_slot_gen[1] == 0;
 
     if (!healthy) {
@@ -326,9 +362,12 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 tc_fence_after();
                 const int valid = keys - j * kBlockN;      // keys of this tile that exist
                 const bool masked = valid < kBlockN;
-                // O_g holds the sum over tiles < j once the previous P V has completed
-                err = softmax_tile<D>(tS, tO, bar_o_full(g), (uint32_t)(i - 1) & 1, i == 0, valid, c, m_ref, l_run);
-                if (err) break;
+                softmax_tile<D>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
+                    if (kBlock && masked) return;          // not before the value rows below are clear
+                    tmem_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(bar_p_early(g));
+                });
                 if (kBlock && masked) {
                     // Keys past the end of the sequence have weight zero, but 0 x NaN is NaN in the
                     // product P V, and padding may hold any bit pattern: clear their value rows in
@@ -350,9 +389,10 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 }
                 tmem_wait_st();
                 tc_fence_before();
+                if (kBlock && masked) mbar_arrive(bar_p_early(g));
                 mbar_arrive(bar_p_full(g));
             }
-            if (err == 0 && (!kBlock || nkv > 0) && !mbar_wait(bar_o_full(g), (my_tiles - 1) & 1)) err = kErrWaitO;
+            if (err == 0 && (!kBlock || nkv > 0) && !mbar_wait(bar_o_full(g), 0)) err = kErrWaitO;
             // ---- split keys: group 1 hands its reference point and row sum to group 0 (through its
             // own Q buffer, which no MMA reads any more) and is done; group 0 adds group 1's
             // accumulator, read from tensor memory, to its own.  Every thread of both groups takes
@@ -368,7 +408,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 } else {
                     named_bar_sync(3, 2 * kBlockM);
                     const float2 other = hand_over[r];
-                    if (err == 0 && !mbar_wait(bar_o_full(1), ((nkv / 2) - 1) & 1)) err = kErrWaitO;
+                    if (err == 0 && !mbar_wait(bar_o_full(1), 0)) err = kErrWaitO;
                     const float m_all = fmaxf(m_ref, other.x);
                     scale_own = ex2(m_ref - m_all);
                     scale_other = ex2(other.x - m_all);
@@ -431,7 +471,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         }
     } else {
         reg_dec<72>();
-        if (warp == kLoadWarp && lane == 0) {
+        if (warp == kLoadWarp && elect_one()) {
             // =============================================================== TMA producer
             // what the first MMA needs comes first: Q tile 0, K tile 0, then Q tile 1
             // buffer g takes query tile g, or, with split keys, a second copy of tile 0
@@ -442,9 +482,8 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                     load_box(sQ + g * kTileBytes + cx * kBoxBytes, &tm_q, bar_q(g), cx * 64,
                              row0 + (split ? 0 : g * kBlockM));
             };
-            if (!early_sent && (!kBlock || nkv > 0)) load_q(0);      // without keys the Q buffers only stage the zero output
             // ring items: 2j = K tile j, 2j+1 = V tile j
-            for (int item = early_sent ? 1 : 0; item < 2 * nkv; ++item) {
+            for (int item = 1; item < 2 * nkv; ++item) {
                 if (item == 1 && groups > 1) load_q(1);
                 const int slot = item % kStages, use = item / kStages;
                 if (use > 0 && !mbar_wait(bar_kv_empty(slot), (use - 1) & 1)) { report(p, kErrWaitSlot); break; }
@@ -455,7 +494,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 for (int cx = 0; cx < kBoxes; ++cx)
                     load_box(dst + cx * kBoxBytes, tm, bar_kv_full(slot), cx * 64, (item >> 1) * kBlockN);
             }
-        } else if (warp == kMmaWarp && lane == 0) {
+        } else if (warp == kMmaWarp && elect_one()) {
             // =============================================================== MMA issuer
             constexpr uint32_t kIdescS = idesc_bf16(kBlockM, kBlockN, false);
             constexpr uint32_t kIdescO = idesc_bf16(kBlockM, D, true);
@@ -477,15 +516,21 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 mma_commit(bar_s_full(g));
             };
             // O_g (+)= P_g V for the V tile in `slot`
-            auto issue_o = [&](int g, int slot, bool first) {
+            // (three quarters of the keys' weights are there, the rest when parity `par` of p_full completes)
+            auto issue_o = [&](int g, int slot, bool first, bool last, uint32_t par) -> bool {
                 const uint64_t b = desc_v0 + (uint64_t)(slot * (kTileBytes >> 4));
                 const uint32_t tS = tmem + kColS + g * kBlockN, tO = tmem + kColO + g * D;
 #pragma unroll
                 for (int ks = 0; ks < kBlockN / 16; ++ks) {
                     // 16 keys = two 8-row groups of 1024 bytes; column blocks of 64 are one box apart
+                    if (ks == 6) {
+                        if (!mbar_wait(bar_p_full(g), par)) return false;
+                        tc_fence_after();
+                    }
                     mma_ts(tO, tS + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (!first || ks > 0));
                 }
-                mma_commit(bar_o_full(g));
+                if (last) mma_commit(bar_o_full(g));
+                return true;
             };
             auto wait_item = [&](int item) {
                 return mbar_wait(bar_kv_full(item % kStages), (item / kStages) & 1);
@@ -505,9 +550,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                         const int g = t & 1, i = t >> 1;
                         const int item_v = 2 * t + 1, item_k = 2 * (t + 2);
                         if (!wait_item(item_v)) { err = kErrWaitKV; break; }
-                        if (!mbar_wait(bar_p_full(g), i & 1)) { err = kErrWaitP; break; }
+                        if (!mbar_wait(bar_p_early(g), i & 1)) { err = kErrWaitP; break; }
                         tc_fence_after();
-                        issue_o(g, item_v % kStages, i == 0);
+                        if (!issue_o(g, item_v % kStages, i == 0, t + 2 >= nkv, i & 1)) { err = kErrWaitP; break; }
                         mma_commit(bar_kv_empty(item_v % kStages));
                         if (t + 2 < nkv) {
                             if (!wait_item(item_k)) { err = kErrWaitKV; break; }
@@ -538,9 +583,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                     if (!wait_item(item_v)) { err = kErrWaitKV; break; }
                     if (more && !wait_item(item_k)) { err = kErrWaitKV; break; }
                     for (int g = 0; g < ntiles; ++g) {
-                        if (!mbar_wait(bar_p_full(g), j & 1)) { err = kErrWaitP; break; }
+                        if (!mbar_wait(bar_p_early(g), j & 1)) { err = kErrWaitP; break; }
                         tc_fence_after();
-                        issue_o(g, item_v % kStages, j == 0);
+                        if (!issue_o(g, item_v % kStages, j == 0, !more, j & 1)) { err = kErrWaitP; break; }
                         if (more) issue_s(g, item_k % kStages);
                     }
                     if (err) break;
@@ -564,6 +609,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 }
 
 #include "dd_attention_persistent.cuh"
+#include "dd_attention_short.cuh"
 
 // ---------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -636,26 +682,23 @@ int launch(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, 
     return DD_OK;
 }
 
-// The persistent kernel: one CTA per SM (or per item, if there are fewer).
-template <int D>
-int launch_persistent(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const CUtensorMap &to,
-                      const AttnParams &p, int sms, cudaStream_t s)
+// The persistent kernels: one CTA per SM (or per item, if there are fewer).
+template <typename Kernel, typename... Args>
+int launch_persistent(Kernel kernel, int smem, bool (&attr_done)[64], const AttnParams &p, int sms, cudaStream_t s, const Args &...maps)
 {
-    static bool attr_done[64] = {};
     static std::mutex attr_mu;
     int dev = 0;
     DD_CUDA_TRY(cudaGetDevice(&dev));
-    const int smem = SmemP<D>::kTotal + 1024;
     {
         std::lock_guard<std::mutex> lock(attr_mu);
         if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-            DD_CUDA_TRY(cudaFuncSetAttribute(attention_persistent_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            DD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             attr_done[dev] = true;
         }
     }
     const long items = (long)p.BH * p.m_blocks;
     const unsigned grid = (unsigned)(items < sms ? items : sms);
-    attention_persistent_kernel<D><<<grid, kThreads, smem, s>>>(tq, tk, tv, to, p);
+    kernel<<<grid, kThreads, smem, s>>>(maps..., p);
     DD_CUDA_TRY(cudaGetLastError());
     dd::count_launch();
     return DD_OK;
@@ -712,16 +755,27 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     p.scale_log2 = scale * 1.4426950408889634f;
     p.status = ctx->attn_status;
     p.mirror = ctx->mirror_dev;
+    p.out = out;
     cudaStream_t s = (cudaStream_t)stream;
     const bool general = kv_len != nullptr || !head_major || Nq != Nkv;
     if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
-    // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in
-    // every item): the persistent kernel overlaps each item's start and end with its neighbours.
+    // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in every item):
+    // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four key tiles or
+    // more: the kernel whose rounds run across items (16 x 32 heads of 512 tokens 101 us with a CTA per item,
+    // 87 with the short kernel, 81 with this one; of 1024 299, 313 and 276).  Two key tiles, and D = 64: the short
+    // kernel (64 x 32 heads of 256 tokens at D = 128: 148, 99 and 113; 16 x 32 of 512 at D = 64: 73, 61 and 63).
+    // Items of one query tile among those of two: a CTA per item (3 x 24 heads of 1357: 80 against 89).
     int sms = 0;
     if ((rc = sm_count(&sms)) != DD_OK) return rc;
     const int nkv = (Nkv + kBlockN - 1) / kBlockN;
-    if (BH * m_blocks > sms && nkv <= 16 && (Nq - 1) % (kQTiles * kBlockM) >= kBlockM)
-        return D == 64 ? launch_persistent<64>(tq, tk, tv, to, p, sms, s) : launch_persistent<128>(tq, tk, tv, to, p, sms, s);
+    if (BH * m_blocks > sms && nkv <= 16 && (Nq - 1) % (kQTiles * kBlockM) >= kBlockM) {
+        static bool attr_done[3][64] = {};
+        if (D == 64)
+            return launch_persistent(attention_short_kernel<64>, SmemP<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv, to);
+        if (nkv < 4)
+            return launch_persistent(attention_short_kernel<128>, SmemP<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv, to);
+        return launch_persistent(attention_persistent_kernel<128>, SmemL<128>::kTotal + 1024, attr_done[2], p, sms, s, tq, tk, tv);
+    }
     return D == 64 ? launch<64, false>(tq, tk, tv, to, p, s) : launch<128, false>(tq, tk, tv, to, p, s);
 }
 

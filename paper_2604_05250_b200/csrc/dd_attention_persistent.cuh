@@ -1,92 +1,137 @@
-// Persistent form of the attention kernel for many short work items (Section 2.2; Eq. 3): the
-// square, head-major case of dd_bidir_attention when there are more (head, 256-row block) items
-// than SMs and each item has few key tiles.  A CTA of the one-item kernel spends 5-6 us per item
-// outside its steady state: Q and the first K tile have to arrive, the first S product and the
-// first softmax run with nothing to overlap them, and at the end the tensor core waits for the
-// epilogue.  With four key tiles per item (N = 512) that is a third of the item.
+// The square, head-major case of dd_bidir_attention (Section 2.2; Eq. 3) for many items of four to sixteen
+// key tiles at D = 128: persistent CTAs, one per SM, each walking over work items blockIdx.x,
+// blockIdx.x + gridDim.x, ...  An item is up to two tiles of 128 query rows of one head.  Roles and
+// arithmetic are those of attention_kernel; the pipeline never drains between items.
 //
-// Here one CTA per SM walks over items blockIdx.x, blockIdx.x + gridDim.x, ...  The roles and the
-// arithmetic are those of attention_kernel (same softmax code, same MMA shapes); what changes:
-//   * four Q buffers, two per item parity: the producer loads the next item's Q tiles and first
-//     K/V tiles while the current item is still being worked on (ring of three K/V tiles);
-//   * barriers, ring positions and tensor memory live across items, every phase is a running
-//     count;
-//   * the MMA thread issues the next item's first S products right behind the current item's last
-//     P V, so that the softmax groups find scores waiting when their epilogue is done; the first
-//     P V of an item waits until the group has read the previous accumulator out of tensor memory
-//     (o_free);
-//   * the output tile is staged in the item's own Q buffer as before; the buffer is handed back
-//     to the producer (q_free) once the TMA store has read it, which the storing thread checks
-//     after its next key tile, not before.
+// One stream of rounds.  Round r of a CTA is one key tile of one item, for both query tiles g:
+// O_g += P_g V, and the S_g that follows.  The K tile a round needs beside its V tile is the one of the
+// next round, whichever item that belongs to, so V of round r and K of round r + 1 form a pair: one
+// barrier announces both, and one commit at the end of the round releases both.  Items therefore
+// follow each other like rounds do: the next item's first scores are computed while the softmax
+// groups still work on the current item's last tile or write its result.
+//   * A barrier wait costs the issuing thread 170 cycles even when its phase is complete, which the
+//     tensor core spends on products already queued, but only so many; so there are few of them: one
+//     per round for the pair and two per group for its weights.
+//   * The weights of a tile are handed over in two parts: the product starts with the first three
+//     quarters of the keys while the softmax group still computes the last.
+//   * A group that has received S of round r + 1 knows that P V of round r has completed (same thread,
+//     issued earlier), so O has a barrier of its own only at an item's end.
+//   * Q buffers: Q_g of the next item goes into a buffer whose last S product has been committed
+//     (q_free), a round before the item ends, not into one whose result has been written: results go from
+//     registers straight to global memory, a full 32-byte sector per thread and store, so that five
+//     key/value tiles fit beside two query tiles.  (Staged in shared memory, with four: 16 x 32 heads of 512
+//     tokens 83 -> 88 us, of 1024 269 -> 289.)
+//   * o_free: the group has read the finished accumulator out of tensor memory; the next item's
+//     first P V may overwrite it.
 // Every wait is bounded and reports to the attention health word.  Included by dd_attention.cu
 // (inside its unnamed namespace, after the softmax helpers).
 #pragma once
 
-constexpr int kPStages = 3;          // K/V ring slots of the persistent kernel
+constexpr int kReleases = 8;         // release barriers: round r completes phase r / 8 of barrier r % 8
 
 template <int D>
-struct SmemP {
+struct SmemL {
     static constexpr int kTileBytes = kBlockN * D * 2;
-    static constexpr int kQ = 0;                                    // q[parity][group]: four tiles
-    static constexpr int kRing = 4 * kTileBytes;
-    static constexpr int kBars = kRing + kPStages * kTileBytes;
-    // q_full[4], q_free[4], kv_full[3], kv_empty[3], s_full[2], p_full[2], o_full[2], o_free[2]
-    static constexpr int kNumBars = 8 + 2 * kPStages + 8;
+    static constexpr int kQ = 2;                                    // query tiles
+    static constexpr int kSlots = 5;                                // key and value tiles
+    static constexpr int kPairs = kSlots / 2 + 1;                   // pair barriers
+    static constexpr int kRing = kQ * kTileBytes;
+    static constexpr int kBars = kRing + kSlots * kTileBytes;
+    // q_full[kQ], q_free[kQ], pair[kPairs], release[kReleases], k0_full,
+    // s_full[2], p_early[2], p_full[2], o_full[2], o_free[2]
+    static constexpr int kNumBars = 2 * kQ + kPairs + kReleases + 1 + 10;
     static constexpr int kTmemSlot = kBars + 8 * kNumBars;
     static constexpr int kTotal = kTmemSlot + 16;
     static_assert(kTileBytes % 1024 == 0 && kBars % 8 == 0, "tiles on swizzle boundaries, barriers on 8 bytes");
     static_assert(kTotal + 1024 <= 227 * 1024, "shared memory of one CTA");
+    // A barrier may not get two phases ahead of a waiter: the producer is at most (kSlots - 1) / 2 + 1 rounds
+    // past the release it waits for, and at most kPairs pairs past the one the issuing thread waits for.
+    static_assert((kSlots - 1) / 2 + 1 <= kReleases, "release barriers");
 };
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                            const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
-                            const AttnParams p)
+                            const __grid_constant__ CUtensorMap tm_v, const AttnParams p)
 {
+    using L = SmemL<D>;
+    constexpr uint32_t kQ = L::kQ, kSlots = L::kSlots;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char *smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));
-    constexpr uint32_t kTileBytes = SmemP<D>::kTileBytes;
-    const uint32_t sQ = smem_base + SmemP<D>::kQ, sRing = smem_base + SmemP<D>::kRing;
-    const uint32_t bars = smem_base + SmemP<D>::kBars;
-    auto bar_q_full = [&](int par, int g) { return bars + 8u * (par * 2 + g); };
-    auto bar_q_free = [&](int par, int g) { return bars + 8u * (4 + par * 2 + g); };
-    auto bar_kv_full = [&](int s) { return bars + 8u * (8 + s); };
-    auto bar_kv_empty = [&](int s) { return bars + 8u * (8 + kPStages + s); };
-    auto bar_s_full = [&](int g) { return bars + 8u * (8 + 2 * kPStages + g); };
-    auto bar_p_full = [&](int g) { return bars + 8u * (10 + 2 * kPStages + g); };
-    auto bar_o_full = [&](int g) { return bars + 8u * (12 + 2 * kPStages + g); };
-    auto bar_o_free = [&](int g) { return bars + 8u * (14 + 2 * kPStages + g); };
-    const uint32_t tmem_slot = smem_base + SmemP<D>::kTmemSlot;
-    volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + SmemP<D>::kTmemSlot);
+    constexpr uint32_t kTileBytes = L::kTileBytes;
+    const uint32_t sQ = smem_base, sRing = smem_base + L::kRing;
+    const uint32_t bars = smem_base + L::kBars;
+    auto bar_q_full = [&](uint32_t b) { return bars + 8u * b; };
+    auto bar_q_free = [&](uint32_t b) { return bars + 8u * (kQ + b); };
+    auto bar_pair = [&](uint32_t i) { return bars + 8u * (2 * kQ + i); };
+    auto bar_release = [&](uint32_t i) { return bars + 8u * (2 * kQ + L::kPairs + i); };
+    constexpr uint32_t kFixed = 2 * kQ + L::kPairs + kReleases;
+    const uint32_t bar_k0 = bars + 8u * kFixed;
+    auto bar_s_full = [&](int g) { return bars + 8u * (kFixed + 1 + g); };
+    auto bar_p_early = [&](int g) { return bars + 8u * (kFixed + 3 + g); };
+    auto bar_p_full = [&](int g) { return bars + 8u * (kFixed + 5 + g); };
+    auto bar_o_full = [&](int g) { return bars + 8u * (kFixed + 7 + g); };
+    auto bar_o_free = [&](int g) { return bars + 8u * (kFixed + 9 + g); };
+    const uint32_t tmem_slot = smem_base + L::kTmemSlot;
+    volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + L::kTmemSlot);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int n_items = p.BH * p.m_blocks;
-    const int nkv = (p.Nkv + kBlockN - 1) / kBlockN;            // key tiles per item (>= 1)
+    const int nkv = (p.Nkv + kBlockN - 1) / kBlockN;            // rounds per item (>= 1)
+    const int my_items = (n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kBoxBytes = 128 * 128;
-    constexpr uint32_t kColS = 0, kColO = 256;
-    auto q_buf = [&](int par, int g) { return sQ + (uint32_t)(par * 2 + g) * kTileBytes; };
+    constexpr uint32_t kColS = 0, kColO = 256;       // S_0, S_1 (128 columns each, P over them), O_0, O_1 (D each)
+    struct Item { int bh, row0, tiles; };
+    auto item_at = [&](int n) {
+        const int item = (int)blockIdx.x + n * (int)gridDim.x;
+        Item t;
+        t.bh = item / p.m_blocks;
+        t.row0 = (item - t.bh * p.m_blocks) * (kQTiles * kBlockM);
+        t.tiles = p.Nq - t.row0 > kBlockM ? 2 : 1;             // query tiles that hold rows
+        return t;
+    };
+    auto load_tile = [&](uint32_t dst, const CUtensorMap *tm, uint32_t bar, int row, int bh) {
+#pragma unroll
+        for (int cx = 0; cx < kBoxes; ++cx) tma_load_3d(dst + cx * kBoxBytes, tm, bar, cx * 64, row, bh);
+    };
 
+    // The producer thread sets up the barriers its copies complete on and sends Q tile 0 and K tile 0
+    // on their way before the CTA's first barrier: they travel while tensor memory is allocated and
+    // the other barriers are set up.  (Also when an earlier wait has expired and the CTA will do
+    // nothing: such a CTA lingers at its end until copies in flight have landed.)
+    if (warp == kLoadWarp && elect_one()) {
+        prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
+        for (uint32_t i = 0; i < kQ; ++i) mbar_init(bar_q_full(i), 1);
+        for (int i = 0; i < L::kPairs; ++i) mbar_init(bar_pair(i), 1);
+        mbar_init(bar_k0, 1);
+        fence_mbar_init();
+        const Item t = item_at(0);
+        mbar_expect_tx(bar_q_full(0), kTileBytes);
+        load_tile(sQ, &tm_q, bar_q_full(0), t.row0, t.bh);
+        mbar_expect_tx(bar_k0, kTileBytes);
+        load_tile(sRing, &tm_k, bar_k0, 0, t.bh);
+    }
     if (tid == 0) {
-        prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v); prefetch_tmap(&tm_o);
-        for (int i = 0; i < 4; ++i) { mbar_init(bars + 8u * i, 1); mbar_init(bars + 8u * (4 + i), 1); }
-        for (int s = 0; s < kPStages; ++s) { mbar_init(bar_kv_full(s), 1); mbar_init(bar_kv_empty(s), 1); }
+        for (uint32_t i = 0; i < kQ; ++i) mbar_init(bar_q_free(i), 1);
+        for (int i = 0; i < kReleases; ++i) mbar_init(bar_release(i), 1);
         for (int g = 0; g < kQTiles; ++g) {
             mbar_init(bar_s_full(g), 1);
+            mbar_init(bar_p_early(g), kBlockM);
             mbar_init(bar_p_full(g), kBlockM);
             mbar_init(bar_o_full(g), 1);
             mbar_init(bar_o_free(g), kBlockM);
         }
         fence_mbar_init();
+        // a wait that expired in an earlier CTA or launch stops the rest from queueing up behind it
         tmem_slot_gen[1] = *reinterpret_cast<volatile unsigned int *>(p.status);
     }
     if (warp == 0) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot_gen;
+    const uint32_t tmem = warp_uniform(*tmem_slot_gen);
     const bool healthy = tmem_slot_gen[1] == 0;
 
     if (!healthy) {
@@ -99,162 +144,200 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
         const uint32_t tS = tmem + lane_off + kColS + g * kBlockN;
         const uint32_t tO = tmem + lane_off + kColO + g * D;
         const float c = p.scale_log2;
-        const bool storer = (warp & 3) == 0 && lane == 0;
+        const bool sectors = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;     // rows start on 32-byte boundaries
+        uint32_t t_run = 0, i_run = 0;   // key tiles and items of this group so far: phases
         unsigned err = 0;
-        uint32_t t_run = 0;              // key tiles of this group so far, over all items: phase of s/p/o_full
-        int pending_free = -1;           // parity of the Q buffer whose store this thread has committed
-        int n = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
-            const int par = n & 1;
-            const int bh = item / p.m_blocks, mb = item - bh * p.m_blocks;
-            const int row0 = mb * (kQTiles * kBlockM);
+        for (int n = 0; n < my_items; ++n) {
+            const Item t = item_at(n);
+            if (g >= t.tiles) continue;
             float m_ref = -INFINITY, l_run = 0.f;
             for (int j = 0; j < nkv; ++j, ++t_run) {
                 if (!mbar_wait(bar_s_full(g), t_run & 1)) { err = kErrWaitS; break; }
                 tc_fence_after();
-                // O_g holds the sum over this item's tiles < j once the previous P V has completed
-                err = softmax_tile<D>(tS, tO, bar_o_full(g), (t_run - 1) & 1, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run);
-                if (err) break;
+                softmax_tile<D>(tS, tO, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run,
+                    [&] {                        // three quarters of the weights are stored
+                        tmem_wait_st();
+                        tc_fence_before();
+                        mbar_arrive(bar_p_early(g));
+                    });
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive(bar_p_full(g));
-                if (storer && pending_free >= 0) {
-                    // the previous item's store has long read its staging buffer: hand it back
-                    tma_store_wait_read();
-                    mbar_arrive(bar_q_free(pending_free, g));
-                    pending_free = -1;
-                }
             }
-            if (err == 0 && !mbar_wait(bar_o_full(g), (t_run - 1) & 1)) err = kErrWaitO;
-            if (err != 0) report(p, err);
-            if (err == 0) {
-                // ---- epilogue: O / l -> bf16 -> this item's Q buffer (every MMA that read it has
-                // completed) in the swizzled layout of the tensor map -> global by TMA
-                tc_fence_after();
-                const int r = (warp & 3) * 32 + lane;
+            if (err == 0 && !mbar_wait(bar_o_full(g), i_run & 1)) err = kErrWaitO;
+            ++i_run;
+            if (err != 0) { report(p, err); break; }
+            // ---- epilogue: O / l -> bf16 -> global
+            tc_fence_after();
+            uint32_t acc[D];
+#pragma unroll
+            for (int cb = 0; cb < D / 32; ++cb)
+                tmem_ld32(tO + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[cb * 32]));
+            tmem_wait_ld();
+            tc_fence_before();
+            mbar_arrive(bar_o_free(g));      // the next item's first P V may overwrite the accumulator
+            const int row = t.row0 + g * kBlockM + (warp & 3) * 32 + lane;
+            if (row < p.Nq) {
                 const float inv = 1.f / l_run;
-                const uint32_t stage = q_buf(par, g) + r * 128;
-                // the whole accumulator row in one go; once it is in registers the next item's first
-                // P V may overwrite the accumulator
-                uint32_t acc[D];
+                unsigned char *dst = reinterpret_cast<unsigned char *>(p.out) + ((size_t)t.bh * p.Nq + row) * (D * 2);
 #pragma unroll
-                for (int cb = 0; cb < D / 32; ++cb)
-                    tmem_ld32(tO + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[cb * 32]));
-                tmem_wait_ld();
-                tc_fence_before();
-                mbar_arrive(bar_o_free(g));
+                for (int i = 0; i < D; i += 16) {
+                    uint32_t w[8];
 #pragma unroll
-                for (int cb = 0; cb < D / 32; ++cb) columns_to_staging(&acc[cb * 32], inv, stage, r, cb);
-                fence_proxy_async_smem();
-            }
-            // every thread of the warpgroup comes here, also after an expired wait
-            named_bar_sync(1 + g, kBlockM);
-            if (err != 0) break;
-            if (storer) {
-#pragma unroll
-                for (int cx = 0; cx < kBoxes; ++cx)
-                    tma_store_3d(&tm_o, q_buf(par, g) + cx * kBoxBytes, cx * 64, row0 + g * kBlockM, bh);
-                tma_store_commit();
-                pending_free = par;
+                    for (int h = 0; h < 8; ++h) {
+                        __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(acc[i + 2 * h]) * inv,
+                                                                 __uint_as_float(acc[i + 2 * h + 1]) * inv);
+                        w[h] = *reinterpret_cast<uint32_t *>(&v);
+                    }
+                    if (sectors) st_global_v8(dst + 2 * i, w);
+                    else {
+                        reinterpret_cast<uint4 *>(dst + 2 * i)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                        reinterpret_cast<uint4 *>(dst + 2 * i)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    }
+                }
             }
         }
-        if (storer) tma_store_wait_read();          // shared memory must outlive the last store's reads
     } else {
         reg_dec<72>();
-        if (warp == kLoadWarp && lane == 0) {
+        if (warp == kLoadWarp && elect_one()) {
             // =============================================================== TMA producer
-            uint32_t ring = 0;           // ring items so far, over all items
-            int n = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++n) {
-                const int par = n & 1;
-                const int bh = item / p.m_blocks, mb = item - bh * p.m_blocks;
-                const int row0 = mb * (kQTiles * kBlockM);
-                auto load_q = [&](int g) -> bool {
-                    // the buffer staged the output of item n - 2
-                    if (n >= 2 && !mbar_wait(bar_q_free(par, g), ((n >> 1) - 1) & 1)) return false;
-                    mbar_expect_tx(bar_q_full(par, g), kTileBytes);
-#pragma unroll
-                    for (int cx = 0; cx < kBoxes; ++cx)
-                        tma_load_3d(q_buf(par, g) + cx * kBoxBytes, &tm_q, bar_q_full(par, g), cx * 64, row0 + g * kBlockM, bh);
-                    return true;
-                };
-                if (!load_q(0)) { report(p, kErrWaitSlot); break; }
-                for (int it = 0; it < 2 * nkv; ++it, ++ring) {
-                    if (it == 1 && !load_q(1)) { report(p, kErrWaitSlot); ok = false; break; }
-                    const int slot = ring % kPStages;
-                    const uint32_t use = ring / kPStages;
-                    if (use > 0 && !mbar_wait(bar_kv_empty(slot), (use - 1) & 1)) { report(p, kErrWaitSlot); ok = false; break; }
-                    const uint32_t dst = sRing + slot * kTileBytes;
-                    const CUtensorMap *tm = (it & 1) ? &tm_v : &tm_k;
-                    mbar_expect_tx(bar_kv_full(slot), kTileBytes);
-#pragma unroll
-                    for (int cx = 0; cx < kBoxes; ++cx)
-                        tma_load_3d(dst + cx * kBoxBytes, tm, bar_kv_full(slot), cx * 64, (it >> 1) * kBlockN, bh);
+            uint32_t qi = 1;             // query tiles sent so far
+            auto load_q = [&](const Item &t, int g) -> bool {
+                const uint32_t b = qi % kQ, use = qi / kQ;
+                if (use > 0 && !mbar_wait(bar_q_free(b), (use - 1) & 1)) return false;
+                mbar_expect_tx(bar_q_full(b), kTileBytes);
+                load_tile(sQ + b * kTileBytes, &tm_q, bar_q_full(b), t.row0 + g * kBlockM, t.bh);
+                ++qi;
+                return true;
+            };
+            // ring position i: 0 is the first K tile, 2r + 1 the V tile of round r, 2r + 2 the K tile of
+            // round r + 1; the slot is free once the round that read position i - kSlots has completed
+            uint32_t released = 0;       // rounds known to have completed
+            auto slot_free = [&](uint32_t i) -> bool {
+                if (i < kSlots) return true;
+                const uint32_t r = i == kSlots ? 0u : (i - kSlots - 1) >> 1;
+                for (; released <= r; ++released)
+                    if (!mbar_wait(bar_release(released % kReleases), (released / kReleases) & 1)) return false;
+                return true;
+            };
+            Item t = item_at(0);
+            bool ok = t.tiles < 2 || load_q(t, 1);
+            uint32_t r = 0;
+            for (int n = 0; n < my_items && ok; ++n) {
+                const bool more_items = n + 1 < my_items;
+                const Item next = more_items ? item_at(n + 1) : t;
+                for (int j = 0; j < nkv && ok; ++j, ++r) {
+                    const bool last = j + 1 == nkv, with_k = !last || more_items;
+                    const uint32_t bar = bar_pair(r % L::kPairs);
+                    if (!slot_free(2 * r + 1)) { ok = false; break; }
+                    mbar_expect_tx(bar, with_k ? 2 * kTileBytes : kTileBytes);
+                    load_tile(sRing + ((2 * r + 1) % kSlots) * kTileBytes, &tm_v, bar, j * kBlockN, t.bh);
+                    if (with_k) {
+                        if (!slot_free(2 * r + 2)) { ok = false; break; }
+                        load_tile(sRing + ((2 * r + 2) % kSlots) * kTileBytes, &tm_k, bar, last ? 0 : (j + 1) * kBlockN,
+                                  last ? next.bh : t.bh);
+                    }
+                    if (last && more_items) {
+                        ok = load_q(next, 0);
+                        if (ok && next.tiles > 1) ok = load_q(next, 1);
+                    }
                 }
+                t = next;
             }
-        } else if (warp == kMmaWarp && lane == 0) {
+            if (!ok) report(p, kErrWaitSlot);
+        } else if (warp == kMmaWarp && elect_one()) {
             // =============================================================== MMA issuer
             constexpr uint32_t kIdescS = idesc_bf16(kBlockM, kBlockN, false);
             constexpr uint32_t kIdescO = idesc_bf16(kBlockM, D, true);
             const uint64_t desc_q0 = smem_desc_sw128(sQ, 16, 1024);
-            const uint64_t desc_k0 = smem_desc_sw128(sRing, 16, 1024);
-            const uint64_t desc_v0 = smem_desc_sw128(sRing, kBoxBytes, 1024);
+            const uint64_t desc_k0 = smem_desc_sw128(sRing, 16, 1024);            // K-major operand (K tile)
+            const uint64_t desc_v0 = smem_desc_sw128(sRing, kBoxBytes, 1024);     // MN-major operand (V tile)
             unsigned err = 0;
-            auto issue_s = [&](int par, int g, int slot) {
-                const uint64_t a = desc_q0 + (uint64_t)((par * 2 + g) * (kTileBytes >> 4));
+            auto issue_s = [&](int g, uint32_t q_buf, uint32_t slot) {
+                const uint64_t a = desc_q0 + (uint64_t)(q_buf * (kTileBytes >> 4));
                 const uint64_t b = desc_k0 + (uint64_t)(slot * (kTileBytes >> 4));
                 const uint32_t tS = tmem + kColS + g * kBlockN;
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
-                    const uint32_t off = ((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4;
+                    const uint32_t off = ((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4;   // 16 bf16 = 32 bytes per k-step
                     mma_ss(tS, a + off, b + off, kIdescS, ks > 0);
                 }
                 mma_commit(bar_s_full(g));
             };
-            auto issue_o = [&](int g, int slot, bool first) {
+            // O_g (+)= P_g V, the weights of the last quarter of the keys as soon as they are there
+            auto issue_o = [&](int g, uint32_t slot, bool first, uint32_t parity) -> bool {
                 const uint64_t b = desc_v0 + (uint64_t)(slot * (kTileBytes >> 4));
-                const uint32_t tS = tmem + kColS + g * kBlockN, tO = tmem + kColO + g * D;
+                const uint32_t tP = tmem + kColS + g * kBlockN, tO = tmem + kColO + g * D;
 #pragma unroll
-                for (int ks = 0; ks < kBlockN / 16; ++ks)
-                    mma_ts(tO, tS + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (!first || ks > 0));
-                mma_commit(bar_o_full(g));
-            };
-            uint32_t ring = 0;           // ring items consumed so far, over all items
-            uint32_t t_run = 0;          // key tiles so far (the same for both groups)
-            auto wait_ring = [&](uint32_t r) { return mbar_wait(bar_kv_full(r % kPStages), (r / kPStages) & 1); };
-            int n = 0;
-            for (int item = blockIdx.x; item < n_items && err == 0; item += gridDim.x, ++n) {
-                const int par = n & 1;
-                const uint32_t q_phase = (uint32_t)(n >> 1) & 1;
-                // ring items of this work item: ring + 2j = K tile j, ring + 2j + 1 = V tile j
-                if (!mbar_wait(bar_q_full(par, 0), q_phase)) { err = kErrWaitQ; break; }
-                if (!wait_ring(ring)) { err = kErrWaitKV; break; }
-                tc_fence_after();
-                issue_s(par, 0, ring % kPStages);
-                if (!mbar_wait(bar_q_full(par, 1), q_phase)) { err = kErrWaitQ; break; }
-                tc_fence_after();
-                issue_s(par, 1, ring % kPStages);
-                mma_commit(bar_kv_empty(ring % kPStages));
-                for (int j = 0; j < nkv && err == 0; ++j, ++t_run) {
-                    const uint32_t r_v = ring + 2 * j + 1, r_k = ring + 2 * j + 2;
-                    const bool more = j + 1 < nkv;
-                    if (!wait_ring(r_v)) { err = kErrWaitKV; break; }
-                    if (more && !wait_ring(r_k)) { err = kErrWaitKV; break; }
-                    for (int g = 0; g < kQTiles; ++g) {
-                        if (!mbar_wait(bar_p_full(g), t_run & 1)) { err = kErrWaitP; break; }
-                        // the first product of an item overwrites the accumulator: the group must
-                        // have read the previous item's result out of it
-                        if (j == 0 && n > 0 && !mbar_wait(bar_o_free(g), (uint32_t)(n - 1) & 1)) { err = kErrWaitO; break; }
+                for (int ks = 0; ks < kBlockN / 16; ++ks) {
+                    // 16 keys = two 8-row groups of 1024 bytes; column blocks of 64 are one box apart
+                    if (ks == 6) {
+                        if (!mbar_wait(bar_p_full(g), parity)) return false;
                         tc_fence_after();
-                        issue_o(g, r_v % kPStages, j == 0);
-                        if (more) issue_s(par, g, r_k % kPStages);
                     }
-                    if (err) break;
-                    mma_commit(bar_kv_empty(r_v % kPStages));
-                    if (more) mma_commit(bar_kv_empty(r_k % kPStages));
+                    mma_ts(tO, tP + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (!first || ks > 0));
                 }
-                ring += 2 * (uint32_t)nkv;
+                return true;
+            };
+            uint32_t qi = 0;                       // query tiles taken over so far
+            uint32_t q_cur[2] = {0, 0};            // their buffers, of the item whose scores are being issued
+            uint32_t pc[2] = {0, 0}, ic[2] = {0, 0};   // P tiles and items per group so far: phases
+            auto take_q = [&](int g) -> bool {
+                const uint32_t b = qi % kQ;
+                if (!mbar_wait(bar_q_full(b), (qi / kQ) & 1)) return false;
+                q_cur[g] = b;
+                ++qi;
+                return true;
+            };
+            Item t = item_at(0);
+            // first scores of the first item
+            for (int g = 0; g < t.tiles && !err; ++g) {
+                if (!take_q(g)) { err = kErrWaitQ; break; }
+                if (g == 0 && !mbar_wait(bar_k0, 0)) { err = kErrWaitKV; break; }
+                tc_fence_after();
+                issue_s(g, q_cur[g], 0);
+                if (nkv == 1) mma_commit(bar_q_free(q_cur[g]));
+            }
+            uint32_t r = 0;
+            for (int n = 0; n < my_items && !err; ++n) {
+                const bool more_items = n + 1 < my_items;
+                const Item next = more_items ? item_at(n + 1) : t;
+                for (int j = 0; j < nkv && !err; ++j, ++r) {
+                    const bool last = j + 1 == nkv;
+                    const int tiles_s = last ? (more_items ? next.tiles : 0) : t.tiles;   // groups with a next S
+                    const bool q_last = last ? nkv == 1 : j + 2 == nkv;                   // that S is its query tile's last
+                    const uint32_t slot_v = (2 * r + 1) % kSlots, slot_k = (2 * r + 2) % kSlots;
+                    // V of this round, K of the next
+                    if (!mbar_wait(bar_pair(r % L::kPairs), (r / L::kPairs) & 1)) { err = kErrWaitKV; break; }
+                    auto next_s = [&](int g) {
+                        if (g >= tiles_s) return;
+                        if (last && !take_q(g)) { err = kErrWaitQ; return; }
+                        if (last) tc_fence_after();
+                        issue_s(g, q_cur[g], slot_k);
+                        if (q_last) mma_commit(bar_q_free(q_cur[g]));
+                    };
+#pragma unroll
+                    for (int g = 0; g < kQTiles; ++g) {
+                        if (err) break;
+                        if (g < t.tiles) {
+                            const uint32_t parity = pc[g] & 1;
+                            if (!mbar_wait(bar_p_early(g), parity)) { err = kErrWaitP; break; }
+                            ++pc[g];
+                            // the first product of an item overwrites the accumulator: the group must
+                            // have read the previous item's result out of it
+                            if (j == 0) {
+                                if (ic[g] > 0 && !mbar_wait(bar_o_free(g), (ic[g] - 1) & 1)) { err = kErrWaitO; break; }
+                                ++ic[g];
+                            }
+                            tc_fence_after();
+                            if (!issue_o(g, slot_v, j == 0, parity)) { err = kErrWaitP; break; }
+                            if (last) mma_commit(bar_o_full(g));
+                        }
+                        next_s(g);
+                    }
+                    mma_commit(bar_release(r % kReleases));
+                }
+                t = next;
             }
             if (err) report(p, err);
         }

@@ -383,7 +383,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + (tmem_slot - smem_base));
     volatile uint32_t *abort_flag = tmem_slot_gen + 1;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5);
     const LmPlan plan = *q.plan;
     const int k_steps = q.K / kBlockK;
     // a stage: one or two tiles of hidden states (two unless no item has more than 128 rows), one of weights
@@ -405,7 +405,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot_gen;
+    const uint32_t tmem = warp_uniform(*tmem_slot_gen);
 
     // a wait that gives up: the code goes to the health word, every role winds down
     auto give_up = [&](unsigned code) {
@@ -423,7 +423,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
         return false;
     };
 
-    if (warp == kLoadWarp && lane == 0) {
+    if (warp == kLoadWarp && elect_one()) {
         // ===================================================================== TMA producer
         const int width = (Widths<KL>::max_n - plan.N) / 32;
         const CUtensorMap *h = plan.gathered ? &maps.h_gathered : &maps.h, *w = &maps.w[width];
@@ -448,7 +448,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
                 if (++s == stages) { s = 0; ++round; }
             }
         }
-    } else if (warp == kMmaWarp && lane == 0) {
+    } else if (warp == kMmaWarp && elect_one()) {
         // ===================================================================== MMA issuer
         const uint32_t idesc = idesc_bf16(128, plan.N, false);
         uint32_t s = 0, round = 0;
