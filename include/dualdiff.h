@@ -93,7 +93,7 @@ int dd_bidir_attention(const void *q, const void *k, const void *v, void *out,
  *                     id) or if DD_FLAG_EMIT_DRAFTER; otherwise a_i
  *   out_score[b,i]  = KL_i (KL mode) or c_i (CONF and TRUST modes)
  * Positions with mask_flags == 0 pass through: out_tokens = tokens,
- * out_mask = 0, out_score = 0, and their logits are never read.
+ * out_mask = 0, out_score = 0, and nothing is computed from their logits.
  * A logit of -inf is an excluded token (probability 0, an ordinary input: a banned or
  * padded vocabulary entry, the mask token): it contributes no term to Eq. 5 where the
  * drafter excludes it (the sum runs over the support of p_D), and KL_i = +inf where
@@ -104,8 +104,9 @@ int dd_bidir_attention(const void *q, const void *k, const void *v, void *out,
  * drafter_logits, verifier_logits: [B,P,V] bf16 (drafter_logits may be NULL
  * unless the mode is KL); tokens int32 [B,P]; mask_flags uint8 [B,P];
  * out_tokens int32 [B,P] (may alias tokens); out_mask uint8 [B,P]; out_score
- * fp32 [B,P], nullable.  The streaming path needs V % 8 == 0 and 16-byte
- * aligned logits; otherwise a slower element-wise path is taken.
+ * fp32 [B,P], nullable.  The streaming path needs 16-byte aligned
+ * logits (any V); otherwise a slower element-wise path is taken.  Where V is not a multiple of eight,
+ * logits of an unflagged position that share a 16-byte block with a flagged one's are loaded and discarded.
  * Supported: P <= 8192; V < 2^31 / 2.
  * Errors: DD_ERR_INVALID_ARG (null required pointer, B/P/V <= 0, k < 0, unknown
  * mode or flag bit, tau NaN), DD_ERR_UNSUPPORTED (P too large), DD_ERR_CUDA.

@@ -41,7 +41,7 @@
 #include <cuda.h>
 
 #include "dd_ptx.cuh"
-#include "dd_verify_common.cuh"
+#include "dd_verify_decide_block.cuh"
 
 namespace ddlm {
 
@@ -183,39 +183,18 @@ __device__ __forceinline__ void store_partial(const ddv::VerifyParams &p, const 
     __stcg(reinterpret_cast<float4 *>(dst) + 1, make_float4(c.s_d, c.t, 0.f, 0.f));
 }
 
-// n more rows of sequence b are accounted for (warp-level); the warp that accounts for the last
-// of the P rows decides the sequence.
-__device__ __forceinline__ void rows_done(const ddv::VerifyParams &p, int b, int n, ddv::DecideStage *stage)
-{
-    const int lane = threadIdx.x & 31;
-    int last = 0;
-    if (lane == 0) {
-        __threadfence();
-        last = atomicAdd(p.seq_counter + ddv::checked(p, b, p.B, ddv::kSiteSeq), (unsigned)n) + (unsigned)n == (unsigned)p.P;
-    }
-    last = __shfl_sync(0xFFFFFFFFu, last, 0);
-    if (!last) return;
-    __threadfence();
-    if (lane == 0) p.seq_counter[b] = 0u;      // ready for the next launch
-    ddv::decide_sequence(p, b, stage);
-}
-
-// Last launch of dd_lm_head_verify: one warp per row folds the row's tile partials (fp64, tile
-// order: the streaming kernel's fold) and stores score and argmax; one warp per sequence accounts
-// for the rows that are not flagged; the warp that accounts for a sequence's last row runs the
-// decision stage.  The partials were written by the previous kernel on the stream.
-constexpr int kFoldThreads = 128;
-constexpr int kFoldDecideKeys = 2048;      // keys of one sequence each warp can keep in shared memory
+// Last launch of dd_lm_head_verify: one warp per row folds the row's tile partials (fp64, tile order: the
+// streaming kernel's fold) and stores score and argmax; the CTA counts its rows in their sequences and decides
+// those it completes with all its threads (a warp per deciding sequence took 12-16 us from a cold
+// instruction cache: 16 rows of 126464 entries 204 -> 194 us, 8 x 512 of 8000 41.5 -> 39.8).  The partials were written by the previous kernel on the stream.
+constexpr int kFoldThreads = 256;
 template <bool KL>
-__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::VerifyParams p, int rows, const LmPlan *plan)
+__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const __grid_constant__ ddv::VerifyParams p, int rows, const LmPlan *plan)
 {
-    __shared__ uint32_t s_keys[kFoldThreads / 32][kFoldDecideKeys];
-    ddv::DecideStage stage;
-    stage.key = s_keys[threadIdx.x >> 5];
-    stage.capacity = kFoldDecideKeys;
-    const int w = blockIdx.x * (kFoldThreads / 32) + (threadIdx.x >> 5);     // rows first, then sequences
-    if (w < rows) {
-        if (!p.flags[w]) return;
+    __shared__ ddv::BlockReport s_report;
+    const int row0 = blockIdx.x * (kFoldThreads / 32);
+    const int w = row0 + (threadIdx.x >> 5);
+    if (w < rows && p.flags[w]) {
         float score;
         int argmax;
         const int n_tiles = plan->n_tiles;
@@ -226,14 +205,8 @@ __global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const ddv::V
             __stcg(p.row_score + row_at, score);
             __stcg(p.row_argmax + row_at, argmax);
         }
-        __syncwarp();
-        rows_done(p, w / p.P, 1, &stage);
-    } else {
-        const int b = w - rows;
-        if (b >= p.B) return;
-        const int unflagged = p.P - ddv::count_flagged(p, b);
-        if (unflagged > 0) rows_done(p, b, unflagged, &stage);
     }
+    ddv::report_rows(p, row0, kFoldThreads / 32, s_report);
 }
 
 // The work items of a CTA, in order: every role walks the same way.  Items that follow each other share a

@@ -9,11 +9,13 @@
 // (M = m*log2e rounded once; any reference works as long as it is reused), and
 // each logit is read from HBM exactly once.
 //
-// Streaming kernel (V % 8 == 0, 16-byte aligned logits; dd_verify_stream.cuh):
+// Row kernel (16-byte aligned logits, any V, small and middle-sized problems; dd_verify_rows.cuh): a row per
+// warp, CTA or cluster, read straight into registers.
+// Streaming kernel (the same, large problems; dd_verify_stream.cuh):
 // persistent CTAs; a producer warp feeds per-warp rings in shared memory with bulk
 // asynchronous copies, consumer warps accumulate chunks of up to 8192 logits from
 // them, a publishing warp counts, folds and decides.
-// Element-wise kernel (any V, any alignment; this file): one CTA of 256 threads
+// Element-wise kernel (logits off 16-byte boundaries; this file): one CTA of 256 threads
 // per chunk of at most 8192 logits, 2-byte loads with bounds checks.
 //
 // The warp that sees a row's last chunk folds the row's chunk partials in chunk
@@ -31,6 +33,7 @@
 #include <mutex>
 
 #include "dd_verify_stream.cuh"
+#include "dd_verify_rows.cuh"
 #include "dd_lm_head_kernel.cuh"
 
 namespace {
@@ -210,9 +213,12 @@ size_t workspace_bytes(int B, int P, int nchunks)
     return bytes;
 }
 
-bool streaming_path(const void *drafter, const void *verifier, int V, bool kl)
+// Rows may start anywhere (V need not be a multiple of eight), the tensors themselves on 16 bytes.  V = 32001,
+// 2 x 300 positions, half of them flagged, KL: element-wise kernel 41.5 us, streaming 37.6, row kernel 23.1;
+// V = 50001, 8 x 256, CONF: element-wise 108, streaming 40.1.
+bool streaming_path(const void *drafter, const void *verifier, bool kl)
 {
-    return (V % 8 == 0) && (((uintptr_t)verifier & 15) == 0) && (!kl || ((uintptr_t)drafter & 15) == 0);
+    return ((uintptr_t)verifier & 15) == 0 && (!kl || ((uintptr_t)drafter & 15) == 0);
 }
 
 // Streaming path: stages per chunk (a chunk is the work of one warp and yields one partial).
@@ -253,7 +259,6 @@ void chunking(int V, bool streaming, bool kl, int pieces, int *nchunks, int *chu
 
 std::mutex g_mu;                 // guards the per-device caches below
 int g_sm_count[64] = {};
-bool g_smem_attr_done[64][2] = {};
 std::atomic<int> g_max_ctas{0};  // 0: one CTA per SM; otherwise a cap on the streaming kernel's grid
 
 // Number of SMs of the current device (cached), or a negative status.
@@ -267,7 +272,7 @@ int sm_count_of_current_device()
     return g_sm_count[dev];
 }
 
-template <bool KL>
+template <bool KL, bool kRagged>
 int launch_stream(const VerifyParams &p, cudaStream_t stream)
 {
     const int sms = sm_count_of_current_device();
@@ -275,22 +280,63 @@ int launch_stream(const VerifyParams &p, cudaStream_t stream)
     int dev = 0;
     DD_CUDA_TRY(cudaGetDevice(&dev));
     {
+        static bool attr_done[64] = {};
         std::lock_guard<std::mutex> lock(g_mu);
-        if (!g_smem_attr_done[dev][KL ? 1 : 0]) {
-            DD_CUDA_TRY(cudaFuncSetAttribute(verify_stream_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (!attr_done[dev]) {
+            DD_CUDA_TRY(cudaFuncSetAttribute(verify_stream_kernel<KL, kRagged>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kSRingBytes));
             // the same split of the SM's memory as the attention kernel that runs before and after
-            DD_CUDA_TRY(cudaFuncSetAttribute(verify_stream_kernel<KL>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            DD_CUDA_TRY(cudaFuncSetAttribute(verify_stream_kernel<KL, kRagged>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                              cudaSharedmemCarveoutMaxShared));
-            g_smem_attr_done[dev][KL ? 1 : 0] = true;
+            attr_done[dev] = true;
         }
     }
     const long units = (long)p.B * p.P * p.nchunks;
     long grid = units < sms ? units : sms;
     const int cap = g_max_ctas.load(std::memory_order_relaxed);
     if (cap > 0 && grid > cap) grid = cap;
-    verify_stream_kernel<KL><<<(unsigned)grid, kSThreads, kSRingBytes, stream>>>(p);
+    verify_stream_kernel<KL, kRagged><<<(unsigned)grid, kSThreads, kSRingBytes, stream>>>(p);
     DD_CUDA_TRY(cudaGetLastError());
+    dd::count_launch();
+    return DD_OK;
+}
+
+// The row kernel or the streaming kernel.  In pieces of 4 KB (1024 logits of both tensors, 2048 of one), whatever
+// share of the rows is flagged (the host does not know): up to 160 pieces per SM the row kernel.
+// Measured (us, row against streaming kernel; B x P, V, share flagged): 1 x 128, 1024, KL 25 %: 10.0 / 13.9;
+// 4 x 128, 4096, KL: 11.6 / 21.9; 1 x 256, 16000, KL: 12.9 / 21.9; 1 x 512, 32000, KL 100 %: 30.0 / 34.1, 25 %: 21.7 /
+// 29.9; 1 x 32, 126464, KL: 14.2 / 24.2; 1 x 128: 25.9 / 31.9; 16 x 512, 1000, CONF: 23.0 / 38.3.  Beyond the line: 8 x
+// 256, 32000, CONF: 36.6 / 31.7; 1 x 256, 126464, KL: 38.7 / 37.5; 16 x 512, 8000, KL 50 %: 58.4 / 51.1.
+long row_pieces(int V, bool kl) { return ((long)V + 7) / (kl ? kPiece : 2 * kPiece) + 1; }
+bool rows_path(int V, long rows, int sms, bool kl) { return rows * row_pieces(V, kl) <= 160L * sms && rows <= 32L * 1024; }
+
+template <bool KL>
+int launch_rows(const VerifyParams &p, cudaStream_t stream)
+{
+    const int sms = sm_count_of_current_device();
+    if (sms < 0) return sms;
+    const long rows = (long)p.B * p.P;
+    const long pieces = row_pieces(p.V, KL);
+    // Warps per row: enough to fill the GPU (24 per SM), but at least two pieces for each.  Few rows: clusters
+    // of CTAs, as long as two CTAs per SM hold them all (32 rows of 126464: 27 us with eight warps a row,
+    // 14 with clusters of eight; 128 rows: clusters of two 25.9, of four 30.1).
+    RowsShape shape = {1, 1};
+    while (shape.wpr < kRWarps && 4 * shape.wpr <= pieces + 1 && rows * shape.wpr < 24L * sms) shape.wpr *= 2;
+    while (shape.wpr == kRWarps && shape.cluster < kRMaxCluster && 4 * kRWarps * shape.cluster <= pieces + 1 &&
+           2 * shape.cluster * rows <= 2L * sms)
+        shape.cluster *= 2;
+    const long groups = (rows + kRWarps / shape.wpr - 1) / (kRWarps / shape.wpr);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(groups * shape.cluster));
+    cfg.blockDim = dim3(32 * kRWarps);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = shape.cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
+    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL>, p, shape));
     dd::count_launch();
     return DD_OK;
 }
@@ -308,8 +354,12 @@ int launch_elementwise(const VerifyParams &p, cudaStream_t stream)
 int launch(const VerifyParams &p, bool streaming, cudaStream_t s)
 {
     const bool kl = p.algo == DD_MODE_KL;
-    if (streaming) return kl ? launch_stream<true>(p, s) : launch_stream<false>(p, s);
-    return kl ? launch_elementwise<true>(p, s) : launch_elementwise<false>(p, s);
+    if (!streaming) return kl ? launch_elementwise<true>(p, s) : launch_elementwise<false>(p, s);
+    const int sms = sm_count_of_current_device();
+    if (sms < 0) return sms;
+    if (rows_path(p.V, (long)p.B * p.P, sms, kl)) return kl ? launch_rows<true>(p, s) : launch_rows<false>(p, s);
+    if (p.V % 8 != 0) return kl ? launch_stream<true, true>(p, s) : launch_stream<false, true>(p, s);
+    return kl ? launch_stream<true, false>(p, s) : launch_stream<false, false>(p, s);
 }
 
 int check_args(const void *drafter_logits, const void *verifier_logits, const int32_t *tokens,
@@ -355,7 +405,7 @@ extern "C" size_t dd_verify_workspace_bytes(int B, int P, int V)
 {
     if (B <= 0 || P <= 0 || V <= 0) return 0;
     int nchunks, chunk;
-    chunking(V, V % 8 == 0, true, 1, &nchunks, &chunk);       // the finest cut a launch may choose
+    chunking(V, true, true, 1, &nchunks, &chunk);             // the finest cut a launch may choose
     return workspace_bytes(B, P, nchunks) + counter_bytes(B, P) + kControlBytes;
 }
 
@@ -369,7 +419,7 @@ extern "C" int dd_verify(const void *drafter_logits, const void *verifier_logits
                         B, P, V);
     if (rc != DD_OK) return rc;
     const bool kl = (mode & 0xFF) == DD_MODE_KL;
-    const bool streaming = streaming_path(drafter_logits, verifier_logits, V, kl);
+    const bool streaming = streaming_path(drafter_logits, verifier_logits, kl);
 
     VerifyParams p;
     int pieces = 4;
@@ -496,8 +546,8 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
     DD_CUDA_TRY(cudaGetLastError());
     lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
     DD_CUDA_TRY(cudaGetLastError());
-    // one warp per row, then one per sequence
-    const unsigned fold_grid = (unsigned)(((long)q.rows + p.B + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
+    // one warp per row
+    const unsigned fold_grid = (unsigned)(((long)q.rows + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
     lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q.rows, q.plan);
     DD_CUDA_TRY(cudaGetLastError());
     dd::count_launch(3);
@@ -625,7 +675,7 @@ extern "C" int dd_verify_static(const void *drafter_logits, const void *verifier
                         B, P, V);
     if (rc != DD_OK) return rc;
     const bool kl = (mode & 0xFF) == DD_MODE_KL;
-    const bool streaming = streaming_path(drafter_logits, verifier_logits, V, kl);
+    const bool streaming = streaming_path(drafter_logits, verifier_logits, kl);
 
     VerifyParams p;
     // the fixed scratch bounds the problem size (stated for chunks of 8192 logits; a finer cut is

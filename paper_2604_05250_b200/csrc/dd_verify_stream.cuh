@@ -1,4 +1,4 @@
-// Streaming kernel of dd_verify (V % 8 == 0, 16-byte aligned logits).
+// Streaming kernel of dd_verify (16-byte aligned logits, any V).
 //
 // One persistent CTA per SM: fifteen streaming warps and one publishing warp.
 //
@@ -260,15 +260,16 @@ __device__ __forceinline__ void lane_pass2(LaneState &L, const uint4 (&rv)[kVecP
 // The chunk has ended: the 32 lane states become one partial (the same bits in every lane):
 // the warp's maxima first, then every lane's sums moved to them and added up.  The drafter's
 // "maximum" is the largest of the lanes' reference points: the sums only need a common one.
+// Pieces are `stride` logits apart.
 template <bool KL>
-__device__ __forceinline__ Partial lanes_to_partial(const LaneState &L, int chunk_begin, int lane)
+__device__ __forceinline__ Partial lanes_to_partial(const LaneState &L, int chunk_begin, int lane, int stride = PieceOf<KL>::value)
 {
     Partial c;
     const float lo_m = bf16lo(L.max2_v), hi_m = bf16hi(L.max2_v);
     auto element_of = [&](uint32_t q, int odd) {     // q = piece * 16 + j * 4 + h (KL), piece * 32 + j * 4 + h
         const int piece = KL ? (int)(q >> 4) : (int)(q >> 5);
         const int vec = KL ? (int)((q >> 2) & 3u) : (int)((q >> 2) & 7u);
-        return chunk_begin + piece * PieceOf<KL>::value + (lane + 32 * vec) * 8 + 2 * (int)(q & 3u) + odd;
+        return chunk_begin + piece * stride + (lane + 32 * vec) * 8 + 2 * (int)(q & 3u) + odd;
     };
     const int e_lo = element_of(L.where2_v & 0xFFFFu, 0), e_hi = element_of(L.where2_v >> 16, 1);
     const float my_m = fmaxf(lo_m, hi_m);
@@ -329,6 +330,11 @@ __device__ __noinline__ Partial careful_chunk_partial(const uint16_t *verifier_r
     c.pad0 = c.pad1 = 0.f;
     return c;
 }
+
+// Elements between the 16-byte boundary at or before row `row` and the row itself.  A vocabulary that is not
+// a multiple of eight puts most rows off that boundary; the kernel then walks over the aligned vectors that
+// hold the row and sets what is not the row's to -inf.
+__device__ __forceinline__ int row_head(int row, int V) { return (int)(((unsigned)row * (unsigned)V) & 7u); }
 
 // A finished row (or a range's share of a row cut by a range boundary), handed from a
 // streaming warp to the publishing warp.

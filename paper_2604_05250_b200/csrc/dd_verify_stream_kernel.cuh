@@ -66,7 +66,8 @@ __device__ __forceinline__ void pending_add(const VerifyParams &p, Pending &pend
     ++pend.used;
 }
 
-template <bool KL>
+// kRagged: V is not a multiple of eight.
+template <bool KL, bool kRagged>
 __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const VerifyParams p)
 {
     extern __shared__ __align__(128) unsigned char s_ring[];     // [warp][stage][kSStageBytes]
@@ -285,7 +286,8 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
             const unsigned char *ring_gen = s_ring + warp * kSStages * kSStageBytes;
             const uint32_t ring = s_addr(s_ring) + (uint32_t)(warp * kSStages * kSStageBytes);
             const int chunk_pieces = p.chunk / kStep;
-            const int last_pieces = (p.V - (nch - 1) * p.chunk + kStep - 1) / kStep;     // of a row's last chunk
+            const int last_pieces = (p.V - (nch - 1) * p.chunk + kStep - 1) / kStep;     // of a row's last chunk (V a multiple of eight)
+            const unsigned last_row = (unsigned)n_rows - 1u;
             // The order in which the range's units are handed out starts with the range's share of
             // its last row, then its share of its first row (the two rows it may share with a
             // neighbour), then everything in between.
@@ -294,6 +296,7 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
 
             // ---- lane 0 feeds the ring: the piece it will issue next
             int i_row = 0, i_chunk = 0, i_piece = 0, i_npieces = 0, i_where = 0;
+            int i_head = 0;                   // elements in front of the row in its first vector
             bool i_more = true;               // false once the end marker has been posted
             const uint64_t policy = l2_evict_first_policy();
             auto issue = [&](unsigned stage) {
@@ -315,19 +318,42 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
                     const int local_row = (int)(f - f_lo);
                     i_row = s_rows[local_row];
                     i_where = t | (local_row << 16);
-                    i_npieces = i_chunk == nch - 1 ? last_pieces : chunk_pieces;
+                    if constexpr (kRagged) {
+                        i_head = row_head(i_row, p.V);
+                        i_npieces = i_chunk == nch - 1 ? (i_head + p.V - i_chunk * p.chunk + kStep - 1) / kStep : chunk_pieces;
+                    } else {
+                        i_npieces = i_chunk == nch - 1 ? last_pieces : chunk_pieces;
+                    }
                     i_piece = 0;
                 }
-                const int e_begin = i_chunk * p.chunk + i_piece * kStep;
-                const int n = min(kStep, p.V - e_begin);
-                const int fl = n | (i_piece == 0 ? 1 << 16 : 0) | (i_piece == i_npieces - 1 ? 1 << 17 : 0) | (i_piece << 20);
-                s_meta[warp][stage] = make_int4(fl, i_where, i_row, i_chunk);
-                const uint32_t bytes = (uint32_t)n * 2u;
-                const uint32_t dst = ring + stage * kSStageBytes;
-                const size_t off = checked_run(p, (long)i_row * p.V + e_begin, n, n_rows * p.V, kSiteLogit);
-                sbar_expect_tx(bar, KL ? 2u * bytes : bytes);
-                bulk_load(dst, p.verifier + off, bytes, bar, policy);
-                if (KL) bulk_load(dst + kSStageBytes / 2, p.drafter + off, bytes, bar, policy);
+                if constexpr (!kRagged) {
+                    const int e_begin = i_chunk * p.chunk + i_piece * kStep;
+                    const int n = min(kStep, p.V - e_begin);
+                    const int fl = n | (i_piece == 0 ? 1 << 16 : 0) | (i_piece == i_npieces - 1 ? 1 << 17 : 0) | (i_piece << 20);
+                    s_meta[warp][stage] = make_int4(fl, i_where, i_row, i_chunk);
+                    const uint32_t bytes = (uint32_t)n * 2u;
+                    const uint32_t dst = ring + stage * kSStageBytes;
+                    const size_t off = checked_run(p, (long)i_row * p.V + e_begin, n, n_rows * p.V, kSiteLogit);
+                    sbar_expect_tx(bar, KL ? 2u * bytes : bytes);
+                    bulk_load(dst, p.verifier + off, bytes, bar, policy);
+                    if (KL) bulk_load(dst + kSStageBytes / 2, p.drafter + off, bytes, bar, policy);
+                } else {
+                    const int x_begin = i_chunk * p.chunk + i_piece * kStep;         // from the row's first vector on
+                    const int n = min(kStep, i_head + p.V - x_begin);
+                    const bool edge = n < kStep || (i_head != 0 && x_begin == 0);
+                    const int fl = n | (i_piece == 0 ? 1 << 16 : 0) | (i_piece == i_npieces - 1 ? 1 << 17 : 0) | (edge ? 1 << 18 : 0) | (i_piece << 20);
+                    s_meta[warp][stage] = make_int4(fl, i_where, i_row, i_chunk);
+                    // whole vectors; one that the tensor's last row fills only in part is left out (see below)
+                    const int vecs = (unsigned)i_row == last_row ? n >> 3 : (n + 7) >> 3;
+                    const uint32_t bytes = (uint32_t)vecs * 16u;
+                    const uint32_t dst = ring + stage * kSStageBytes;
+                    sbar_expect_tx(bar, KL ? 2u * bytes : bytes);
+                    if (vecs > 0) {
+                        const size_t off = checked_run(p, (long)i_row * p.V - i_head + x_begin, 8L * vecs, n_rows * p.V, kSiteLogit);
+                        bulk_load(dst, p.verifier + off, bytes, bar, policy);
+                        if (KL) bulk_load(dst + kSStageBytes / 2, p.drafter + off, bytes, bar, policy);
+                    }
+                }
                 ++i_piece;
             };
             if (lane == 0) {
@@ -353,7 +379,7 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
                     }
                     if (!arrived) { err = kErrWaitFull; break; }
                 }
-                // n logits | first << 16 | last << 17 | piece << 20;  slot | local row << 16;  row;  chunk
+                // n logits | first << 16 | last << 17 | edge of the row << 18 | piece << 20;  slot | local row << 16;  row;  chunk
                 const int4 meta = s_meta[warp][stage];
                 const int n = meta.x & 0xFFFF;
                 if (n == 0) { ++it; break; }                      // the range has no more units for this warp
@@ -367,13 +393,52 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
                         rv[j] = sv[32 * j];
                         rd[j] = sd[32 * j];
                     }
-                    if (n < kStep) {
-                        // what lies beyond the row's end in the stage is stale: -inf instead
-                        const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+                    if constexpr (!kRagged) {
+                        if (n < kStep) {
+                            // what lies beyond the row's end in the stage is stale: -inf instead
+                            const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+#pragma unroll
+                            for (int j = 0; j < kVecPerThread; ++j) {
+                                if ((lane + 32 * j) * 8 >= n) rv[j] = ninf;
+                                if ((lane + 32 * (KL ? j : kVecPerThread + j)) * 8 >= n) rd[j] = ninf;
+                            }
+                        }
+                    } else if (meta.x & (1 << 18)) {
+                        // -inf for what is not the row's: stale data beyond the vectors copied, and the neighbours'
+                        // logits in the vectors that the row shares with them
+                        const int head = (kRagged ? row_head(meta.z, p.V) : 0);
+                        const int x_begin = meta.w * p.chunk + ((meta.x >> 20) & 0xF) * kStep;
+                        const long at = (long)meta.z * p.V - head + x_begin;          // of the piece, in the tensor
+                        const bool last_row_tail = meta.z == (int)last_row && (n & 7) != 0;
+                        auto edge_vector = [&](uint4 &r, int vec, const uint16_t *logits) {
+                            const int e0 = vec * 8;
+                            if (last_row_tail && e0 < n && e0 + 8 > n) {
+                                // the vector that was not copied: its logits one by one
+                                uint32_t w[4] = {0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u};
+#pragma unroll
+                                for (int i = 0; i < 7; ++i)
+                                    if (e0 + i < n) {
+                                        const uint32_t v = __ldg(logits + checked(p, at + e0 + i, n_rows * p.V, kSiteLogit));
+                                        w[i / 2] = (w[i / 2] & (i & 1 ? 0x0000FFFFu : 0xFFFF0000u)) | (i & 1 ? v << 16 : v);
+                                    }
+                                r = make_uint4(w[0], w[1], w[2], w[3]);
+                            }
+                            const int from = x_begin == 0 ? head : 0;                  // first element that is the row's
+                            if (e0 + 8 > n || e0 < from) {
+                                uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                                for (int h = 0; h < 4; ++h) {
+                                    const int e = e0 + 2 * h;
+                                    if (e >= n || e < from) w[h] = (w[h] & 0xFFFF0000u) | 0xFF80u;
+                                    if (e + 1 >= n || e + 1 < from) w[h] = (w[h] & 0x0000FFFFu) | 0xFF800000u;
+                                }
+                                r = make_uint4(w[0], w[1], w[2], w[3]);
+                            }
+                        };
 #pragma unroll
                         for (int j = 0; j < kVecPerThread; ++j) {
-                            if ((lane + 32 * j) * 8 >= n) rv[j] = ninf;
-                            if ((lane + 32 * (KL ? j : kVecPerThread + j)) * 8 >= n) rd[j] = ninf;
+                            edge_vector(rv[j], lane + 32 * j, p.verifier);
+                            edge_vector(rd[j], lane + 32 * (KL ? j : kVecPerThread + j), KL ? p.drafter : p.verifier);
                         }
                     }
                 }
@@ -388,14 +453,15 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
 
                 // ---- the chunk is complete: into the table; the warp that completes the range's share
                 // of a row hands the row on
-                Partial part = lanes_to_partial<KL>(L, meta.w * p.chunk, lane);
+                const int head = (kRagged ? row_head(meta.z, p.V) : 0);
+                Partial part = lanes_to_partial<KL>(L, meta.w * p.chunk - head, lane);
                 lane_reset(L);
                 if (!(isfinite(part.s_v) && isfinite(part.s_d) && isfinite(part.t) && part.m_v > -INFINITY) ||
                     (KL && fabsf(part.t) > kExcludedExcess * part.s_d)) {
-                    const int begin = meta.w * p.chunk;
+                    const int begin = kRagged ? max(0, meta.w * p.chunk - head) : meta.w * p.chunk;
+                    const int end = kRagged && meta.w == nch - 1 ? p.V : min(p.V, begin + p.chunk - (begin == 0 ? head : 0));
                     const size_t row_off = checked_run(p, (long)meta.z * p.V, p.V, n_rows * p.V, kSiteLogit);
-                    part = careful_chunk_partial<KL>(p.verifier + row_off, KL ? p.drafter + row_off : nullptr,
-                                                     begin, min(p.V, begin + p.chunk));
+                    part = careful_chunk_partial<KL>(p.verifier + row_off, KL ? p.drafter + row_off : nullptr, begin, end);
                 }
                 const int slot = meta.y & 0xFFFF, local_row = meta.y >> 16;
                 const unsigned row_first = (f_lo + (unsigned)local_row) * (unsigned)nch;   // the row's unit 0

@@ -60,3 +60,23 @@ def test_loop_matches_oracle_loop(dd, oracle_mod, mode, tau, k, K):
     if not mode & 0x200:
         # kept positions carry the verifier's token, and the toy verifier knows the target
         np.testing.assert_array_equal(x.cpu().numpy(), target)
+
+
+@pytest.mark.parametrize("mode,tau,k,K,unmask_k", [(KL, 0.5, 2, 3, 2), (TRUST, 0.0, 0, 8, 5), (CONF, 0.6, 1, 2, 40)])
+def test_loop_with_a_fixed_number_per_step(dd, oracle_mod, mode, tau, k, K, unmask_k):
+    """No threshold: the host follows the number of masked positions by itself within a cycle.  Prompts of
+    unequal length, a sequence with nothing to generate, a last step with fewer positions than unmask_k."""
+    import torch
+    from paper_2604_05250_b200.pipeline import dualdiffusion_generate
+    target, start, drafter, verifier = problem(7)
+    start[1] = target[1]
+    start[2, :23] = target[2, :23]
+    ref_x, ref_stats, near = oracle_mod.dualdiffusion_loop(drafter, verifier, start, MASK_ID, K, mode, tau, k, seed=9,
+                                                           unmask_tau=float("inf"), unmask_k=unmask_k, max_cycles=200)
+    assert near == 0
+    x, stats = dualdiffusion_generate(on_device(drafter), on_device(verifier), torch.from_numpy(start).cuda(),
+                                      MASK_ID, K, mode, tau, k, seed=9, unmask_k=unmask_k, max_cycles=200)
+    np.testing.assert_array_equal(x.cpu().numpy(), ref_x)
+    for key in ("cycles", "drafter_calls", "verifier_calls", "unmasked_by_drafter", "remasked_by_verifier",
+                "masked_after_cycle"):
+        assert getattr(stats, key) == ref_stats[key], key

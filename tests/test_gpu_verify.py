@@ -293,3 +293,80 @@ def test_excluded_tokens(dd, oracle_mod, V):
         for mode in (KL, CONF, KL | PROB):
             _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 3, 7)
             assert np.isfinite(ref["out_score"]).all() and np.isfinite(got[2]).all()
+
+
+# vocabularies that put rows anywhere between 16-byte boundaries: fewer logits than a vector, one vector more
+# or less than a stage (1024 logits of both tensors, 2048 of one), a chunk's last stage of a few logits
+@pytest.mark.parametrize("V", [1, 3, 7, 9, 15, 1017, 1023, 1025, 1031, 2041, 2047, 2050, 4089, 4095, 4097, 8190, 8193, 16385])
+@pytest.mark.parametrize("mode", [KL, CONF])
+def test_rows_off_vector_boundaries(dd, oracle_mod, V, mode):
+    dra, ver, tokens, flags = synth.verify_inputs(2, 37, V, 23, 0.3, seed=V + 1)
+    flags[1, -1] = 1                         # the tensor's last row, whose last vector is not whole
+    flags[0, 0] = 1
+    # the neighbours' logits share vectors with a flagged row's and must not reach it
+    ver[flags == 0] = 0x7FC0
+    dra[flags == 0] = 0x7F80
+    compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 4, 1)
+
+
+@pytest.mark.parametrize("V", [1000, 1003])
+@pytest.mark.parametrize("mode", [KL, CONF])
+def test_logits_off_16_byte_boundaries(dd, oracle_mod, V, mode):
+    """Tensors that start in the middle of a vector take the element-wise kernel."""
+    import torch
+    dra, ver, tokens, flags = synth.verify_inputs(2, 24, V, 17, 0.2, seed=V)
+    ref = oracle_mod.verify(dra if mode == KL else None, ver, tokens, flags, mode, 0.5, 4, 1)
+
+    def off(bits):
+        big = torch.zeros(bits.size + 8, dtype=torch.bfloat16, device="cuda")
+        view = big[3:3 + bits.size].view(bits.shape)
+        view.copy_(to_torch_bf16(bits, "cuda"))
+        assert view.data_ptr() % 16 != 0
+        return view
+    out = dd.verify(off(dra) if mode == KL else None, off(ver), torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda(),
+                    mode, 0.5, 4, 1)
+    torch.cuda.synchronize()
+    assert dd.verify_status() == 0
+    check_verify(*(x.cpu().numpy() for x in out), ref, flags, tokens)
+
+
+# shapes on both sides of the line between the row kernel and the streaming kernel (23680 pieces of 1024 logits of
+# both tensors or 2048 of one on 148 SMs), rows on and off vector boundaries; in the streaming kernel rows cut
+# by range boundaries and grids of any size; in the row kernel clusters, CTAs, warps per row
+@pytest.mark.parametrize("B,P,V,flagged,mode", [
+    (2, 200, 65000, 150, KL), (2, 200, 65003, 150, KL),              # streaming
+    (4, 256, 65000, 40, CONF), (4, 256, 65003, 40, CONF | PROB),     # streaming
+    (1, 20, 126464, 20, KL | PROB), (1, 40, 65003, 33, KL), (2, 70, 40003, 60, CONF),   # clusters of eight, four and two
+    (1, 300, 20003, 77, KL), (4, 200, 9001, 150, KL), (6, 512, 4100, 100, KL), (24, 300, 1001, 100, CONF),   # 8, 4, 2 and 1 warps
+])
+def test_row_and_streaming_kernels(dd, oracle_mod, B, P, V, flagged, mode):
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=V + P)
+    hot = np.argmax(synth.bf16_bits_to_f32(ver[0, :1]), axis=1)
+    flags[0, 0] = 1
+    for row in ver.reshape(-1, V)[::7]:      # a token excluded by the verifier, somewhere
+        row[(int(hot[0]) + 5) % V] = 0xFF80
+    for row in dra.reshape(-1, V)[::7]:      # and by the drafter
+        row[(int(hot[0]) + 5) % V] = 0xFF80
+    _, _, whole = compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 9, 3)
+    try:
+        for cap in (1, 61):
+            dd.debug_set_max_ctas(cap)
+            got = run_gpu(dd, dra if (mode & 0xFF) == KL else None, ver, tokens, flags, mode, 0.5, 9, 3)
+            for a, b in zip(whole, got):
+                np.testing.assert_array_equal(a, b)
+    finally:
+        dd.debug_set_max_ctas(0)
+
+
+@pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 100, 299, 300, 301])
+def test_minimum_keep_with_many_equal_scores(dd, oracle_mod, k):
+    """300 rows of which many are the same: ties at every place of the order, kept lowest index first."""
+    dra, ver, tokens, flags = synth.verify_inputs(1, 300, 256, 300, 0.5, seed=3)
+    same = np.random.default_rng(k).integers(0, 12, size=300)
+    dra, ver = dra[:, same], ver[:, same]
+    for mode in (KL, CONF):
+        ref = oracle_mod.verify(dra if mode == KL else None, ver, tokens, flags, mode, 0.0 if mode == KL else 1.0, k, 0)
+        ot, om, osc = run_gpu(dd, dra if mode == KL else None, ver, tokens, flags, mode, 0.0 if mode == KL else 1.0, k, 0)
+        # equal rows have equal scores on either side, so the order is the same and so is the kept set
+        np.testing.assert_array_equal(om, ref["out_mask"])
+        np.testing.assert_array_equal(ot, ref["out_tokens"])
