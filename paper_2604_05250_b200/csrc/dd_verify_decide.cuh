@@ -324,8 +324,10 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
             sc = (float)fmax(kl, 0.0);
         }
     } else if (lane == 0) {
-        // the maximum's own term is 2^(m*log2e - M), not exactly 1
-        sc = (float)(exp2((double)bm_v * (double)kLog2e - (double)Mv) / sv);
+        // The maximum's own term is 2^d, d = m*log2e - M, not exactly 1: d is the rounding of M, so four terms of
+        // the series are exact in fp64 for |m| < 2^16 (a call of exp2 costs a microsecond at the end of a launch).
+        const double d = (double)bm_v * (double)kLog2e - (double)Mv, x = d * kLn2;
+        sc = (float)((fabs(d) < 0.00390625 ? 1.0 + x * (1.0 + x * (0.5 + x * (1.0 / 6.0))) : exp2(d)) / sv);
     }
     score = __shfl_sync(0xFFFFFFFFu, sc, 0);
     argmax = bidx;
