@@ -113,6 +113,22 @@ def load(path) -> ctypes.CDLL:
     return L
 
 
+try:
+    from . import _host_call as _fast        # the native form of the wrappers below (csrc/host_call.cpp)
+except ImportError:
+    _fast = None                             # not built: the Python form serves every call
+
+
+def _addresses(L):
+    """Addresses of the entry points that _fast calls, looked up once per library."""
+    try:
+        return L._dd_addresses
+    except AttributeError:
+        L._dd_addresses = {name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+                           for name in ("dd_bidir_attention", "dd_block_attention", "dd_verify", "dd_verify_static", "dd_unmask")}
+        return L._dd_addresses
+
+
 def _check(status: int):
     if status != DD_OK:
         L = lib()
@@ -125,8 +141,9 @@ def _check(status: int):
 # A call on small tensors is bound by what happens here, so the wrappers below check all tensors in one
 # expression and only go through _require, which words the error, when something is wrong; addresses and
 # the stream are passed as plain integers, and outputs are made like an input of the same shape.
-# (dd_verify on the tiny workload, host side of a call: 23.2 us before, 12.9 now; attention
-# 14.9 and 8.3.)
+# (dd_verify on the tiny workload, host side of a call: 23.2 us at first, 12.9 so; attention 14.9 and 8.3.)
+# Calls on device tensors on the current stream go through _fast, which does the same natively (5.7 us, the
+# launch itself included) and returns None for whatever it does not take, so that every error is worded here.
 
 _BF16, _I32, _U8, _F32 = torch.bfloat16, torch.int32, torch.uint8, torch.float32
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
@@ -164,6 +181,12 @@ def bidir_attention(q, k, v, out=None, scale=None, stream=None, host=False):
     """dd_bidir_attention (dd_bidir_attention_host if host=True).
 
     q, k, v: [B,H,N,D] torch.bfloat16.  Returns out (allocated if None)."""
+    if _fast is not None and stream is None and not host:
+        r = _fast.attention(_addresses(_lib or lib())["dd_bidir_attention"], q, k, v, out, scale)
+        if r is not None:
+            if type(r) is int:
+                _check(r)
+            return r
     shape = q.shape
     B, H, N, D = shape
     cuda = not host
@@ -190,6 +213,13 @@ def block_attention(q, k, v, kv_len=None, layout="bhnd", out=None, scale=None, s
     layout "bhnd": q [B,H,Nq,D], k, v [B,H,Nkv,D]; "bnhd": q [B,Nq,H,D], k, v [B,Nkv,H,D];
     torch.bfloat16 device tensors.  kv_len: int32 [B] device tensor (valid keys per sequence)
     or None.  Returns out (allocated if None), in the layout of q."""
+    if _fast is not None and stream is None and (layout == "bhnd" or layout == "bnhd"):
+        r = _fast.block(_addresses(_lib or lib())["dd_block_attention"], q, k, v, kv_len,
+                        DD_LAYOUT_BHND if layout == "bhnd" else DD_LAYOUT_BNHD, out, scale)
+        if r is not None:
+            if type(r) is int:
+                _check(r)
+            return r
     shape = q.shape
     if layout == "bhnd":
         B, H, Nq, D = shape
@@ -258,6 +288,13 @@ def verify(drafter_logits, verifier_logits, tokens, mask_flags, mode, tau, k, se
     nothing, if static_scratch=True and every output tensor is passed in).
 
     Returns (out_tokens int32 [B,P], out_mask uint8 [B,P], out_score float32 [B,P] or None)."""
+    if _fast is not None and stream is None and not host:
+        r = _fast.verify(_addresses(_lib or lib())["dd_verify_static" if static_scratch else "dd_verify"], drafter_logits,
+                         verifier_logits, tokens, mask_flags, mode, tau, k, seed, out_tokens, out_mask, out_score, want_score)
+        if r is not None:
+            if type(r) is int:
+                _check(r)
+            return r
     B, P, V = full = verifier_logits.shape
     cuda = not host
     if not _fits(verifier_logits, _BF16, full, cuda):
@@ -310,6 +347,12 @@ def unmask(logits, tokens, mask_flags, tau, k, out_tokens=None, out_mask=None, o
     """dd_unmask: one confidence-based unmasking step on logits [B,P,V] (device tensors).
 
     Returns (out_tokens int32 [B,P], out_mask uint8 [B,P] with 1 = still masked, out_conf float32 [B,P])."""
+    if _fast is not None and stream is None:
+        r = _fast.unmask(_addresses(_lib or lib())["dd_unmask"], logits, tokens, mask_flags, tau, k, out_tokens, out_mask, out_conf)
+        if r is not None:
+            if type(r) is int:
+                _check(r)
+            return r
     B, P, V = full = logits.shape
     if not _fits(logits, _BF16, full, True):
         _require(logits, _BF16, (B, P, V), True, "logits")

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> libdualdiff.so (sm_100a only)."""
+"""Builds in-tree: csrc/*.cu -> libdualdiff.so (sm_100a only), csrc/host_call.cpp -> _host_call.so (the
+native host side of the Python calls)."""
 from __future__ import annotations
 
 import glob
@@ -10,6 +11,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdualdiff.so")
+HOST_SRC = os.path.join(CSRC, "host_call.cpp")
+HOST = os.path.join(HERE, "_host_call.so")
 LIB_CHECK = os.path.join(HERE, "libdualdiff_check.so")      # the same sources with -DDD_BOUNDS_CHECK
 
 NVCC_FLAGS = [
@@ -46,7 +49,27 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if verbose:
             print(" ".join(cmd), flush=True)
         subprocess.run(cmd, check=True)
+    build_host(force, verbose)
     return LIB
+
+
+def build_host(force: bool = False, verbose: bool = False) -> str:
+    """The module behind binding.py's calls on device tensors: torch's headers and libraries, no CUDA code."""
+    if force or not os.path.exists(HOST) or os.path.getmtime(HOST) < os.path.getmtime(HOST_SRC):
+        import sysconfig
+
+        import torch
+        root = os.path.dirname(torch.__file__)
+        cuda = os.path.dirname(os.path.dirname(_nvcc()))
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"],
+               "-o", HOST, HOST_SRC, "-L" + os.path.join(root, "lib"),
+               "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
+        if verbose:
+            print(" ".join(cmd), flush=True)
+        subprocess.run(cmd, check=True)
+    return HOST
 
 
 def build_check(force: bool = False, verbose: bool = False) -> str:

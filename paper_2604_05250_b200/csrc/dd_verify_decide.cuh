@@ -325,7 +325,7 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
         }
     } else if (lane == 0) {
         // The maximum's own term is 2^d, d = m*log2e - M, not exactly 1: d is the rounding of M, so four terms of
-        // the series are exact in fp64 for |m| < 2^16 (a call of exp2 costs a microsecond at the end of a launch).
+        // the series give it to 2e-12 (a call of exp2 costs a microsecond at the end of a launch).
         const double d = (double)bm_v * (double)kLog2e - (double)Mv, x = d * kLn2;
         sc = (float)((fabs(d) < 0.00390625 ? 1.0 + x * (1.0 + x * (0.5 + x * (1.0 / 6.0))) : exp2(d)) / sv);
     }
