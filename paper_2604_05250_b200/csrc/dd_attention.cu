@@ -2,7 +2,8 @@
 // evaluated over the whole key range) for sm_100a, and dd_block_attention: the same
 // equation for a block of Nq queries against Nkv (cached) keys, with a per-sequence
 // number of valid keys and either memory layout.  One kernel serves both; two persistent forms of
-// it take many short items (see attention_impl).
+// it take many short items, and a form with one query tile and two CTAs per SM takes short query blocks and
+// problems too small to fill the chip, whose keys it splits over clusters (see attention_impl, split_parts).
 //
 // One CTA owns two tiles of 128 query rows of one (batch, head) and walks over
 // the keys in tiles of 128.  The CTA is warp-specialised:
@@ -610,6 +611,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 
 #include "dd_attention_persistent.cuh"
 #include "dd_attention_short.cuh"
+#include "dd_attention_split.cuh"
 
 // ---------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -634,12 +636,12 @@ EncodeTiledFn encode_fn()
 // dimension) or of a [B,N,H,D] tensor as (D, N, H, B); box = 64 columns x 128 rows x 1 (x 1),
 // 128-byte swizzle, zero fill: a tile never reaches into the next head or sequence, and rows
 // past N read as zero / are not written.
-int make_tmap(CUtensorMap *m, const void *base, int B, int H, int N, int D, bool head_major)
+int make_tmap(CUtensorMap *m, const void *base, int B, int H, int N, int D, bool head_major, int box_rows = 128)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return dd::cuda_fail(cudaErrorSymbolNotFound, "cuTensorMapEncodeTiled entry point");
     const cuuint64_t row = (cuuint64_t)D * 2;
-    const cuuint32_t box[4] = {64, 128, 1, 1};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r;
     if (head_major) {
@@ -704,6 +706,38 @@ int launch_persistent(Kernel kernel, int smem, bool (&attr_done)[64], const Attn
     return DD_OK;
 }
 
+// Short query blocks: `parts` CTAs (a cluster) per head and tile of 128 query rows.
+template <int D>
+int launch_split(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const AttnParams &p, int q_rows, int parts,
+                 cudaStream_t s)
+{
+    static bool attr_done[64] = {};
+    static std::mutex attr_mu;
+    int dev = 0;
+    DD_CUDA_TRY(cudaGetDevice(&dev));
+    {
+        std::lock_guard<std::mutex> lock(attr_mu);
+        if (dev >= 0 && dev < 64 && !attr_done[dev]) {
+            DD_CUDA_TRY(cudaFuncSetAttribute(attention_split_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
+            attr_done[dev] = true;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((long)p.BH * p.m_blocks * parts));
+    cfg.blockDim = dim3(kSplitThreads);
+    cfg.dynamicSmemBytes = kSplitSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute cluster;
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = (unsigned)parts;
+    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = parts > 1 ? 1 : 0;
+    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_split_kernel<D>, tq, tk, tv, p, q_rows, parts));
+    dd::count_launch();
+    return DD_OK;
+}
+
 int sm_count(int *out)
 {
     static int cached[64] = {};
@@ -715,6 +749,34 @@ int sm_count(int *out)
     if (cached[dev] == 0) DD_CUDA_TRY(cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev));
     *out = cached[dev];
     return DD_OK;
+}
+
+// How many CTAs of attention_split_kernel share one query tile's keys; 0: one of the other kernels is faster.
+// `tiles`: query tiles of 128 rows over all heads.  Figures in us on 148 SMs at D = 128, head-major, this
+// kernel : attention_kernel; n: key tiles.
+//   * More tiles than SMs, one per head: a CTA per tile, two on an SM.  Two of them take 1.2 (short keys) to 1.9
+//     times (long ones) as long as one CTA of attention_kernel with the SM to itself, so from n = 9 on waves are
+//     compared, and beyond 16 there is nothing to win.  32 queries, n = 2: 256 heads 10.9 : 15.1; n = 8: 176 heads
+//     22.3 : 27.5, 256 26.3 : 30.2, 400 44.7 : 44.8 (two waves to three), 512 47.7 : 57.7; n = 16: 256 heads 45.7 :
+//     50.1, 400 87 : 78, 512 89 : 101; n = 32, unequal lengths: 296 heads 81.5 : 77.9, 1024 242 : 239.
+//   * Too few tiles to fill the chip: eight CTAs a tile while that leaves an SM to each, four up to two on an SM, two
+//     beyond that (only heads of several tiles, of which attention_kernel gives a CTA two).  32 queries: 8 heads,
+//     n = 32 14.7 : 31.3, n = 16 11.6 : 18.3; 32 heads, n = 32 21.5 : 32.7, n = 8 10.6 : 12.0; 64 heads, n = 16 19.4 :
+//     20.3, n = 8 13.7 : 12.8.  128 queries (a ring of two tiles): 32 heads, n = 16 17.4 : 19.6, n = 8 13.5 : 12.4; 64
+//     heads, n = 32 33.3 : 35.2, n = 16 23.3 : 21.1.  256 queries: 8 heads, n = 8 12.5 : 18.5; 32 heads, n = 8 17.2 :
+//     19.1; 64 heads, n = 16 29.4 : 34.0, n = 8 21.5 : 20.4.  With two key tiles a part or fewer the meeting of the
+//     parts (some 3 us) is hardly earned back.
+int split_parts(long tiles, int nkv, int Nq, int sms)
+{
+    if (tiles > sms && Nq <= kBlockM) {
+        const long waves = (tiles + sms - 1) / sms, waves2 = (tiles + 2 * sms - 1) / (2 * sms);
+        return nkv > 1 && nkv <= 16 && (nkv <= 8 || 9 * waves2 < 5 * waves) ? 1 : 0;
+    }
+    int parts = tiles * 8 <= sms ? 8 : tiles * 4 <= 2 * sms ? 4 : tiles <= sms && Nq > kBlockM ? 2 : 0;
+    if (parts == 8 && nkv < 16) parts = 4;
+    const bool roomy = tiles * parts <= sms;
+    const int least = Nq > kBlockM ? (parts == 2 ? 16 : 8) : Nq > 64 ? (roomy ? 16 : 32) : roomy ? 8 : 16;
+    return nkv >= least ? parts : 0;
 }
 
 int attention_impl(const void *q, const void *k, const void *v, void *out, int B, int H, int Nq, int Nkv, int D,
@@ -742,10 +804,8 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     }
     const bool head_major = layout == DD_LAYOUT_BHND;
     CUtensorMap tq, tk, tv, to;
-    if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
     if ((rc = make_tmap(&tk, k, B, H, Nkv, D, head_major)) != DD_OK) return rc;
     if ((rc = make_tmap(&tv, v, B, H, Nkv, D, head_major)) != DD_OK) return rc;
-    if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
 
     AttnParams p;
     p.BH = (int)BH; p.H = H; p.Nq = Nq; p.Nkv = Nkv; p.D = D;
@@ -758,6 +818,18 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     p.out = out;
     cudaStream_t s = (cudaStream_t)stream;
     const bool general = kv_len != nullptr || !head_major || Nq != Nkv;
+    int sms = 0;
+    if ((rc = sm_count(&sms)) != DD_OK) return rc;
+    const int nkv = (Nkv + kBlockN - 1) / kBlockN;
+    const long tiles = BH * ((Nq + kBlockM - 1) / kBlockM);
+    if (const int parts = split_parts(tiles, nkv, Nq, sms)) {
+        const int q_rows = Nq <= 64 ? 64 : 128;
+        if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major, q_rows)) != DD_OK) return rc;
+        p.m_blocks = (Nq + kBlockM - 1) / kBlockM;
+        return D == 64 ? launch_split<64>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128>(tq, tk, tv, p, q_rows, parts, s);
+    }
+    if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
+    if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
     if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
     // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in every item):
     // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four key tiles or
@@ -765,9 +837,6 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     // 87 with the short kernel, 81 with this one; of 1024 299, 313 and 276).  Two key tiles, and D = 64: the short
     // kernel (64 x 32 heads of 256 tokens at D = 128: 148, 99 and 113; 16 x 32 of 512 at D = 64: 73, 61 and 63).
     // Items of one query tile among those of two: a CTA per item (3 x 24 heads of 1357: 80 against 89).
-    int sms = 0;
-    if ((rc = sm_count(&sms)) != DD_OK) return rc;
-    const int nkv = (Nkv + kBlockN - 1) / kBlockN;
     if (BH * m_blocks > sms && nkv <= 16 && (Nq - 1) % (kQTiles * kBlockM) >= kBlockM) {
         static bool attr_done[3][64] = {};
         if (D == 64)

@@ -194,3 +194,45 @@ def test_drafter_shape_full_size(dd, oracle_mod, layout):
         q, k, v = (np.ascontiguousarray(a.transpose(0, 2, 1, 3)) for a in (q, k, v))
     got = run_gpu(dd, q, k, v, D ** -0.5, kv_len=kv_len, layout=layout)
     check_attention(got, oracle_mod.block_attention(q, k, v, D ** -0.5, kv_len=kv_len, layout=layout))
+
+
+# The kernel for one query tile per CTA: keys shared by 2, 4 and 8 CTAs of a cluster (parts of unequal
+# length, and without a tile where a sequence is short), both sizes of the query buffer (up to 64 rows and up
+# to 128), a last query tile that is not full, and more items than SMs, where no keys are shared.
+@pytest.mark.parametrize("B,H,Nq,Nkv,D,kv_len", [
+    (2, 4, 1, 2050, 128, [2050, 700]), (2, 3, 64, 4096, 64, [4095, 1]), (1, 8, 65, 2048, 128, None),
+    (3, 8, 33, 1100, 128, [1100, 0, 129]), (2, 8, 130, 1000, 64, [900, 128]), (1, 8, 600, 1030, 128, None),
+    (2, 32, 150, 2048, 64, [64, 2048]), (10, 16, 5, 300, 128, [300, 0, 1, 127, 128, 129, 256, 257, 299, 300]),
+    (6, 32, 128, 260, 64, [260, 3, 128, 0, 250, 129]),
+])
+@pytest.mark.parametrize("layout", ["bhnd", "bnhd"])
+def test_one_query_tile_per_cta(dd, oracle_mod, B, H, Nq, Nkv, D, kv_len, layout):
+    q, k, v = block_inputs(B, H, Nq, Nkv, D, 300 + Nq)
+    if kv_len is not None:
+        kv_len = np.array(kv_len, dtype=np.int32)
+        for b in range(B):                          # what lies behind the keys is not read as numbers
+            k[b, :, kv_len[b]:] = 0x7FC0
+            v[b, :, kv_len[b]:] = 0xFF80
+    ref = oracle_mod.block_attention(q, k, v, D ** -0.5, kv_len=kv_len)
+    if layout == "bnhd":
+        q, k, v, ref = (np.ascontiguousarray(a.transpose(0, 2, 1, 3)) for a in (q, k, v, ref))
+    got = run_gpu(dd, q, k, v, D ** -0.5, kv_len=kv_len, layout=layout)
+    check_attention(got, ref)
+    np.testing.assert_array_equal(run_gpu(dd, q, k, v, D ** -0.5, kv_len=kv_len, layout=layout), got)
+
+
+def test_split_keys_with_peaked_rows_and_an_output_on_16_bytes(dd, oracle_mod):
+    """The parts' reference points differ by far more than the step between two rescalings, and the output
+    starts on a 16-byte boundary that is not one of 32 bytes."""
+    import torch
+    q, k, v = block_inputs(1, 4, 40, 2000, 128, 7)
+    for t, f in ((0, 0.1), (700, 4.0), (1500, 8.0)):                 # later keys outweigh earlier ones, and the first part nothing
+        k[:, :, t:t + 500] = synth.f32_to_bf16_bits(synth.bf16_bits_to_f32(k[:, :, t:t + 500]) * np.float32(f))
+    tq, tk, tv = (to_torch_bf16(x, "cuda") for x in (q, k, v))
+    buf = torch.empty(tq.numel() + 8, dtype=torch.bfloat16, device="cuda")
+    out = buf[8:].view(tq.shape)
+    dd.block_attention(tq, tk, tv, out=out, scale=0.2)
+    torch.cuda.synchronize()
+    assert dd.attention_status() == 0
+    assert out.data_ptr() % 32 == 16
+    check_attention(bf16_tensor_to_f64(out), oracle_mod.block_attention(q, k, v, 0.2), stress=True)
