@@ -72,6 +72,7 @@ struct AttnParams {
     float scale_log2;          // scale * log2(e)
     unsigned int *status;      // health word of the attention kernel on this device
     unsigned int *mirror;      // its copy in mapped host memory (written only when a wait expires)
+    int longest_first;         // 1: sequences by falling number of keys (kv_len given; see attention_impl)
     void *out;                 // where attention_persistent_kernel stores its result (the others through a tensor map)
 };
 
@@ -249,6 +250,29 @@ __device__ __forceinline__ void columns_to_staging(const uint32_t *acc, float f,
     }
 }
 
+// The sequence that the `pos`-th group of CTAs works on, and how many keys it has.  With p.longest_first the
+// sequences of unequal length are taken longest first (within runs of 32, by key tiles; ties in order), so that the
+// launch does not end with a long one that began late.  Every warp finds this out for itself: 32 lengths are one
+// load, and a lane's place is the number of lanes with a longer one.
+__device__ __forceinline__ int sequence_at(const AttnParams &p, int pos, int &keys)
+{
+    auto clamped = [&](int b) { return min(max(p.kv_len[b], 0), p.Nkv); };
+    if (!p.kv_len) { keys = p.Nkv; return pos; }
+    if (!p.longest_first) { keys = clamped(pos); return pos; }
+    const int lane = threadIdx.x & 31, run = pos & ~31, B = p.BH / p.H;
+    const int n = min(32, B - run);
+    const int own = lane < n ? clamped(run + lane) : -1;
+    const int tiles = (own + kBlockN - 1) / kBlockN;             // 0 for a lane without a sequence, as for an empty one
+    int place = 0;
+    for (int i = 0; i < n; ++i) {
+        const int other = __shfl_sync(0xFFFFFFFFu, tiles, i);
+        place += other > tiles || (other == tiles && i < lane);
+    }
+    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, lane < n && place == (pos & 31))) - 1;
+    keys = __shfl_sync(0xFFFFFFFFu, own, src);
+    return run + src;
+}
+
 // kBlock = false: the square, head-major, unpadded case of dd_bidir_attention with nothing of the
 // general case compiled in.
 template <int D, bool kBlock>
@@ -275,17 +299,18 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(smem_gen + Smem<D>::kTmemSlot);
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
-    const int bh = blockIdx.x / p.m_blocks;
-    const int mb = blockIdx.x - bh * p.m_blocks;
+    const int head = blockIdx.x / p.m_blocks;
+    const int mb = blockIdx.x - head * p.m_blocks;
     const int row0 = mb * (kQTiles * kBlockM);
-    const int b_idx = kBlock ? bh / p.H : 0, h_idx = kBlock ? bh - b_idx * p.H : 0;
+    int keys = p.Nkv;                                     // keys that exist
+    const int b_idx = kBlock ? sequence_at(p, head / p.H, keys) : 0, h_idx = kBlock ? head % p.H : 0;
+    const int bh = kBlock ? b_idx * p.H + h_idx : head;
     const bool hm = !kBlock || p.head_major != 0;
     // one tile of 128 rows x 64 columns of head (b_idx, h_idx), rows from n0
     auto load_box = [&](uint32_t dst, const CUtensorMap *tm, uint32_t bar, int c0, int n0) {
         if (hm) tma_load_3d(dst, tm, bar, c0, n0, bh);
         else tma_load_4d(dst, tm, bar, c0, n0, h_idx, b_idx);
     };
-    const int keys = (kBlock && p.kv_len) ? min(max(p.kv_len[b_idx], 0), p.Nkv) : p.Nkv;   // keys that exist
     const int nkv = (keys + kBlockN - 1) / kBlockN;       // 0: the sequence has no key, the output is zero
     const int ntiles = (p.Nq - row0 > kBlockM) ? 2 : 1;   // query tiles of this CTA that hold rows
     // A CTA with a single query tile (a short query block) gives its key tiles to the two softmax
@@ -816,20 +841,28 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     p.status = ctx->attn_status;
     p.mirror = ctx->mirror_dev;
     p.out = out;
+    p.longest_first = 0;
     cudaStream_t s = (cudaStream_t)stream;
     const bool general = kv_len != nullptr || !head_major || Nq != Nkv;
     int sms = 0;
     if ((rc = sm_count(&sms)) != DD_OK) return rc;
     const int nkv = (Nkv + kBlockN - 1) / kBlockN;
+    // Sequences of unequal length, longest first: where the launch takes more than one round of CTAs and no more than
+    // two, what starts in the second is then short (16 x 32 heads, 32 queries over 256-1024 keys: 45.0 -> 41.6 us; 8 x
+    // 32 heads, 256 queries over 512-2048: 66.7 -> 62.0).  With more rounds, CTAs of equal length start and end
+    // together, which costs more (20 x 32 heads of the former 51.1 -> 55.0, 64 x 32 151 -> 156).
+    auto longest_first = [&](long ctas, long at_a_time) { return kv_len && B > 1 && ctas > at_a_time && ctas <= 2 * at_a_time; };
     const long tiles = BH * ((Nq + kBlockM - 1) / kBlockM);
     if (const int parts = split_parts(tiles, nkv, Nq, sms)) {
         const int q_rows = Nq <= 64 ? 64 : 128;
         if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major, q_rows)) != DD_OK) return rc;
         p.m_blocks = (Nq + kBlockM - 1) / kBlockM;
+        p.longest_first = longest_first(tiles * parts, 2 * sms);
         return D == 64 ? launch_split<64>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128>(tq, tk, tv, p, q_rows, parts, s);
     }
     if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
     if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
+    p.longest_first = longest_first(BH * m_blocks, sms);
     if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
     // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in every item):
     // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four key tiles or

@@ -69,12 +69,12 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int item = (int)blockIdx.x / parts, part = (int)blockIdx.x - item * parts;
-    const int bh = item / p.m_blocks, row0 = (item - bh * p.m_blocks) * kBlockM;
-    const int b_idx = bh / p.H, h_idx = bh - b_idx * p.H;
+    const int head = item / p.m_blocks, row0 = (item - head * p.m_blocks) * kBlockM;
+    int keys;
+    const int b_idx = sequence_at(p, head / p.H, keys), h_idx = head % p.H, bh = b_idx * p.H + h_idx;
     const bool hm = p.head_major != 0;
     const int rows = min(p.Nq - row0, kBlockM);                   // query rows of this tile (>= 1)
     const int row_warps = (rows + 31) / 32;
-    const int keys = p.kv_len ? min(max(p.kv_len[b_idx], 0), p.Nkv) : p.Nkv;
     const int nkv = (keys + kBlockN - 1) / kBlockN;
     const int j_begin = part * nkv / parts, n_tiles = (part + 1) * nkv / parts - j_begin;      // key tiles of this CTA
     auto load_box = [&](uint32_t dst, const CUtensorMap *tm, uint32_t bar, int c0, int n0) {

@@ -236,3 +236,23 @@ def test_split_keys_with_peaked_rows_and_an_output_on_16_bytes(dd, oracle_mod):
     assert dd.attention_status() == 0
     assert out.data_ptr() % 32 == 16
     check_attention(bf16_tensor_to_f64(out), oracle_mod.block_attention(q, k, v, 0.2), stress=True)
+
+
+# Sequences of unequal length taken longest first (more CTAs than fit at a time, no more than twice as many):
+# fewer than a run of 32 sequences, a whole one, and one more than a run; ties, empty and clamped lengths.
+@pytest.mark.parametrize("B,H,Nq,Nkv", [(20, 16, 4, 260), (32, 12, 7, 200), (33, 10, 3, 300), (40, 4, 140, 257)])
+def test_sequences_taken_longest_first(dd, oracle_mod, B, H, Nq, Nkv):
+    q, k, v = block_inputs(B, H, Nq, Nkv, 64, 500 + B)
+    rng = np.random.default_rng(B)
+    kv_len = rng.integers(0, Nkv + 1, B).astype(np.int32)
+    kv_len[:4] = [0, Nkv, 128, 128]
+    kv_len[-1] = Nkv
+    passed = kv_len.copy()
+    passed[1] = Nkv + 50
+    passed[0] = -7
+    for layout in ("bhnd", "bnhd"):
+        ref = oracle_mod.block_attention(q, k, v, 0.125, kv_len=kv_len)
+        a = [q, k, v, ref]
+        if layout == "bnhd":
+            a = [np.ascontiguousarray(x.transpose(0, 2, 1, 3)) for x in a]
+        check_attention(run_gpu(dd, *a[:3], 0.125, kv_len=passed, layout=layout), a[3])
