@@ -129,12 +129,12 @@ __device__ __forceinline__ float2 ex2_poly(float2 x)
 }
 
 // Row maximum of the raw scores of one key tile (keys past the sequence end excluded).
-template <bool kMasked>
-__device__ __forceinline__ float row_max(const float (&s)[kBlockN], int valid)
+template <bool kMasked, int N>
+__device__ __forceinline__ float row_max(const float (&s)[N], int valid)
 {
     float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int i = 0; i < kBlockN; i += 8)
+    for (int i = 0; i < N; i += 8)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int e = i + 2 * u;
@@ -152,8 +152,8 @@ __device__ __forceinline__ float row_max(const float (&s)[kBlockN], int valid)
 // columns); adds the weights as rounded to sum_a + sum_b, so that O / l is an exact convex combination.  Two
 // values per instruction where the hardware has a packed form; one pair in kPoly (0: none) goes to the
 // FMA pipe.
-template <bool kMasked, int kPoly>
-__device__ __forceinline__ void weights_to_tmem(const float (&s)[kBlockN], int q, int valid, float c, float m_ref,
+template <bool kMasked, int kPoly, int N>
+__device__ __forceinline__ void weights_to_tmem(const float (&s)[N], int q, int valid, float c, float m_ref,
                                                 uint32_t tmem_p, float2 &sum_a, float2 &sum_b)
 {
     const float2 c2 = make_float2(c, c), nm2 = make_float2(-m_ref, -m_ref);
@@ -179,6 +179,30 @@ __device__ __forceinline__ void weights_to_tmem(const float (&s)[kBlockN], int q
     tmem_st16(tmem_p + q * 16, pk);
 }
 
+// A key tile with maximum mx (times scale) meets a row: the first tile sets the row's reference point, a later one
+// moves it if it outgrows it by more than the allowed step; then O is rescaled in tensor memory.
+template <int D>
+__device__ __forceinline__ void move_reference(uint32_t tO, bool first, float mx, float &m_ref, float &l_run)
+{
+    if (first) {
+        m_ref = mx;
+    } else if (__any_sync(0xffffffffu, mx > m_ref + kRescaleStep)) {
+        const float m_new = mx > m_ref + kRescaleStep ? mx : m_ref;
+        const float alpha = ex2(m_ref - m_new);       // 1 where the row does not move
+        m_ref = m_new;
+        l_run *= alpha;
+#pragma unroll
+        for (int cb = 0; cb < D / 32; ++cb) {
+            uint32_t r[32];
+            tmem_ld32(tO + cb * 32, r);
+            tmem_wait_ld(r);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+            tmem_st32(tO + cb * 32, r);
+        }
+    }
+}
+
 // One key tile of one query row, shared by both attention kernels: reads the row's 128 scores from tensor
 // memory (the S product has completed), moves the row's reference point if the tile's maximum outgrows
 // it by more than the allowed step (the first tile sets it), and writes the weights over S.  They are handed
@@ -197,23 +221,7 @@ __device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, bool firs
     tmem_wait_ld();
     const bool masked = valid < kBlockN;
     const float mx = (masked ? row_max<true>(s, valid) : row_max<false>(s, valid)) * c;
-    if (first) {
-        m_ref = mx;
-    } else if (__any_sync(0xffffffffu, mx > m_ref + kRescaleStep)) {
-        const float m_new = mx > m_ref + kRescaleStep ? mx : m_ref;
-        const float alpha = ex2(m_ref - m_new);       // 1 where the row does not move
-        m_ref = m_new;
-        l_run *= alpha;
-#pragma unroll
-        for (int cb = 0; cb < D / 32; ++cb) {
-            uint32_t r[32];
-            tmem_ld32(tO + cb * 32, r);
-            tmem_wait_ld(r);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-            tmem_st32(tO + cb * 32, r);
-        }
-    }
+    move_reference<D>(tO, first, mx, m_ref, l_run);
     float2 sum_a = make_float2(0.f, 0.f), sum_b = sum_a;
     auto weights = [&](auto is_masked, auto poly) {
 #pragma unroll
@@ -732,7 +740,7 @@ int launch_persistent(Kernel kernel, int smem, bool (&attr_done)[64], const Attn
 }
 
 // Short query blocks: `parts` CTAs (a cluster) per head and tile of 128 query rows.
-template <int D>
+template <int D, int G>
 int launch_split(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const AttnParams &p, int q_rows, int parts,
                  cudaStream_t s)
 {
@@ -743,7 +751,7 @@ int launch_split(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap
     {
         std::lock_guard<std::mutex> lock(attr_mu);
         if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-            DD_CUDA_TRY(cudaFuncSetAttribute(attention_split_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
+            DD_CUDA_TRY(cudaFuncSetAttribute(attention_split_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
             attr_done[dev] = true;
         }
     }
@@ -758,7 +766,7 @@ int launch_split(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap
     cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
     cfg.attrs = &cluster;
     cfg.numAttrs = parts > 1 ? 1 : 0;
-    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_split_kernel<D>, tq, tk, tv, p, q_rows, parts));
+    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_split_kernel<D, G>, tq, tk, tv, p, q_rows, parts));
     dd::count_launch();
     return DD_OK;
 }
@@ -854,11 +862,15 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     auto longest_first = [&](long ctas, long at_a_time) { return kv_len && B > 1 && ctas > at_a_time && ctas <= 2 * at_a_time; };
     const long tiles = BH * ((Nq + kBlockM - 1) / kBlockM);
     if (const int parts = split_parts(tiles, nkv, Nq, sms)) {
-        const int q_rows = Nq <= 64 ? 64 : 128;
-        if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major, q_rows)) != DD_OK) return rc;
+        // copies of the query rows in a tile (see attention_split_kernel)
+        const int copies = Nq > 32 ? 1 : D == 64 ? 4 : 2;
+        const int q_rows = copies > 1 ? 32 * copies : Nq <= 64 ? 64 : 128;
+        if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major, copies > 1 ? 32 : q_rows)) != DD_OK) return rc;
         p.m_blocks = (Nq + kBlockM - 1) / kBlockM;
         p.longest_first = longest_first(tiles * parts, 2 * sms);
-        return D == 64 ? launch_split<64>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128>(tq, tk, tv, p, q_rows, parts, s);
+        if (copies > 1)
+            return D == 64 ? launch_split<64, 4>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128, 2>(tq, tk, tv, p, q_rows, parts, s);
+        return D == 64 ? launch_split<64, 1>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128, 1>(tq, tk, tv, p, q_rows, parts, s);
     }
     if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
     if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;

@@ -4,7 +4,7 @@
 //   warps 0-3   softmax (thread = query row = TMEM lane); warps without a query row sit out
 //   warp  4     one thread feeds a ring of K/V tiles by TMA
 //   warp  5     one thread issues every tcgen05 MMA
-//   warps 6-7   only fill the register-allocation group
+//   warps 6-7   clear the value rows behind a sequence's end
 // The parts of a split item meet at the end: every CTA leaves its accumulator in fp32 (the ring's memory,
 // which no copy or product uses any more) and its rows' reference points and sums in its own shared memory,
 // and after a cluster barrier each CTA combines its share of the columns over distributed shared memory, in
@@ -14,8 +14,9 @@
 // What bounds it.  One tile's chain (copy -> S -> softmax -> P V, some 2600 cycles a key tile, and 4-5 us of start and
 // end) keeps neither the memory nor the tensor core busy; the SM's other CTA fills in.  attention_kernel has an SM to
 // itself with two query tiles' worth of shared memory and, for a single tile, both softmax groups on it: faster for one
-// item, but the next one's start is exposed.  16 sequences x 32 heads, 32 queries over 256-1024 keys: 49.7 -> 43.5 us;
-// 64 x 32 heads 174.8 -> 134.7; 40 x 16 heads of 200 keys at D = 64 30.0 -> 21.7.  Where there are few items the
+// item, but the next one's start is exposed.  16 sequences x 32 heads, 32 queries over 256-1024 keys: 49.7 -> 43.5 us
+// (before copies and order, below and in sequence_at: 37.7 now); 64 x 32 heads 174.8 -> 134.7; 40 x 16 heads of up to 200
+// keys at D = 64 30.0 -> 21.7.  Where there are few items the
 // splitting is what counts: 2 x 8 heads, 16 queries over 4096 keys 32.3 -> 17.0 us.  Built and not faster: persistent
 // CTAs that take the next item over from the launch queue (clusterlaunchcontrol) and load it behind the current
 // one's tiles, 51 against 43.5 and 160 against 135 us.
@@ -36,15 +37,55 @@ struct SplitLayout {
     static __host__ __device__ constexpr int q_bytes(int q_rows) { return q_rows * D * 2; }
     static __host__ __device__ constexpr int slots(int q_rows) { return (112 * 1024 - q_bytes(q_rows)) / kTileBytes; }
     static constexpr int kMaxSlots = (112 * 1024 - 64 * D * 2) / kTileBytes;
-    // q_full, s_full, p_early, p_full, o_full, kv_full[], kv_empty[]
-    static constexpr int kNumBars = 5 + 2 * kMaxSlots;
+    // q_full, s_full, p_early, p_full, o_full, v_last, v_clear, kv_full[], kv_empty[]
+    static constexpr int kFixedBars = 7;
+    static constexpr int kNumBars = kFixedBars + 2 * kMaxSlots;
     static constexpr int kBarBytes = 8 * kNumBars + 16;
     static_assert(kBarBytes <= 256, "barriers fit whichever side of the tiles the alignment leaves free");
     static_assert(slots(128) * kTileBytes >= 128 * D * 4, "the ring holds a whole accumulator in fp32");
-    static_assert(q_bytes(64) >= 128 * 8, "the query buffer holds the rows' reference points and sums");
+    static_assert(q_bytes(64) >= 2 * 128 * 8, "the query buffer holds the rows' reference points and sums");
 };
 
-template <int D>
+// softmax_tile for a row that takes only the tile's keys key0 .. key0 + K - 1: weight zero for the others.
+template <int D, int K>
+__device__ __forceinline__ void softmax_part(uint32_t tS, uint32_t tO, int key0, bool first, int valid, float c, float &m_ref,
+                                             float &l_run)
+{
+    float s[K];
+#pragma unroll
+    for (int cb = 0; cb < K / 32; ++cb)
+        tmem_ld32(tS + key0 + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[cb * 32]));
+    tmem_wait_ld();
+    const int own = valid - key0;
+    const bool masked = own < K;
+    const float mx = own <= 0 ? -INFINITY : (masked ? row_max<true>(s, own) : row_max<false>(s, own)) * c;
+    move_reference<D>(tO, first, mx, m_ref, l_run);
+    float2 sum_a = make_float2(0.f, 0.f), sum_b = sum_a;
+    auto weights = [&](auto is_masked, auto poly) {
+#pragma unroll
+        for (int q = 0; q < K / 32; ++q)
+            weights_to_tmem<decltype(is_masked)::value, decltype(poly)::value>(s, q, own, c, m_ref, tS + key0 / 2, sum_a, sum_b);
+    };
+    if (masked) weights(std::true_type(), std::integral_constant<int, 0>());
+    else weights(std::false_type(), std::integral_constant<int, kPolyOneIn<D>>());
+    uint32_t zero[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) zero[i] = 0u;
+#pragma unroll
+    for (int q = 0; q < kBlockN / 32; ++q)
+        if (q * 32 < key0 || q * 32 >= key0 + K) tmem_st16(tS + q * 16, zero);
+    sum_a = __fadd2_rn(sum_a, sum_b);
+    l_run += sum_a.x + sum_a.y;
+}
+
+// G > 1 (up to 32 query rows): the query tile holds G copies of them, one above the other, and copy g (one warp)
+// takes the g-th part of every tile's keys, with weight zero for the others and an accumulator, reference point and
+// sum of its own; the copies are combined at the end like the parts of a cluster.  A tile's softmax is then the work
+// of G warps instead of one, and so is the masked tile at a sequence's end: 16 x 32 heads, 32 queries over 256-1024
+// keys 42.3 -> 37.7 us, 64 x 32 157.8 -> 130.2, 50 x 32 with one query over 125-500 75.7 -> 59.6, 40 x 16 over 50-200
+// at D = 64 22.3 -> 15.4; whole tiles only: 64 x 8 over 1024 51.2 -> 47.8.  Two copies at D = 128, where a fourth of
+// the buffer's rows would cost a key tile, four at D = 64.
+template <int D, int G>
 __global__ void __launch_bounds__(kSplitThreads, 2)
 attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const AttnParams p, const int q_rows, const int parts)
@@ -61,9 +102,10 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     unsigned char *bars_gen = pad >= 256 ? smem_dyn : tiles_gen + 112 * 1024;
     const uint32_t bars = smem_u32(bars_gen);
     const int slots = L::slots(q_rows);
-    const uint32_t bar_q = bars, bar_s_full = bars + 8, bar_p_early = bars + 16, bar_p_full = bars + 24, bar_o_full = bars + 32;
-    auto bar_kv_full = [&](int s) { return bars + 8u * (5 + s); };
-    auto bar_kv_empty = [&](int s) { return bars + 8u * (5 + L::kMaxSlots + s); };
+    const uint32_t bar_q = bars, bar_s_full = bars + 8, bar_p_early = bars + 16, bar_p_full = bars + 24, bar_o_full = bars + 32,
+                   bar_v_last = bars + 40, bar_v_clear = bars + 48;
+    auto bar_kv_full = [&](int s) { return bars + 8u * (L::kFixedBars + s); };
+    auto bar_kv_empty = [&](int s) { return bars + 8u * (L::kFixedBars + L::kMaxSlots + s); };
     const uint32_t tmem_slot = bars + 8u * L::kNumBars;
     volatile uint32_t *tmem_slot_gen = reinterpret_cast<volatile uint32_t *>(bars_gen + 8 * L::kNumBars);
 
@@ -75,17 +117,23 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const bool hm = p.head_major != 0;
     const int rows = min(p.Nq - row0, kBlockM);                   // query rows of this tile (>= 1)
     const int row_warps = (rows + 31) / 32;
+    const int soft_warps = G > 1 ? G : row_warps;                 // softmax warps at work
     const int nkv = (keys + kBlockN - 1) / kBlockN;
     const int j_begin = part * nkv / parts, n_tiles = (part + 1) * nkv / parts - j_begin;      // key tiles of this CTA
     auto load_box = [&](uint32_t dst, const CUtensorMap *tm, uint32_t bar, int c0, int n0) {
         if (hm) tma_load_3d(dst, tm, bar, c0, n0, bh);
         else tma_load_4d(dst, tm, bar, c0, n0, h_idx, b_idx);
     };
-    auto load_tile = [&](int slot, const CUtensorMap *tm, int j) {
-        mbar_expect_tx(bar_kv_full(slot), kTileBytes);
+    // Keys past the sequence's end have weight zero, but 0 x NaN is NaN in the product P V, and padding may
+    // hold any bit pattern: the last value tile's rows behind the end are cleared before the product reads it, by
+    // warps 6-7, which wait for this tile on a barrier of its own.  (Rows past the end of the tensor were zero-filled
+    // by the copy.)  The softmax warps doing it behind their weights: 1-3 % slower on sequences of a few tiles.
+    const bool clear = n_tiles > 0 && j_begin + n_tiles == nkv && keys % kBlockN != 0 && keys < p.Nkv;
+    auto load_tile = [&](int slot, const CUtensorMap *tm, int j, bool last_v) {
+        const uint32_t bar = last_v ? bar_v_last : bar_kv_full(slot);
+        mbar_expect_tx(bar, kTileBytes);
 #pragma unroll
-        for (int cx = 0; cx < kBoxes; ++cx)
-            load_box(sRing + slot * kTileBytes + cx * kBoxBytes, tm, bar_kv_full(slot), cx * 64, j * kBlockN);
+        for (int cx = 0; cx < kBoxes; ++cx) load_box(sRing + slot * kTileBytes + cx * kBoxBytes, tm, bar, cx * 64, j * kBlockN);
     };
 
     // The producer thread sets up the barriers its copies complete on and sends the query tile, the first key
@@ -93,22 +141,27 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     if (warp == kSplitLoadWarp && elect_one()) {
         prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
         mbar_init(bar_q, 1);
+        mbar_init(bar_v_last, 1);
         for (int s = 0; s < slots; ++s) mbar_init(bar_kv_full(s), 1);
         fence_mbar_init();
         if (n_tiles > 0) {
             mbar_expect_tx(bar_q, (uint32_t)L::q_bytes(q_rows));
 #pragma unroll
-            for (int cx = 0; cx < kBoxes; ++cx) load_box(sQ + cx * (q_rows * 128), &tm_q, bar_q, cx * 64, row0);
-            load_tile(0, &tm_k, j_begin);
-            load_tile(1, &tm_v, j_begin);
+            for (int cx = 0; cx < kBoxes; ++cx)
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    load_box(sQ + cx * (q_rows * 128) + g * (32 * 128), &tm_q, bar_q, cx * 64, row0);
+            load_tile(0, &tm_k, j_begin, false);
+            load_tile(1, &tm_v, j_begin, clear && n_tiles == 1);
         }
     }
     if (tid == 0) {
         for (int s = 0; s < slots; ++s) mbar_init(bar_kv_empty(s), 1);
         mbar_init(bar_s_full, 1);
-        mbar_init(bar_p_early, row_warps * 32);
-        mbar_init(bar_p_full, row_warps * 32);
+        mbar_init(bar_p_early, soft_warps * 32);
+        mbar_init(bar_p_full, soft_warps * 32);
         mbar_init(bar_o_full, 1);
+        mbar_init(bar_v_clear, 64);
         fence_mbar_init();
         // a wait that expired in an earlier CTA or launch stops the rest from queueing up behind it
         tmem_slot_gen[1] = *reinterpret_cast<volatile unsigned int *>(p.status);
@@ -141,7 +194,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
     if (warp < 4) {
         reg_inc<200>();
-        if (healthy && warp < row_warps) {
+        if (healthy && warp < soft_warps) {
             // =============================================================== softmax warps
             const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
             const uint32_t tS = tmem + lane_off + kColS, tO = tmem + lane_off + kColO;
@@ -153,29 +206,14 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 if (!mbar_wait(bar_s_full, i & 1)) { err = kErrWaitS; break; }
                 tc_fence_after();
                 const int valid = keys - (j_begin + i) * kBlockN;
-                // Keys past the sequence's end have weight zero, but 0 x NaN is NaN in the product P V, and
-                // padding may hold any bit pattern: its value rows are cleared in the ring slot (whole
-                // 128-byte rows, which the swizzle maps onto themselves) before the weights are handed over.
-                // Rows past the end of the tensor were zero-filled by the copy.
-                const bool clear = valid < kBlockN && keys < p.Nkv;
-                softmax_tile<D>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
-                    if (clear) return;
+                if constexpr (G > 1) softmax_part<D, kBlockN / G>(tS, tO, warp * (kBlockN / G), i == 0, valid, c, m_ref, l_run);
+                else softmax_tile<D>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
                     tmem_wait_st();
                     tc_fence_before();
                     mbar_arrive(bar_p_early);
                 });
-                if (clear) {
-                    const int tile_v = 2 * i + 1, slot_v = tile_v % slots;
-                    if (!mbar_wait(bar_kv_full(slot_v), (tile_v / slots) & 1)) { err = kErrWaitKV; break; }
-                    for (int r = valid + warp * 4 + (lane >> 3); r < kBlockN; r += row_warps * 4)
-#pragma unroll
-                        for (int cx = 0; cx < kBoxes; ++cx)
-                            st_shared_v4(sRing + slot_v * kTileBytes + cx * kBoxBytes + r * 128 + (lane & 7) * 16, 0u, 0u, 0u, 0u);
-                    fence_proxy_async_smem();
-                }
                 tmem_wait_st();
                 tc_fence_before();
-                if (clear) mbar_arrive(bar_p_early);
                 mbar_arrive(bar_p_full);
             }
             if (err == 0 && n_tiles > 0 && !mbar_wait(bar_o_full, 0)) err = kErrWaitO;
@@ -192,7 +230,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 #pragma unroll
                 for (int i = 0; i < D; ++i) acc[i] = 0u;
             }
-            if (parts == 1) {
+            if (G == 1 && parts == 1) {
                 const float inv = nkv > 0 ? 1.f / l_run : 0.f;
                 if (err == 0 && row < rows)
 #pragma unroll
@@ -205,6 +243,37 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     st_shared_v4(sRing + ((i / 4) * kBlockM + row) * 16, acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
             }
         }
+        if (G > 1) {
+            // ---- the copies meet: each warp combines its share of the columns, for the result or for the cluster
+            named_bar_sync(1, 128);
+            const float2 *ml = reinterpret_cast<const float2 *>(tiles_gen);
+            float4 *o = reinterpret_cast<float4 *>(tiles_gen + L::q_bytes(q_rows));
+            float m_all = -INFINITY, sum = 0.f, w[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) m_all = fmaxf(m_all, ml[g * 32 + lane].x);
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                w[g] = n_tiles > 0 ? ex2(ml[g * 32 + lane].x - m_all) : 0.f;
+                sum += ml[g * 32 + lane].y * w[g];
+            }
+            const float inv = nkv > 0 ? 1.f / sum : 0.f;
+            for (int c0 = warp * 16; healthy && c0 < D; c0 += 64) {
+                float acc[16];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const float4 v = o[(c0 / 4 + k) * kBlockM + g * 32 + lane];
+                        a.x += v.x * w[g]; a.y += v.y * w[g]; a.z += v.z * w[g]; a.w += v.w * w[g];
+                    }
+                    if (parts > 1) o[(c0 / 4 + k) * kBlockM + lane] = a;             // over the first copy's
+                    acc[4 * k] = a.x; acc[4 * k + 1] = a.y; acc[4 * k + 2] = a.z; acc[4 * k + 3] = a.w;
+                }
+                if (parts == 1 && lane < rows) store16(lane, c0, acc, inv);
+            }
+            if (parts > 1 && warp == 0) reinterpret_cast<float2 *>(tiles_gen)[kBlockM + lane] = make_float2(m_all, sum);
+        }
     } else {
         reg_dec<56>();
         if (healthy && warp == kSplitLoadWarp && elect_one()) {
@@ -212,7 +281,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             // ring tiles: 2i = K tile i, 2i + 1 = V tile i; the first two are on their way
             for (int t = 2, slot = 2 % slots, use = 2 / slots; t < 2 * n_tiles; ++t) {
                 if (use > 0 && !mbar_wait(bar_kv_empty(slot), (use - 1) & 1)) { report(p, kErrWaitSlot); break; }
-                load_tile(slot, (t & 1) ? &tm_v : &tm_k, j_begin + (t >> 1));
+                load_tile(slot, (t & 1) ? &tm_v : &tm_k, j_begin + (t >> 1), clear && t + 1 == 2 * n_tiles);
                 if (++slot == slots) { slot = 0; ++use; }
             }
         } else if (healthy && warp == kSplitMmaWarp && elect_one()) {
@@ -247,15 +316,17 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 issue_s();
                 next_slot();
                 for (int i = 0; i < n_tiles; ++i) {
-                    if (!mbar_wait(bar_kv_full(slot), phase)) { err = kErrWaitKV; break; }
-                    if (!mbar_wait(bar_p_early, i & 1)) { err = kErrWaitP; break; }
+                    const bool last = clear && i + 1 == n_tiles;
+                    if (!mbar_wait(last ? bar_v_last : bar_kv_full(slot), last ? 0 : phase)) { err = kErrWaitKV; break; }
+                    if (last && !mbar_wait(bar_v_clear, 0)) { err = kErrWaitKV; break; }
+                    if (!mbar_wait(G > 1 ? bar_p_full : bar_p_early, i & 1)) { err = kErrWaitP; break; }
                     tc_fence_after();
                     const uint64_t b = desc_v0 + (uint64_t)(slot * (kTileBytes >> 4));
                     bool ok = true;
 #pragma unroll
                     for (int ks = 0; ks < kBlockN / 16; ++ks) {
                         // 16 keys = two 8-row groups of 1024 bytes; column blocks of 64 are one box apart
-                        if (ks == 6) {
+                        if (G == 1 && ks == 6) {
                             if (!mbar_wait(bar_p_full, i & 1)) { ok = false; break; }
                             tc_fence_after();
                         }
@@ -272,6 +343,18 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 }
             } while (false);
             if (err) report(p, err);
+        } else if (healthy && warp > kSplitMmaWarp && clear) {
+            // =============================================================== value rows behind the end
+            if (!mbar_wait(bar_v_last, 0)) report(p, kErrWaitKV);
+            else {
+                // whole 128-byte rows, which the swizzle maps onto themselves
+                const uint32_t tile = sRing + ((2 * n_tiles - 1) % slots) * kTileBytes;
+                for (int r = keys % kBlockN + (warp - kSplitMmaWarp - 1) * 4 + (lane >> 3); r < kBlockN; r += 8)
+#pragma unroll
+                    for (int cx = 0; cx < kBoxes; ++cx) st_shared_v4(tile + cx * kBoxBytes + r * 128 + (lane & 7) * 16, 0u, 0u, 0u, 0u);
+                fence_proxy_async_smem();
+                mbar_arrive(bar_v_clear);
+            }
         }
     }
 
@@ -297,7 +380,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 for (int i = 0; i < parts; ++i) {
                     ml[i] = make_float2(-INFINITY, 0.f);
                     if ((i + 1) * nkv / parts == i * nkv / parts) continue;       // no key tile, nothing written
-                    ml[i] = ld_cluster_v2(cluster_addr(sQ + row * 8, i));
+                    ml[i] = ld_cluster_v2(cluster_addr(sQ + ((G > 1 ? kBlockM : 0) + row) * 8, i));
                     m_all = fmaxf(m_all, ml[i].x);
                 }
                 float sum = 0.f, acc[16];
