@@ -785,30 +785,46 @@ int sm_count(int *out)
 }
 
 // How many CTAs of attention_split_kernel share one query tile's keys; 0: one of the other kernels is faster.
-// `tiles`: query tiles of 128 rows over all heads.  Figures in us on 148 SMs at D = 128, head-major, this
-// kernel : attention_kernel; n: key tiles.
-//   * More tiles than SMs, one per head: a CTA per tile, two on an SM.  Two of them take 1.2 (short keys) to 1.9
-//     times (long ones) as long as one CTA of attention_kernel with the SM to itself, so from n = 9 on waves are
-//     compared, and beyond 16 there is nothing to win.  32 queries, n = 2: 256 heads 10.9 : 15.1; n = 8: 176 heads
-//     22.3 : 27.5, 256 26.3 : 30.2, 400 44.7 : 44.8 (two waves to three), 512 47.7 : 57.7; n = 16: 256 heads 45.7 :
-//     50.1, 400 87 : 78, 512 89 : 101; n = 32, unequal lengths: 296 heads 81.5 : 77.9, 1024 242 : 239.
-//   * Too few tiles to fill the chip: eight CTAs a tile while that leaves an SM to each, four up to two on an SM, two
-//     beyond that (only heads of several tiles, of which attention_kernel gives a CTA two).  32 queries: 8 heads,
-//     n = 32 14.7 : 31.3, n = 16 11.6 : 18.3; 32 heads, n = 32 21.5 : 32.7, n = 8 10.6 : 12.0; 64 heads, n = 16 19.4 :
-//     20.3, n = 8 13.7 : 12.8.  128 queries (a ring of two tiles): 32 heads, n = 16 17.4 : 19.6, n = 8 13.5 : 12.4; 64
-//     heads, n = 32 33.3 : 35.2, n = 16 23.3 : 21.1.  256 queries: 8 heads, n = 8 12.5 : 18.5; 32 heads, n = 8 17.2 :
-//     19.1; 64 heads, n = 16 29.4 : 34.0, n = 8 21.5 : 20.4.  With two key tiles a part or fewer the meeting of the
-//     parts (some 3 us) is hardly earned back.
-int split_parts(long tiles, int nkv, int Nq, int sms)
+// `tiles`: query tiles of 128 rows over all heads; n: key tiles.  Figures in us on 148 SMs, D = 128 unless noted, this
+// kernel : attention_kernel.
+//   * One key tile: where attention_kernel's general form is the other side, or it takes more than one round (the
+//     start and end of a CTA are all there is; the square form is quicker in one, 4 x 128 4.5 : 5.3).  8 heads, 8 queries 5.5 : 6.0, 1024 heads 22.7 :
+//     39.8, of unequal length 26.6 : 51.3; 128 queries, 160 heads 7.9 : 10.0, 1024 29.8 : 39.7.
+//   * More tiles than SMs, one per head: a CTA per tile, two on an SM.  Up to 32 queries (keys shared by a CTA's
+//     warps): 320 heads, n = 12 52.9 : 56.2, of unequal length 35.4 : 44.2; 1024, n = 16 175 : 193 and 118 : 141; 256,
+//     n = 32 84 : 95; 1024 at D = 64, n = 16 93 : 139 and 63 : 108.  Not where long sequences of unequal length take one
+//     round, which attention_kernel's faster single item wins at D = 128 (160 heads, n = 32 50 : 44; 256 65 : 61).
+//     33 to 128 queries: two CTAs on an SM take 1.2 (short keys) to 1.9 times (long ones) as long as one of
+//     attention_kernel, so from n = 9 on waves are compared, and beyond 16 there is nothing to win.  128 queries, n = 8:
+//     256 heads 29 : 32, 400 51 : 48 (two waves to three), 512 55 : 61; n = 16: 256 heads 51 : 53, 400 93 : 81, 512
+//     97 : 107; n = 32: 512 heads 194 : 195.
+//   * Too few tiles to fill the chip: eight CTAs a tile while that leaves an SM to each, four up to 1.75 an SM (288 CTAs
+//     in clusters of four are not resident at a time: 72 heads, n = 16 27.7 : 20.7, 64 19.0 : 20.3), two beyond that
+//     (only heads of several tiles, of which attention_kernel gives a CTA two).  With two key tiles a part
+//     or fewer the meeting of the parts (some 3 us) is hardly earned back.  Up to 32 queries: 8 heads, n = 32 14.7 :
+//     31.3, n = 16 11.3 : 18.3, n = 4 8.3 : 9.0; 32 heads, n = 32 19.4 : 32.7, n = 8 10.4 : 12.0, n = 4 8.8 : 9.1; 64
+//     heads, n = 12 16.2 : 16.7, n = 8 13.4 : 12.8; D = 64, 64 heads, n = 8 10.2 : 11.5, and without splitting n = 4 7.5 :
+//     8.1, 128 heads n = 16 18.6 : 19.4.  128 queries (a ring of two tiles): 32 heads, n = 16 17.4 : 19.6, n = 8 13.5 :
+//     12.4; 64 heads, n = 32 33.3 : 35.2, n = 16 23.3 : 21.1.  256 queries: 8 heads, n = 8 12.5 : 18.5; 32 heads, n = 8
+//     17.2 : 19.1; 64 heads, n = 16 29.4 : 34.0, n = 8 21.5 : 20.4.
+int split_parts(long tiles, int nkv, int Nq, int D, bool general, bool unequal, int sms)
 {
-    if (tiles > sms && Nq <= kBlockM) {
+    const bool copies = Nq <= 32, one_tile = Nq <= kBlockM;
+    if (one_tile && nkv == 1) return general || tiles > sms ? 1 : 0;
+    if (one_tile && tiles > sms) {
+        if (copies) return unequal && D == 128 && nkv > 16 && 4 * tiles <= 7L * sms ? 0 : 1;
         const long waves = (tiles + sms - 1) / sms, waves2 = (tiles + 2 * sms - 1) / (2 * sms);
-        return nkv > 1 && nkv <= 16 && (nkv <= 8 || 9 * waves2 < 5 * waves) ? 1 : 0;
+        return nkv <= 16 && (nkv <= 8 || 9 * waves2 < 5 * waves) ? 1 : 0;
     }
-    int parts = tiles * 8 <= sms ? 8 : tiles * 4 <= 2 * sms ? 4 : tiles <= sms && Nq > kBlockM ? 2 : 0;
-    if (parts == 8 && nkv < 16) parts = 4;
-    const bool roomy = tiles * parts <= sms;
-    const int least = Nq > kBlockM ? (parts == 2 ? 16 : 8) : Nq > 64 ? (roomy ? 16 : 32) : roomy ? 8 : 16;
+    int parts = tiles * 8 <= sms ? 8 : tiles * 16 <= 7L * sms ? 4 : tiles * 8 <= 7L * sms && !one_tile ? 2 : 0;
+    if (parts == 8 && nkv < (tiles * 16 <= sms ? 16 : 24)) parts = 4;
+    const bool roomy = tiles * parts <= sms;              // an SM for each CTA
+    if (copies) {
+        const int least = D == 64 ? 6 : roomy ? 4 : 12;
+        if (parts && nkv >= least) return parts;
+        return D == 64 || nkv == 2 ? 1 : 0;
+    }
+    const int least = !one_tile ? (parts == 2 ? 16 : 8) : Nq > 64 ? (roomy ? 16 : 32) : roomy ? 8 : 16;
     return nkv >= least ? parts : 0;
 }
 
@@ -861,7 +877,7 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     // together, which costs more (20 x 32 heads of the former 51.1 -> 55.0, 64 x 32 151 -> 156).
     auto longest_first = [&](long ctas, long at_a_time) { return kv_len && B > 1 && ctas > at_a_time && ctas <= 2 * at_a_time; };
     const long tiles = BH * ((Nq + kBlockM - 1) / kBlockM);
-    if (const int parts = split_parts(tiles, nkv, Nq, sms)) {
+    if (const int parts = split_parts(tiles, nkv, Nq, D, general, kv_len && B > 1, sms)) {
         // copies of the query rows in a tile (see attention_split_kernel)
         const int copies = Nq > 32 ? 1 : D == 64 ? 4 : 2;
         const int q_rows = copies > 1 ? 32 * copies : Nq <= 64 ? 64 : 128;

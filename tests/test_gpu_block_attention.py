@@ -203,7 +203,8 @@ def test_drafter_shape_full_size(dd, oracle_mod, layout):
     (2, 4, 1, 2050, 128, [2050, 700]), (2, 3, 64, 4096, 64, [4095, 1]), (1, 8, 65, 2048, 128, None),
     (3, 8, 33, 1100, 128, [1100, 0, 129]), (2, 8, 130, 1000, 64, [900, 128]), (1, 8, 600, 1030, 128, None),
     (2, 32, 150, 2048, 64, [64, 2048]), (10, 16, 5, 300, 128, [300, 0, 1, 127, 128, 129, 256, 257, 299, 300]),
-    (6, 32, 128, 260, 64, [260, 3, 128, 0, 250, 129]),
+    (6, 32, 128, 260, 64, [260, 3, 128, 0, 250, 129]), (2, 3, 32, 128, 64, [1, 128]), (3, 5, 1, 128, 128, [0, 31, 33]),
+    (2, 3, 100, 77, 128, [77, 0]), (2, 90, 31, 100, 64, [100, 65]), (2, 3, 17, 500, 64, [500, 289]), (2, 2, 32, 600, 128, [513, 100]),
 ])
 @pytest.mark.parametrize("layout", ["bhnd", "bnhd"])
 def test_one_query_tile_per_cta(dd, oracle_mod, B, H, Nq, Nkv, D, kv_len, layout):
