@@ -1,13 +1,17 @@
 // The host side of one call, native: checks the tensors, makes the outputs, asks torch for the current
 // stream and calls an entry point of libdualdiff.so by its address.  binding.py does the same in Python, at
 // 8 to 13 us a call, which is more than the small launches take on the device; it remains for everything
-// this file does not take (another stream, host buffers, tensors that are not as they should be: the
-// functions below then return None, and the words of the error are the binding's).
+// this file does not take: another stream, host buffers, subclasses of torch.Tensor (FakeTensor among
+// them) and tensors without storage, calls under a torch function or dispatch mode, tensors that are not as
+// they should be, and whatever throws before the launch (an allocation that fails).  The functions below
+// then return None, having launched nothing, and the words of the error are the binding's.
 // Marshalling only: no arithmetic of the method.
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <ATen/PythonTorchFunctionTLS.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -23,12 +27,16 @@ struct Shape {
     int n;
 };
 
-const at::Tensor *tensor_of(PyObject *o) { return THPVariable_Check(o) ? &THPVariable_Unpack(o) : nullptr; }
+// A torch.Tensor or torch.nn.Parameter itself: what a subclass makes of a call is decided in Python.
+const at::Tensor *tensor_of(PyObject *o) { return THPVariable_CheckExact(o) ? &THPVariable_Unpack(o) : nullptr; }
+
+// No mode that would have a say in what torch.empty or Tensor.data_ptr do here.
+bool plain_call() { return !at::impl::torch_function_mode_enabled() && !c10::impl::TorchDispatchModeTLS::any_modes_set(); }
 
 // A contiguous tensor on the given device (device < 0: any, which is then the one to compare with).
 bool fits(const at::Tensor *t, at::ScalarType type, const Shape &s, int &device)
 {
-    if (!t || !t->is_cuda() || t->scalar_type() != type || t->dim() != s.n || !t->is_contiguous()) return false;
+    if (!t || !t->has_storage() || !t->is_cuda() || t->scalar_type() != type || t->dim() != s.n || !t->is_contiguous()) return false;
     for (int i = 0; i < s.n; ++i)
         if (t->size(i) != s.d[i]) return false;
     if (device < 0) device = t->get_device();
@@ -56,12 +64,14 @@ void *stream_now() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
 void *ptr(const at::Tensor &t) { return t.data_ptr(); }
 
-template <typename Call>
-int without_gil(Call call)
+// Calls an entry point of the library, which throws nothing, without the GIL.  The arguments are values: whatever
+// can throw (data_ptr, the current stream, an allocation) comes before, with the GIL held.
+template <typename Fn, typename... Args>
+int without_gil(Fn fn, Args... args)
 {
     int status;
     Py_BEGIN_ALLOW_THREADS
-    status = call();
+    status = fn(args...);
     Py_END_ALLOW_THREADS
     return status;
 }
@@ -86,13 +96,19 @@ uintptr_t address(PyObject *o) { return (uintptr_t)PyLong_AsVoidPtr(o); }
 
 bool is_none(PyObject *o) { return o == Py_None; }
 
-#define GUARD_BEGIN try {
+// What is thrown before the launch is the Python form's to meet again and to word; behind it (wrapping the
+// results) there is nothing to repeat.
+#define GUARD_BEGIN bool launched = false; try {
 #define GUARD_END                                            \
     }                                                        \
     catch (const std::exception &e)                          \
     {                                                        \
-        PyErr_SetString(PyExc_RuntimeError, e.what());       \
-        return nullptr;                                      \
+        if (launched) {                                      \
+            PyErr_SetString(PyExc_RuntimeError, e.what());   \
+            return nullptr;                                  \
+        }                                                    \
+        PyErr_Clear();                                       \
+        Py_RETURN_NONE;                                      \
     }
 
 // The output of an attention call: the one given, or a new one.
@@ -124,20 +140,21 @@ PyObject *attention_result(int status, PyObject *given, at::Tensor &out)
 PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     GUARD_BEGIN
-    if (n != 6) Py_RETURN_NONE;
+    if (n != 6 || !plain_call()) Py_RETURN_NONE;
     const at::Tensor *q = tensor_of(a[1]), *k = tensor_of(a[2]), *v = tensor_of(a[3]);
     Shape s;
     int dev = -1;
     double scale;
     at::Tensor out;
     if (!shape_of(q, 4, s) || !fits(q, at::kBFloat16, s, dev) || !fits(k, at::kBFloat16, s, dev) || !fits(v, at::kBFloat16, s, dev) ||
-        !scale_of(a[5], s.d[3], scale) || !attention_output(a[4], s, dev, out))
+        !scale_of(a[5], s.d[3], scale))
         Py_RETURN_NONE;
+    const void *pq = ptr(*q), *pk = ptr(*k), *pv = ptr(*v);
+    if (!attention_output(a[4], s, dev, out)) Py_RETURN_NONE;
     using Fn = int (*)(const void *, const void *, const void *, void *, int, int, int, int, float, void *);
-    const Fn fn = (Fn)address(a[0]);
-    const int status = without_gil([&] {
-        return fn(ptr(*q), ptr(*k), ptr(*v), ptr(out), (int)s.d[0], (int)s.d[1], (int)s.d[2], (int)s.d[3], (float)scale, stream_now());
-    });
+    const int status = without_gil((Fn)address(a[0]), pq, pk, pv, ptr(out), (int)s.d[0], (int)s.d[1], (int)s.d[2], (int)s.d[3],
+                                   (float)scale, stream_now());
+    launched = true;
     return attention_result(status, a[4], out);
     GUARD_END
 }
@@ -146,7 +163,7 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n)
 PyObject *block(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     GUARD_BEGIN
-    if (n != 8) Py_RETURN_NONE;
+    if (n != 8 || !plain_call()) Py_RETURN_NONE;
     const at::Tensor *q = tensor_of(a[1]), *k = tensor_of(a[2]), *v = tensor_of(a[3]);
     long layout;
     Shape s, ks;
@@ -160,19 +177,18 @@ PyObject *block(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (!fits(q, at::kBFloat16, s, dev) || !fits(k, at::kBFloat16, ks, dev) || !fits(v, at::kBFloat16, ks, dev) ||
         !scale_of(a[7], s.d[3], scale))
         Py_RETURN_NONE;
-    const void *lens = nullptr;
+    const int32_t *lens = nullptr;
     if (!is_none(a[4])) {
         const at::Tensor *l = tensor_of(a[4]);
         if (!fits(l, at::kInt, Shape{{s.d[0], 0, 0, 0}, 1}, dev)) Py_RETURN_NONE;
-        lens = ptr(*l);
+        lens = (const int32_t *)ptr(*l);
     }
+    const void *pq = ptr(*q), *pk = ptr(*k), *pv = ptr(*v);
     if (!attention_output(a[6], s, dev, out)) Py_RETURN_NONE;
     using Fn = int (*)(const void *, const void *, const void *, void *, int, int, int, int, int, const int32_t *, int, float, void *);
-    const Fn fn = (Fn)address(a[0]);
-    const int status = without_gil([&] {
-        return fn(ptr(*q), ptr(*k), ptr(*v), ptr(out), (int)s.d[0], (int)s.d[at_h], (int)s.d[at_n], (int)ks.d[at_n], (int)s.d[3],
-                  (const int32_t *)lens, (int)layout, (float)scale, stream_now());
-    });
+    const int status = without_gil((Fn)address(a[0]), pq, pk, pv, ptr(out), (int)s.d[0], (int)s.d[at_h], (int)s.d[at_n], (int)ks.d[at_n],
+                                   (int)s.d[3], lens, (int)layout, (float)scale, stream_now());
+    launched = true;
     return attention_result(status, a[6], out);
     GUARD_END
 }
@@ -181,6 +197,9 @@ PyObject *block(PyObject *, PyObject *const *a, Py_ssize_t n)
 struct Decision {
     at::Tensor t[3];                 // tokens, mask, score
     PyObject *given[3];
+    int32_t *tokens;
+    uint8_t *mask;
+    float *score;                    // null: not wanted
 };
 bool outputs(Decision &o, PyObject *const *a, const Shape &s, int dev, bool want_score)
 {
@@ -194,6 +213,9 @@ bool outputs(Decision &o, PyObject *const *a, const Shape &s, int dev, bool want
     }
     for (int i = 0; i < 3; ++i)
         if (!o.given[i] && (i < 2 || want_score)) o.t[i] = make(s, types[i], dev);
+    o.tokens = (int32_t *)ptr(o.t[0]);
+    o.mask = (uint8_t *)ptr(o.t[1]);
+    o.score = o.t[2].defined() ? (float *)ptr(o.t[2]) : nullptr;
     return true;
 }
 PyObject *result(Decision &o)
@@ -212,7 +234,7 @@ PyObject *result(Decision &o)
 PyObject *verify(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     GUARD_BEGIN
-    if (n != 13) Py_RETURN_NONE;
+    if (n != 13 || !plain_call()) Py_RETURN_NONE;
     const at::Tensor *dra = is_none(a[1]) ? nullptr : tensor_of(a[1]), *ver = tensor_of(a[2]);
     const at::Tensor *tok = tensor_of(a[3]), *fl = tensor_of(a[4]);
     Shape full;
@@ -225,16 +247,18 @@ PyObject *verify(PyObject *, PyObject *const *a, Py_ssize_t n)
         !fits(fl, at::kByte, s, dev) || !integer(a[5], mode) || !number(a[6], tau) || !integer(a[7], k) || !PyLong_Check(a[8]))
         Py_RETURN_NONE;
     const uint64_t seed = PyLong_AsUnsignedLongLongMask(a[8]);
+    const int want_score = PyObject_IsTrue(a[12]);
+    if (want_score < 0) { PyErr_Clear(); Py_RETURN_NONE; }
+    const void *pd = dra ? ptr(*dra) : nullptr, *pv = ptr(*ver);
+    const int32_t *pt = (const int32_t *)ptr(*tok);
+    const uint8_t *pf = (const uint8_t *)ptr(*fl);
     Decision o;
-    if (!outputs(o, a + 9, s, dev, PyObject_IsTrue(a[12]) == 1)) Py_RETURN_NONE;
+    if (!outputs(o, a + 9, s, dev, want_score == 1)) Py_RETURN_NONE;
     using Fn = int (*)(const void *, const void *, const int32_t *, const uint8_t *, int, float, int, uint64_t, int32_t *, uint8_t *,
                        float *, int, int, int, void *);
-    const Fn fn = (Fn)address(a[0]);
-    const int status = without_gil([&] {
-        return fn(dra ? ptr(*dra) : nullptr, ptr(*ver), (const int32_t *)ptr(*tok), (const uint8_t *)ptr(*fl), (int)mode, (float)tau,
-                  (int)k, seed, (int32_t *)ptr(o.t[0]), (uint8_t *)ptr(o.t[1]), o.t[2].defined() ? (float *)ptr(o.t[2]) : nullptr,
-                  (int)full.d[0], (int)full.d[1], (int)full.d[2], stream_now());
-    });
+    const int status = without_gil((Fn)address(a[0]), pd, pv, pt, pf, (int)mode, (float)tau, (int)k, seed, o.tokens, o.mask, o.score,
+                                   (int)full.d[0], (int)full.d[1], (int)full.d[2], stream_now());
+    launched = true;
     if (status) return PyLong_FromLong(status);
     return result(o);
     GUARD_END
@@ -244,7 +268,7 @@ PyObject *verify(PyObject *, PyObject *const *a, Py_ssize_t n)
 PyObject *unmask(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     GUARD_BEGIN
-    if (n != 9) Py_RETURN_NONE;
+    if (n != 9 || !plain_call()) Py_RETURN_NONE;
     const at::Tensor *logits = tensor_of(a[1]), *tok = tensor_of(a[2]), *fl = tensor_of(a[3]);
     Shape full;
     if (!shape_of(logits, 3, full)) Py_RETURN_NONE;
@@ -255,14 +279,15 @@ PyObject *unmask(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (!fits(logits, at::kBFloat16, full, dev) || !fits(tok, at::kInt, s, dev) || !fits(fl, at::kByte, s, dev) || !number(a[4], tau) ||
         !integer(a[5], k))
         Py_RETURN_NONE;
+    const void *pl = ptr(*logits);
+    const int32_t *pt = (const int32_t *)ptr(*tok);
+    const uint8_t *pf = (const uint8_t *)ptr(*fl);
     Decision o;
     if (!outputs(o, a + 6, s, dev, true)) Py_RETURN_NONE;
     using Fn = int (*)(const void *, const int32_t *, const uint8_t *, float, int, int32_t *, uint8_t *, float *, int, int, int, void *);
-    const Fn fn = (Fn)address(a[0]);
-    const int status = without_gil([&] {
-        return fn(ptr(*logits), (const int32_t *)ptr(*tok), (const uint8_t *)ptr(*fl), (float)tau, (int)k, (int32_t *)ptr(o.t[0]),
-                  (uint8_t *)ptr(o.t[1]), (float *)ptr(o.t[2]), (int)full.d[0], (int)full.d[1], (int)full.d[2], stream_now());
-    });
+    const int status = without_gil((Fn)address(a[0]), pl, pt, pf, (float)tau, (int)k, o.tokens, o.mask, o.score, (int)full.d[0],
+                                   (int)full.d[1], (int)full.d[2], stream_now());
+    launched = true;
     if (status) return PyLong_FromLong(status);
     return result(o);
     GUARD_END

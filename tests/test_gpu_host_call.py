@@ -83,3 +83,42 @@ def test_same_errors(dd, monkeypatch):
     native = [outcome(c) for c in bad]
     monkeypatch.setattr(dd, "_fast", None)
     assert [outcome(c) for c in bad] == native
+
+
+def test_what_is_left_to_the_python_form(dd, monkeypatch):
+    """Wrapped tensors, a torch function mode and an allocation that fails: as without the native side."""
+    import torch
+    from torch.overrides import TorchFunctionMode
+    q = torch.zeros(2, 2, 16, 64, dtype=torch.bfloat16, device="cuda")
+
+    class Seen(TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            names.append(getattr(func, "__name__", str(func)))
+            return func(*args, **(kwargs or {}))
+
+    def no_memory():
+        big = torch.empty(64, 32, 2048, 64, dtype=torch.bfloat16, device="cuda")
+        torch.cuda.empty_cache()
+        total = torch.cuda.get_device_properties(0).total_memory
+        torch.cuda.set_per_process_memory_fraction(torch.cuda.memory_reserved() / total)
+        try:
+            dd.bidir_attention(big, big, big)
+        finally:
+            torch.cuda.set_per_process_memory_fraction(1.0)
+
+    def outcomes():
+        seen = []
+        with pytest.raises(RuntimeError) as e:
+            torch.vmap(lambda t: dd.bidir_attention(t[None], t[None], t[None]))(q)
+        seen.append(str(e.value))
+        with pytest.raises(torch.OutOfMemoryError):
+            no_memory()
+        names.clear()
+        with Seen():
+            dd.bidir_attention(q, q, q)
+        return seen, sorted(set(names))
+    names = []
+    native = outcomes()
+    assert "empty_like" in native[1]
+    monkeypatch.setattr(dd, "_fast", None)
+    assert outcomes() == native
