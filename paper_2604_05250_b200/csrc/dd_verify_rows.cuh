@@ -71,8 +71,10 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
         LaneState L;
         lane_reset(L);
         const int head = row_head(row, p.V), extent = head + p.V;      // from the row's first vector on
-        const bool last_row = row == n_rows - 1;
         const size_t off = (size_t)row * p.V - head;
+        // what the tensor holds from there on, as far as the row's vectors reach: a vector that goes beyond is not loaded
+        // whole (the last row's last one; of fewer than eight logits also that of the rows before it)
+        const int present = (int)min(n_rows * p.V - (long)off, (long)extent + 7);
         const uint16_t *ver = p.verifier + off, *dra = KL ? p.drafter + off : p.verifier + off;
         const uint64_t policy = l2_evict_first_policy();
         int ordinal = 0;
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
             const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             auto load = [&](const uint16_t *src, int vec) {
                 const int e = vec * 8;
-                if (e >= n || (e + 8 > n && last_row)) return ninf;      // (the tensor's last vector may not be whole)
+                if (e >= n || x + e + 8 > present) return ninf;
                 return ld_streamed(src + checked_run(p, x + e, 8, n_rows * p.V - (long)off, kSiteLogit), policy);
             };
 #pragma unroll
@@ -92,13 +94,13 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
                 rd[j] = load(dra, lane + 32 * (KL ? j : kVecPerThread + j));
             }
             if (n < kStep || (head != 0 && x == 0)) {
-                // the vectors that the row shares with its neighbours, and the tensor's last
+                // the vectors that the row shares with its neighbours, and one that the tensor does not fill
                 const int from = x == 0 ? head : 0;
                 auto edge = [&](uint4 &r, int vec, const uint16_t *src) {
                     const int e0 = vec * 8;
                     if (e0 >= n || (e0 + 8 <= n && e0 >= from)) return;
                     uint32_t w[4] = {r.x, r.y, r.z, r.w};
-                    const bool apart = last_row && e0 + 8 > n;
+                    const bool apart = x + e0 + 8 > present;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int e = e0 + i;

@@ -287,7 +287,6 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
             const uint32_t ring = s_addr(s_ring) + (uint32_t)(warp * kSStages * kSStageBytes);
             const int chunk_pieces = p.chunk / kStep;
             const int last_pieces = (p.V - (nch - 1) * p.chunk + kStep - 1) / kStep;     // of a row's last chunk (V a multiple of eight)
-            const unsigned last_row = (unsigned)n_rows - 1u;
             // The order in which the range's units are handed out starts with the range's share of
             // its last row, then its share of its first row (the two rows it may share with a
             // neighbour), then everything in between.
@@ -343,13 +342,14 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
                     const bool edge = n < kStep || (i_head != 0 && x_begin == 0);
                     const int fl = n | (i_piece == 0 ? 1 << 16 : 0) | (i_piece == i_npieces - 1 ? 1 << 17 : 0) | (edge ? 1 << 18 : 0) | (i_piece << 20);
                     s_meta[warp][stage] = make_int4(fl, i_where, i_row, i_chunk);
-                    // whole vectors; one that the tensor's last row fills only in part is left out (see below)
-                    const int vecs = (unsigned)i_row == last_row ? n >> 3 : (n + 7) >> 3;
+                    // whole vectors; one that the tensor's last logits fill only in part is left out (see below)
+                    const long begin = (long)i_row * p.V - i_head + x_begin;
+                    const int vecs = (int)min((long)((n + 7) >> 3), (n_rows * p.V - begin) >> 3);
                     const uint32_t bytes = (uint32_t)vecs * 16u;
                     const uint32_t dst = ring + stage * kSStageBytes;
                     sbar_expect_tx(bar, KL ? 2u * bytes : bytes);
                     if (vecs > 0) {
-                        const size_t off = checked_run(p, (long)i_row * p.V - i_head + x_begin, 8L * vecs, n_rows * p.V, kSiteLogit);
+                        const size_t off = checked_run(p, begin, 8L * vecs, n_rows * p.V, kSiteLogit);
                         bulk_load(dst, p.verifier + off, bytes, bar, policy);
                         if (KL) bulk_load(dst + kSStageBytes / 2, p.drafter + off, bytes, bar, policy);
                     }
@@ -409,10 +409,10 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
                         const int head = (kRagged ? row_head(meta.z, p.V) : 0);
                         const int x_begin = meta.w * p.chunk + ((meta.x >> 20) & 0xF) * kStep;
                         const long at = (long)meta.z * p.V - head + x_begin;          // of the piece, in the tensor
-                        const bool last_row_tail = meta.z == (int)last_row && (n & 7) != 0;
+                        const bool part_of_vector = at + ((n + 7) & ~7) > n_rows * p.V;
                         auto edge_vector = [&](uint4 &r, int vec, const uint16_t *logits) {
                             const int e0 = vec * 8;
-                            if (last_row_tail && e0 < n && e0 + 8 > n) {
+                            if (part_of_vector && e0 < n && e0 + 8 > n) {
                                 // the vector that was not copied: its logits one by one
                                 uint32_t w[4] = {0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u};
 #pragma unroll

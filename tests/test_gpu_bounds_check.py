@@ -81,3 +81,17 @@ def test_fused_heads(libs, mode):
     tok, fl = torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()
     d = t[:2] if mode == KL else [None, None]
     both_builds(binding, check_path, lambda: binding.lm_head_verify(d[0], d[1], t[2], t[3], tok, fl, mode, 0.3, 3, 5))
+
+
+@pytest.mark.parametrize("B,P", [(2, 37), (5, 8000)])          # row kernel; beyond its 32768 rows the streaming kernel
+@pytest.mark.parametrize("V", [1, 2, 3, 5, 7])
+@pytest.mark.parametrize("mode", [KL, CONF])
+def test_last_logits_of_rows_shorter_than_a_vector(libs, B, P, V, mode):
+    """The last vector of several rows reaches beyond the tensor."""
+    import torch
+    binding, check_path = libs
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, P // 2, 0.2, seed=V)
+    flags[-1, -9:] = 1
+    t = [to_torch_bf16(dra, "cuda") if mode == KL else None, to_torch_bf16(ver, "cuda"),
+         torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()]
+    both_builds(binding, check_path, lambda: binding.verify(t[0], t[1], t[2], t[3], mode, 0.5, 4, 9))
