@@ -34,6 +34,8 @@
 // twice in rolled loops instead of kept in 128 registers.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <float.h>
+#include <math_constants.h>
 #include <math.h>
 
 #include <mutex>
@@ -110,13 +112,14 @@ template <int D> constexpr int kPolyOneIn = D == 64 ? 4 : 0;
 
 // 2^x of two values on the FMA pipe: x = n + f with n the nearest integer (read off the low bits of
 // x + 1.5 * 2^23), 2^f on [-1/2, 1/2] as a polynomial of degree five (relative error 1.5e-7, fitted
-// by weighted least squares; ex2.approx has 2^-22 = 2.4e-7), n added to the exponent.  Below 2^-125
-// the result is 2^-125 instead of zero.
+// by weighted least squares; ex2.approx has 2^-22 = 2.4e-7), n added to the exponent.  From x = -127 downwards (-inf
+// included) the result is 2^-149, which is 0 as bf16; between that and -125.5 it is a number below 2^-125.  A NaN gives the
+// largest float: infinite as bf16, so that the row's sum is infinite and its result NaN.
 __device__ __forceinline__ float2 ex2_poly(float2 x)
 {
     auto c = [](float v) { return make_float2(v, v); };
-    x.x = max_nan(x.x, -125.f);      // a NaN stays one (and its row becomes NaN, whichever pair it falls into)
-    x.y = max_nan(x.y, -125.f);
+    x.x = max_nan(x.x, -127.f);
+    x.y = max_nan(x.y, -127.f);
     const float2 t = __fadd2_rn(x, c(12582912.f));
     const float2 f = __ffma2_rn(__fadd2_rn(t, c(-12582912.f)), c(-1.f), x);
     float2 y = __ffma2_rn(f, c(0.001327647129073739f), c(0.009675541892647743f));
@@ -185,7 +188,8 @@ template <int D>
 __device__ __forceinline__ void move_reference(uint32_t tO, bool first, float mx, float &m_ref, float &l_run)
 {
     if (first) {
-        m_ref = mx;
+        // (a row of which every score so far is -inf: the lowest number, so that their weights are 0 and not NaN)
+        m_ref = mx == -INFINITY ? -FLT_MAX : mx;
     } else if (__any_sync(0xffffffffu, mx > m_ref + kRescaleStep)) {
         const float m_new = mx > m_ref + kRescaleStep ? mx : m_ref;
         const float alpha = ex2(m_ref - m_new);       // 1 where the row does not move

@@ -257,3 +257,44 @@ def test_sequences_taken_longest_first(dd, oracle_mod, B, H, Nq, Nkv):
         if layout == "bnhd":
             a = [np.ascontiguousarray(x.transpose(0, 2, 1, 3)) for x in a]
         check_attention(run_gpu(dd, *a[:3], 0.125, kv_len=passed, layout=layout), a[3])
+
+
+def check_with_infinities(got, ref):
+    """Infinities where the exact result has them, everything else as usual (bars of check_attention)."""
+    assert not np.isnan(ref).any()
+    inf = np.isinf(ref)
+    np.testing.assert_array_equal(got[inf], ref[inf])
+    check_attention(np.where(inf, 0.0, got), np.where(inf, 0.0, ref))
+
+
+# one warp, two and four warps per key tile; one CTA, clusters and heads of several query tiles; sequences that leave some
+# of the warps without a key
+INFINITE = [(3, 2, 32, 600, 128, [600, 513, 40]), (3, 2, 8, 300, 64, [300, 129, 20]), (2, 3, 1, 2050, 64, [2050, 70]),
+            (2, 4, 64, 2048, 128, None), (1, 8, 600, 1030, 64, None), (2, 90, 100, 520, 64, None), (1, 4, 20, 4096, 128, None)]
+
+
+@pytest.mark.parametrize("B,H,Nq,Nkv,D,kv_len", INFINITE)
+def test_infinite_values(dd, oracle_mod, B, H, Nq, Nkv, D, kv_len):
+    """A value of +-inf at a key that exists makes its column of the result +-inf (every weight is positive), nothing else."""
+    q, k, v = block_inputs(B, H, Nq, Nkv, D, 900 + Nq)
+    q = synth.f32_to_bf16_bits(synth.bf16_bits_to_f32(q) * np.float32(0.25))      # no weight underflows
+    for n, (key, col) in enumerate([(0, 3), (17, 40), (Nkv // 2 + 33, 17), (Nkv - 1, D - 1)]):
+        v[:, :, key, col] = 0xFF80 if n & 1 else 0x7F80
+    kv = None if kv_len is None else np.array(kv_len, dtype=np.int32)
+    got = run_gpu(dd, q, k, v, D ** -0.5, kv_len=kv)
+    check_with_infinities(got, oracle_mod.block_attention(q, k, v, D ** -0.5, kv_len=kv))
+
+
+@pytest.mark.parametrize("B,H,Nq,Nkv,D,kv_len", INFINITE)
+def test_scores_of_minus_infinity(dd, oracle_mod, B, H, Nq, Nkv, D, kv_len):
+    """Keys at -inf from every query have no weight, also where they are all that a warp, a CTA or a tile begins with."""
+    q, k, v = block_inputs(B, H, Nq, Nkv, D, 950 + Nq)
+    q &= 0x7FFF                                                                    # positive
+    q[q == 0] = 0x3F00
+    k[:, :, :32] = 0xFF80
+    k[:, :, 64:96] = 0xFF80
+    if Nkv > 1024:
+        k[:, :, 256:1024] = 0xFF80                                                 # whole tiles, and whole parts of a cluster
+    kv = None if kv_len is None else np.maximum(np.array(kv_len, dtype=np.int32), 33)
+    got = run_gpu(dd, q, k, v, D ** -0.5, kv_len=kv)
+    check_attention(got, oracle_mod.block_attention(q, k, v, D ** -0.5, kv_len=kv))
