@@ -156,8 +156,11 @@ int dd_unmask(const void *logits, const int32_t *tokens, const uint8_t *mask_fla
  * positions with mask_flags == 0 may be read (they share tiles with their neighbours) but nothing is
  * computed from them.  Three kernels per call, in stream order: a small one that gathers the flagged
  * rows where that saves products, the products with their per-tile reductions, and a small one that
- * combines the tiles of every row and decides the sequences.  The library's scratch then holds a copy
- * of the hidden states as well (where there is no room for it, every row is multiplied).
+ * combines the tiles of every row and decides the sequences.  Scratch: 32 bytes for each row and vocabulary
+ * tile, of 128 entries (KL: 64) at the narrowest; where that is more than a quarter of the free memory, for the tiles picked where
+ * every row is multiplied, of 128 to 256 (64 to 128).  And a copy of the hidden states as large as they are (KL: both
+ * models'), without which every row is multiplied; it is not allocated beyond a quarter of the free memory, nor while
+ * `stream` is captured.
  * Supported: K a multiple of 64; any V >= 1; P <= 8192.
  */
 int dd_lm_head_verify(const void *drafter_hidden, const void *drafter_weight,

@@ -86,6 +86,33 @@ int ensure_bytes(void **ptr, size_t *have, size_t need)
     return DD_OK;
 }
 
+int try_bytes(void **ptr, size_t *have, size_t need, cudaStream_t stream)
+{
+    if (need <= *have && *ptr) return DD_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    size_t free_now = 0, total = 0;
+    const size_t bytes = (need + 255) & ~size_t(255);
+    // No more than a quarter of what is free: the rest of the program goes first.  (Asking costs a few microseconds
+    // and no synchronisation, and what was refused is not tried on every call.)
+    DD_CUDA_TRY(cudaStreamIsCapturing(stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return DD_ERR_UNSUPPORTED;
+    DD_CUDA_TRY(cudaMemGetInfo(&free_now, &total));
+    if (bytes > free_now / 4) return DD_ERR_UNSUPPORTED;
+    void *block = nullptr;
+    DD_CUDA_TRY(cudaMalloc(&block, bytes));
+    cudaError_t e = cudaMemset(block, 0, bytes);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();     // (earlier launches may still use the old block)
+    if (e != cudaSuccess) {
+        cudaFree(block);
+        return cuda_fail(e, "scratch");
+    }
+    void *old = *ptr;
+    *ptr = block;
+    *have = bytes;
+    if (old) DD_CUDA_TRY(cudaFree(old));
+    return DD_OK;
+}
+
 }  // namespace dd
 
 using namespace dd;

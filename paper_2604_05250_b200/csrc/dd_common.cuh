@@ -16,7 +16,7 @@ struct DeviceCtx {
     size_t verify_ws_bytes = 0;
     void *verify_cnt = nullptr;     // dd_verify completion counters: all zero between launches
     size_t verify_cnt_bytes = 0;
-    void *head_ws = nullptr;        // dd_lm_head_verify: plan, list of flagged rows, their hidden states
+    void *head_ws = nullptr;        // dd_lm_head_verify: the flagged rows' hidden states, where there is room for them
     size_t head_ws_bytes = 0;
     void *staging = nullptr;        // device copies of host buffers (the *_host calls)
     size_t staging_bytes = 0;
@@ -41,6 +41,9 @@ int check_mirror(const DeviceCtx *ctx, int which);
 
 // Grows (never shrinks) a scratch buffer; new memory is zero-filled.
 int ensure_bytes(void **ptr, size_t *have, size_t need);
+// The same for scratch that a call can do without, a quarter of the free memory at most and never while `stream` is
+// being captured: DD_OK if it is there; if not, nothing has changed.
+int try_bytes(void **ptr, size_t *have, size_t need, cudaStream_t stream);
 
 // Records a CUDA error text for dd_last_cuda_error() and returns DD_ERR_CUDA.
 int cuda_fail(cudaError_t e, const char *where);

@@ -192,10 +192,11 @@ __global__ void __launch_bounds__(kThreads, 3) verify_elementwise_kernel(const V
 // Host side.
 
 // Counters live in their own allocation: it holds nothing else, so it is all zero whenever no
-// launch is in flight, whatever (B, P) the previous call used.  Its last 256 bytes hold the
-// streaming kernel's health word.
+// launch is in flight, whatever (B, P) the previous call used.  Its last 256 bytes are not
+// counters: they hold the health word and the plan of the fused heads.
 constexpr size_t kControlBytes = 256;
 constexpr size_t kStatusOffset = 0;
+constexpr size_t kPlanOffset = 128;              // dd_lm_head_verify: what its kernels tell each other
 
 size_t counter_bytes(int B, int P)
 {
@@ -580,28 +581,36 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     const int ctas = cap > 0 && cap < sms ? cap : sms;
 
     // the narrowest tiles that the device may choose bound the partials
+    constexpr long kMaxPartials = (1L << 31) - (1L << 24);
     const int max_n = kl ? ddlm::Widths<true>::max_n : ddlm::Widths<false>::max_n;
+    auto tiles_of = [&](int n) { return (V + n - 1) / n; };
     int min_n = max_n / 2;
-    while (rows * ((V + min_n - 1) / min_n) >= (1L << 31) - (1L << 24)) {
+    while (rows * tiles_of(min_n) >= kMaxPartials) {
         if (min_n == max_n) return DD_ERR_UNSUPPORTED;
         min_n += 32;
     }
 
     VerifyParams p;
-    p.nchunks = (V + min_n - 1) / min_n;
-    p.chunk = min_n;
     dd::DeviceCtx *ctx = dd::current_ctx();
     if (!ctx) return DD_ERR_CUDA;
     if ((rc = dd::ensure_mirror(ctx)) != DD_OK) return rc;
     if ((rc = dd::check_mirror(ctx, 1)) != DD_OK) return rc;
-    rc = dd::ensure_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, p.nchunks));
-    if (rc != DD_OK) return rc;
+    if (dd::try_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)), (cudaStream_t)stream) != DD_OK) {
+        // no room for the narrowest: no narrower than what is picked where every row is multiplied
+        const long row_blocks = (rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem;
+        min_n = kl ? ddlm::pick_tile_n<true>(V, row_blocks, sms, min_n) : ddlm::pick_tile_n<false>(V, row_blocks, sms, min_n);
+        rc = dd::ensure_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)));
+        if (rc != DD_OK) return rc;
+    }
     rc = dd::ensure_bytes(&ctx->verify_cnt, &ctx->verify_cnt_bytes, counter_bytes(B, P) + kControlBytes);
     if (rc != DD_OK) return rc;
     const size_t bp = (size_t)rows;
+    char *control = (char *)ctx->verify_cnt + ctx->verify_cnt_bytes - kControlBytes;
+    p.nchunks = tiles_of(min_n);
+    p.chunk = min_n;
     p.row_counter = (unsigned int *)ctx->verify_cnt;
     p.seq_counter = (unsigned int *)((char *)ctx->verify_cnt + ((bp * 4 + 255) & ~size_t(255)));
-    p.status = (unsigned int *)((char *)ctx->verify_cnt + ctx->verify_cnt_bytes - kControlBytes + kStatusOffset);
+    p.status = (unsigned int *)(control + kStatusOffset);
     p.mirror = ctx->mirror_dev + 1;
     char *w = (char *)ctx->verify_ws;
     p.row_score = (float *)w;          w += (bp * 4 + 255) & ~size_t(255);
@@ -609,18 +618,17 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     p.partials = (Partial *)w;
     fill_params(p, nullptr, nullptr, tokens, mask_flags, mode, tau, k, seed, out_tokens, out_mask, out_score, B, P, V);
 
-    // scratch of this entry point: the plan, the list of flagged rows, their hidden states
-    const size_t map_bytes = ((size_t)rows * 4 + 255) & ~size_t(255), gathered_bytes = ((size_t)rows * K * 2 + 255) & ~size_t(255);
+    // A copy of the flagged rows' hidden states; without room for it every row is multiplied.  The list of those rows
+    // stands where the last kernel will put the rows' maxima, when nothing reads the list any more.
+    const size_t gathered_bytes = ((size_t)rows * K * 2 + 255) & ~size_t(255);
     ddlm::LmParams q;
-    q.can_gather = dd::ensure_bytes(&ctx->head_ws, &ctx->head_ws_bytes, 256 + map_bytes + (kl ? 2 : 1) * gathered_bytes) == DD_OK;
-    // no room for a copy of the hidden states: every row is multiplied
-    if (!q.can_gather && (rc = dd::ensure_bytes(&ctx->head_ws, &ctx->head_ws_bytes, 256 + map_bytes)) != DD_OK) return rc;
+    q.can_gather = dd::try_bytes(&ctx->head_ws, &ctx->head_ws_bytes, (kl ? 2 : 1) * gathered_bytes, (cudaStream_t)stream) == DD_OK;
     q.rows = (int)rows; q.K = K; q.V = V;
     q.min_n = min_n;
     q.ctas = sms;
-    q.plan = (ddlm::LmPlan *)ctx->head_ws;
-    q.row_map = (int *)((char *)ctx->head_ws + 256);
-    char *gathered = (char *)ctx->head_ws + (q.can_gather ? 256 + map_bytes : 0);
+    q.plan = (ddlm::LmPlan *)(control + kPlanOffset);
+    q.row_map = p.row_argmax;
+    char *gathered = (char *)(q.can_gather ? ctx->head_ws : ctx->verify_ws);
     return kl ? launch_lm_head<true>(q, p, drafter_hidden, drafter_weight, verifier_hidden, verifier_weight, gathered,
                                      gathered_bytes, ctas, (cudaStream_t)stream)
               : launch_lm_head<false>(q, p, nullptr, nullptr, verifier_hidden, verifier_weight, gathered, 0, ctas,

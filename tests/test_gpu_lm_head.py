@@ -203,3 +203,51 @@ def test_argument_errors(dd):
     assert call(CONF, 0) == dd.DD_ERR_INVALID_ARG
     assert call(7, 64) == dd.DD_ERR_INVALID_ARG
     assert L.dd_lm_head_verify(None, None, None, p(w), p(t), p(f), CONF, 0.5, 0, 0, p(t), p(f), p(o), 1, 4, 64, 16, None) == dd.DD_ERR_INVALID_ARG
+
+
+def test_without_room_for_the_gathered_rows(dd):
+    """Little free memory: no copy of the hidden states is made, every row is multiplied, the results are the same, no
+    call allocates or waits (one can be captured), and the copy is made again once there is room."""
+    import torch
+    dd.release()
+    B, P, K, V = 24, 2048, 4096, 500
+    g = torch.Generator(device="cuda").manual_seed(3)
+    hidden = torch.randn(B, P, K, device="cuda", generator=g, dtype=torch.bfloat16)           # 403 MB
+    weight = torch.randn(V, K, device="cuda", generator=g).mul_(K ** -0.5).to(torch.bfloat16)
+    tok = torch.zeros(B, P, dtype=torch.int32, device="cuda")
+    fl = (torch.rand(B, P, device="cuda", generator=g) < 0.3).to(torch.uint8)
+    outs = dict(out_tokens=torch.empty_like(tok), out_mask=torch.empty_like(fl), out_score=torch.empty(B, P, device="cuda"))
+    call = lambda: [x.clone() for x in dd.lm_head_verify(None, None, hidden, weight, tok, fl, CONF, 0.0, 0, 0, **outs)]
+    free = lambda: torch.cuda.mem_get_info()[0]
+
+    def same(a, b):
+        # the products are the same numbers; sums over tiles of another width differ in their order only
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+        torch.testing.assert_close(a[2], b[2], rtol=1e-5, atol=0)
+    roomy = call()
+    torch.cuda.synchronize()
+    dd.release()
+    torch.cuda.empty_cache()
+    filler = torch.empty(free() - (1 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        first = call()
+        torch.cuda.synchronize()
+        before = free()
+        same(call(), roomy)
+        same(first, roomy)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            dd.lm_head_verify(None, None, hidden, weight, tok, fl, CONF, 0.0, 0, 0, **outs)
+        outs["out_score"].fill_(-1.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        same([outs["out_tokens"], outs["out_mask"], outs["out_score"]], roomy)
+        assert before - free() < hidden.numel()                  # (less than half of the copy)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    before = free()
+    same(call(), roomy)
+    torch.cuda.synchronize()
+    assert before - free() >= hidden.numel() * 2
+    assert dd.verify_status() == 0
