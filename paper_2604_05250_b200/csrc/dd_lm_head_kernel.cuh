@@ -15,7 +15,7 @@
 // every flagged row's partials in fp64 with the streaming kernel's fold and runs dd_verify's
 // decision stage per sequence.
 //
-// Only flagged positions need logits.  A first small kernel (lm_head_rows_kernel) lists the flagged
+// Only flagged positions need logits.  Where that can pay, a first small kernel (lm_head_rows_kernel) lists the flagged
 // rows and, where that leaves fewer 128-row tiles, copies their hidden states one after the other
 // into scratch; the products then run over those.  How many there are is known on the device only:
 // it picks the width N of the vocabulary tiles too (a tensor map per width travels with the launch).
@@ -54,6 +54,7 @@ constexpr int kTileRows = 128;
 constexpr int kRowsPerItem = 2 * kTileRows; // two accumulators
 constexpr int kBlockK = 64;                // one 128-byte swizzled box per k-step
 constexpr int kMaxStages = 6;
+constexpr int kCheckedRows = 4 * kThreads;
 constexpr int kMaxN = 256;
 constexpr uint32_t kTmemCols = 512;        // see the layout above
 constexpr int kATileBytes = kTileRows * kBlockK * 2;                  // 16 KB: 128 rows x 64 bf16
@@ -80,8 +81,9 @@ struct LmParams {
     int rows, K, V;            // rows = B * P
     int ctas;                  // CTAs the tile width is chosen for
     int min_n;                 // the narrowest width the scratch has partials for
-    int can_gather;            // the scratch has room for the hidden states
-    LmPlan *plan;
+    int rows_per_block;        // rows that a block of the first kernel copies: a multiple of kRowsWarps
+    LmPlan *plan;              // null: nothing is gathered, the plan is all_rows and the first kernel is not launched
+    LmPlan all_rows;
     int *row_map;              // [rows]: the row that gathered row i is (not written where nothing is gathered)
 };
 
@@ -113,12 +115,26 @@ __host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int
     return best;
 }
 
-// First launch of dd_lm_head_verify.  Every block counts all flags (a few KB) and the flags before its
+template <bool KL>
+__host__ __device__ inline LmPlan plan_for(const LmParams &q, int n_rows, bool gathered)
+{
+    LmPlan plan;
+    plan.n_rows = n_rows;
+    plan.gathered = gathered;
+    plan.N = pick_tile_n<KL>(q.V, (n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n);
+    plan.n_tiles = (q.V + plan.N - 1) / plan.N;
+    return plan;
+}
+
+// First launch of dd_lm_head_verify, where gathering can pay.  Every block counts all flags and the flags before its
 // own rows; the first one writes the plan.  Gathering pays where it leaves fewer 128-row tiles (at
-// K = 4096, V = 126464 a tile of rows costs 85 us, copying 128 rows less than one); elsewhere nothing is
-// copied.  One warp per row.
+// K = 4096, V = 126464 a tile of rows costs 85 us, copying 128 rows less than one), and with one or two tiles of the
+// vocabulary, whose products are no more than reading the rows, where few are flagged: a gathered row is read twice
+// and written once (105150 rows, 60 %, K = 320, V = 102: 131 us without, 169 with; 38520, 5 %, 3072, 242: 118 and 79).
+// Elsewhere nothing is copied.  One warp per row; at most kRowsBlocks blocks, so that the counting stays linear in the rows.
 constexpr int kRowsThreads = 256;
-constexpr int kRowsPerBlock = kRowsThreads / 32;
+constexpr int kRowsWarps = kRowsThreads / 32;
+constexpr int kRowsBlocks = 1024;
 template <bool KL>
 __global__ void __launch_bounds__(kRowsThreads)
 lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden, uint4 *gathered,
@@ -126,7 +142,7 @@ lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden,
 {
     __shared__ int s_before, s_all;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int first = blockIdx.x * kRowsPerBlock;
+    const int first = blockIdx.x * q.rows_per_block;
     if (tid == 0) s_before = s_all = 0;
     __syncthreads();
     int before = 0, all = 0;
@@ -134,6 +150,7 @@ lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden,
     int done = 0;
     if ((reinterpret_cast<uintptr_t>(flags) & 7) == 0) {           // eight flags at a time (first is a multiple of eight)
         done = q.rows & ~7;
+#pragma unroll 4
         for (int i = 8 * tid; i < done; i += 8 * kRowsThreads) {
             const uint2 w = *reinterpret_cast<const uint2 *>(flags + i);
             count(i, __popc(__vsetne4(w.x, 0u)) + __popc(__vsetne4(w.y, 0u)));
@@ -145,30 +162,29 @@ lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden,
     if (lane == 0) { atomicAdd(&s_before, before); atomicAdd(&s_all, all); }
     __syncthreads();
     all = s_all;
-    const bool gather = q.can_gather && (all + kTileRows - 1) / kTileRows < (q.rows + kTileRows - 1) / kTileRows;
-    if (blockIdx.x == 0 && tid == 0) {
-        LmPlan plan;
-        plan.n_rows = gather ? all : q.rows;
-        plan.gathered = gather;
-        plan.N = pick_tile_n<KL>(q.V, (plan.n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n);
-        plan.n_tiles = (q.V + plan.N - 1) / plan.N;
-        *q.plan = plan;
-    }
+    const bool gather = (all + kTileRows - 1) / kTileRows < (q.rows + kTileRows - 1) / kTileRows &&
+                        (q.all_rows.n_tiles > 2 || 3L * all < (long)q.rows * q.all_rows.n_tiles);
+    if (blockIdx.x == 0 && tid == 0) *q.plan = plan_for<KL>(q, gather ? all : q.rows, gather);
     if (!gather) return;
-    const int row = first + warp;
-    if (row >= q.rows || !flags[row]) return;
-    const bool mine = lane < warp && flags[first + lane] != 0;
-    const int at = s_before + __popc(__ballot_sync(0xFFFFFFFFu, mine));
-    if (lane == 0) q.row_map[at] = row;
     const int vecs = q.K / 8;                                      // 16-byte vectors per row
-    auto copy = [&](uint4 *dst, const uint4 *src) {
-        dst += (size_t)at * vecs;
-        src += (size_t)row * vecs;
+    int seen = s_before;                                           // flags before the warps' next rows
+    for (int row0 = first; row0 < min(first + q.rows_per_block, q.rows); row0 += kRowsWarps) {
+        const bool flagged = lane < kRowsWarps && row0 + lane < q.rows && flags[row0 + lane] != 0;
+        const unsigned mask = __ballot_sync(0xFFFFFFFFu, flagged);
+        const int at = seen + __popc(mask & ((1u << warp) - 1u));
+        seen += __popc(mask);
+        if (!(mask >> warp & 1u)) continue;
+        const int row = row0 + warp;
+        if (lane == 0) q.row_map[at] = row;
+        auto copy = [&](uint4 *dst, const uint4 *src) {
+            dst += (size_t)at * vecs;
+            src += (size_t)row * vecs;
 #pragma unroll 8
-        for (int i = lane; i < vecs; i += 32) dst[i] = src[i];
-    };
-    copy(gathered, hidden);
-    if (KL) copy(gathered_d, hidden_d);
+            for (int i = lane; i < vecs; i += 32) dst[i] = src[i];
+        };
+        copy(gathered, hidden);
+        if (KL) copy(gathered_d, hidden_d);
+    }
 }
 
 // One row's partial of one vocabulary tile into the global table.  Nothing else happens in this
@@ -189,15 +205,16 @@ __device__ __forceinline__ void store_partial(const ddv::VerifyParams &p, const 
 // instruction cache: 16 rows of 126464 entries 204 -> 194 us, 8 x 512 of 8000 41.5 -> 39.8).  The partials were written by the previous kernel on the stream.
 constexpr int kFoldThreads = 256;
 template <bool KL>
-__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const __grid_constant__ ddv::VerifyParams p, int rows, const LmPlan *plan)
+__global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const __grid_constant__ ddv::VerifyParams p, const LmParams q)
 {
+    const int rows = q.rows;
     __shared__ ddv::BlockReport s_report;
     const int row0 = blockIdx.x * (kFoldThreads / 32);
     const int w = row0 + (threadIdx.x >> 5);
     if (w < rows && p.flags[w]) {
         float score;
         int argmax;
-        const int n_tiles = plan->n_tiles;
+        const int n_tiles = q.plan ? q.plan->n_tiles : q.all_rows.n_tiles;
         ddv::fold_partials<KL>(p.partials + ddv::checked_run(p, (long)w * n_tiles, n_tiles, (long)rows * n_tiles, ddv::kSitePartial),
                                n_tiles, score, argmax);
         if ((threadIdx.x & 31) == 0) {
@@ -357,7 +374,13 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     volatile uint32_t *abort_flag = tmem_slot_gen + 1;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5);
-    const LmPlan plan = *q.plan;
+    LmPlan plan = q.plan ? *q.plan : q.all_rows;
+    // few rows, none listed: perhaps none of them is flagged, and there is nothing to multiply
+    int any = 1;
+    if (!q.plan && q.rows <= kCheckedRows) {
+        any = 0;
+        for (int i = tid; i < q.rows; i += kThreads) any |= p.flags[i];
+    }
     const int k_steps = q.K / kBlockK;
     // a stage: one or two tiles of hidden states (two unless no item has more than 128 rows), one of weights
     const uint32_t a_bytes = plan.n_rows > kTileRows ? 2 * kATileBytes : kATileBytes;
@@ -376,7 +399,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     }
     if (warp == 0) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
     tc_fence_before();
-    __syncthreads();
+    if (!__syncthreads_or(any)) plan.n_rows = 0;
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot_gen);
 

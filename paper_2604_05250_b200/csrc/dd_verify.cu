@@ -511,6 +511,21 @@ int make_matrix_tmap(CUtensorMap *m, const void *base, long n_rows, int K, int b
     return DD_OK;
 }
 
+// Whether multiplying fewer rows can earn back the launch that finds out which (2 to 4 us; the host does not know how
+// many are flagged).  It cannot where there is one tile of rows, and hardly where all items run at the same time: with
+// fewer rows there are then fewer at work.  Measured over 400 calls, shares flagged 5 % to 100 % (us, every row against flagged
+// rows only; rows, K, V): one round 52, 64, 863 12.2 : 15.7; 6980, 64, 150 28.9 : 34.4; nearly full rounds of long items
+// 456, 2624, 17002 43.9 : 32.5, 2923, 1280, 2689 32.0 : 24.8; more rounds 4320, 320, 2259 24.7 : 21.7, 868, 192, 83158 KL
+// 149 : 57; with nothing to leave out some 3 us are lost, 903, 1920, 19487 71.0 : 74.7.
+bool gathering_can_pay(const ddlm::LmParams &q, bool kl)
+{
+    if (q.rows <= ddlm::kTileRows) return false;
+    const long items = (long)q.all_rows.n_tiles * ((q.rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem);
+    if (items > q.ctas) return true;
+    const long item_cost = (kl ? 2L : 1L) * q.K * (150 + q.all_rows.N);      // 30 to 35 us a million
+    return q.all_rows.n_tiles > 2 && 5 * items >= 4 * q.ctas && item_cost >= 400000;
+}
+
 template <bool KL>
 int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void *dw, const void *vh, const void *vw,
                    char *gathered, size_t gathered_bytes, int ctas, cudaStream_t stream)
@@ -528,11 +543,12 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
     }
     LmMaps<KL> m;
     if ((rc = make_matrix_tmap(&m.h, vh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
+    if (!q.plan) { gathered = (char *)const_cast<void *>(vh); gathered_bytes = 0; }      // (the maps are not read)
     if ((rc = make_matrix_tmap(&m.h_gathered, gathered, q.rows, q.K, kTileRows)) != DD_OK) return rc;
     m.hd = m.h; m.hd_gathered = m.h_gathered;          // not read outside the KL mode
     if (KL) {
         if ((rc = make_matrix_tmap(&m.hd, dh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
-        if ((rc = make_matrix_tmap(&m.hd_gathered, gathered + (q.can_gather ? gathered_bytes : 0), q.rows, q.K, kTileRows)) != DD_OK) return rc;
+        if ((rc = make_matrix_tmap(&m.hd_gathered, gathered + gathered_bytes, q.rows, q.K, kTileRows)) != DD_OK) return rc;
     }
     for (int i = 0; i < Widths<KL>::count; ++i) {
         if ((rc = make_matrix_tmap(&m.w[i], vw, q.V, q.K, Widths<KL>::max_n - 32 * i)) != DD_OK) return rc;
@@ -541,17 +557,20 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
     // One CTA per SM, fewer if even the narrowest tiles of all rows do not make that many items.
     const long items = (long)((q.V + Widths<KL>::max_n / 2 - 1) / (Widths<KL>::max_n / 2)) * ((q.rows + kRowsPerItem - 1) / kRowsPerItem);
     const unsigned grid = (unsigned)(items < ctas ? items : ctas);
-    lm_head_rows_kernel<KL><<<(unsigned)((q.rows + kRowsPerBlock - 1) / kRowsPerBlock), kRowsThreads, 0, stream>>>(
-        q, p.flags, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
-        static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
-    DD_CUDA_TRY(cudaGetLastError());
+    if (q.plan) {
+        q.rows_per_block = kRowsWarps * ((q.rows + kRowsWarps * kRowsBlocks - 1) / (kRowsWarps * kRowsBlocks));
+        lm_head_rows_kernel<KL><<<(unsigned)((q.rows + q.rows_per_block - 1) / q.rows_per_block), kRowsThreads, 0, stream>>>(
+            q, p.flags, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
+            static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
+        DD_CUDA_TRY(cudaGetLastError());
+    }
     lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
     DD_CUDA_TRY(cudaGetLastError());
     // one warp per row
     const unsigned fold_grid = (unsigned)(((long)q.rows + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
-    lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q.rows, q.plan);
+    lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q);
     DD_CUDA_TRY(cudaGetLastError());
-    dd::count_launch(3);
+    dd::count_launch(q.plan ? 3 : 2);
     return DD_OK;
 }
 
@@ -618,17 +637,21 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     p.partials = (Partial *)w;
     fill_params(p, nullptr, nullptr, tokens, mask_flags, mode, tau, k, seed, out_tokens, out_mask, out_score, B, P, V);
 
-    // A copy of the flagged rows' hidden states; without room for it every row is multiplied.  The list of those rows
-    // stands where the last kernel will put the rows' maxima, when nothing reads the list any more.
-    const size_t gathered_bytes = ((size_t)rows * K * 2 + 255) & ~size_t(255);
     ddlm::LmParams q;
-    q.can_gather = dd::try_bytes(&ctx->head_ws, &ctx->head_ws_bytes, (kl ? 2 : 1) * gathered_bytes, (cudaStream_t)stream) == DD_OK;
     q.rows = (int)rows; q.K = K; q.V = V;
     q.min_n = min_n;
     q.ctas = sms;
-    q.plan = (ddlm::LmPlan *)(control + kPlanOffset);
+    q.plan = nullptr;
+    q.all_rows = kl ? ddlm::plan_for<true>(q, q.rows, false) : ddlm::plan_for<false>(q, q.rows, false);
+    // A copy of the flagged rows' hidden states, where multiplying fewer rows can pay for it; without room for it every
+    // row is multiplied.  The list of those rows stands where the last kernel will put the rows' maxima, when nothing
+    // reads the list any more.
+    const size_t gathered_bytes = ((size_t)rows * K * 2 + 255) & ~size_t(255);
+    if (gathering_can_pay(q, kl) &&
+        dd::try_bytes(&ctx->head_ws, &ctx->head_ws_bytes, (kl ? 2 : 1) * gathered_bytes, (cudaStream_t)stream) == DD_OK)
+        q.plan = (ddlm::LmPlan *)(control + kPlanOffset);
     q.row_map = p.row_argmax;
-    char *gathered = (char *)(q.can_gather ? ctx->head_ws : ctx->verify_ws);
+    char *gathered = (char *)ctx->head_ws;
     return kl ? launch_lm_head<true>(q, p, drafter_hidden, drafter_weight, verifier_hidden, verifier_weight, gathered,
                                      gathered_bytes, ctas, (cudaStream_t)stream)
               : launch_lm_head<false>(q, p, nullptr, nullptr, verifier_hidden, verifier_weight, gathered, 0, ctas,

@@ -251,3 +251,14 @@ def test_without_room_for_the_gathered_rows(dd):
     torch.cuda.synchronize()
     assert before - free() >= hidden.numel() * 2
     assert dd.verify_status() == 0
+
+
+# Rows gathered or not: nothing flagged where rows are not listed; many rows (more than one for a warp of the listing
+# kernel) with two tiles of the vocabulary, where few and where most of them are flagged, and with three.
+@pytest.mark.parametrize("B,P,K,V,share", [(1, 20, 128, 1000, 0.0), (2, 500, 64, 300, 0.0), (3, 8000, 64, 300, 0.15),
+                                           (3, 8000, 64, 300, 0.8), (3, 8000, 64, 700, 0.3)])
+@pytest.mark.parametrize("mode", [CONF, KL])
+def test_rows_gathered_or_not(dd, oracle_mod, B, P, K, V, share, mode):
+    dh, dw, vh, vw, tokens, flags = synth.lm_head_pair_inputs(B, P, K, V, "all", 0.2, seed=P + V)
+    flags[:] = np.random.default_rng(P).random((B, P)) < share
+    compare(dd, oracle_mod, vh, vw, tokens, flags, mode, 0.3, 5, 1, drafter=(dh, dw) if mode == KL else (None, None))
