@@ -9,10 +9,13 @@ missing the first call raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import torch
 from torch import Tensor
+
+from .build import host_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdualdiff.so")
@@ -113,10 +116,25 @@ def load(path) -> ctypes.CDLL:
     return L
 
 
-try:
-    from . import _host_call as _fast        # the native form of the wrappers below (csrc/host_call.cpp)
-except ImportError:
-    _fast = None                             # not built: the Python form serves every call
+_fast = None        # the native form of the wrappers below (csrc/host_call.cpp); None: the Python form serves every call
+
+
+def load_native():
+    """Loads the native form if it has been built for this Python and torch; build.build() calls it again."""
+    global _fast
+    path = host_path()
+    if _fast is None and os.path.exists(path):
+        name = __package__ + "._host_call"
+        spec = importlib.util.spec_from_file_location(name, path)
+        try:
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+        except ImportError:
+            return
+        _fast = module
+
+
+load_native()
 
 
 def _addresses(L):
