@@ -24,6 +24,16 @@ def to_torch_bf16(bits, device=None, pin=False):
     return t.pin_memory() if pin else t
 
 
+def off_vector_boundary(bits):
+    """The same numbers on the device in a tensor that starts in the middle of a 16-byte vector."""
+    import torch
+    big = torch.zeros(bits.size + 8, dtype=torch.bfloat16, device="cuda")
+    view = big[3:3 + bits.size].view(bits.shape)
+    view.copy_(to_torch_bf16(bits, "cuda"))
+    assert view.data_ptr() % 16 != 0
+    return view
+
+
 def bf16_tensor_to_f64(t):
     import torch
     return t.detach().to("cpu").to(torch.float64).numpy()

@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 from paper_2604_05250_b200 import synth
-from tests._parity import to_torch_bf16
+from tests._parity import off_vector_boundary, to_torch_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -22,6 +22,13 @@ def libs():
     from paper_2604_05250_b200 import binding, build
     build.build()
     return binding, build.build_check()
+
+
+def fresh_outputs(B, P):
+    import torch
+    return dict(out_tokens=torch.empty(B, P, dtype=torch.int32, device="cuda"),
+                out_mask=torch.empty(B, P, dtype=torch.uint8, device="cuda"),
+                out_score=torch.empty(B, P, dtype=torch.float32, device="cuda"))
 
 
 def both_builds(binding, check_path, call):
@@ -40,13 +47,22 @@ def both_builds(binding, check_path, call):
 
 
 @pytest.mark.parametrize("B,P,V,flagged,mode", [
+    # the row kernel
     (1, 128, 1024, 32, KL),                      # cfg0
-    (2, 96, 20000, 61, KL | PROB),               # ragged last chunk, rows cut by range boundaries
+    (2, 96, 20000, 61, KL | PROB),               # two CTAs a row, ragged last piece
     (3, 40, 126464, 33, CONF),                   # the LLaDA vocabulary
-    (2, 50, 1003, 31, KL),                       # V % 8 != 0: the element-wise kernel
-    (15, 700, 64, 380, CONF | PROB),             # many short rows, sequences beyond the register-resident decision
-    (1, 1500, 4104, 900, TRUST | EMIT),          # a sequence beyond the register-resident decision
+    (1, 20, 126464, 20, KL),                     # clusters of eight
+    (2, 50, 1003, 31, KL),                       # rows off vector boundaries
+    (15, 700, 64, 380, CONF | PROB),             # many short rows, sequences beyond the short decision
+    (1, 1500, 4104, 900, TRUST | EMIT),          # a sequence beyond the short decision
     (4, 8, 8, 0, KL),                            # nothing flagged: every sequence passes through
+    # the streaming kernel: rows cut by range boundaries, on and off vector boundaries; short rows, several rounds
+    (2, 200, 65000, 150, KL | PROB),
+    (2, 200, 65003, 150, KL),
+    (4, 256, 65003, 40, CONF),
+    (60, 700, 64, 500, KL),
+    (24, 1500, 37, 900, CONF | PROB),
+    (6, 6000, 1003, 0, KL),
 ])
 def test_verify_addresses_stay_inside(libs, B, P, V, flagged, mode):
     import torch
@@ -57,26 +73,38 @@ def test_verify_addresses_stay_inside(libs, B, P, V, flagged, mode):
     both_builds(binding, check_path, lambda: binding.verify(t[0], t[1], t[2], t[3], mode, 0.5, 4, 9))
 
 
-def test_static_scratch_and_unmask(libs):
+@pytest.mark.parametrize("B,P,V,flagged,mode", [
+    (2, 50, 1003, 31, KL), (1, 24, 20000, 17, CONF), (1, 1900, 203, 1000, KL | PROB), (1, 2500, 203, 1200, CONF),
+])
+@pytest.mark.parametrize("static", [False, True])
+def test_element_wise_kernel(libs, B, P, V, flagged, mode, static):
+    """Logits off 16-byte boundaries, sequences inside its key area and beyond it, both scratches."""
     import torch
     binding, check_path = libs
-    dra, ver, tokens, flags = synth.verify_inputs(2, 96, 20000, 61, 0.2, seed=3)
-    t = [to_torch_bf16(dra, "cuda"), to_torch_bf16(ver, "cuda"), torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()]
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=P + V)
+    t = [off_vector_boundary(dra) if (mode & 0xFF) == KL else None, off_vector_boundary(ver),
+         torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()]
+    both_builds(binding, check_path, lambda: binding.verify(t[0], t[1], t[2], t[3], mode, 0.5, 4, 9, static_scratch=static,
+                                                            **(fresh_outputs(B, P) if static else {})))
 
-    def static_call():
-        outs = dict(out_tokens=torch.empty(2, 96, dtype=torch.int32, device="cuda"),
-                    out_mask=torch.empty(2, 96, dtype=torch.uint8, device="cuda"),
-                    out_score=torch.empty(2, 96, dtype=torch.float32, device="cuda"))
-        return binding.verify(t[0], t[1], t[2], t[3], KL, 0.5, 4, 9, static_scratch=True, **outs)
-    both_builds(binding, check_path, static_call)
+
+@pytest.mark.parametrize("B,P,V,flagged", [(2, 96, 20000, 61), (2, 200, 65003, 150)])      # row and streaming kernel
+def test_static_scratch_and_unmask(libs, B, P, V, flagged):
+    import torch
+    binding, check_path = libs
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=3)
+    t = [to_torch_bf16(dra, "cuda"), to_torch_bf16(ver, "cuda"), torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()]
+    both_builds(binding, check_path, lambda: binding.verify(t[0], t[1], t[2], t[3], KL, 0.5, 4, 9, static_scratch=True,
+                                                            **fresh_outputs(B, P)))
     both_builds(binding, check_path, lambda: binding.unmask(t[1], t[2], t[3], 0.3, 2))
 
 
+@pytest.mark.parametrize("B,P,K,V", [(2, 300, 128, 4100), (3, 700, 64, 20000)])        # every row; flagged rows only
 @pytest.mark.parametrize("mode", [CONF | PROB, KL])
-def test_fused_heads(libs, mode):
+def test_fused_heads(libs, mode, B, P, K, V):
     import torch
     binding, check_path = libs
-    dh, dw, vh, vw, tokens, flags = synth.lm_head_pair_inputs(2, 300, 128, 4100, "uniform_25_100", 0.2, seed=8)
+    dh, dw, vh, vw, tokens, flags = synth.lm_head_pair_inputs(B, P, K, V, "uniform_25_100", 0.2, seed=8)
     t = [to_torch_bf16(x, "cuda") for x in (dh, dw, vh, vw)]
     tok, fl = torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()
     d = t[:2] if mode == KL else [None, None]

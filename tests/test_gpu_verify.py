@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2604_05250_b200 import synth
-from tests._parity import Guarded, check_verify, to_torch_bf16
+from tests._parity import Guarded, check_verify, off_vector_boundary, to_torch_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -21,11 +21,13 @@ def dd():
     return binding
 
 
-def run_gpu(dd, dra, ver, tokens, flags, mode, tau, k, seed, host=False):
+def run_gpu(dd, dra, ver, tokens, flags, mode, tau, k, seed, host=False, off=False):
+    """off: logits off 16-byte boundaries, which take the element-wise kernel."""
     import torch
     dev = None if host else "cuda"
-    t_ver = to_torch_bf16(ver, dev, pin=host)
-    t_dra = None if dra is None else to_torch_bf16(dra, dev, pin=host)
+    logits = off_vector_boundary if off else (lambda bits: to_torch_bf16(bits, dev, pin=host))
+    t_ver = logits(ver)
+    t_dra = None if dra is None else logits(dra)
     t_tok = torch.from_numpy(tokens)
     t_fl = torch.from_numpy(flags)
     if host:
@@ -44,11 +46,11 @@ def run_gpu(dd, dra, ver, tokens, flags, mode, tau, k, seed, host=False):
     return ot.cpu().numpy(), om.cpu().numpy(), osc.cpu().numpy()
 
 
-def compare(dd, oracle_mod, dra, ver, tokens, flags, mode, tau, k, seed, host=False):
+def compare(dd, oracle_mod, dra, ver, tokens, flags, mode, tau, k, seed, host=False, off=False):
     algo = mode & 0xFF
     d_in = dra if algo == KL else None
     ref = oracle_mod.verify(d_in, ver, tokens, flags, mode, tau, k, seed)
-    ot, om, osc = run_gpu(dd, d_in, ver, tokens, flags, mode, tau, k, seed, host=host)
+    ot, om, osc = run_gpu(dd, d_in, ver, tokens, flags, mode, tau, k, seed, host=host, off=off)
     return check_verify(ot, om, osc, ref, flags, tokens), ref, (ot, om, osc)
 
 
@@ -66,9 +68,10 @@ def test_config0_tiny(dd, oracle_mod, mode):
 @pytest.mark.parametrize("V", [8, 1000, 1003, 8192, 8200, 8201, 20000, 32000])
 @pytest.mark.parametrize("mode", [KL, CONF])
 def test_vocab_sizes_and_ragged_tails(dd, oracle_mod, V, mode):
-    """Several chunks plus a ragged tail; V % 8 != 0 takes the element-wise path."""
+    """Several pieces or chunks plus a ragged tail, in the row kernel and in the element-wise kernel."""
     dra, ver, tokens, flags = synth.verify_inputs(2, 24, V, 17, 0.2, seed=V)
     compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 4, 1)
+    compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 4, 1, off=True)
 
 
 def test_config1_llada_shaped_full_size(dd, oracle_mod):
@@ -145,15 +148,24 @@ def test_many_short_rows_and_long_sequences(dd, oracle_mod):
     dra, ver, tokens, flags = synth.verify_inputs(15, 8192, 64, 5700, 0.2, seed=31)
     compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 0.5, 40, 3)
     compare(dd, oracle_mod, dra, ver, tokens, flags, CONF | PROB, 0.5, 7, 3)
-    # longer than what a lane keeps in registers (1024 keys), inside the key area
+    # the row kernel's decision of sequences longer than 512 positions
     dra, ver, tokens, flags = synth.verify_inputs(2, 1500, 4104, 900, 0.2, seed=32)
     compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 0.5, 33, 1)
-    # the element-wise kernel (V % 8 != 0): inside its key area (2048 keys) and beyond it, where
-    # every pass of the decision stage re-reads the scores from memory (the streaming kernel's
+    # the element-wise kernel (logits off 16-byte boundaries): inside its key area (2048 keys) and beyond
+    # it, where every pass of the decision stage re-reads the scores from memory (the streaming kernel's
     # area holds the longest sequence the library accepts)
     for P, nflag in ((1900, 1000), (2500, 1200)):
         dra, ver, tokens, flags = synth.verify_inputs(1, P, 203, nflag, 0.2, seed=P)
         compare(dd, oracle_mod, dra, ver, tokens, flags, KL | PROB, 0.5, 21, 5)
+        compare(dd, oracle_mod, dra, ver, tokens, flags, KL | PROB, 0.5, 21, 5, off=True)
+
+
+@pytest.mark.parametrize("B,P,V,flagged", [(60, 700, 64, 500), (24, 1500, 37, 900), (6, 6000, 64, 3000)])
+@pytest.mark.parametrize("mode", [KL, CONF | PROB])
+def test_long_sequences_in_the_streaming_kernel(dd, oracle_mod, B, P, V, flagged, mode):
+    """More than 32768 rows: the streaming kernel, its decision from registers (up to 1024 positions) and from its key area."""
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=P)
+    compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 33, 1)
 
 
 def test_exact_ties_in_verifier_row(dd, oracle_mod):
@@ -236,6 +248,12 @@ def test_results_do_not_depend_on_the_grid(dd, oracle_mod, cta_cap):
     """Same inputs on 1, 7, 37 CTAs and on every SM: tokens, masks and scores bit-identical (which
     warp computes a unit, and in which order units finish, must not matter)."""
     cases = [
+        # the streaming kernel: rows on and off vector boundaries, long and short
+        (synth.verify_inputs(2, 200, 65000, 150, 0.2, seed=43), KL | PROB, 0.5, 8, 0),
+        (synth.verify_inputs(2, 200, 65003, 150, 0.2, seed=44), KL, 0.5, 4, 1),
+        (synth.verify_inputs(4, 256, 65003, 40, 0.2, seed=45), CONF | PROB, 0.5, 4, 2),
+        (synth.verify_inputs(6, 6000, 41, 3000, 0.2, seed=46), KL, 0.5, 40, 3),
+        # the row kernel, whose grid the cap leaves alone
         (synth.verify_config_inputs(0), KL | PROB, 0.5, 8, 0),
         (synth.verify_inputs(2, 40, 20000 + 8 * 37, 29, 0.2, seed=41), KL, 0.5, 4, 1),       # ragged last chunk
         (synth.verify_inputs(2, 40, 20000 + 8 * 37, 29, 0.2, seed=41), CONF | PROB, 0.5, 4, 2),
@@ -258,7 +276,7 @@ def test_results_do_not_depend_on_the_grid(dd, oracle_mod, cta_cap):
 @pytest.mark.parametrize("V", [20000, 1003])
 def test_token_excluded_by_the_verifier_alone(dd, oracle_mod, V):
     """p_V(x) = 0 where p_D(x) > 0: the divergence of Eq. 5 is infinite, in the oracle and in both
-    kernels (the streaming path meets the token as a finite logit of -3.4e38 and must notice)."""
+    kernels (the vector paths meet the token as a finite logit of -3.4e38 and must notice)."""
     ninf = np.uint16(0xFF80)
     dra, ver, tokens, flags = synth.verify_inputs(2, 12, V, 12, 0.25, seed=77 + V)
     rng = np.random.default_rng(V + 1)
@@ -268,11 +286,12 @@ def test_token_excluded_by_the_verifier_alone(dd, oracle_mod, V):
     both = rng.choice(V, size=40, replace=False)
     dra[1, 4, both] = ninf; ver[1, 4, both] = ninf                     # a row that stays finite
     tokens[:] = np.argmax(synth.bf16_bits_to_f32(dra), axis=2)
-    _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 0.5, 3, 7)
-    inf_at = np.zeros((2, 12), dtype=bool)
-    inf_at[0, 2] = inf_at[1, 3] = True
-    assert np.isposinf(ref["out_score"][inf_at]).all() and np.isposinf(got[2][inf_at]).all()
-    assert np.isfinite(ref["out_score"][~inf_at]).all() and np.isfinite(got[2][~inf_at]).all()
+    for off in (False, True):
+        _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 0.5, 3, 7, off=off)
+        inf_at = np.zeros((2, 12), dtype=bool)
+        inf_at[0, 2] = inf_at[1, 3] = True
+        assert np.isposinf(ref["out_score"][inf_at]).all() and np.isposinf(got[2][inf_at]).all()
+        assert np.isfinite(ref["out_score"][~inf_at]).all() and np.isfinite(got[2][~inf_at]).all()
 
 
 @pytest.mark.parametrize("V", [4096, 20000, 1003])
@@ -291,8 +310,9 @@ def test_excluded_tokens(dd, oracle_mod, V):
         dra[1, 7, :V - 3] = ninf; ver[1, 7, :V - 3] = ninf             # nearly everything
         tokens[:] = np.argmax(synth.bf16_bits_to_f32(dra), axis=2)
         for mode in (KL, CONF, KL | PROB):
-            _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 3, 7)
-            assert np.isfinite(ref["out_score"]).all() and np.isfinite(got[2]).all()
+            for off in (False, True):
+                _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 3, 7, off=off)
+                assert np.isfinite(ref["out_score"]).all() and np.isfinite(got[2]).all()
 
 
 # vocabularies that put rows anywhere between 16-byte boundaries: fewer logits than a vector, one vector more
@@ -316,13 +336,7 @@ def test_logits_off_16_byte_boundaries(dd, oracle_mod, V, mode):
     import torch
     dra, ver, tokens, flags = synth.verify_inputs(2, 24, V, 17, 0.2, seed=V)
     ref = oracle_mod.verify(dra if mode == KL else None, ver, tokens, flags, mode, 0.5, 4, 1)
-
-    def off(bits):
-        big = torch.zeros(bits.size + 8, dtype=torch.bfloat16, device="cuda")
-        view = big[3:3 + bits.size].view(bits.shape)
-        view.copy_(to_torch_bf16(bits, "cuda"))
-        assert view.data_ptr() % 16 != 0
-        return view
+    off = off_vector_boundary
     out = dd.verify(off(dra) if mode == KL else None, off(ver), torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda(),
                     mode, 0.5, 4, 1)
     torch.cuda.synchronize()

@@ -13,18 +13,18 @@ import numpy as np
 import pytest
 
 from paper_2604_05250_b200 import synth
-from tests._parity import SCORE_ABS_FLOOR, SCORE_REL, check_verify, to_torch_bf16
+from tests._parity import SCORE_ABS_FLOOR, SCORE_REL, check_verify, off_vector_boundary, to_torch_bf16
 
 pytestmark = pytest.mark.gpu
 
 KL, CONF, PROB = 1, 2, 0x100
 
 
-def both_entry_points(dd, oracle_mod, shape, mode, seed):
+def both_entry_points(dd, oracle_mod, shape, mode, seed, off=False):
     import torch
     B, P, V, nflag = shape
     dra, ver, tokens, flags = synth.verify_inputs(B, P, V, nflag, 0.2, seed=seed)
-    t_dra, t_ver = to_torch_bf16(dra, "cuda"), to_torch_bf16(ver, "cuda")
+    t_dra, t_ver = (off_vector_boundary(x) if off else to_torch_bf16(x, "cuda") for x in (dra, ver))
     t_tok, t_fl = torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()
     if (mode & 0xFF) != KL:
         t_dra, dra = None, None
@@ -62,8 +62,10 @@ def test_static_scratch_matches_dd_verify_on_two_calls_in_a_row(oracle_mod):
     both_entry_points(dd, oracle_mod, (2, 96, 20000, 61), KL | PROB, seed=21)
     frees = [both_entry_points(dd, oracle_mod, (3, 40, 126464, 33), KL, seed=22),
              both_entry_points(dd, oracle_mod, (1, 128, 1024, 32), CONF, seed=23),
-             # V % 8 != 0: the element-wise kernel runs on the fixed array as well
-             both_entry_points(dd, oracle_mod, (2, 50, 1003, 31), KL, seed=24)]
+             # rows off vector boundaries; tensors off them, which take the element-wise kernel; the streaming kernel
+             both_entry_points(dd, oracle_mod, (2, 50, 1003, 31), KL, seed=24),
+             both_entry_points(dd, oracle_mod, (2, 50, 1003, 31), KL, seed=25, off=True),
+             both_entry_points(dd, oracle_mod, (2, 200, 65003, 150), KL, seed=26)]
     # once the first call on the device has looked up the array, a call takes no device memory
     for before, after in frees:
         assert after == before
