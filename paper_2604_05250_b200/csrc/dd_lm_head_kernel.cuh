@@ -137,9 +137,10 @@ constexpr int kRowsWarps = kRowsThreads / 32;
 constexpr int kRowsBlocks = 1024;
 template <bool KL>
 __global__ void __launch_bounds__(kRowsThreads)
-lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden, uint4 *gathered,
+lm_head_rows_kernel(const LmParams q, const ddv::VerifyParams p, const uint4 *hidden, uint4 *gathered,
                     const uint4 *hidden_d, uint4 *gathered_d)
 {
+    const uint8_t *flags = p.flags;
     __shared__ int s_before, s_all;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int first = blockIdx.x * q.rows_per_block;
@@ -175,10 +176,10 @@ lm_head_rows_kernel(const LmParams q, const uint8_t *flags, const uint4 *hidden,
         seen += __popc(mask);
         if (!(mask >> warp & 1u)) continue;
         const int row = row0 + warp;
-        if (lane == 0) q.row_map[at] = row;
+        if (lane == 0) q.row_map[ddv::checked(p, at, q.rows, ddv::kSiteRow)] = row;
         auto copy = [&](uint4 *dst, const uint4 *src) {
-            dst += (size_t)at * vecs;
-            src += (size_t)row * vecs;
+            dst += ddv::checked_run(p, (long)at * vecs, vecs, (long)q.rows * vecs, ddv::kSiteHidden);
+            src += ddv::checked_run(p, (long)row * vecs, vecs, (long)q.rows * vecs, ddv::kSiteHidden);
 #pragma unroll 8
             for (int i = lane; i < vecs; i += 32) dst[i] = src[i];
         };
@@ -276,7 +277,7 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const LmPlan &plan, 
         int row = walk.row0 + (walk.two ? acc * kTileRows : 0) + (warp & 3) * 32 + lane;
         // the row of the caller's tensors, or -1: nothing to store
         if (row >= plan.n_rows) row = -1;
-        else if (plan.gathered) row = q.row_map[row];
+        else if (plan.gathered) row = q.row_map[ddv::checked(p, row, q.rows, ddv::kSiteRow)];
         else if (!p.flags[row]) row = -1;
         bool arrived = false;
         for (uint32_t it = 0; it < (1u << 22); ++it) {

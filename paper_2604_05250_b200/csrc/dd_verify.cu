@@ -560,7 +560,7 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
     if (q.plan) {
         q.rows_per_block = kRowsWarps * ((q.rows + kRowsWarps * kRowsBlocks - 1) / (kRowsWarps * kRowsBlocks));
         lm_head_rows_kernel<KL><<<(unsigned)((q.rows + q.rows_per_block - 1) / q.rows_per_block), kRowsThreads, 0, stream>>>(
-            q, p.flags, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
+            q, p, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
             static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
         DD_CUDA_TRY(cudaGetLastError());
     }

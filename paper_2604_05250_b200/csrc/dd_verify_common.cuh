@@ -65,10 +65,11 @@ __device__ __forceinline__ void report_expired(const VerifyParams &p, unsigned c
 // index these kernels form into a caller's tensor or into the library's scratch goes through
 // checked(), which compares it with the extent, records kErrBounds | site << 8 in the health word
 // and substitutes index 0 (a legal one) on a violation, so that the launch finishes and the host
-// reads the word.  In the normal build checked() is the identity.  (The attention kernels address
-// global memory through tensor maps only, which the hardware clips.)
+// reads the word.  In the normal build checked() is the identity.  (The attention kernels load through tensor
+// maps, which the hardware clips, and two of them store through one; the others store whole rows of the output
+// whose number has just been compared with the number of queries.)
 constexpr unsigned kErrBounds = 0xB000;
-enum : unsigned { kSitePartial = 1, kSiteRow = 2, kSiteSeq = 3, kSiteLogit = 4, kSiteOut = 5, kSiteFlag = 6 };
+enum : unsigned { kSitePartial = 1, kSiteRow = 2, kSiteSeq = 3, kSiteLogit = 4, kSiteOut = 5, kSiteFlag = 6, kSiteHidden = 7 };
 #ifdef DD_BOUNDS_CHECK
 constexpr bool kBoundsChecked = true;
 #else
