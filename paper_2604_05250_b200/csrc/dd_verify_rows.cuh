@@ -80,12 +80,12 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
         int ordinal = 0;
 #pragma unroll 1
         for (int x = first * kStep; x < extent; x += stride, ++ordinal) {
-            const int n = min(kStep, extent - x);
+            const int n = min(kStep, extent - x), whole = min((n + 7) & ~7, present - x);      // logits in vectors loaded whole
             uint4 rv[kVecPerThread], rd[kVecPerThread];
             const uint4 ninf = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             auto load = [&](const uint16_t *src, int vec) {
                 const int e = vec * 8;
-                if (e >= n || x + e + 8 > present) return ninf;
+                if (e + 8 > whole) return ninf;
                 return ld_streamed(src + checked_run(p, x + e, 8, n_rows * p.V - (long)off, kSiteLogit), policy);
             };
 #pragma unroll
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
                     const int e0 = vec * 8;
                     if (e0 >= n || (e0 + 8 <= n && e0 >= from)) return;
                     uint32_t w[4] = {r.x, r.y, r.z, r.w};
-                    const bool apart = x + e0 + 8 > present;
+                    const bool apart = e0 + 8 > whole;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int e = e0 + i;
