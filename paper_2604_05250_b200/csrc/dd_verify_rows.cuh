@@ -10,6 +10,7 @@
 // that completes a sequence decides it with all its threads.  Results do not depend on which CTA runs when.
 #pragma once
 
+#include "dd_ptx.cuh"
 #include "dd_verify_decide_block.cuh"
 #include "dd_verify_stream.cuh"
 
@@ -17,24 +18,6 @@ namespace ddv {
 
 constexpr int kRWarps = 8;
 constexpr int kRMaxCluster = 8;
-
-__device__ __forceinline__ void named_sync(uint32_t id, uint32_t count)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
-// 16 bytes of the same shared variable in another CTA of the cluster.
-__device__ __forceinline__ float4 ld_cluster(const void *ptr, int rank)
-{
-    float4 r;
-    uint32_t addr;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(s_addr(ptr)), "r"(rank));
-    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(addr) : "memory");
-    return r;
-}
 
 __device__ __forceinline__ uint4 ld_streamed(const uint16_t *ptr, uint64_t policy)
 {
@@ -136,24 +119,26 @@ __global__ void __launch_bounds__(32 * kRWarps, 3) verify_rows_kernel(const __gr
         }
         if (lane == 0) s_part[warp] = part;
         __syncwarp();
-        if (wpr > 1 && cluster == 1) named_sync(1 + warp / wpr, 32 * wpr);
+        if (wpr > 1 && cluster == 1) cta_bar_sync(1 + warp / wpr, 32 * wpr);
     }
     const int pieces = (row_head(row, p.V) + p.V + kStep - 1) / kStep;
     const Partial *parts = s_part + warp - warp % wpr;
     if (cluster > 1) {
         // (the flag is the same in the whole cluster)
         if (mine) {
-            cluster_sync();
+            ddptx::cluster_arrive();
+            ddptx::cluster_wait();
             if (rank == 0 && warp == 0) {
                 // 32 bytes of every warp of the cluster, in the order of their pieces
                 for (int i = lane; i < cluster * kRWarps; i += 32) {
-                    const float4 *src = reinterpret_cast<const float4 *>(s_part + i % kRWarps);
-                    reinterpret_cast<float4 *>(s_all + i)[0] = ld_cluster(src, i / kRWarps);
-                    reinterpret_cast<float4 *>(s_all + i)[1] = ld_cluster(src + 1, i / kRWarps);
+                    const uint32_t src = ddptx::cluster_addr(s_addr(s_part + i % kRWarps), i / kRWarps);
+                    reinterpret_cast<float4 *>(s_all + i)[0] = ddptx::ld_cluster_v4(src);
+                    reinterpret_cast<float4 *>(s_all + i)[1] = ddptx::ld_cluster_v4(src + 16);
                 }
                 __syncwarp();
             }
-            cluster_sync();                                          // a peer's shared memory outlives its reads
+            ddptx::cluster_arrive();                                 // a peer's shared memory outlives its reads
+            ddptx::cluster_wait();
         }
         if (rank != 0) return;
         parts = s_all;
