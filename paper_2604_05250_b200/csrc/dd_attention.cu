@@ -897,16 +897,19 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     p.longest_first = longest_first(BH * m_blocks, sms);
     if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
     // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in every item):
-    // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four key tiles or
+    // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four whole key tiles or
     // more: the kernel whose rounds run across items (16 x 32 heads of 512 tokens 101 us with a CTA per item,
-    // 87 with the short kernel, 81 with this one; of 1024 299, 313 and 276).  Two key tiles, and D = 64: the short
+    // 75 with the short kernel, 71 with this one; of 1024 299, 294 and 264).  Fewer, and D = 64: the short
     // kernel (64 x 32 heads of 256 tokens at D = 128: 148, 99 and 113; 16 x 32 of 512 at D = 64: 73, 61 and 63).
+    // A fourth tile that is not nearly whole counts as none (short : this kernel, 64 x 32 heads of 385 tokens 286 :
+    // 339, of 400 287 : 388; 16 x 32 of 460 79 : 92, of 470 78.9 : 80.3, of 480 80.8 : 80.3, of 490 81.2 : 79.8); from six tiles
+    // on it makes no difference (40 x 32 of 641 420 : 392, of 660 418 : 412, of 700 435 : 433).
     // Items of one query tile among those of two: a CTA per item (3 x 24 heads of 1357: 80 against 89).
     if (BH * m_blocks > sms && nkv <= 16 && (Nq - 1) % (kQTiles * kBlockM) >= kBlockM) {
         static bool attr_done[3][64] = {};
         if (D == 64)
             return launch_persistent(attention_short_kernel<64>, SmemP<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv, to);
-        if (nkv < 4)
+        if (Nkv < 480)
             return launch_persistent(attention_short_kernel<128>, SmemP<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv, to);
         return launch_persistent(attention_persistent_kernel<128>, SmemL<128>::kTotal + 1024, attr_done[2], p, sms, s, tq, tk, tv);
     }

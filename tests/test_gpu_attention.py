@@ -182,9 +182,10 @@ def test_many_short_items_match_one_item_per_cta(dd):
     assert torch.equal(whole, torch.cat(parts, dim=1))
 
 
-# where the choice of kernel changes (more items than SMs; 4 and 16 key tiles), one key in the last tile,
-# one query tile in the last item, and D = 64, whose exponentials are partly computed as a polynomial
+# where the choice of kernel changes (more items than SMs; 480 keys and 16 key tiles), one key in the last tile,
+# heads whose last 256 rows are one query tile, and D = 64, whose exponentials are partly computed as a polynomial
 @pytest.mark.parametrize("B,H,N,D", [(1, 80, 385, 128), (1, 38, 897, 128), (2, 80, 300, 128), (1, 19, 2048, 128),
+                                     (1, 80, 479, 128), (1, 80, 480, 128),
                                      (1, 17, 2177, 128), (1, 80, 385, 64), (1, 75, 500, 64), (1, 50, 600, 64)])
 def test_kernel_choice(dd, oracle_mod, B, H, N, D):
     import torch
