@@ -35,7 +35,6 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <float.h>
-#include <math_constants.h>
 #include <math.h>
 
 #include <mutex>
@@ -184,12 +183,13 @@ __device__ __forceinline__ void weights_to_tmem(const float (&s)[N], int q, int 
 
 // A key tile with maximum mx (times scale) meets a row: the first tile sets the row's reference point, a later one
 // moves it if it outgrows it by more than the allowed step; then O is rescaled in tensor memory.
-template <int D>
+// kPart: the row's keys are shared out, and these may all have a score of -inf where others do not; the reference point is
+// then the lowest number, so that their weights are 0 and not NaN.
+template <int D, bool kPart>
 __device__ __forceinline__ void move_reference(uint32_t tO, bool first, float mx, float &m_ref, float &l_run)
 {
     if (first) {
-        // (a row of which every score so far is -inf: the lowest number, so that their weights are 0 and not NaN)
-        m_ref = mx == -INFINITY ? -FLT_MAX : mx;
+        m_ref = kPart ? fmaxf(mx, -FLT_MAX) : mx;
     } else if (__any_sync(0xffffffffu, mx > m_ref + kRescaleStep)) {
         const float m_new = mx > m_ref + kRescaleStep ? mx : m_ref;
         const float alpha = ex2(m_ref - m_new);       // 1 where the row does not move
@@ -214,7 +214,7 @@ __device__ __forceinline__ void move_reference(uint32_t tO, bool first, float mx
 // (each time: wait for the stores, fence, arrive), so that P V runs while the last quarter is computed.  A
 // row that moves rescales O in tensor memory.  O then holds the sum over the earlier tiles: their P V
 // products were issued before this S product by the same thread, so they had completed when S arrived.
-template <int D, typename Early>
+template <int D, bool kPart, typename Early>
 __device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, bool first, int valid, float c, float &m_ref,
                                              float &l_run, Early early)
 {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, bool firs
     tmem_wait_ld();
     const bool masked = valid < kBlockN;
     const float mx = (masked ? row_max<true>(s, valid) : row_max<false>(s, valid)) * c;
-    move_reference<D>(tO, first, mx, m_ref, l_run);
+    move_reference<D, kPart>(tO, first, mx, m_ref, l_run);
     float2 sum_a = make_float2(0.f, 0.f), sum_b = sum_a;
     auto weights = [&](auto is_masked, auto poly) {
 #pragma unroll
@@ -400,7 +400,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 tc_fence_after();
                 const int valid = keys - j * kBlockN;      // keys of this tile that exist
                 const bool masked = valid < kBlockN;
-                softmax_tile<D>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
+                softmax_tile<D, false>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
                     if (kBlock && masked) return;          // not before the value rows below are clear
                     tmem_wait_st();
                     tc_fence_before();

@@ -154,7 +154,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
             for (int j = 0; j < nkv; ++j, ++t_run) {
                 if (!mbar_wait(bar_s_full(g), t_run & 1)) { err = kErrWaitS; break; }
                 tc_fence_after();
-                softmax_tile<D>(tS, tO, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run,
+                softmax_tile<D, false>(tS, tO, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run,
                     [&] {                        // three quarters of the weights are stored
                         tmem_wait_st();
                         tc_fence_before();

@@ -46,12 +46,8 @@ struct SplitLayout {
     static_assert(q_bytes(64) >= 2 * 128 * 8, "the query buffer holds the rows' reference points and sums");
 };
 
-// softmax_tile for a row that takes only the tile's keys key0 .. key0 + K - 1.  The others' weights are not 0 but
-// the smallest normal bf16 number: their values are the other copies' to weigh, and an infinite one times 0 would be a
-// NaN in this copy.  2^-126 of any finite value is nothing beside a row whose largest weight is 1 or more.
-constexpr uint32_t kOthersWeights = 0x00800080u;
-// Of a row that no key has a weight in, NaN and not infinity: its accumulator holds the others' values.
-__device__ __forceinline__ float normaliser(float sum) { return sum == 0.f ? CUDART_NAN_F : 1.f / sum; }
+// softmax_tile for a row that takes only the tile's keys key0 .. key0 + K - 1; the others' weights are not written, and
+// the products with those keys leave the row alone.
 template <int D, int K>
 __device__ __forceinline__ void softmax_part(uint32_t tS, uint32_t tO, int key0, bool first, int valid, float c, float &m_ref,
                                              float &l_run)
@@ -64,7 +60,7 @@ __device__ __forceinline__ void softmax_part(uint32_t tS, uint32_t tO, int key0,
     const int own = valid - key0;
     const bool masked = own < K;
     const float mx = own <= 0 ? -INFINITY : (masked ? row_max<true>(s, own) : row_max<false>(s, own)) * c;
-    move_reference<D>(tO, first, mx, m_ref, l_run);
+    move_reference<D, true>(tO, first, mx, m_ref, l_run);
     float2 sum_a = make_float2(0.f, 0.f), sum_b = sum_a;
     auto weights = [&](auto is_masked, auto poly) {
 #pragma unroll
@@ -73,18 +69,12 @@ __device__ __forceinline__ void softmax_part(uint32_t tS, uint32_t tO, int key0,
     };
     if (masked) weights(std::true_type(), std::integral_constant<int, 0>());
     else weights(std::false_type(), std::integral_constant<int, kPolyOneIn<D>>());
-    uint32_t others[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) others[i] = kOthersWeights;
-#pragma unroll
-    for (int q = 0; q < kBlockN / 32; ++q)
-        if (q * 32 < key0 || q * 32 >= key0 + K) tmem_st16(tS + q * 16, others);
     sum_a = __fadd2_rn(sum_a, sum_b);
     l_run += sum_a.x + sum_a.y;
 }
 
 // G > 1 (up to 32 query rows): the query tile holds G copies of them, one above the other, and copy g (one warp)
-// takes the g-th part of every tile's keys, with next to no weight for the others and an accumulator, reference point and
+// takes the g-th part of every tile's keys (the products with those keys are for its rows only), with an accumulator, reference point and
 // sum of its own; the copies are combined at the end like the parts of a cluster.  A tile's softmax is then the work
 // of G warps instead of one, and so is the masked tile at a sequence's end: 16 x 32 heads, 32 queries over 256-1024
 // keys 42.3 -> 37.7 us, 64 x 32 157.8 -> 130.2, 50 x 32 with one query over 125-500 75.7 -> 59.6, 40 x 16 over 50-200
@@ -212,7 +202,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 tc_fence_after();
                 const int valid = keys - (j_begin + i) * kBlockN;
                 if constexpr (G > 1) softmax_part<D, kBlockN / G>(tS, tO, warp * (kBlockN / G), i == 0, valid, c, m_ref, l_run);
-                else softmax_tile<D>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
+                else softmax_tile<D, true>(tS, tO, i == 0, valid, c, m_ref, l_run, [&] {
                     tmem_wait_st();
                     tc_fence_before();
                     mbar_arrive(bar_p_early);
@@ -258,12 +248,10 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             for (int g = 0; g < G; ++g) m_all = fmaxf(m_all, ml[g * 32 + lane].x);
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-                // never 0: a copy without keys of its own holds next to nothing of the others' finite values, but
-                // their infinite ones, which 0 would turn into a NaN
-                w[g] = n_tiles > 0 ? fmaxf(ex2(ml[g * 32 + lane].x - m_all), FLT_MIN) : 0.f;
+                w[g] = n_tiles > 0 ? ex2(ml[g * 32 + lane].x - m_all) : 0.f;
                 sum += ml[g * 32 + lane].y * w[g];
             }
-            const float inv = nkv > 0 ? normaliser(sum) : 0.f;
+            const float inv = nkv > 0 ? 1.f / sum : 0.f;
             for (int c0 = warp * 16; healthy && c0 < D; c0 += 64) {
                 float acc[16];
 #pragma unroll
@@ -330,14 +318,32 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     tc_fence_after();
                     const uint64_t b = desc_v0 + (uint64_t)(slot * (kTileBytes >> 4));
                     bool ok = true;
+                    // 16 keys = two 8-row groups of 1024 bytes; column blocks of 64 are one box apart
+                    if constexpr (G == 1) {
 #pragma unroll
-                    for (int ks = 0; ks < kBlockN / 16; ++ks) {
-                        // 16 keys = two 8-row groups of 1024 bytes; column blocks of 64 are one box apart
-                        if (G == 1 && ks == 6) {
-                            if (!mbar_wait(bar_p_full, i & 1)) { ok = false; break; }
-                            tc_fence_after();
+                        for (int ks = 0; ks < kBlockN / 16; ++ks) {
+                            if (ks == 6) {
+                                if (!mbar_wait(bar_p_full, i & 1)) { ok = false; break; }
+                                tc_fence_after();
+                            }
+                            mma_ts(tmem + kColO, tmem + kColS + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (i > 0 || ks > 0));
                         }
-                        mma_ts(tmem + kColO, tmem + kColS + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (i > 0 || ks > 0));
+                    } else {
+                        constexpr int kSteps = kBlockN / 16 / G;
+                        auto product = [&](auto copy) {
+                            constexpr int g = decltype(copy)::value;
+#pragma unroll
+                            for (int k = 0; k < kSteps; ++k) {
+                                const int ks = g * kSteps + k;
+                                mma_ts_rows<g>(tmem + kColO, tmem + kColS + ks * 8, b + (uint32_t)(ks * (2048 >> 4)), kIdescO, (i > 0 || k > 0));
+                            }
+                        };
+                        product(std::integral_constant<int, 0>());
+                        product(std::integral_constant<int, 1>());
+                        if constexpr (G == 4) {
+                            product(std::integral_constant<int, 2>());
+                            product(std::integral_constant<int, 3>());
+                        }
                     }
                     if (!ok) { err = kErrWaitP; break; }
                     if (i + 1 == n_tiles) { mma_commit(bar_o_full); break; }
@@ -403,7 +409,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                         acc[4 * k] += v.x * w; acc[4 * k + 1] += v.y * w; acc[4 * k + 2] += v.z * w; acc[4 * k + 3] += v.w * w;
                     }
                 }
-                if (row < rows) store16(row, c0, acc, nkv > 0 ? normaliser(sum) : 0.f);
+                if (row < rows) store16(row, c0, acc, nkv > 0 ? 1.f / sum : 0.f);
             }
         }
         __syncwarp();
