@@ -911,7 +911,7 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
             return launch_persistent(attention_short_kernel<64>, SmemP<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv, to);
         if (Nkv < 480)
             return launch_persistent(attention_short_kernel<128>, SmemP<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv, to);
-        return launch_persistent(attention_persistent_kernel<128>, SmemL<128>::kTotal + 1024, attr_done[2], p, sms, s, tq, tk, tv);
+        return launch_persistent(attention_persistent_kernel, SmemL::kTotal + 1024, attr_done[2], p, sms, s, tq, tk, tv);
     }
     return D == 64 ? launch<64, false>(tq, tk, tv, to, p, s) : launch<128, false>(tq, tk, tv, to, p, s);
 }

@@ -1,6 +1,6 @@
 // The square, head-major case of dd_bidir_attention (Section 2.2; Eq. 3) for many items of four to sixteen
 // key tiles at D = 128: persistent CTAs, one per SM, each walking over work items blockIdx.x,
-// blockIdx.x + gridDim.x, ...  An item is up to two tiles of 128 query rows of one head.  Roles and
+// blockIdx.x + gridDim.x, ...  An item is two tiles of 128 query rows of one head.  Roles and
 // arithmetic are those of attention_kernel; the pipeline never drains between items.
 //
 // One stream of rounds.  Round r of a CTA is one key tile of one item, for both query tiles g:
@@ -9,8 +9,8 @@
 // barrier announces both, and one commit at the end of the round releases both.  Items therefore
 // follow each other like rounds do: the next item's first scores are computed while the softmax
 // groups still work on the current item's last tile or write its result.
-//   * A barrier wait costs the issuing thread 170 cycles even when its phase is complete, which the
-//     tensor core spends on products already queued, but only so many; so there are few of them: one
+//   * A barrier wait costs the issuing thread some cycles (10-40 under elect.sync) even when its phase is complete,
+//     which the tensor core spends on products already queued, but only so many; so there are few of them: one
 //     per round for the pair and two per group for its weights.
 //   * The weights of a tile are handed over in two parts: the product starts with the first three
 //     quarters of the keys while the softmax group still computes the last.
@@ -29,8 +29,8 @@
 
 constexpr int kReleases = 8;         // release barriers: round r completes phase r / 8 of barrier r % 8
 
-template <int D>
 struct SmemL {
+    static constexpr int D = 128;
     static constexpr int kTileBytes = kBlockN * D * 2;
     static constexpr int kQ = 2;                                    // query tiles
     static constexpr int kSlots = 5;                                // key and value tiles
@@ -49,12 +49,12 @@ struct SmemL {
     static_assert((kSlots - 1) / 2 + 1 <= kReleases, "release barriers");
 };
 
-template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                             const __grid_constant__ CUtensorMap tm_v, const AttnParams p)
 {
-    using L = SmemL<D>;
+    using L = SmemL;
+    constexpr int D = L::D;
     constexpr uint32_t kQ = L::kQ, kSlots = L::kSlots;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -78,18 +78,17 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int n_items = p.BH * p.m_blocks;
-    const int nkv = (p.Nkv + kBlockN - 1) / kBlockN;            // rounds per item (>= 1)
+    const int nkv = (p.Nkv + kBlockN - 1) / kBlockN;            // rounds per item (>= 2)
     const int my_items = (n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kBoxBytes = 128 * 128;
     constexpr uint32_t kColS = 0, kColO = 256;       // S_0, S_1 (128 columns each, P over them), O_0, O_1 (D each)
-    struct Item { int bh, row0, tiles; };
+    struct Item { int bh, row0; };
     auto item_at = [&](int n) {
         const int item = (int)blockIdx.x + n * (int)gridDim.x;
         Item t;
         t.bh = item / p.m_blocks;
         t.row0 = (item - t.bh * p.m_blocks) * (kQTiles * kBlockM);
-        t.tiles = p.Nq - t.row0 > kBlockM ? 2 : 1;             // query tiles that hold rows
         return t;
     };
     auto load_tile = [&](uint32_t dst, const CUtensorMap *tm, uint32_t bar, int row, int bh) {
@@ -145,11 +144,10 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
         const uint32_t tO = tmem + lane_off + kColO + g * D;
         const float c = p.scale_log2;
         const bool sectors = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;     // rows start on 32-byte boundaries
-        uint32_t t_run = 0, i_run = 0;   // key tiles and items of this group so far: phases
+        uint32_t t_run = 0;              // key tiles so far: phase
         unsigned err = 0;
         for (int n = 0; n < my_items; ++n) {
             const Item t = item_at(n);
-            if (g >= t.tiles) continue;
             float m_ref = -INFINITY, l_run = 0.f;
             for (int j = 0; j < nkv; ++j, ++t_run) {
                 if (!mbar_wait(bar_s_full(g), t_run & 1)) { err = kErrWaitS; break; }
@@ -164,8 +162,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
                 tc_fence_before();
                 mbar_arrive(bar_p_full(g));
             }
-            if (err == 0 && !mbar_wait(bar_o_full(g), i_run & 1)) err = kErrWaitO;
-            ++i_run;
+            if (err == 0 && !mbar_wait(bar_o_full(g), n & 1)) err = kErrWaitO;
             if (err != 0) { report(p, err); break; }
             // ---- epilogue: O / l -> bf16 -> global
             tc_fence_after();
@@ -221,7 +218,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
                 return true;
             };
             Item t = item_at(0);
-            bool ok = t.tiles < 2 || load_q(t, 1);
+            bool ok = load_q(t, 1);
             uint32_t r = 0;
             for (int n = 0; n < my_items && ok; ++n) {
                 const bool more_items = n + 1 < my_items;
@@ -237,10 +234,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
                         load_tile(sRing + ((2 * r + 2) % kSlots) * kTileBytes, &tm_k, bar, last ? 0 : (j + 1) * kBlockN,
                                   last ? next.bh : t.bh);
                     }
-                    if (last && more_items) {
-                        ok = load_q(next, 0);
-                        if (ok && next.tiles > 1) ok = load_q(next, 1);
-                    }
+                    if (last && more_items) ok = load_q(next, 0) && load_q(next, 1);
                 }
                 t = next;
             }
@@ -281,7 +275,6 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
             };
             uint32_t qi = 0;                       // query tiles taken over so far
             uint32_t q_cur[2] = {0, 0};            // their buffers, of the item whose scores are being issued
-            uint32_t pc[2] = {0, 0}, ic[2] = {0, 0};   // P tiles and items per group so far: phases
             auto take_q = [&](int g) -> bool {
                 const uint32_t b = qi % kQ;
                 if (!mbar_wait(bar_q_full(b), (qi / kQ) & 1)) return false;
@@ -289,55 +282,42 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
                 ++qi;
                 return true;
             };
-            Item t = item_at(0);
             // first scores of the first item
-            for (int g = 0; g < t.tiles && !err; ++g) {
+            for (int g = 0; g < kQTiles && !err; ++g) {
                 if (!take_q(g)) { err = kErrWaitQ; break; }
                 if (g == 0 && !mbar_wait(bar_k0, 0)) { err = kErrWaitKV; break; }
                 tc_fence_after();
                 issue_s(g, q_cur[g], 0);
-                if (nkv == 1) mma_commit(bar_q_free(q_cur[g]));
             }
-            uint32_t r = 0;
+            uint32_t r = 0;                        // rounds so far: the phase of the weights' barriers
             for (int n = 0; n < my_items && !err; ++n) {
-                const bool more_items = n + 1 < my_items;
-                const Item next = more_items ? item_at(n + 1) : t;
                 for (int j = 0; j < nkv && !err; ++j, ++r) {
                     const bool last = j + 1 == nkv;
-                    const int tiles_s = last ? (more_items ? next.tiles : 0) : t.tiles;   // groups with a next S
-                    const bool q_last = last ? nkv == 1 : j + 2 == nkv;                   // that S is its query tile's last
+                    const bool more = !last || n + 1 < my_items;         // there is a next S
                     const uint32_t slot_v = (2 * r + 1) % kSlots, slot_k = (2 * r + 2) % kSlots;
                     // V of this round, K of the next
                     if (!mbar_wait(bar_pair(r % L::kPairs), (r / L::kPairs) & 1)) { err = kErrWaitKV; break; }
                     auto next_s = [&](int g) {
-                        if (g >= tiles_s) return;
+                        if (!more) return;
                         if (last && !take_q(g)) { err = kErrWaitQ; return; }
                         if (last) tc_fence_after();
                         issue_s(g, q_cur[g], slot_k);
-                        if (q_last) mma_commit(bar_q_free(q_cur[g]));
+                        if (j + 2 == nkv) mma_commit(bar_q_free(q_cur[g]));      // its query tile's last
                     };
 #pragma unroll
                     for (int g = 0; g < kQTiles; ++g) {
                         if (err) break;
-                        if (g < t.tiles) {
-                            const uint32_t parity = pc[g] & 1;
-                            if (!mbar_wait(bar_p_early(g), parity)) { err = kErrWaitP; break; }
-                            ++pc[g];
-                            // the first product of an item overwrites the accumulator: the group must
-                            // have read the previous item's result out of it
-                            if (j == 0) {
-                                if (ic[g] > 0 && !mbar_wait(bar_o_free(g), (ic[g] - 1) & 1)) { err = kErrWaitO; break; }
-                                ++ic[g];
-                            }
-                            tc_fence_after();
-                            if (!issue_o(g, slot_v, j == 0, parity)) { err = kErrWaitP; break; }
-                            if (last) mma_commit(bar_o_full(g));
-                        }
+                        if (!mbar_wait(bar_p_early(g), r & 1)) { err = kErrWaitP; break; }
+                        // the first product of an item overwrites the accumulator: the group must
+                        // have read the previous item's result out of it
+                        if (j == 0 && n > 0 && !mbar_wait(bar_o_free(g), (uint32_t)(n - 1) & 1)) { err = kErrWaitO; break; }
+                        tc_fence_after();
+                        if (!issue_o(g, slot_v, j == 0, r & 1)) { err = kErrWaitP; break; }
+                        if (last) mma_commit(bar_o_full(g));
                         next_s(g);
                     }
                     mma_commit(bar_release(r % kReleases));
                 }
-                t = next;
             }
             if (err) report(p, err);
         }
