@@ -14,10 +14,11 @@ is replayed until the timed window is at least a quarter of a second, every
 replay between two CUDA events, and the median over replays is reported (with
 the 10th and 90th percentiles, and the eagerly launched latency beside it).
 `e2e` is the same step through the host-buffer entry points with the
-host<->device copies inside the timed region.  At one GPU the line also carries
-`other_configs`: every other workload shape (batched serving, long context, the
-sequence-length and vocabulary sweeps, the tiny case, the drafter's block
-attention), each timed the same way with its own clock record.
+host<->device copies inside the timed region.  At one GPU every other workload
+shape (batched serving, long context, the sequence-length and vocabulary sweeps,
+the tiny case, the drafter's block attention) is timed the same way, each with its
+own clock record: one short line each on stderr, and --out FILE takes the whole
+record, the headline with `other_configs` in it.
 --impl reference times the CPU oracle on the host cores instead (a deliberately
 slow baseline, not a target).
 """
@@ -768,9 +769,12 @@ def run_ours(args):
             "kernels": kernels,
             "cpu_baseline": cpu,
         }
-        if others is not None:
-            line["other_configs"] = others
-        print(json.dumps(line), flush=True)
+        if args.out:
+            with open(args.out, "w") as f:
+                f.write(json.dumps(dict(line, other_configs=others or [])) + "\n")
+        for e in others or []:
+            print(f"{e['name']} ({e['op']}): {1e3 * e['ms']:.1f} us", file=sys.stderr)
+        print(json.dumps(line), flush=True)          # the headline, last and alone on stdout
     else:
         sampler.stop()
     if distributed:
@@ -822,8 +826,9 @@ def main():
     ap.add_argument("--quick", action="store_true", help="shorter timing windows for the other configurations")
     ap.add_argument("--eager-only", nargs="?", const="step", default=None, choices=["step", "drafter_block", "unmask_cfg1", "lm_head_small", "lm_head_small_kl", "attention_cfg2"],
                     help="launch K steps (or calls on one of the other shapes) eagerly and exit: for profilers")
+    ap.add_argument("--out", metavar="FILE", default=None, help="write the whole record, other workloads included, to FILE")
     ap.add_argument("--tables", metavar="FILE", default=None,
-                    help="print markdown tables of a stored JSON line of this program and exit (no GPU needed)")
+                    help="print markdown tables of a record that --out wrote and exit (no GPU needed)")
     args = ap.parse_args()
     if args.tables:
         return print_tables(args.tables)
