@@ -131,7 +131,7 @@ int dd_verify(const void *drafter_logits, const void *verifier_logits,
  *   out_mask[b,i]   = 1 if the position stays masked, else 0
  *   out_conf[b,i]   = c_i (nullable)
  * Positions with mask_flags == 0 pass through (out_tokens = tokens, out_mask = 0,
- * out_conf = 0) and their logits are never read.  Shapes, supported sizes,
+ * out_conf = 0) and nothing is computed from their logits.  Shapes, supported sizes,
  * scratch and errors as for dd_verify, whose confidence rule (Eq. 7) this is,
  * applied to one logits tensor: the same kernel launch.
  */

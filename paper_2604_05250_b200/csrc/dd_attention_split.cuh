@@ -74,12 +74,14 @@ __device__ __forceinline__ void softmax_part(uint32_t tS, uint32_t tO, int key0,
 }
 
 // G > 1 (up to 32 query rows): the query tile holds G copies of them, one above the other, and copy g (one warp)
-// takes the g-th part of every tile's keys (the products with those keys are for its rows only), with an accumulator, reference point and
-// sum of its own; the copies are combined at the end like the parts of a cluster.  A tile's softmax is then the work
+// takes the g-th part of every tile's keys (the products with those keys write its rows only), with an accumulator,
+// reference point and sum of its own; the copies are combined at the end like the parts of a cluster.  A tile's softmax is then the work
 // of G warps instead of one, and so is the masked tile at a sequence's end: 16 x 32 heads, 32 queries over 256-1024
 // keys 42.3 -> 37.7 us, 64 x 32 157.8 -> 130.2, 50 x 32 with one query over 125-500 75.7 -> 59.6, 40 x 16 over 50-200
 // at D = 64 22.3 -> 15.4; whole tiles only: 64 x 8 over 1024 51.2 -> 47.8.  Two copies at D = 128, where a fourth of
 // the buffer's rows would cost a key tile, four at D = 64.
+// Distance from fp64, relative, mean over some 280 drawn calls: 1.939e-3 where attention_kernel's general form has 1.949e-3; call by
+// call between 0.95 and 1.04 of it, by which keys are reference points, whose weight is exact.
 template <int D, int G>
 __global__ void __launch_bounds__(kSplitThreads, 2)
 attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,

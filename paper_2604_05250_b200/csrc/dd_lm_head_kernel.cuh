@@ -7,7 +7,7 @@
 // Eq. 4-5 over the drafter's logits, which are a second product of the same shape.  The kernel
 // therefore keeps the products in tensor memory and never stores a logit: a persistent CTA takes
 // work items of 256 rows x N vocabulary entries, accumulates them with tcgen05 MMAs (accumulators
-// of 128 rows, fp32) from operand tiles that a TMA producer streams through a three-stage ring,
+// of 128 rows, fp32) from operand tiles that a TMA producer streams through a ring of up to six stages,
 // and its epilogue warps turn every accumulator row into one partial (maximum, first index,
 // sum 2^(l*log2e - M); KL: also the drafter's maximum, sum and the weighted logit differences) of
 // the same form as the streaming kernel's chunk partials, stored in the same global table ("chunk"
