@@ -111,7 +111,7 @@ def test_fused_heads(libs, mode, B, P, K, V):
     both_builds(binding, check_path, lambda: binding.lm_head_verify(d[0], d[1], t[2], t[3], tok, fl, mode, 0.3, 3, 5))
 
 
-@pytest.mark.parametrize("B,P", [(2, 37), (5, 8000)])          # row kernel; beyond its 32768 rows the streaming kernel
+@pytest.mark.parametrize("B,P", [(2, 37), (5, 8000)])          # row kernel; beyond its line the streaming kernel
 @pytest.mark.parametrize("V", [1, 2, 3, 5, 7])
 @pytest.mark.parametrize("mode", [KL, CONF])
 def test_last_logits_of_rows_shorter_than_a_vector(libs, B, P, V, mode):

@@ -163,7 +163,7 @@ def test_many_short_rows_and_long_sequences(dd, oracle_mod):
 @pytest.mark.parametrize("B,P,V,flagged", [(60, 700, 64, 500), (24, 1500, 37, 900), (6, 6000, 64, 3000)])
 @pytest.mark.parametrize("mode", [KL, CONF | PROB])
 def test_long_sequences_in_the_streaming_kernel(dd, oracle_mod, B, P, V, flagged, mode):
-    """More than 32768 rows: the streaming kernel, its decision from registers (up to 1024 positions) and from its key area."""
+    """Beyond the row kernel's line: the streaming kernel, its decision from registers (up to 1024 positions) and from its key area."""
     dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=P)
     compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 33, 1)
 
