@@ -303,4 +303,11 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
+// Both halves of a bf16 pair added to fp32 values (low half to x): exact conversion, one fp32 rounding each.
+__device__ __forceinline__ void add_bf16x2(float2 &s, uint32_t pair)
+{
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.f32.bf16 %0, l, %0;\n\tadd.f32.bf16 %1, h, %1;\n\t}"
+        : "+f"(s.x), "+f"(s.y) : "r"(pair));
+}
+
 }  // namespace ddptx
