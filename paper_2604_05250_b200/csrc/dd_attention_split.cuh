@@ -377,6 +377,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     if (*reinterpret_cast<volatile unsigned int *>(p.status) != 0) {
         // a wait expired somewhere: give copies that may still be in flight time to land before the
         // shared memory is released
+#pragma unroll 1
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     tc_fence_before();

@@ -280,6 +280,7 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const LmPlan &plan, 
         else if (plan.gathered) row = q.row_map[ddv::checked(p, row, q.rows, ddv::kSiteRow)];
         else if (!p.flags[row]) row = -1;
         bool arrived = false;
+#pragma unroll 1
         for (uint32_t it = 0; it < (1u << 22); ++it) {
             if (mbar_try_wait(bars_acc_full + 8u * acc, n_done & 1)) { arrived = true; break; }
             if (it > 64) {
@@ -410,6 +411,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
         ddv::report_expired(p, code);
     };
     auto wait = [&](uint32_t bar, uint32_t parity) {
+#pragma unroll 1
         for (uint32_t it = 0; it < (1u << 22); ++it) {
             if (mbar_try_wait(bar, parity)) return true;
             if (it > 64) {
@@ -493,6 +495,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     if (*abort_flag) {
         // a wait expired: give copies that may still be in flight time to land before the shared
         // memory is released
+#pragma unroll 1
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     }
     if (warp == 0) { __syncwarp(); tmem_dealloc(tmem, kTmemCols); }
