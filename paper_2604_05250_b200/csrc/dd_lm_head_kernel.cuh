@@ -22,6 +22,8 @@
 // 16 sequences of 256 positions, 62 % of them flagged, K = 4096, V = 126464: 3024 us
 // with every row multiplied, 1961 us so.
 //
+// The KL mode of more than 128 rows is lm_head_pair_kernel's (dd_lm_head_pair.cuh).
+//
 // Tensor memory (512 columns): TRUST/CONF, N <= 256: the verifier's two accumulators at columns 0
 // and 256.  KL, N <= 128: the drafter's at 0 and 128, the verifier's at 256 and 384; a work item
 // runs the k loop over the drafter's operands first, then over the verifier's.  An item with no more
@@ -80,6 +82,7 @@ struct LmPlan {
 struct LmParams {
     int rows, K, V;            // rows = B * P
     int ctas;                  // CTAs the tile width is chosen for
+    int pairs;                 // 1: the products are lm_head_pair_kernel's
     int min_n;                 // the narrowest width the scratch has partials for
     int rows_per_block;        // rows that a block of the first kernel copies: a multiple of kRowsWarps
     LmPlan *plan;              // null: nothing is gathered, the plan is all_rows and the first kernel is not launched
@@ -96,11 +99,12 @@ struct LmMaps {
 
 // Vocabulary entries per work item: the width for which the slowest of `ctas` CTAs finishes first.
 // A work item of n entries takes about (fixed + n) units of time: the hidden-state tiles it loads and
-// the MMAs' shared-memory reads of them do not shrink with n.  Measured at K = 4096 (time per item
+// the MMAs' shared-memory reads of them do not shrink with n.  `pairs`: pairs of CTAs work on two tiles at a time
+// (dd_lm_head_pair.cuh; any constant from 60 to 250 picks as well there).  Measured at K = 4096 (time per item
 // against n, tile widths forced): fixed = 140 for one product per item, 157 for the KL mode's two.
 // Counting n alone picked tiles of 128 entries at 4096 rows, 25 % slower than 256.
 template <bool KL>
-__host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int min_n)
+__host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int min_n, bool pairs)
 {
     constexpr int fixed = KL ? 157 : 140;
     int best = Widths<KL>::max_n;
@@ -108,8 +112,9 @@ __host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int
     for (int i = 0; i < Widths<KL>::count; ++i) {
         const int n = Widths<KL>::max_n - 32 * i;
         if (n < min_n) break;
-        const long items = ((V + n - 1) / n) * row_blocks;
-        const long cost = ((items + ctas - 1) / ctas) * (fixed + n);
+        const long tiles = (V + n - 1) / n;
+        const long items = (pairs ? (tiles + 1) / 2 : tiles) * row_blocks, workers = pairs ? (ctas + 1) / 2 : ctas;
+        const long cost = ((items + workers - 1) / workers) * (fixed + n);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = n; }
     }
     return best;
@@ -121,7 +126,7 @@ __host__ __device__ inline LmPlan plan_for(const LmParams &q, int n_rows, bool g
     LmPlan plan;
     plan.n_rows = n_rows;
     plan.gathered = gathered;
-    plan.N = pick_tile_n<KL>(q.V, (n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n);
+    plan.N = pick_tile_n<KL>(q.V, (n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n, q.pairs != 0);
     plan.n_tiles = (q.V + plan.N - 1) / plan.N;
     return plan;
 }
@@ -256,11 +261,67 @@ struct Walk {
     __device__ __forceinline__ bool uses(int acc) const { return two || one == acc; }
 };
 
-// Epilogue warps: every accumulator row becomes one partial.  Columns are visited in index order
-// with a strict comparison, so the index kept is the lowest index of the maximum.  KL (Eq. 4-5):
-// the drafter's accumulator is read beside the verifier's, and the row also keeps the drafter's
-// running maximum m_d, s_d = sum 2^(d*log2e - M_d) and t = sum 2^(d*log2e - M_d) * (d - v), both
-// rescaled whenever the maximum moves.
+// One row of a tile of N entries: its columns of the accumulators (dacc: the drafter's, KL only) become a partial.  Columns are
+// visited in index order with a strict comparison, so the index kept is the lowest index of the maximum.  KL (Eq. 4-5): the
+// row also keeps the drafter's running maximum m_d, s_d = sum 2^(d*log2e - M_d) and t = sum 2^(d*log2e - M_d) * (d - v),
+// both rescaled whenever the maximum moves.
+template <bool KL>
+__device__ __forceinline__ ddv::Partial reduce_columns(uint32_t tacc, uint32_t dacc, int N, int col0, int V)
+{
+    float m = -INFINITY, M = -INFINITY, s = 0.f;
+    float m_d = -INFINITY, M_d = -INFINITY, s_d = 0.f, t = 0.f;
+    int idx = 0x7FFFFFFF;
+    for (int cb = 0; cb < N / 32; ++cb) {
+        uint32_t r[32], rd[32];              // rd: the drafter's logits, KL only
+        tmem_ld32(tacc + cb * 32, r);
+        if constexpr (KL) tmem_ld32(dacc + cb * 32, rd);
+        tmem_wait_ld();
+        const int valid = V - (col0 + cb * 32);                 // columns of this group that exist
+        if (valid <= 0) break;
+        float cm = -INFINITY;
+        int ci = 0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const float v = __uint_as_float(r[i]);
+            if (i < valid && v > cm) { cm = v; ci = i; }
+        }
+        if (cm > m) {
+            const float M_new = cm * ddv::kLog2e;
+            s *= ddv::rescale_factor(M, M_new);
+            m = cm; M = M_new;
+            idx = col0 + cb * 32 + ci;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < valid) s += ddv::ex2_approx(fmaf(__uint_as_float(r[i]), ddv::kLog2e, -M));
+        if constexpr (KL) {
+            float cd = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < valid) cd = fmaxf(cd, __uint_as_float(rd[i]));
+            if (cd > m_d) {
+                const float M_new = cd * ddv::kLog2e;
+                const float f = ddv::rescale_factor(M_d, M_new);
+                s_d *= f; t *= f;
+                m_d = cd; M_d = M_new;
+            }
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < valid) {
+                    const float d = __uint_as_float(rd[i]);
+                    const float e = ddv::ex2_approx(fmaf(d, ddv::kLog2e, -M_d));
+                    s_d += e;
+                    t = fmaf(e, d - __uint_as_float(r[i]), t);
+                }
+        }
+    }
+    ddv::Partial c;
+    c.m_v = m; c.s_v = s; c.idx = idx;
+    c.m_d = KL ? m_d : 0.f; c.s_d = s_d; c.t = t; c.pad0 = c.pad1 = 0.f;
+    return c;
+}
+
+// Epilogue warps: every accumulator row becomes one partial; KL: the drafter's accumulator is read beside the verifier's.
 template <bool KL>
 __device__ __forceinline__ void epilogue(const LmParams &q, const LmPlan &plan, const ddv::VerifyParams &p, uint32_t tmem,
                                          uint32_t bars_acc_full, uint32_t bars_acc_empty, volatile uint32_t *abort_flag)
@@ -297,61 +358,11 @@ __device__ __forceinline__ void epilogue(const LmParams &q, const LmPlan &plan, 
             return;
         }
         tc_fence_after();
-        float m = -INFINITY, M = -INFINITY, s = 0.f;
-        float m_d = -INFINITY, M_d = -INFINITY, s_d = 0.f, t = 0.f;
-        int idx = 0x7FFFFFFF;
-        for (int cb = 0; cb < plan.N / 32; ++cb) {
-            uint32_t r[32], rd[32];              // rd: the drafter's logits, KL only
-            tmem_ld32(tacc + cb * 32, r);
-            if constexpr (KL) tmem_ld32(dacc + cb * 32, rd);
-            tmem_wait_ld();
-            const int valid = q.V - (col0 + cb * 32);                 // columns of this group that exist
-            if (valid <= 0) break;
-            float cm = -INFINITY;
-            int ci = 0;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const float v = __uint_as_float(r[i]);
-                if (i < valid && v > cm) { cm = v; ci = i; }
-            }
-            if (cm > m) {
-                const float M_new = cm * ddv::kLog2e;
-                s *= ddv::rescale_factor(M, M_new);
-                m = cm; M = M_new;
-                idx = col0 + cb * 32 + ci;
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i < valid) s += ddv::ex2_approx(fmaf(__uint_as_float(r[i]), ddv::kLog2e, -M));
-            if constexpr (KL) {
-                float cd = -INFINITY;
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (i < valid) cd = fmaxf(cd, __uint_as_float(rd[i]));
-                if (cd > m_d) {
-                    const float M_new = cd * ddv::kLog2e;
-                    const float f = ddv::rescale_factor(M_d, M_new);
-                    s_d *= f; t *= f;
-                    m_d = cd; M_d = M_new;
-                }
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (i < valid) {
-                        const float d = __uint_as_float(rd[i]);
-                        const float e = ddv::ex2_approx(fmaf(d, ddv::kLog2e, -M_d));
-                        s_d += e;
-                        t = fmaf(e, d - __uint_as_float(r[i]), t);
-                    }
-            }
-        }
+        const ddv::Partial c = reduce_columns<KL>(tacc, dacc, plan.N, col0, q.V);
         // the accumulator may be overwritten once its four epilogue warps have read their lanes
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bars_acc_empty + 8u * acc);
-
-        ddv::Partial c;
-        c.m_v = m; c.s_v = s; c.idx = idx;
-        c.m_d = KL ? m_d : 0.f; c.s_d = s_d; c.t = t; c.pad0 = c.pad1 = 0.f;
         if (row >= 0) store_partial(p, c, row, tile, plan.n_tiles);
     }
 }

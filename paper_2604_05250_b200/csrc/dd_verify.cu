@@ -35,6 +35,7 @@
 #include "dd_verify_stream.cuh"
 #include "dd_verify_rows.cuh"
 #include "dd_lm_head_kernel.cuh"
+#include "dd_lm_head_pair.cuh"
 
 namespace {
 
@@ -538,6 +539,7 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
         std::lock_guard<std::mutex> lock(g_mu);
         if (!attr_done[dev]) {
             DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+            if (KL) DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
             attr_done[dev] = true;
         }
     }
@@ -564,8 +566,28 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
             static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
         DD_CUDA_TRY(cudaGetLastError());
     }
-    lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
-    DD_CUDA_TRY(cudaGetLastError());
+    bool launched = false;
+    if constexpr (KL) {
+        if (q.pairs) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(grid + (grid & 1));
+            cfg.blockDim = dim3(ddlm::kThreads);
+            cfg.dynamicSmemBytes = kSmemBytes;
+            cfg.stream = stream;
+            cudaLaunchAttribute cluster;
+            cluster.id = cudaLaunchAttributeClusterDimension;
+            cluster.val.clusterDim.x = 2;
+            cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+            cfg.attrs = &cluster;
+            cfg.numAttrs = 1;
+            DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, lm_head_pair_kernel, m, q, p));
+            launched = true;
+        }
+    }
+    if (!launched) {
+        lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
+        DD_CUDA_TRY(cudaGetLastError());
+    }
     // one warp per row
     const unsigned fold_grid = (unsigned)(((long)q.rows + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
     lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q);
@@ -601,6 +623,7 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
 
     // the narrowest tiles that the device may choose bound the partials
     constexpr long kMaxPartials = (1L << 31) - (1L << 24);
+    const bool pairs = kl && rows > ddlm::kTileRows;
     const int max_n = kl ? ddlm::Widths<true>::max_n : ddlm::Widths<false>::max_n;
     auto tiles_of = [&](int n) { return (V + n - 1) / n; };
     int min_n = max_n / 2;
@@ -617,7 +640,7 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     if (dd::try_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)), (cudaStream_t)stream) != DD_OK) {
         // no room for the narrowest: no narrower than what is picked where every row is multiplied
         const long row_blocks = (rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem;
-        min_n = kl ? ddlm::pick_tile_n<true>(V, row_blocks, sms, min_n) : ddlm::pick_tile_n<false>(V, row_blocks, sms, min_n);
+        min_n = kl ? ddlm::pick_tile_n<true>(V, row_blocks, sms, min_n, pairs) : ddlm::pick_tile_n<false>(V, row_blocks, sms, min_n, false);
         rc = dd::ensure_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)));
         if (rc != DD_OK) return rc;
     }
@@ -640,6 +663,7 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     ddlm::LmParams q;
     q.rows = (int)rows; q.K = K; q.V = V;
     q.min_n = min_n;
+    q.pairs = pairs;
     q.ctas = sms;
     q.plan = nullptr;
     q.all_rows = kl ? ddlm::plan_for<true>(q, q.rows, false) : ddlm::plan_for<false>(q, q.rows, false);

@@ -82,6 +82,19 @@ def test_small_shapes_kl(dd, oracle_mod, B, P, K, V, flagged, mode):
             assert ref["out_mask"][fl].any() and not ref["out_mask"][fl].all()
 
 
+@pytest.mark.parametrize("P,K,V,flagged", [
+    (129, 64, 8, 129),                 # one row in the second CTA of a pair; one tile, its neighbour beyond the vocabulary
+    (256, 128, 321, 256),              # whole blocks of rows; an odd number of tiles
+    (257, 192, 256, 257),              # a second block of one row
+    (600, 256, 20011, 130),            # the flagged rows gathered, in one block
+    (700, 128, 40000, 390),            # and in two
+])
+def test_pairs_of_ctas(dd, oracle_mod, P, K, V, flagged):
+    """The KL mode beyond 128 rows: 256 rows by two tiles of the vocabulary per pair of CTAs."""
+    dh, dw, vh, vw, tokens, flags = synth.lm_head_pair_inputs(1, P, K, V, flagged, 0.2, seed=P)
+    compare(dd, oracle_mod, vh, vw, tokens, flags, KL, 0.5, 9, 3, drafter=(dh, dw))
+
+
 @pytest.mark.parametrize("P", [700, 1100, 2100])
 def test_long_sequences(dd, oracle_mod, P):
     """Sequences longer than the register-resident decision stage holds (512 positions), longer
