@@ -7,7 +7,7 @@
 // Eq. 4-5 over the drafter's logits, which are a second product of the same shape.  The kernel
 // therefore keeps the products in tensor memory and never stores a logit: a persistent CTA takes
 // work items of 256 rows x N vocabulary entries, accumulates them with tcgen05 MMAs (accumulators
-// of 128 rows, fp32) from operand tiles that a TMA producer streams through a ring of up to six stages,
+// of 128 rows, fp32) from operand tiles that a TMA producer streams through a ring of up to nine stages,
 // and its epilogue warps turn every accumulator row into one partial (maximum, first index,
 // sum 2^(l*log2e - M); KL: also the drafter's maximum, sum and the weighted logit differences) of
 // the same form as the streaming kernel's chunk partials, stored in the same global table ("chunk"
@@ -22,7 +22,7 @@
 // 16 sequences of 256 positions, 62 % of them flagged, K = 4096, V = 126464: 3024 us
 // with every row multiplied, 1961 us so.
 //
-// The KL mode of more than 128 rows is lm_head_pair_kernel's (dd_lm_head_pair.cuh).
+// More than 128 rows are multiplied by pairs of CTAs where that is faster, always in the KL mode (dd_lm_head_pair.cuh).
 //
 // Tensor memory (512 columns): TRUST/CONF, N <= 256: the verifier's two accumulators at columns 0
 // and 256.  KL, N <= 128: the drafter's at 0 and 128, the verifier's at 256 and 384; a work item
@@ -42,6 +42,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "dd_ptx.cuh"
 #include "dd_verify_decide_block.cuh"
 
@@ -55,7 +57,7 @@ constexpr int kLoadWarp = 8, kMmaWarp = 9;
 constexpr int kTileRows = 128;
 constexpr int kRowsPerItem = 2 * kTileRows; // two accumulators
 constexpr int kBlockK = 64;                // one 128-byte swizzled box per k-step
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 9;
 constexpr int kCheckedRows = 4 * kThreads;
 constexpr int kMaxN = 256;
 constexpr uint32_t kTmemCols = 512;        // see the layout above
@@ -64,11 +66,12 @@ constexpr int kRingBytes = 3 * (2 * kATileBytes + kMaxN * kBlockK * 2);   // 192
 constexpr int kSmemBytes = kRingBytes + 1024 + 256;
 constexpr unsigned kErrLmFull = 0xC00, kErrLmEmpty = 0xD00, kErrLmAcc = 0xE00;
 
-// Widths of the vocabulary tiles: kWidths multiples of 32 downwards from the largest.
+// Widths of the vocabulary tiles: multiples of 32 downwards from the largest.  Below half of it only where that leaves SMs idle
+// (dd_lm_head_verify).
 template <bool KL>
 struct Widths {
     static constexpr int max_n = KL ? kMaxN / 2 : kMaxN;
-    static constexpr int count = max_n / 64 + 1;              // down to half of it
+    static constexpr int count = max_n / 32;
 };
 
 // What the first kernel finds out, for the two behind it.
@@ -104,16 +107,20 @@ struct LmMaps {
 // against n, tile widths forced): fixed = 140 for one product per item, 157 for the KL mode's two.
 // Counting n alone picked tiles of 128 entries at 4096 rows, 25 % slower than 256.
 template <bool KL>
-__host__ __device__ inline int pick_tile_n(int V, long row_blocks, int ctas, int min_n, bool pairs)
+__host__ __device__ inline int pick_tile_n(int V, long n_rows, int ctas, int min_n, bool pairs)
 {
     constexpr int fixed = KL ? 157 : 140;
+    const long row_blocks = (n_rows + kRowsPerItem - 1) / kRowsPerItem;
     int best = Widths<KL>::max_n;
     long best_cost = -1;
     for (int i = 0; i < Widths<KL>::count; ++i) {
         const int n = Widths<KL>::max_n - 32 * i;
         if (n < min_n) break;
         const long tiles = (V + n - 1) / n;
-        const long items = (pairs ? (tiles + 1) / 2 : tiles) * row_blocks, workers = pairs ? (ctas + 1) / 2 : ctas;
+        const long items = !pairs ? tiles * row_blocks
+                         : KL ? (tiles + 1) / 2 * row_blocks
+                              : tiles * (row_blocks / 2) + (row_blocks % 2 ? (tiles + 1) / 2 : 0);
+        const long workers = pairs ? (ctas + 1) / 2 : ctas;
         const long cost = ((items + workers - 1) / workers) * (fixed + n);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = n; }
     }
@@ -126,7 +133,7 @@ __host__ __device__ inline LmPlan plan_for(const LmParams &q, int n_rows, bool g
     LmPlan plan;
     plan.n_rows = n_rows;
     plan.gathered = gathered;
-    plan.N = pick_tile_n<KL>(q.V, (n_rows + kRowsPerItem - 1) / kRowsPerItem, q.ctas, q.min_n, q.pairs != 0);
+    plan.N = pick_tile_n<KL>(q.V, n_rows, q.ctas, q.min_n, q.pairs != 0);
     plan.n_tiles = (q.V + plan.N - 1) / plan.N;
     return plan;
 }
@@ -168,7 +175,8 @@ lm_head_rows_kernel(const LmParams q, const ddv::VerifyParams p, const uint4 *hi
     if (lane == 0) { atomicAdd(&s_before, before); atomicAdd(&s_all, all); }
     __syncthreads();
     all = s_all;
-    const bool gather = (all + kTileRows - 1) / kTileRows < (q.rows + kTileRows - 1) / kTileRows &&
+    const int unit = q.pairs ? kRowsPerItem : kTileRows;           // rows that cost as much as one
+    const bool gather = (all + unit - 1) / unit < (q.rows + unit - 1) / unit &&
                         (q.all_rows.n_tiles > 2 || 3L * all < (long)q.rows * q.all_rows.n_tiles);
     if (blockIdx.x == 0 && tid == 0) *q.plan = plan_for<KL>(q, gather ? all : q.rows, gather);
     if (!gather) return;
@@ -261,63 +269,80 @@ struct Walk {
     __device__ __forceinline__ bool uses(int acc) const { return two || one == acc; }
 };
 
-// One row of a tile of N entries: its columns of the accumulators (dacc: the drafter's, KL only) become a partial.  Columns are
-// visited in index order with a strict comparison, so the index kept is the lowest index of the maximum.  KL (Eq. 4-5): the
-// row also keeps the drafter's running maximum m_d, s_d = sum 2^(d*log2e - M_d) and t = sum 2^(d*log2e - M_d) * (d - v),
-// both rescaled whenever the maximum moves.
+// One row of a tile of N entries: its columns of the accumulators (dacc: the drafter's, KL only) become a partial: the
+// verifier's maximum m_v, its lowest index and s_v = sum 2^(l*log2e - M); KL (Eq. 4-5): also the drafter's maximum m_d, s_d = sum
+// 2^(d*log2e - M_d) and t = sum 2^(d*log2e - M_d) * (d - v).
+// The columns are read twice, for the maxima and for the sums.  Nothing else of the CTA hides this, so what counts is the length of the chains (as one
+// pass with a running maximum and its index it was 32 dependent steps per 32 columns) and the size of the code, which is
+// cold every time: two short loops, four chains for every sum.  256 columns, eight warps 7400 -> 6200 cycles (8960 -> 6420 the
+// first time; one pass with four chains 5900 and 7300), KL 128 columns 7200 -> 5800; 8192 rows, K = 512, V = 2000 38.7 -> 36.5 us,
+// KL 62.0 -> 58.8; 1024, 2048, 50000 172 -> 164.
 template <bool KL>
 __device__ __forceinline__ ddv::Partial reduce_columns(uint32_t tacc, uint32_t dacc, int N, int col0, int V)
 {
-    float m = -INFINITY, M = -INFINITY, s = 0.f;
-    float m_d = -INFINITY, M_d = -INFINITY, s_d = 0.f, t = 0.f;
+    const int columns = min(N, V - col0);                        // that exist
+    float m = -INFINITY, m_d = -INFINITY;
+    uint32_t r[32], rd[32];                                      // rd: the drafter's logits, KL only
+    auto load = [&](int cb) {
+        tmem_ld32(tacc + cb, r);
+        if constexpr (KL) tmem_ld32(dacc + cb, rd);
+        tmem_wait_ld(r);
+        if constexpr (KL) tmem_wait_ld(rd);
+    };
+    auto top = [&](const uint32_t (&x)[32], float m) {
+        float c[4] = {m, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) c[i / 2 % 4] = max3(c[i / 2 % 4], __uint_as_float(x[i]), __uint_as_float(x[i + 1]));
+        return max3(c[0], c[1], fmaxf(c[2], c[3]));
+    };
+    // 32 columns of which `valid` exist: the others are out of every maximum and sum
+    auto clip = [&](uint32_t (&x)[32], int valid, uint32_t with) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = i < valid ? x[i] : with;
+    };
+    constexpr uint32_t kMinusInf = 0xFF800000u;
+#pragma unroll 1
+    for (int cb = 0; cb < columns; cb += 32) {
+        load(cb);
+        if (columns - cb < 32) { clip(r, columns - cb, kMinusInf); if constexpr (KL) clip(rd, columns - cb, kMinusInf); }
+        m = top(r, m);
+        if constexpr (KL) m_d = top(rd, m_d);
+    }
+    const float M = m * ddv::kLog2e, M_d = m_d * ddv::kLog2e;
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, s_d[4] = {0.f, 0.f, 0.f, 0.f}, t[4] = {0.f, 0.f, 0.f, 0.f};
     int idx = 0x7FFFFFFF;
-    for (int cb = 0; cb < N / 32; ++cb) {
-        uint32_t r[32], rd[32];              // rd: the drafter's logits, KL only
-        tmem_ld32(tacc + cb * 32, r);
-        if constexpr (KL) tmem_ld32(dacc + cb * 32, rd);
-        tmem_wait_ld();
-        const int valid = V - (col0 + cb * 32);                 // columns of this group that exist
-        if (valid <= 0) break;
-        float cm = -INFINITY;
-        int ci = 0;
+#pragma unroll 1
+    for (int cb = 0; cb < columns; cb += 32) {
+        load(cb);
+        int at[4] = {32, 32, 32, 32};
+        auto sums = [&](auto is_masked) {
+            const int valid = columns - cb;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float v = __uint_as_float(r[i]);
-            if (i < valid && v > cm) { cm = v; ci = i; }
-        }
-        if (cm > m) {
-            const float M_new = cm * ddv::kLog2e;
-            s *= ddv::rescale_factor(M, M_new);
-            m = cm; M = M_new;
-            idx = col0 + cb * 32 + ci;
-        }
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (i < valid) s += ddv::ex2_approx(fmaf(__uint_as_float(r[i]), ddv::kLog2e, -M));
-        if constexpr (KL) {
-            float cd = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i < valid) cd = fmaxf(cd, __uint_as_float(rd[i]));
-            if (cd > m_d) {
-                const float M_new = cd * ddv::kLog2e;
-                const float f = ddv::rescale_factor(M_d, M_new);
-                s_d *= f; t *= f;
-                m_d = cd; M_d = M_new;
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i < valid) {
-                    const float d = __uint_as_float(rd[i]);
-                    const float e = ddv::ex2_approx(fmaf(d, ddv::kLog2e, -M_d));
-                    s_d += e;
-                    t = fmaf(e, d - __uint_as_float(r[i]), t);
+            for (int i = 31; i >= 0; --i) {
+                if (decltype(is_masked)::value && i >= valid) continue;
+                const float v = __uint_as_float(r[i]);
+                if (v == m) at[i / 8] = i;
+                s[i % 4] += ex2(fmaf(v, ddv::kLog2e, -M));
+                if constexpr (KL) {
+                    const float d = __uint_as_float(rd[i]), e = ex2(fmaf(d, ddv::kLog2e, -M_d));
+                    s_d[i % 4] += e;
+                    t[i % 4] = fmaf(e, d - v, t[i % 4]);
                 }
-        }
+            }
+        };
+        if (columns - cb >= 32) sums(std::false_type());
+        else sums(std::true_type());
+        const int first = min(min(at[0], at[1]), min(at[2], at[3]));
+        if (first < 32) idx = min(idx, col0 + cb + first);
     }
     ddv::Partial c;
-    c.m_v = m; c.s_v = s; c.idx = idx;
-    c.m_d = KL ? m_d : 0.f; c.s_d = s_d; c.t = t; c.pad0 = c.pad1 = 0.f;
+    c.m_v = m;
+    c.s_v = (s[0] + s[1]) + (s[2] + s[3]);
+    c.idx = m == -INFINITY ? 0x7FFFFFFF : idx;               // nothing above -inf: no token
+    c.m_d = KL ? m_d : 0.f;
+    c.s_d = (s_d[0] + s_d[1]) + (s_d[2] + s_d[3]);
+    c.t = (t[0] + t[1]) + (t[2] + t[3]);
+    c.pad0 = c.pad1 = 0.f;
     return c;
 }
 

@@ -539,7 +539,7 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
         std::lock_guard<std::mutex> lock(g_mu);
         if (!attr_done[dev]) {
             DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-            if (KL) DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+            DD_CUDA_TRY(cudaFuncSetAttribute(lm_head_pair_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
             attr_done[dev] = true;
         }
     }
@@ -552,12 +552,15 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
         if ((rc = make_matrix_tmap(&m.hd, dh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
         if ((rc = make_matrix_tmap(&m.hd_gathered, gathered + gathered_bytes, q.rows, q.K, kTileRows)) != DD_OK) return rc;
     }
+    // a map per width that the device may choose; one where the host has chosen
     for (int i = 0; i < Widths<KL>::count; ++i) {
-        if ((rc = make_matrix_tmap(&m.w[i], vw, q.V, q.K, Widths<KL>::max_n - 32 * i)) != DD_OK) return rc;
-        if (KL && (rc = make_matrix_tmap(&m.wd[i], dw, q.V, q.K, Widths<KL>::max_n - 32 * i)) != DD_OK) return rc;
+        if (q.plan ? Widths<KL>::max_n - 32 * i < q.min_n : Widths<KL>::max_n - 32 * i != q.all_rows.N) continue;
+        const int width = Widths<KL>::max_n - 32 * i, box = q.pairs && !KL ? width / 2 : width;      // what one CTA loads at a time
+        if ((rc = make_matrix_tmap(&m.w[i], vw, q.V, q.K, box)) != DD_OK) return rc;
+        if (KL && (rc = make_matrix_tmap(&m.wd[i], dw, q.V, q.K, box)) != DD_OK) return rc;
     }
     // One CTA per SM, fewer if even the narrowest tiles of all rows do not make that many items.
-    const long items = (long)((q.V + Widths<KL>::max_n / 2 - 1) / (Widths<KL>::max_n / 2)) * ((q.rows + kRowsPerItem - 1) / kRowsPerItem);
+    const long items = (long)((q.V + q.min_n - 1) / q.min_n) * ((q.rows + kRowsPerItem - 1) / kRowsPerItem);
     const unsigned grid = (unsigned)(items < ctas ? items : ctas);
     if (q.plan) {
         q.rows_per_block = kRowsWarps * ((q.rows + kRowsWarps * kRowsBlocks - 1) / (kRowsWarps * kRowsBlocks));
@@ -566,25 +569,20 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
             static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
         DD_CUDA_TRY(cudaGetLastError());
     }
-    bool launched = false;
-    if constexpr (KL) {
-        if (q.pairs) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(grid + (grid & 1));
-            cfg.blockDim = dim3(ddlm::kThreads);
-            cfg.dynamicSmemBytes = kSmemBytes;
-            cfg.stream = stream;
-            cudaLaunchAttribute cluster;
-            cluster.id = cudaLaunchAttributeClusterDimension;
-            cluster.val.clusterDim.x = 2;
-            cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
-            cfg.attrs = &cluster;
-            cfg.numAttrs = 1;
-            DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, lm_head_pair_kernel, m, q, p));
-            launched = true;
-        }
-    }
-    if (!launched) {
+    if (q.pairs) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid + (grid & 1));
+        cfg.blockDim = dim3(ddlm::kThreads);
+        cfg.dynamicSmemBytes = kSmemBytes;
+        cfg.stream = stream;
+        cudaLaunchAttribute cluster;
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim.x = 2;
+        cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+        cfg.attrs = &cluster;
+        cfg.numAttrs = 1;
+        DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, lm_head_pair_kernel<KL>, m, q, p));
+    } else {
         lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
         DD_CUDA_TRY(cudaGetLastError());
     }
@@ -623,10 +621,22 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
 
     // the narrowest tiles that the device may choose bound the partials
     constexpr long kMaxPartials = (1L << 31) - (1L << 24);
-    const bool pairs = kl && rows > ddlm::kTileRows;
+    // Pairs of CTAs (dd_lm_head_pair.cuh): beyond one tile of rows; outside the KL mode, whose single CTAs have the smaller items, where the k
+    // loop is long enough to pay for the meeting of the two and there are items for half of the SMs.  us, lm_head_kernel : pairs (rows, K, V):
+    // 256, 4096, 126464 262 : 239 (short bursts 240 : 219); 150, 4096, 126464 243 : 224; 300, 2048, 128256 245 : 216; 1000 of 4000,
+    // 4096, 32000 221 : 207; 256, 2048, 126464 149 : 136; 512, 3072, 10000 42.5 : 39.9; 2540 of 4096, 4096, 126464 the same; 400, 4096, 3000
+    // 32.3 : 34.1; 960 of 2400, 1024, 12000 38.7 : 40.9; 8192, 512, 2000 38.7 : 40.9.
+    const bool pairs = rows > ddlm::kTileRows &&
+                       (kl || (K >= 2048 && 2 * ((V + ddlm::kMaxN - 1) / ddlm::kMaxN) * ((rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem) >= sms));
     const int max_n = kl ? ddlm::Widths<true>::max_n : ddlm::Widths<false>::max_n;
     auto tiles_of = [&](int n) { return (V + n - 1) / n; };
+    // Half of the widest, or, where that leaves SMs without an item, narrower ones: an SM takes 45 to 55 bytes per clock, whoever
+    // is idle beside it.  Every tile costs the fold a partial per row, though, so with short rows of weights only while a lane has one
+    // (us, half : narrower; rows, K, V: 100, 4096, 3072 28.6 : 25.1; 400, 4096, 3000 34.3 : 31.5; 512, 1024, 6000 19.4 : 18.7; 64, 512, 1000
+    // 13.1 : 11.7, KL 13.5 : 12.7; 16, 512, 4000 13.2 : 14.9).
     int min_n = max_n / 2;
+    const long row_blocks = (rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem;
+    while (min_n > 32 && tiles_of(min_n) * row_blocks < sms && (K >= 1024 || tiles_of(min_n - 32) <= 32)) min_n -= 32;
     while (rows * tiles_of(min_n) >= kMaxPartials) {
         if (min_n == max_n) return DD_ERR_UNSUPPORTED;
         min_n += 32;
@@ -639,8 +649,7 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     if ((rc = dd::check_mirror(ctx, 1)) != DD_OK) return rc;
     if (dd::try_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)), (cudaStream_t)stream) != DD_OK) {
         // no room for the narrowest: no narrower than what is picked where every row is multiplied
-        const long row_blocks = (rows + ddlm::kRowsPerItem - 1) / ddlm::kRowsPerItem;
-        min_n = kl ? ddlm::pick_tile_n<true>(V, row_blocks, sms, min_n, pairs) : ddlm::pick_tile_n<false>(V, row_blocks, sms, min_n, false);
+        min_n = kl ? ddlm::pick_tile_n<true>(V, rows, sms, min_n, pairs) : ddlm::pick_tile_n<false>(V, rows, sms, min_n, pairs);
         rc = dd::ensure_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)));
         if (rc != DD_OK) return rc;
     }

@@ -95,6 +95,19 @@ def test_pairs_of_ctas(dd, oracle_mod, P, K, V, flagged):
     compare(dd, oracle_mod, vh, vw, tokens, flags, KL, 0.5, 9, 3, drafter=(dh, dw))
 
 
+@pytest.mark.parametrize("P,K,V,flagged", [
+    (129, 2048, 19000, 129),           # one block of rows, two tiles of the vocabulary at a time; an odd number of tiles
+    (513, 2048, 6500, 513),            # 512 rows a tile at a time, one row two tiles at a time
+    (300, 2112, 9500, 300),            # 512 rows that are not all there
+    (1000, 2048, 6500, 200),           # the flagged rows gathered
+    (70, 1088, 1100, 70),              # not in pairs: tiles narrower than 128, to have more of them
+])
+def test_pairs_of_ctas_verifier_only(dd, oracle_mod, P, K, V, flagged):
+    """The other modes in pairs, and the narrow tiles of problems with few items."""
+    hidden, weight, tokens, flags = synth.lm_head_inputs(1, P, K, V, flagged, seed=P)
+    compare(dd, oracle_mod, hidden, weight, tokens, flags, CONF | PROB, 0.05, 9, 11)
+
+
 @pytest.mark.parametrize("P", [700, 1100, 2100])
 def test_long_sequences(dd, oracle_mod, P):
     """Sequences longer than the register-resident decision stage holds (512 positions), longer
