@@ -281,15 +281,17 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
     const int lane = threadIdx.x & 31;
     float bm_v = -INFINITY, bm_d = -INFINITY;
     int bidx = 0x7FFFFFFF;
-    for (int ch = lane; ch < n; ch += 32) {
+    // up to 16 partials: every `width` lanes take all of them, and as many steps of the exchange are left out
+    const int width = n > 16 ? 32 : n <= 1 ? 1 : 2 << (31 - __clz(n - 1)), ch0 = lane & (width - 1);
+    for (int ch = ch0; ch < n; ch += width) {
         const float4 a = ld_volatile16(src + ch);
         const float mv = a.x, md = a.w;
         const int ix = __float_as_int(a.z);
         if (mv > bm_v || (mv == bm_v && ix < bidx)) { bm_v = mv; bidx = ix; }
         bm_d = fmaxf(bm_d, md);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll 1
+    for (int o = width >> 1; o > 0; o >>= 1) {
         const float om = __shfl_xor_sync(0xFFFFFFFFu, bm_v, o);
         const int oi = __shfl_xor_sync(0xFFFFFFFFu, bidx, o);
         if (om > bm_v || (om == bm_v && oi < bidx)) { bm_v = om; bidx = oi; }
@@ -297,7 +299,7 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
     }
     const float Mv = __fmul_rn(bm_v, kLog2e), Md = __fmul_rn(bm_d, kLog2e);
     double sv = 0.0, sd = 0.0, tt = 0.0;
-    for (int ch = lane; ch < n; ch += 32) {
+    for (int ch = ch0; ch < n; ch += width) {
         const float4 a = ld_volatile16(src + ch);
         const float4 bq = ld_volatile16(reinterpret_cast<const float4 *>(src + ch) + 1);
         // the factor that moves a chunk's sums to the row's reference point is a power of two with a
@@ -312,8 +314,14 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
             tt += (double)bq.y * f;
         }
     }
-    sv = warp_sum(sv);
-    if (KL) { sd = warp_sum(sd); tt = warp_sum(tt); }
+#pragma unroll 1
+    for (int o = width >> 1; o > 0; o >>= 1) {
+        sv += __shfl_xor_sync(0xFFFFFFFFu, sv, o);
+        if (KL) {
+            sd += __shfl_xor_sync(0xFFFFFFFFu, sd, o);
+            tt += __shfl_xor_sync(0xFFFFFFFFu, tt, o);
+        }
+    }
     float sc = 0.f;
     if (KL) {
         // lane 0 takes the verifier's logarithm while lane 1 takes the drafter's

@@ -143,10 +143,13 @@ __device__ __noinline__ void decide_block(const VerifyParams &p, int b, BlockDec
 }
 
 // The same for sequences of at most 512 positions and two per thread: everything about a position is loaded
-// in one batch and stays in registers, and the k-th largest key is found by warp 0 from keys in registers, bit
-// by bit without a barrier, ending as soon as exactly k keys are left above the candidate (12-16 steps; all 32
-// only for ties).  1 x 128 positions: 9700 cycles for the general form, of which 4700 for the selection, 6200 for
-// this one (cold; with the cheaper report below 2 us of a call).
+// in one batch and stays in registers, and the k-th largest key is found from keys in registers, three bits at a time:
+// seven warps count the keys from one candidate each, a barrier, and every warp picks the next three bits.  It begins below the
+// bits that all keys share and ends as soon as exactly k keys are left (4-6 rounds; more only for ties).  Bit by bit in one warp, without
+// barriers, from the highest bit on, it took 1.5 to 2.7 us of a call; together with a report that is prepared while the first
+// warp folds and a fold that exchanges among as many lanes as there are partials: 1 x 128 positions, V = 1024, KL 7.7 -> 7.2 us; 16 x 512,
+// 1000, CONF 19.7 -> 17.9; 1 x 300, 5000 10.4 -> 9.0; 1 x 512, 32000 18.6 -> 17.0; 2 x 300, 32001, KL 20.3 -> 19.8.
+// At least eight warps.
 __device__ __noinline__ void decide_block_short(const VerifyParams &p, int b, BlockDecide &s)
 {
     constexpr int R = 2;
@@ -199,33 +202,52 @@ __device__ __noinline__ void decide_block_short(const VerifyParams &p, int b, Bl
     unsigned last_equal = 0;
     bool keep_all = false;
     if (any) {
-        if (warp == 0) {
-            uint32_t kr[16];
+        uint32_t kr[16];                                 // all keys, in every warp
 #pragma unroll
-            for (int r = 0; r < 16; ++r) kr[r] = r * 32 < p.P ? s.key[lane + 32 * r] : 0u;
-            auto count_above = [&](uint32_t bound) -> int {
-                int c0 = 0, c1 = 0;
+        for (int r = 0; r < 16; ++r) kr[r] = r * 32 < p.P ? s.key[lane + 32 * r] : 0u;
+        auto count_from = [&](uint32_t bound) -> int {   // keys not below it
+            int c0 = 0, c1 = 0;
 #pragma unroll
-                for (int r = 0; r < 4; r += 2) { c0 += kr[r] > bound; c1 += kr[r + 1] > bound; }
-                if (p.P > 128) {
+            for (int r = 0; r < 4; r += 2) { c0 += kr[r] >= bound; c1 += kr[r + 1] >= bound; }
+            if (p.P > 128) {
 #pragma unroll
-                    for (int r = 4; r < 16; r += 2) { c0 += kr[r] > bound; c1 += kr[r + 1] > bound; }
-                }
-                return __reduce_add_sync(full, c0 + c1);
-            };
-            unsigned last = 0xFFFFFFFFu;                 // every position equal to thr
-            if (count_above(0u) > p.k) {
-                bool exact = false;
+                for (int r = 4; r < 16; r += 2) { c0 += kr[r] >= bound; c1 += kr[r + 1] >= bound; }
+            }
+            return __reduce_add_sync(full, c0 + c1);
+        };
+        if (count_from(1u) > p.k) {
+            // every key has the bits above `pos` of the largest
+            uint32_t high = 0u, low = 0xFFFFFFFFu;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                high = max(high, kr[r]);
+                low = min(low, kr[r] - 1u);              // (0, no key, becomes the largest)
+            }
+            high = __reduce_max_sync(full, high);
+            low = __reduce_min_sync(full, low) + 1u;
+            int pos = 32 - __clz(high ^ low);
+            thr = pos < 32 ? high >> pos << pos : 0u;
+            bool exact = false;
 #pragma unroll 1
-                for (int bit = 31; bit >= 0; --bit) {
-                    const uint32_t cand = thr | (1u << bit);
-                    const int n = count_above(cand - 1u);
-                    if (n >= p.k) thr = cand;
-                    if (n == p.k) { exact = true; break; }
-                }
-                if (!exact) {
-                    // ties at the threshold: kept lowest index first
-                    int quota = p.k - count_above(thr), seen = 0;
+            for (unsigned *n = s.hist; pos > 0 && !exact; n = s.hist + ((n - s.hist) ^ 8)) {
+                const int bits = min(pos, 3);
+                pos -= bits;
+                const int mine = count_from(thr | (uint32_t)warp << pos);
+                if (lane == 0 && warp < 8) n[warp] = (unsigned)mine;
+                __syncthreads();
+                unsigned best = 0, left = 0;
+#pragma unroll
+                for (unsigned w = 1; w < 8; ++w)
+                    if (w < (1u << bits) && n[w] >= (unsigned)p.k) { best = w; left = n[w]; }
+                thr |= best << pos;
+                exact = best > 0 && left == (unsigned)p.k;
+            }
+            last_equal = 0xFFFFFFFFu;                    // every position equal to thr
+            if (!exact) {
+                // ties at the threshold: kept lowest index first
+                if (warp == 0) {
+                    unsigned last = 0xFFFFFFFFu;
+                    int quota = p.k - (thr == 0xFFFFFFFFu ? 0 : count_from(thr + 1u)), seen = 0;
 #pragma unroll 1
                     for (int i0 = 0; i0 < p.P; i0 += 32) {
                         const bool eq = s.key[i0 + lane] == thr;
@@ -235,13 +257,12 @@ __device__ __noinline__ void decide_block_short(const VerifyParams &p, int b, Bl
                         if (hit) { last = (unsigned)(i0 + __ffs(hit) - 1); break; }
                         seen += __popc(m);
                     }
+                    if (lane == 0) s.count = last;
                 }
-            }                                            // else: no more than k, all are kept (thr stays 0)
-            if (lane == 0) { s.digit = thr; s.count = last; }
-        }
-        __syncthreads();
-        thr = s.digit;
-        last_equal = s.count;
+                __syncthreads();
+                last_equal = s.count;
+            }
+        }                                                // else: no more than k, all are kept (thr stays 0)
         keep_all = thr == 0u;
     }
 #pragma unroll
@@ -266,7 +287,9 @@ __device__ __forceinline__ unsigned add_acq_rel(unsigned *ptr, unsigned n)
 
 struct BlockReport {                 // in shared memory
     BlockDecide decide;
-    unsigned complete;
+    int seq[32];                     // the sequence that a row belongs to
+    unsigned rows[32];               // how many of the CTA's rows belong to it (with the first of them), else 0
+    unsigned complete;               // bit i: the CTA's row i stands for a complete sequence
 };
 
 // The CTA has finished (folded and stored, or found not flagged) the rows row0 .. row0 + n - 1 (n <= 32, rows past
@@ -276,25 +299,29 @@ __device__ __forceinline__ void report_rows(const VerifyParams &p, int row0, int
 {
     const unsigned full = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
+    if (threadIdx.x >= blockDim.x - 32) {                            // (the first warp may still be folding)
+        const int r = row0 + lane;
+        const int b = lane < n && (long)r < (long)p.B * p.P ? r / p.P : -1;
+        const unsigned same = __match_any_sync(full, b);
+        s.seq[lane] = b;
+        s.rows[lane] = b >= 0 && lane == __ffs(same) - 1 ? __popc(same) : 0;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
-        const int r = row0 + lane;
-        const bool valid = lane < n && (long)r < (long)p.B * p.P;
-        const int b = valid ? r / p.P : -1;
-        const unsigned same = __match_any_sync(full, b);
+        const unsigned count = s.rows[lane];
         bool complete = false;
-        if (valid && lane == __ffs(same) - 1) {
-            const unsigned count = __popc(same);
+        if (count > 0) {
+            const int b = s.seq[lane];
             // (orders what this CTA stored before the count, and what the others stored before theirs after it)
             complete = add_acq_rel(p.seq_counter + checked(p, b, p.B, kSiteSeq), count) + count == (unsigned)p.P;
             if (complete) p.seq_counter[b] = 0u;                     // ready for the next launch
         }
-        const unsigned all = __ballot_sync(full, complete);          // bit i: row0 + i stands for a complete sequence
+        const unsigned all = __ballot_sync(full, complete);
         if (lane == 0) s.complete = all;
     }
     __syncthreads();
     for (unsigned m = s.complete; m; m &= m - 1) {
-        const int b = (row0 + __ffs(m) - 1) / p.P;
+        const int b = s.seq[__ffs(m) - 1];
         if (p.P <= 512 && p.P <= 2 * (int)blockDim.x) decide_block_short(p, b, s.decide);
         else decide_block(p, b, s.decide);
         __syncthreads();

@@ -384,3 +384,21 @@ def test_minimum_keep_with_many_equal_scores(dd, oracle_mod, k):
         # equal rows have equal scores on either side, so the order is the same and so is the kept set
         np.testing.assert_array_equal(om, ref["out_mask"])
         np.testing.assert_array_equal(ot, ref["out_tokens"])
+
+
+@pytest.mark.parametrize("P,ks", [(1, [1]), (31, [1, 30]), (129, [1, 64, 128]), (256, [7, 255]), (257, [1, 8, 200]), (512, [3, 256, 511])])
+def test_threshold_of_the_minimum_keep(dd, oracle_mod, P, ks):
+    """The k-th most reliable position at every size of the short decision stage: scores that differ everywhere, scores
+    of three values (ties at the threshold) and scores that are all the same."""
+    rng = np.random.default_rng(P)
+    distinct = synth.verify_inputs(2, P, 64, P, 0.5, seed=P)
+    for rows in (None, 3, 1):
+        dra, ver, tokens, flags = (x.copy() for x in distinct)
+        if rows:
+            pick = rng.integers(0, min(rows, P), (2, P))
+            for b in range(2):
+                dra[b], ver[b] = distinct[0][b][pick[b]], distinct[1][b][pick[b]]
+            tokens[:] = np.argmax(synth.bf16_bits_to_f32(dra), axis=2)
+        for k in ks:
+            compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 1e-6, k, 1)
+            compare(dd, oracle_mod, dra, ver, tokens, flags, CONF, 0.999999, k, 1)
