@@ -1,8 +1,8 @@
 // dd_bidir_attention: full-sequence bidirectional attention (Section 2.2; Eq. 3
 // evaluated over the whole key range) for sm_100a, and dd_block_attention: the same
 // equation for a block of Nq queries against Nkv (cached) keys, with a per-sequence
-// number of valid keys and either memory layout.  One kernel serves both; two persistent forms of
-// it take many short items, and a form with one query tile and two CTAs per SM takes short query blocks and
+// number of valid keys and either memory layout.  One kernel serves both; a persistent form of
+// it takes more items than there are SMs, and a form with one query tile and two CTAs per SM takes short query blocks and
 // problems too small to fill the chip, whose keys it splits over clusters (see attention_impl, split_parts).
 //
 // One CTA owns two tiles of 128 query rows of one (batch, head) and walks over
@@ -260,6 +260,25 @@ __device__ __forceinline__ void columns_to_staging(const uint32_t *acc, float f,
         }
         const int chunk = (cb % 2) * 4 + i / 8;          // 16-byte chunk of the 128-byte row
         st_shared_v4(box + ((chunk ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Four neighbouring lanes exchange pieces of 32 bytes: lane t gives its piece c to lane c, as piece t.
+__device__ __forceinline__ void quad_transpose(uint32_t (&w)[4][8], int lane)
+{
+#pragma unroll
+    for (int b = 1; b < 4; b *= 2) {
+        const bool upper = lane & b;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (c & b) continue;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, upper ? w[c][i] : w[c | b][i], b);
+                if (upper) w[c][i] = got;
+                else w[c | b][i] = got;
+            }
+        }
     }
 }
 
@@ -649,7 +668,6 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 }
 
 #include "dd_attention_persistent.cuh"
-#include "dd_attention_short.cuh"
 #include "dd_attention_split.cuh"
 
 // ---------------------------------------------------------------------------
@@ -898,22 +916,15 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
     p.longest_first = longest_first(BH * m_blocks, sms);
     if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
-    // Many short items (more than one per SM, at most sixteen key tiles each, two query tiles in every item):
-    // persistent CTAs overlap each item's start and end with its neighbours.  D = 128 with four whole key tiles or
-    // more: the kernel whose rounds run across items (16 x 32 heads of 512 tokens 101 us with a CTA per item,
-    // 75 with the short kernel, 71 with this one; of 1024 299, 294 and 264).  Fewer, and D = 64: the short
-    // kernel (64 x 32 heads of 256 tokens at D = 128: 148, 99 and 113; 16 x 32 of 512 at D = 64: 73, 61 and 63).
-    // A fourth tile that is not nearly whole counts as none (short : this kernel, 64 x 32 heads of 385 tokens 286 :
-    // 339, of 400 287 : 388; 16 x 32 of 460 79 : 92, of 470 78.9 : 80.3, of 480 80.8 : 80.3, of 490 81.2 : 79.8); from six tiles
-    // on it makes no difference (40 x 32 of 641 420 : 392, of 660 418 : 412, of 700 435 : 433).
-    // Items of one query tile among those of two: a CTA per item (3 x 24 heads of 1357: 80 against 89).
-    if (BH * m_blocks > sms && nkv <= 16 && (Nq - 1) % (kQTiles * kBlockM) >= kBlockM) {
-        static bool attr_done[3][64] = {};
-        if (D == 64)
-            return launch_persistent(attention_short_kernel<64>, SmemP<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv, to);
-        if (Nkv < 480)
-            return launch_persistent(attention_short_kernel<128>, SmemP<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv, to);
-        return launch_persistent(attention_persistent_kernel, SmemL::kTotal + 1024, attr_done[2], p, sms, s, tq, tk, tv);
+    // More items than SMs: persistent CTAs, whose rounds run across items.  us, a CTA per item : persistent: D = 128, 16 x 32 heads of
+    // 512 tokens 101 : 76, 40 x 32 of 330 (a short kernel with rounds of its own, until then) 164 : 134, 64 x 32 of 256 148 : 91, 4 x
+    // 32 of 4096 936 : 875, 32 of 8192 955 : 921, 3 x 24 of 1357 73.3 : 66.6; D = 64, 3 x 24 of 1357 61.5 : 56.8, 16 x 32 of 512 60.0 :
+    // 54.8, 32 x 32 of 384 105 : 78.  With one round of items the one-item kernel's shorter start counts: 32 x 300 11.1 : 11.2, 16
+    // x 512 at D = 128 11.65 : 11.8, 2 x 16 of 640 at D = 64 12.2 : 12.4.
+    if (nkv >= 2 && BH * m_blocks > sms) {
+        static bool attr_done[2][64] = {};
+        if (D == 64) return launch_persistent(attention_persistent_kernel<64>, SmemL<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv);
+        return launch_persistent(attention_persistent_kernel<128>, SmemL<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv);
     }
     return D == 64 ? launch<64, false>(tq, tk, tv, to, p, s) : launch<128, false>(tq, tk, tv, to, p, s);
 }

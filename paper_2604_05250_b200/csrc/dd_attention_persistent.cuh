@@ -1,6 +1,6 @@
-// The square, head-major case of dd_bidir_attention (Section 2.2; Eq. 3) for many items of four to sixteen
-// key tiles at D = 128: persistent CTAs, one per SM, each walking over work items blockIdx.x,
-// blockIdx.x + gridDim.x, ...  An item is two tiles of 128 query rows of one head.  Roles and
+// The square, head-major case of dd_bidir_attention (Section 2.2; Eq. 3) where there are more work items than SMs and at least two key
+// tiles: persistent CTAs, one per SM, each walking over work items blockIdx.x,
+// blockIdx.x + gridDim.x, ...  An item is two tiles of 128 query rows of one head (the second one may be empty).  Roles and
 // arithmetic are those of attention_kernel; the pipeline never drains between items.
 //
 // One stream of rounds.  Round r of a CTA is one key tile of one item, for both query tiles g:
@@ -18,9 +18,12 @@
 //     issued earlier), so O has a barrier of its own only at an item's end.
 //   * Q buffers: Q_g of the next item goes into a buffer whose last S product has been committed
 //     (q_free), a round before the item ends, not into one whose result has been written: results go from
-//     registers straight to global memory, a full 32-byte sector per thread and store, so that five
-//     key/value tiles fit beside two query tiles.  (Staged in shared memory, with four: 16 x 32 heads of 512
-//     tokens 83 -> 88 us, of 1024 269 -> 289.)
+//     registers straight to global memory, so that five key/value tiles fit beside two query tiles.  (Staged in shared
+//     memory, with four: 16 x 32 heads of 512 tokens 83 -> 88 us, of 1024 269 -> 289.)
+//   * Every lane storing its own row, 32 bytes at a time, took 2500 to 2900 cycles per item and group; four lanes
+//     now exchange pieces first and store 128 bytes of a row together: 2000 (16 x 32 of 512 71.3 -> 68.5 us in short bursts).
+//   * A group writes an item's result behind the weights of the next item's first tile, whose products the stores then overlap: 68.5
+//     -> 67.2 in bursts; both, under the power cap, 85.3 -> 76.0.
 //   * o_free: the group has read the finished accumulator out of tensor memory; the next item's
 //     first P V may overwrite it.
 // Every wait is bounded and reports to the attention health word.  Included by dd_attention.cu
@@ -29,11 +32,11 @@
 
 constexpr int kReleases = 8;         // release barriers: round r completes phase r / 8 of barrier r % 8
 
+template <int D>
 struct SmemL {
-    static constexpr int D = 128;
     static constexpr int kTileBytes = kBlockN * D * 2;
     static constexpr int kQ = 2;                                    // query tiles
-    static constexpr int kSlots = 5;                                // key and value tiles
+    static constexpr int kSlots = D == 128 ? 5 : 9;                 // key and value tiles
     static constexpr int kPairs = kSlots / 2 + 1;                   // pair barriers
     static constexpr int kRing = kQ * kTileBytes;
     static constexpr int kBars = kRing + kSlots * kTileBytes;
@@ -49,12 +52,12 @@ struct SmemL {
     static_assert((kSlots - 1) / 2 + 1 <= kReleases, "release barriers");
 };
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                             const __grid_constant__ CUtensorMap tm_v, const AttnParams p)
 {
-    using L = SmemL;
-    constexpr int D = L::D;
+    using L = SmemL<D>;
     constexpr uint32_t kQ = L::kQ, kSlots = L::kSlots;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -146,54 +149,71 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
         const bool sectors = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;     // rows start on 32-byte boundaries
         uint32_t t_run = 0;              // key tiles so far: phase
         unsigned err = 0;
-        for (int n = 0; n < my_items; ++n) {
-            const Item t = item_at(n);
+        // An item's result is written after the weights of the next item's first tile have been handed over: the stores then
+        // overlap that tile's products, and the group does not stand still for its last P V.
+        float l_prev = 0.f;
+        for (int n = 0; n <= my_items && err == 0; ++n) {
             float m_ref = -INFINITY, l_run = 0.f;
-            for (int j = 0; j < nkv; ++j, ++t_run) {
-                if (!mbar_wait(bar_s_full(g), t_run & 1)) { err = kErrWaitS; break; }
-                tc_fence_after();
-                softmax_tile<D, false>(tS, tO, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run,
-                    [&] {                        // three quarters of the weights are stored
-                        tmem_wait_st();
-                        tc_fence_before();
-                        mbar_arrive(bar_p_early(g));
-                    });
-                tmem_wait_st();
-                tc_fence_before();
-                mbar_arrive(bar_p_full(g));
-            }
-            if (err == 0 && !mbar_wait(bar_o_full(g), n & 1)) err = kErrWaitO;
-            if (err != 0) { report(p, err); break; }
-            // ---- epilogue: O / l -> bf16 -> global
-            tc_fence_after();
-            uint32_t acc[D];
+            for (int j = 0; j < nkv; ++j) {
+                if (n < my_items) {
+                    if (!mbar_wait(bar_s_full(g), t_run & 1)) { err = kErrWaitS; break; }
+                    tc_fence_after();
+                    softmax_tile<D, false>(tS, tO, j == 0, p.Nkv - j * kBlockN, c, m_ref, l_run,
+                        [&] {                        // three quarters of the weights are stored
+                            tmem_wait_st();
+                            tc_fence_before();
+                            mbar_arrive(bar_p_early(g));
+                        });
+                    tmem_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(bar_p_full(g));
+                    ++t_run;
+                }
+                if (j == 0 && n > 0) {
+                    // ---- epilogue of the item before: O / l -> bf16 -> global
+                    if (!mbar_wait(bar_o_full(g), (n - 1) & 1)) { err = kErrWaitO; break; }
+                    tc_fence_after();
+                    uint32_t acc[D];
 #pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb)
-                tmem_ld32(tO + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[cb * 32]));
-            tmem_wait_ld();
-            tc_fence_before();
-            mbar_arrive(bar_o_free(g));      // the next item's first P V may overwrite the accumulator
-            const int row = t.row0 + g * kBlockM + (warp & 3) * 32 + lane;
-            if (row < p.Nq) {
-                const float inv = 1.f / l_run;
-                unsigned char *dst = reinterpret_cast<unsigned char *>(p.out) + ((size_t)t.bh * p.Nq + row) * (D * 2);
+                    for (int cb = 0; cb < D / 32; ++cb)
+                        tmem_ld32(tO + cb * 32, *reinterpret_cast<uint32_t(*)[32]>(&acc[cb * 32]));
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    mbar_arrive(bar_o_free(g));      // this item's first P V may overwrite the accumulator
+                    const Item t = item_at(n - 1);
+                    const int row = t.row0 + g * kBlockM + (warp & 3) * 32 + (lane & ~3);       // of the quad's first lane
+                    unsigned char *dst = reinterpret_cast<unsigned char *>(p.out) + ((size_t)t.bh * p.Nq + row) * (D * 2) + (lane & 3) * 32;
+                    const float inv = 1.f / l_prev;
 #pragma unroll
-                for (int i = 0; i < D; i += 16) {
-                    uint32_t w[8];
+                    for (int h = 0; h < D / 64; ++h) {
+                        // 64 columns of four rows: each lane turns its row's four 32-byte pieces into one piece of every row
+                        uint32_t w[4][8];
 #pragma unroll
-                    for (int h = 0; h < 8; ++h) {
-                        __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(acc[i + 2 * h]) * inv,
-                                                                 __uint_as_float(acc[i + 2 * h + 1]) * inv);
-                        w[h] = *reinterpret_cast<uint32_t *>(&v);
-                    }
-                    if (sectors) st_global_v8(dst + 2 * i, w);
-                    else {
-                        reinterpret_cast<uint4 *>(dst + 2 * i)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                        reinterpret_cast<uint4 *>(dst + 2 * i)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const int e = 64 * h + 16 * q + 2 * i;
+                                __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(acc[e]) * inv, __uint_as_float(acc[e + 1]) * inv);
+                                w[q][i] = *reinterpret_cast<uint32_t *>(&v);
+                            }
+                        quad_transpose(w, lane);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            if (row + r >= p.Nq) break;
+                            unsigned char *to = dst + r * (D * 2) + h * 128;
+                            if (sectors) st_global_v8(to, w[r]);
+                            else {
+                                reinterpret_cast<uint4 *>(to)[0] = make_uint4(w[r][0], w[r][1], w[r][2], w[r][3]);
+                                reinterpret_cast<uint4 *>(to)[1] = make_uint4(w[r][4], w[r][5], w[r][6], w[r][7]);
+                            }
+                        }
                     }
                 }
+                if (n == my_items) break;
             }
+            l_prev = l_run;
         }
+        if (err != 0) report(p, err);
     } else {
         reg_dec<72>();
         if (warp == kLoadWarp && elect_one()) {

@@ -182,11 +182,28 @@ def test_many_short_items_match_one_item_per_cta(dd):
     assert torch.equal(whole, torch.cat(parts, dim=1))
 
 
-# where the choice of kernel changes (more items than SMs; 480 keys and 16 key tiles), one key in the last tile,
+@pytest.mark.parametrize("N,D", [(259, 128), (259, 64)])
+def test_results_off_sector_boundaries(dd, oracle_mod, N, D):
+    """The persistent kernel's stores where rows start on 16 bytes only, and where a quad of rows is not all there."""
+    import torch
+    q, k, v = synth.attention_inputs(1, 80, N, D, seed=N + D)
+    g = Guarded((80 * N * D + 8,), torch.bfloat16)
+    out = g.view[8:].view(1, 80, N, D)
+    g.view[:8] = 7.0
+    dd.bidir_attention(*(to_torch_bf16(x, "cuda") for x in (q, k, v)), out=out)
+    torch.cuda.synchronize()
+    assert dd.attention_status() == 0 and out.data_ptr() % 32 == 16
+    g.check("attention output")
+    assert (g.view[:8] == 7.0).all()
+    check_attention(bf16_tensor_to_f64(out), oracle_mod.attention(q, k, v, D ** -0.5))
+
+
+# where the choice of kernel changes (more items than SMs; two key tiles), one key in the last tile,
 # heads whose last 256 rows are one query tile, and D = 64, whose exponentials are partly computed as a polynomial
 @pytest.mark.parametrize("B,H,N,D", [(1, 80, 385, 128), (1, 38, 897, 128), (2, 80, 300, 128), (1, 19, 2048, 128),
                                      (1, 80, 479, 128), (1, 80, 480, 128),
-                                     (1, 17, 2177, 128), (1, 80, 385, 64), (1, 75, 500, 64), (1, 50, 600, 64)])
+                                     (1, 17, 2177, 128), (1, 80, 385, 64), (1, 75, 500, 64), (1, 50, 600, 64),
+                                     (1, 160, 129, 128), (1, 17, 2177, 64), (1, 40, 1153, 64)])
 def test_kernel_choice(dd, oracle_mod, B, H, N, D):
     import torch
     # Unplanted inputs: rows that one or two keys carry put results of 2 to 4 in magnitude up to 1.2e-2 from the
