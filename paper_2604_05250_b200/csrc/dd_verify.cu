@@ -310,7 +310,13 @@ int launch_stream(const VerifyParams &p, cudaStream_t stream)
 // 29.9; 1 x 32, 126464, KL: 14.2 / 24.2; 1 x 128: 25.9 / 31.9; 16 x 512, 1000, CONF: 23.0 / 38.3.  Beyond the line: 8 x
 // 256, 32000, CONF: 36.6 / 31.7; 1 x 256, 126464, KL: 38.7 / 37.5; 16 x 512, 8000, KL 50 %: 58.4 / 51.1.
 long row_pieces(int V, bool kl) { return ((long)V + 7) / (kl ? kPiece : 2 * kPiece) + 1; }
-bool rows_path(int V, long rows, int sms, bool kl) { return rows * row_pieces(V, kl) <= 160L * sms && rows <= 32L * 1024; }
+// Beyond it, up to two rounds of the deep form (below), which the streaming kernel's fixed cost does not earn back: 1 x 256,
+// 126464, KL 31.6 / 37.0; 1 x 400, KL 100 % 45.1 / 50.7, 50 % 32.6 / 39.5, CONF 28.4 / 38.2, 20.7 / 34.6; 2 x 256, KL 100 % 56.1 /
+// 57.6, 50 % 34.0 / 37.6, 25 % 32.0 / 31.1.
+bool rows_path(int V, long rows, int sms, bool kl)
+{
+    return (rows * row_pieces(V, kl) <= 160L * sms && rows <= 32L * 1024) || rows <= 4L * sms;
+}
 
 template <bool KL>
 int launch_rows(const VerifyParams &p, cudaStream_t stream)
@@ -322,7 +328,7 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     // Warps per row: enough to fill the GPU (24 per SM), but at least two pieces for each.  Few rows: clusters
     // of CTAs, as long as two CTAs per SM hold them all (32 rows of 126464: 27 us with eight warps a row,
     // 14 with clusters of eight; 128 rows: clusters of two 25.9, of four 30.1).
-    RowsShape shape = {1, 1};
+    RowsShape shape = {1, 1, 0};
     while (shape.wpr < kRWarps && 4 * shape.wpr <= pieces + 1 && rows * shape.wpr < 24L * sms) shape.wpr *= 2;
     while (shape.wpr == kRWarps && shape.cluster < kRMaxCluster && 4 * kRWarps * shape.cluster <= pieces + 1 &&
            2 * shape.cluster * rows <= 2L * sms)
@@ -338,7 +344,16 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
-    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL>, p, shape));
+    // Two CTAs per SM and deep loads (row_part_deep), where all CTAs fit at once and a warp has a few pieces, or rows are few and long;
+    // with more rows a third CTA per SM is worth more than deep loads.  us, three CTAs : deep (B x P, V): 1 x 256, 126464, KL 36.8 : 29.9; 1 x 128
+    // 23.9 : 20.4; 1 x 32 14.1 : 12.8; 1 x 200, 50000, KL 19.9 : 18.2; but 1 x 256, 16000, KL 11.8 : 12.0, 1 x 256, 16001, CONF 8.8 : 9.6; 2 x 300,
+    // 32001, KL 50 % 19.9 : 22.0; 4 x 256, 8000, KL 50 % 13.4 : 16.8; 16 x 512, 1000, CONF 17.8 : 22.4.
+    const bool deep = (groups * shape.cluster <= 2L * sms && (shape.cluster > 1 || pieces >= 3 * shape.wpr)) || rows * pieces > 160L * sms;
+    // flagged rows first (mapped_row): a row per CTA, and long ones (all flagged: 1 x 512, 32000, CONF 16.9 : 18.5, 3 x 200, 60000, CONF 23.8 :
+    // 24.9, 2 x 300, 32001, KL 28.5 : 28.1)
+    shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24));
+    DD_CUDA_TRY(deep ? cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL, true>, p, shape)
+                     : cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL, false>, p, shape));
     dd::count_launch();
     return DD_OK;
 }

@@ -372,6 +372,25 @@ def test_row_and_streaming_kernels(dd, oracle_mod, B, P, V, flagged, mode):
         dd.debug_set_max_ctas(0)
 
 
+# the row kernel's deep form: two pieces to a warp and many, rows on and off vector boundaries (edges at both ends of a row), a last piece of
+# a few logits, of all but one and none at all, clusters; flagged rows first: none, one, the last, more of them than a word of 32
+@pytest.mark.parametrize("B,P,V,flagged,mode", [
+    (1, 256, 24 * 1024, 256, KL), (1, 200, 25 * 1024 + 1, 1, KL | PROB), (1, 130, 51 * 1024 - 1, 130, CONF), (2, 148, 49155, 97, KL),
+    (1, 40, 70001, 40, CONF), (2, 5, 126464, 3, KL), (1, 300, 25 * 1024 + 3, 33, KL), (2, 290, 26001, 580, KL), (3, 60, 50000, 0, KL)])
+def test_row_kernel_with_long_rows(dd, oracle_mod, B, P, V, flagged, mode):
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, min(flagged, P), 0.2, seed=V + P)
+    if flagged == 0:
+        flags[:] = 0
+        flags[1, P - 1] = 1                  # one sequence with its last row only, two without any
+    every = ver.reshape(-1, V)
+    for i, row in enumerate(every[::5]):     # excluded tokens: at the row's ends, a whole lane's vector, a whole piece
+        row[[0, V - 1, 7 * i % V]] = 0xFF80
+        row[1024:1032] = 0xFF80
+        dra.reshape(-1, V)[5 * i, [0, V - 1, 7 * i % V]] = 0xFF80
+        dra.reshape(-1, V)[5 * i, 1024:2048] = 0xFF80
+    compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 9, 3)
+
+
 @pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 100, 299, 300, 301])
 def test_minimum_keep_with_many_equal_scores(dd, oracle_mod, k):
     """300 rows of which many are the same: ties at every place of the order, kept lowest index first."""
