@@ -313,6 +313,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                  const AttnParams p)
 {
+    if (kBlock) grid_wait();                              // the sequences' lengths are read
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     // 128-byte-swizzled tiles must start on a 1024-byte boundary
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -366,6 +367,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         mbar_init(bar_q(0), 1); mbar_init(bar_q(1), 1);
         for (int s = 0; s < kStages; ++s) mbar_init(bar_kv_full(s), 1);
         fence_mbar_init();
+        if (!kBlock) grid_wait();
         // (also when an earlier wait has expired and the CTA will do nothing: such a CTA lingers at
         // its end until copies in flight have landed)
         if (early) {
@@ -387,6 +389,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             mbar_init(bar_o_full(g), 1);
         }
         fence_mbar_init();
+        grid_wait();
         // a wait that expired in an earlier CTA or launch stops the rest from queueing up behind it
         tmem_slot_gen[1] = *reinterpret_cast<volatile unsigned int *>(p.status);
     }
@@ -552,6 +555,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 for (int cx = 0; cx < kBoxes; ++cx)
                     load_box(dst + cx * kBoxBytes, tm, bar_kv_full(slot), cx * 64, (item >> 1) * kBlockN);
             }
+            grid_trigger();
         } else if (warp == kMmaWarp && elect_one()) {
             // =============================================================== MMA issuer
             constexpr uint32_t kIdescS = idesc_bf16(kBlockM, kBlockN, false);
@@ -735,8 +739,7 @@ int launch(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, 
         }
     }
     const long grid = (long)p.BH * p.m_blocks;
-    attention_kernel<D, kBlock><<<(unsigned)grid, kThreads, smem, s>>>(tq, tk, tv, to, p);
-    DD_CUDA_TRY(cudaGetLastError());
+    DD_CUDA_TRY(dd::launch(attention_kernel<D, kBlock>, (unsigned)grid, kThreads, smem, s, 1, tq, tk, tv, to, p));
     dd::count_launch();
     return DD_OK;
 }
@@ -757,8 +760,7 @@ int launch_persistent(Kernel kernel, int smem, bool (&attr_done)[64], const Attn
     }
     const long items = (long)p.BH * p.m_blocks;
     const unsigned grid = (unsigned)(items < sms ? items : sms);
-    kernel<<<grid, kThreads, smem, s>>>(maps..., p);
-    DD_CUDA_TRY(cudaGetLastError());
+    DD_CUDA_TRY(dd::launch(kernel, grid, kThreads, smem, s, 1, maps..., p));
     dd::count_launch();
     return DD_OK;
 }
@@ -779,18 +781,8 @@ int launch_split(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap
             attr_done[dev] = true;
         }
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((long)p.BH * p.m_blocks * parts));
-    cfg.blockDim = dim3(kSplitThreads);
-    cfg.dynamicSmemBytes = kSplitSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute cluster;
-    cluster.id = cudaLaunchAttributeClusterDimension;
-    cluster.val.clusterDim.x = (unsigned)parts;
-    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
-    cfg.attrs = &cluster;
-    cfg.numAttrs = parts > 1 ? 1 : 0;
-    DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_split_kernel<D, G>, tq, tk, tv, p, q_rows, parts));
+    DD_CUDA_TRY(dd::launch(attention_split_kernel<D, G>, (unsigned)((long)p.BH * p.m_blocks * parts), kSplitThreads, kSplitSmem, s, parts,
+                           tq, tk, tv, p, q_rows, parts));
     dd::count_launch();
     return DD_OK;
 }

@@ -109,6 +109,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
         for (int i = 0; i < L::kPairs; ++i) mbar_init(bar_pair(i), 1);
         mbar_init(bar_k0, 1);
         fence_mbar_init();
+        grid_wait();
         const Item t = item_at(0);
         mbar_expect_tx(bar_q_full(0), kTileBytes);
         load_tile(sQ, &tm_q, bar_q_full(0), t.row0, t.bh);
@@ -126,6 +127,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
             mbar_init(bar_o_free(g), kBlockM);
         }
         fence_mbar_init();
+        grid_wait();
         // a wait that expired in an earlier CTA or launch stops the rest from queueing up behind it
         tmem_slot_gen[1] = *reinterpret_cast<volatile unsigned int *>(p.status);
     }
@@ -258,6 +260,7 @@ attention_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
                 }
                 t = next;
             }
+            grid_trigger();
             if (!ok) report(p, kErrWaitSlot);
         } else if (warp == kMmaWarp && elect_one()) {
             // =============================================================== MMA issuer

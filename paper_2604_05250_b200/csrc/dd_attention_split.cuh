@@ -91,6 +91,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     constexpr uint32_t kTileBytes = L::kTileBytes;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kBoxBytes = 128 * 128;
+    grid_wait();                                                 // the sequences' lengths are read
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t pad = (1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u;
     unsigned char *tiles_gen = smem_dyn + pad;
@@ -281,6 +282,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 load_tile(slot, (t & 1) ? &tm_v : &tm_k, j_begin + (t >> 1), clear && t + 1 == 2 * n_tiles);
                 if (++slot == slots) { slot = 0; ++use; }
             }
+            grid_trigger();
         } else if (healthy && warp == kSplitMmaWarp && elect_one()) {
             // =============================================================== MMA issuer
             constexpr uint32_t kIdescS = idesc_bf16(kBlockM, kBlockN, false);

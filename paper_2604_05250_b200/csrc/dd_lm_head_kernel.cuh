@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(kRowsThreads)
 lm_head_rows_kernel(const LmParams q, const ddv::VerifyParams p, const uint4 *hidden, uint4 *gathered,
                     const uint4 *hidden_d, uint4 *gathered_d)
 {
+    grid_trigger();
+    grid_wait();
     const uint8_t *flags = p.flags;
     __shared__ int s_before, s_all;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -221,6 +223,8 @@ constexpr int kFoldThreads = 256;
 template <bool KL>
 __global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const __grid_constant__ ddv::VerifyParams p, const LmParams q)
 {
+    grid_trigger();
+    grid_wait();
     const int rows = q.rows;
     __shared__ ddv::BlockReport s_report;
     const int row0 = blockIdx.x * (kFoldThreads / 32);
@@ -412,6 +416,17 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     volatile uint32_t *abort_flag = tmem_slot_gen + 1;
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5);
+    if (tid == 0) {
+        for (int s = 0; s < kMaxStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(bars_acc_full + 8u * a, 1);
+            mbar_init(bars_acc_empty + 8u * a, kEpilogueWarps / 2);
+        }
+        fence_mbar_init();
+        *abort_flag = 0u;
+    }
+    if (warp == 0) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
+    grid_wait();                                              // what follows reads what the kernels before left
     LmPlan plan = q.plan ? *q.plan : q.all_rows;
     // few rows, none listed: perhaps none of them is flagged, and there is nothing to multiply
     int any = 1;
@@ -426,16 +441,6 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
     const uint32_t stage_bytes = a_bytes + b_bytes;
     const uint32_t stages = min((uint32_t)kMaxStages, kRingBytes / stage_bytes);
 
-    if (tid == 0) {
-        for (int s = 0; s < kMaxStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        for (int a = 0; a < 2; ++a) {
-            mbar_init(bars_acc_full + 8u * a, 1);
-            mbar_init(bars_acc_empty + 8u * a, kEpilogueWarps / 2);
-        }
-        fence_mbar_init();
-        *abort_flag = 0u;
-    }
-    if (warp == 0) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
     tc_fence_before();
     if (!__syncthreads_or(any)) plan.n_rows = 0;
     tc_fence_after();
@@ -483,6 +488,7 @@ lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const 
                 if (++s == stages) { s = 0; ++round; }
             }
         }
+        grid_trigger();
     } else if (warp == kMmaWarp && elect_one()) {
         // ===================================================================== MMA issuer
         const uint32_t idesc = idesc_bf16(128, plan.N, false);

@@ -84,6 +84,15 @@ lm_head_pair_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, c
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int rank = blockIdx.x & 1;
+    if (tid == 0) {
+        for (int s = 0; s < kMaxStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+        mbar_init(bar_acc_full, 1);
+        mbar_init(bar_acc_empty, 2 * kEpilogueWarps);
+        fence_mbar_init();
+        *abort_flag = 0u;
+    }
+    if (warp == 0) { __syncwarp(); tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+    grid_wait();                                              // what follows reads what the kernels before left
     LmPlan plan = q.plan ? *q.plan : q.all_rows;
     // few rows, none listed: perhaps none of them is flagged, and there is nothing to multiply
     int any = 1;
@@ -97,14 +106,6 @@ lm_head_pair_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, c
     const uint32_t stage_bytes = KL ? kATileBytes + b_bytes : max(2 * kATileBytes + b_bytes, kATileBytes + 2 * b_bytes);
     const uint32_t stages = min((uint32_t)kMaxStages, kRingBytes / stage_bytes);
 
-    if (tid == 0) {
-        for (int s = 0; s < kMaxStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        mbar_init(bar_acc_full, 1);
-        mbar_init(bar_acc_empty, 2 * kEpilogueWarps);
-        fence_mbar_init();
-        *abort_flag = 0u;
-    }
-    if (warp == 0) { __syncwarp(); tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
     tc_fence_before();
     if (!__syncthreads_or(any)) plan.n_rows = 0;
     __syncwarp();
@@ -157,6 +158,7 @@ lm_head_pair_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, c
                 if (++s == stages) { s = 0; ++round; }
             }
         }
+        grid_trigger();
     } else if (warp == kMmaWarp && rank == 0 && elect_one()) {
         // ===================================================================== MMA issuer
         const uint32_t idesc = idesc_bf16(256, KL ? 2 * plan.N : plan.N, false);

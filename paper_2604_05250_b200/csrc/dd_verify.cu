@@ -297,8 +297,7 @@ int launch_stream(const VerifyParams &p, cudaStream_t stream)
     long grid = units < sms ? units : sms;
     const int cap = g_max_ctas.load(std::memory_order_relaxed);
     if (cap > 0 && grid > cap) grid = cap;
-    verify_stream_kernel<KL, kRagged><<<(unsigned)grid, kSThreads, kSRingBytes, stream>>>(p);
-    DD_CUDA_TRY(cudaGetLastError());
+    DD_CUDA_TRY(dd::launch(verify_stream_kernel<KL, kRagged>, (unsigned)grid, kSThreads, kSRingBytes, stream, 1, p));
     dd::count_launch();
     return DD_OK;
 }
@@ -334,16 +333,6 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
            2 * shape.cluster * rows <= 2L * sms)
         shape.cluster *= 2;
     const long groups = (rows + kRWarps / shape.wpr - 1) / (kRWarps / shape.wpr);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(groups * shape.cluster));
-    cfg.blockDim = dim3(32 * kRWarps);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = shape.cluster;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
     // Two CTAs per SM and deep loads (row_part_deep), where all CTAs fit at once and a warp has a few pieces, or rows are few and long;
     // with more rows a third CTA per SM is worth more than deep loads.  us, three CTAs : deep (B x P, V): 1 x 256, 126464, KL 36.8 : 29.9; 1 x 128
     // 23.9 : 20.4; 1 x 32 14.1 : 12.8; 1 x 200, 50000, KL 19.9 : 18.2; but 1 x 256, 16000, KL 11.8 : 12.0, 1 x 256, 16001, CONF 8.8 : 9.6; 2 x 300,
@@ -352,8 +341,8 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     // flagged rows first (mapped_row): a row per CTA, and long ones (all flagged: 1 x 512, 32000, CONF 16.9 : 18.5, 3 x 200, 60000, CONF 23.8 :
     // 24.9, 2 x 300, 32001, KL 28.5 : 28.1)
     shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24));
-    DD_CUDA_TRY(deep ? cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL, true>, p, shape)
-                     : cudaLaunchKernelEx(&cfg, verify_rows_kernel<KL, false>, p, shape));
+    DD_CUDA_TRY(dd::launch(deep ? verify_rows_kernel<KL, true> : verify_rows_kernel<KL, false>, (unsigned)(groups * shape.cluster),
+                           32 * kRWarps, 0, stream, shape.cluster, p, shape));
     dd::count_launch();
     return DD_OK;
 }
@@ -579,32 +568,15 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
     const unsigned grid = (unsigned)(items < ctas ? items : ctas);
     if (q.plan) {
         q.rows_per_block = kRowsWarps * ((q.rows + kRowsWarps * kRowsBlocks - 1) / (kRowsWarps * kRowsBlocks));
-        lm_head_rows_kernel<KL><<<(unsigned)((q.rows + q.rows_per_block - 1) / q.rows_per_block), kRowsThreads, 0, stream>>>(
-            q, p, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
-            static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes));
-        DD_CUDA_TRY(cudaGetLastError());
+        DD_CUDA_TRY(dd::launch(lm_head_rows_kernel<KL>, (unsigned)((q.rows + q.rows_per_block - 1) / q.rows_per_block), kRowsThreads, 0, stream, 1,
+                               q, p, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
+                               static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes)));
     }
-    if (q.pairs) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid + (grid & 1));
-        cfg.blockDim = dim3(ddlm::kThreads);
-        cfg.dynamicSmemBytes = kSmemBytes;
-        cfg.stream = stream;
-        cudaLaunchAttribute cluster;
-        cluster.id = cudaLaunchAttributeClusterDimension;
-        cluster.val.clusterDim.x = 2;
-        cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
-        cfg.attrs = &cluster;
-        cfg.numAttrs = 1;
-        DD_CUDA_TRY(cudaLaunchKernelEx(&cfg, lm_head_pair_kernel<KL>, m, q, p));
-    } else {
-        lm_head_kernel<KL><<<grid, ddlm::kThreads, kSmemBytes, stream>>>(m, q, p);
-        DD_CUDA_TRY(cudaGetLastError());
-    }
+    if (q.pairs) DD_CUDA_TRY(dd::launch(lm_head_pair_kernel<KL>, grid + (grid & 1), ddlm::kThreads, kSmemBytes, stream, 2, m, q, p));
+    else DD_CUDA_TRY(dd::launch(lm_head_kernel<KL>, grid, ddlm::kThreads, kSmemBytes, stream, 1, m, q, p));
     // one warp per row
     const unsigned fold_grid = (unsigned)(((long)q.rows + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
-    lm_head_fold_kernel<KL><<<fold_grid, kFoldThreads, 0, stream>>>(p, q);
-    DD_CUDA_TRY(cudaGetLastError());
+    DD_CUDA_TRY(dd::launch(lm_head_fold_kernel<KL>, fold_grid, kFoldThreads, 0, stream, 1, p, q));
     dd::count_launch(q.plan ? 3 : 2);
     return DD_OK;
 }

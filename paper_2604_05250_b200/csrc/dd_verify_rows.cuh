@@ -344,6 +344,7 @@ __global__ void __launch_bounds__(32 * kRWarps, kDeep ? 2 : 3) verify_rows_kerne
     __shared__ __align__(16) Partial s_all[kRMaxCluster * kRWarps];
     __shared__ BlockReport s_report;
     __shared__ uint32_t s_words[kMappedRows / 32];
+    ddptx::grid_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long n_rows = (long)p.B * p.P;
     const int wpr = shape.wpr, cluster = shape.cluster;
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(32 * kRWarps, kDeep ? 2 : 3) verify_rows_kerne
         __syncwarp();
         if (wpr > 1 && cluster == 1) cta_bar_sync(1 + warp / wpr, 32 * wpr);
     }
+    ddptx::grid_trigger();
     const int pieces = (row_head(row, p.V) + p.V + kStep - 1) / kStep;
     const Partial *parts = s_part + warp - warp % wpr;
     if (cluster > 1) {

@@ -38,6 +38,7 @@
 // update per sequence and range) and decides the sequences it completes (Section 3.2).
 #pragma once
 
+#include "dd_ptx.cuh"
 #include "dd_verify_common.cuh"
 
 namespace ddv {
