@@ -70,7 +70,6 @@ __device__ __forceinline__ void pending_add(const VerifyParams &p, Pending &pend
 template <bool KL, bool kRagged>
 __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const VerifyParams p)
 {
-    ddptx::grid_wait();
     extern __shared__ __align__(128) unsigned char s_ring[];     // [warp][stage][kSStageBytes]
     __shared__ __align__(8) unsigned long long s_full[kSConsumers][kSStages];    // mbarriers: the stage holds data
     __shared__ __align__(16) int4 s_meta[kSConsumers][kSStages];  // what the stage holds
@@ -582,7 +581,6 @@ __global__ void __launch_bounds__(kSThreads, 1) verify_stream_kernel(const Verif
         }
     }
 
-    ddptx::grid_trigger();
     __syncthreads();
     if (*abort_flag) {
         // a wait expired: give copies that may still be in flight time to land before the shared
