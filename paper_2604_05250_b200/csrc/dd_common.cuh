@@ -59,10 +59,11 @@ void count_launch(unsigned n = 1);
 // ended and what they wrote can be seen, so that calls on one stream keep their order.  `cluster`: CTAs per cluster.
 // Calls that follow one another directly lose the gap between two kernels and the set-up before the wait (barriers, TMEM, tensor map
 // prefetch): attention 1 x 4 x 128 x 64 4.6 -> 3.6 us a call, 1 x 32 x 1024 x 128 19.7 -> 19.0, verification of 128 rows of 1024 7.5 ->
-// 6.8, 256 of 126464 with two logit streams 37.3 -> 30.3 (1.5 of it the row kernel's), the head's three kernels over 64 rows of 1000
-// 14.8 -> 12.2.  A captured graph keeps these edges.
+// 6.8, the head's three kernels over 64 rows of 1000
+// 14.8 -> 12.2.  A captured graph keeps these edges.  `early` false: an ordinary launch, behind the end of the kernel before.
 template <typename... Params, typename... Args>
-cudaError_t launch(void (*kernel)(Params...), unsigned grid, unsigned threads, int smem, cudaStream_t stream, int cluster, const Args &...args)
+cudaError_t launch_as(bool early, void (*kernel)(Params...), unsigned grid, unsigned threads, int smem, cudaStream_t stream, int cluster,
+                      const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -71,13 +72,19 @@ cudaError_t launch(void (*kernel)(Params...), unsigned grid, unsigned threads, i
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)cluster;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kernel)(Params...), unsigned grid, unsigned threads, int smem, cudaStream_t stream, int cluster, const Args &...args)
+{
+    return launch_as(true, kernel, grid, threads, smem, stream, cluster, args...);
 }
 
 #define DD_CUDA_TRY(expr)                                         \

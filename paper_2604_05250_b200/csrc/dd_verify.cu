@@ -344,8 +344,13 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     // flagged rows first (mapped_row): a row per CTA, and long ones (all flagged: 1 x 512, 32000, CONF 16.9 : 18.5, 3 x 200, 60000, CONF 23.8 :
     // 24.9, 2 x 300, 32001, KL 28.5 : 28.1)
     shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24));
-    DD_CUDA_TRY(dd::launch(deep ? verify_rows_kernel<KL, true> : verify_rows_kernel<KL, false>, (unsigned)(groups * shape.cluster),
-                           32 * kRWarps, 0, stream, shape.cluster, p, shape));
+    // Early only where every CTA has an SM to itself: CTAs that arrive early pile up on the SMs that are free first, and waiting ones of a second
+    // round take up the room of the first one's last.  us, early : ordinary, after attention of 32 heads of 1024: 256 rows of 126464, KL
+    // 55.5 : 53.0, 2 x 300 of 32001 42.7 : 39.3, 1 x 100 of 50000, CONF 35.1 : 33.1, 1 x 512 of 32000, CONF 39.2 : 38.3; but 128 of
+    // 1024, KL 27.1 : 28.4, 64 of 1000 27.9 : 28.5.  One after the other, 1024 of 4000, KL 19.4 : 18.7.
+    const bool early = !deep && groups * shape.cluster <= sms;
+    DD_CUDA_TRY(dd::launch_as(early, deep ? verify_rows_kernel<KL, true> : verify_rows_kernel<KL, false>, (unsigned)(groups * shape.cluster),
+                              32 * kRWarps, 0, stream, shape.cluster, p, shape));
     dd::count_launch();
     return DD_OK;
 }

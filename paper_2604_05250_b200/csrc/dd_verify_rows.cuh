@@ -336,8 +336,6 @@ __device__ __forceinline__ int mapped_row(const VerifyParams &p, int v, uint32_t
     return src * 32 + __ffs(__ballot_sync(full, here)) - 1;
 }
 
-// It does not call the next kernel in: where its CTAs come in more than one round, those of the next call, waiting, took up room that its
-// own last ones could use (1024 rows of 4000, two streams: 18.7 us without, 19.4 with; 3 x 700 of 2000 14.7 and 15.4; one round the same).
 // kDeep: row_part_deep, whose registers leave room for two CTAs on an SM instead of three.
 template <bool KL, bool kDeep>
 __global__ void __launch_bounds__(32 * kRWarps, kDeep ? 2 : 3) verify_rows_kernel(const __grid_constant__ VerifyParams p, const RowsShape shape)
@@ -367,6 +365,7 @@ __global__ void __launch_bounds__(32 * kRWarps, kDeep ? 2 : 3) verify_rows_kerne
         __syncwarp();
         if (wpr > 1 && cluster == 1) cta_bar_sync(1 + warp / wpr, 32 * wpr);
     }
+    ddptx::grid_trigger();
     const int pieces = (row_head(row, p.V) + p.V + kStep - 1) / kStep;
     const Partial *parts = s_part + warp - warp % wpr;
     if (cluster > 1) {
