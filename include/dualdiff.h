@@ -103,8 +103,10 @@ int dd_bidir_attention(const void *q, const void *k, const void *v, void *out,
  *
  * drafter_logits, verifier_logits: [B,P,V] bf16 (drafter_logits may be NULL
  * unless the mode is KL); tokens int32 [B,P]; mask_flags uint8 [B,P];
- * out_tokens int32 [B,P] (may alias tokens); out_mask uint8 [B,P]; out_score
- * fp32 [B,P], nullable.  The streaming path needs 16-byte aligned
+ * out_tokens int32 [B,P] (may alias tokens); out_mask uint8 [B,P], apart from
+ * mask_flags (where the rows are few enough for the row path it may be the same array; in the streaming
+ * path a CTA may look a flag up after the mask of a finished sequence has been written); out_score fp32
+ * [B,P], nullable.  The streaming path needs 16-byte aligned
  * logits (any V); otherwise a slower element-wise path is taken.  Where V is not a multiple of eight,
  * logits of an unflagged position that share a 16-byte block with a flagged one's are loaded and discarded.
  * Supported: P <= 8192; V < 2^31 / 2.

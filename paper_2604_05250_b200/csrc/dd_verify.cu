@@ -343,7 +343,11 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     const bool deep = (groups * shape.cluster <= 2L * sms && (shape.cluster > 1 || pieces >= 3 * shape.wpr)) || rows * pieces > 160L * sms;
     // flagged rows first (mapped_row): a row per CTA, and long ones (all flagged: 1 x 512, 32000, CONF 16.9 : 18.5, 3 x 200, 60000, CONF 23.8 :
     // 24.9, 2 x 300, 32001, KL 28.5 : 28.1)
-    shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24));
+    // Not where the mask is written over the flags: every CTA derives its row from all of them, and would see those of sequences already
+    // decided changed; by its place it reads its own row's only.
+    const uintptr_t flags = (uintptr_t)p.flags, mask = (uintptr_t)p.out_mask;
+    const bool in_place = flags < mask + (size_t)rows && mask < flags + (size_t)rows;
+    shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24)) && !in_place;
     // Early only where every CTA has an SM to itself: CTAs that arrive early pile up on the SMs that are free first, and waiting ones of a second
     // round take up the room of the first one's last.  us, early : ordinary, after attention of 32 heads of 1024: 256 rows of 126464, KL
     // 55.5 : 53.0, 2 x 300 of 32001 42.7 : 39.3, 1 x 100 of 50000, CONF 35.1 : 33.1, 1 x 512 of 32000, CONF 39.2 : 38.3; but 128 of

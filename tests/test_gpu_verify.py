@@ -391,6 +391,23 @@ def test_row_kernel_with_long_rows(dd, oracle_mod, B, P, V, flagged, mode):
     compare(dd, oracle_mod, dra, ver, tokens, flags, mode, 0.5, 9, 3)
 
 
+# more long rows than the GPU holds CTAs of the row kernel at a time: the first sequences are decided before the last rows begin
+@pytest.mark.parametrize("B,P,V,flagged,mode", [(2, 256, 126464, 256, KL), (4, 100, 126464, 60, CONF), (2, 290, 26001, 290, KL | PROB)])
+def test_mask_in_place_of_the_flags(dd, B, P, V, flagged, mode):
+    import torch
+    dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=V + P)
+    dra, ver = to_torch_bf16(dra, "cuda") if (mode & 0xFF) == KL else None, to_torch_bf16(ver, "cuda")
+    tok, fl = torch.from_numpy(tokens).cuda(), torch.from_numpy(flags).cuda()
+    want = dd.verify(dra, ver, tok, fl, mode, 0.5, 9, 3)
+    for _ in range(2):
+        mask = fl.clone()
+        got = dd.verify(dra, ver, tok, mask, mode, 0.5, 9, 3, out_mask=mask)
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+    again = dd.verify(dra, ver, tok, fl, mode, 0.5, 9, 3)         # the counters are as they should be
+    assert all(torch.equal(a, b) for a, b in zip(want, again))
+    assert dd.verify_status() == 0
+
+
 @pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 100, 299, 300, 301])
 def test_minimum_keep_with_many_equal_scores(dd, oracle_mod, k):
     """300 rows of which many are the same: ties at every place of the order, kept lowest index first."""
