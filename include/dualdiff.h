@@ -97,9 +97,9 @@ int dd_bidir_attention(const void *q, const void *k, const void *v, void *out,
  * A logit of -inf is an excluded token (probability 0, an ordinary input: a banned or
  * padded vocabulary entry, the mask token): it contributes no term to Eq. 5 where the
  * drafter excludes it (the sum runs over the support of p_D), and KL_i = +inf where
- * only the verifier does.  In the streaming path that last case is recognised as long
- * as the drafter gives the token at least 3e-35 of the probability mass of its stretch
- * of 4096-8192 logits; below that the token counts as excluded by both.
+ * only the verifier does.  That last case is recognised as long as the drafter gives the
+ * token at least 3e-35 of the probability mass of the logits that are summed together (4096 to 8192 in the
+ * streaming path, up to 20480 in the row path, for V up to a million); below that it counts as excluded by both.
  *
  * drafter_logits, verifier_logits: [B,P,V] bf16 (drafter_logits may be NULL
  * unless the mode is KL); tokens int32 [B,P]; mask_flags uint8 [B,P];

@@ -312,12 +312,35 @@ int launch_stream(const VerifyParams &p, cudaStream_t stream)
 // 29.9; 1 x 32, 126464, KL: 14.2 / 24.2; 1 x 128: 25.9 / 31.9; 16 x 512, 1000, CONF: 23.0 / 38.3.  Beyond the line: 8 x
 // 256, 32000, CONF: 36.6 / 31.7; 1 x 256, 126464, KL: 38.7 / 37.5; 16 x 512, 8000, KL 50 %: 58.4 / 51.1.
 long row_pieces(int V, bool kl) { return ((long)V + 7) / (kl ? kPiece : 2 * kPiece) + 1; }
-// Beyond it, up to two rounds of the deep form (below), which the streaming kernel's fixed cost does not earn back: 1 x 256,
-// 126464, KL 31.6 / 37.0; 1 x 400, KL 100 % 45.1 / 50.7, 50 % 32.6 / 39.5, CONF 28.4 / 38.2, 20.7 / 34.6; 2 x 256, KL 100 % 56.1 /
-// 57.6, 50 % 34.0 / 37.6, 25 % 32.0 / 31.1.
+
+// Warps per row: enough to fill the GPU (24 per SM), but at least two pieces for each.  Few rows: clusters
+// of CTAs, as long as two CTAs per SM hold them all (32 rows of 126464: 27 us with eight warps a row,
+// 14 with clusters of eight; 128 rows: clusters of two 25.9, of four 30.1).
+RowsShape rows_shape(long rows, long pieces, int sms)
+{
+    RowsShape shape = {1, 1, 0};
+    while (shape.wpr < kRWarps && 4 * shape.wpr <= pieces + 1 && rows * shape.wpr < 24L * sms) shape.wpr *= 2;
+    while (shape.wpr == kRWarps && shape.cluster < kRMaxCluster && 4 * kRWarps * shape.cluster <= pieces + 1 &&
+           2 * shape.cluster * rows <= 2L * sms)
+        shape.cluster *= 2;
+    return shape;
+}
+
+// Beyond 160 pieces per SM, up to four rows per SM of no more than kLongShare pieces a warp: the deep form (below), in whose two rounds
+// or so the streaming kernel's fixed cost is not earned back.  us, row : streaming: 1 x 256, 126464, KL 31.6 : 37.0; 1 x 400, KL 100 % 45.1 :
+// 50.7, 50 % 32.6 : 39.5, CONF 28.4 : 38.2, 20.7 : 34.6; 2 x 256, KL 100 % 56.1 : 57.6, 50 % 34.0 : 37.6, 25 % 32.0 : 31.1, but 80 %, where
+// some SMs have a third row, 57.0 : 50.0.  A row is one CTA's, so that an SM with one row more costs the more, the
+// longer the rows: KL, 2 x 75 rows of 180000 (22 pieces a warp) the same, 2 x 100 of 262144 (32) 54 : 52, 2 x 75 of 524288 92 : 70;
+// CONF, 2 x 128 of 262144 (16) 1.26 times as fast, 2 x 150 of 330000 (20) 0.91 to 1.0, of 524288 0.86.  The bound also
+// keeps a warp's sums short, and the places of its maxima far from the 2048 pieces (KL: 4096) that LaneState counts: below the line of 160
+// a warp has at most 160 / 64 per SM (one row in a cluster of eight).
+constexpr long kLongShare = 20;
 bool rows_path(int V, long rows, int sms, bool kl)
 {
-    return (rows * row_pieces(V, kl) <= 160L * sms && rows <= 32L * 1024) || rows <= 4L * sms;
+    const long pieces = row_pieces(V, kl);
+    if (rows * pieces <= 160L * sms && rows <= 32L * 1024) return true;
+    const RowsShape shape = rows_shape(rows, pieces, sms);
+    return rows <= 4L * sms && pieces <= kLongShare * shape.wpr * shape.cluster;
 }
 
 template <bool KL>
@@ -327,14 +350,7 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     if (sms < 0) return sms;
     const long rows = (long)p.B * p.P;
     const long pieces = row_pieces(p.V, KL);
-    // Warps per row: enough to fill the GPU (24 per SM), but at least two pieces for each.  Few rows: clusters
-    // of CTAs, as long as two CTAs per SM hold them all (32 rows of 126464: 27 us with eight warps a row,
-    // 14 with clusters of eight; 128 rows: clusters of two 25.9, of four 30.1).
-    RowsShape shape = {1, 1, 0};
-    while (shape.wpr < kRWarps && 4 * shape.wpr <= pieces + 1 && rows * shape.wpr < 24L * sms) shape.wpr *= 2;
-    while (shape.wpr == kRWarps && shape.cluster < kRMaxCluster && 4 * kRWarps * shape.cluster <= pieces + 1 &&
-           2 * shape.cluster * rows <= 2L * sms)
-        shape.cluster *= 2;
+    RowsShape shape = rows_shape(rows, pieces, sms);
     const long groups = (rows + kRWarps / shape.wpr - 1) / (kRWarps / shape.wpr);
     // Two CTAs per SM and deep loads (row_part_deep), where all CTAs fit at once and a warp has a few pieces, or rows are few and long;
     // with more rows a third CTA per SM is worth more than deep loads.  us, three CTAs : deep (B x P, V): 1 x 256, 126464, KL 36.8 : 29.9; 1 x 128

@@ -134,7 +134,7 @@ constexpr float kExcludedExcess = 1e4f;
 
 struct LaneState {
     uint32_t max2_v;           // packed bf16x2 running maxima of the verifier (even / odd logits of the lane's words)
-    uint32_t where2_v;         // per half: ordinal of the word that first attained that maximum
+    uint32_t where2_v;         // per half: ordinal of the word that first attained that maximum: 16 bits, 2048 pieces (KL: 4096)
     uint32_t max2_d;           // drafter: packed maxima of the lane's first piece (its reference point)
     float M_v, M_d;            // reference points: maximum of the lane's first piece * log2e
     float2 s_v, s_d, t;        // sums of the even / odd logits

@@ -408,6 +408,28 @@ def test_mask_in_place_of_the_flags(dd, B, P, V, flagged, mode):
     assert dd.verify_status() == 0
 
 
+# lengths at the lines between the row kernel and the streaming kernel on 148 SMs (one row: 23680 pieces; 150 and 40 rows: 20 pieces for each of
+# eight and thirty-two warps), and far beyond what a warp of the row kernel could count
+@pytest.mark.parametrize("P,V,mode", [
+    (1, 48_490_000, CONF), (1, 48_500_000, CONF), (1, 300_000_001, CONF), (1, 24_240_000, KL), (1, 24_250_000, KL), (1, 300_000_000, KL),
+    (150, 327_000, CONF), (150, 328_000, CONF), (150, 163_000, KL), (150, 164_000, KL), (40, 654_000, KL), (40, 656_000, KL)])
+def test_place_of_the_maximum_of_very_long_rows(dd, P, V, mode):
+    import torch
+    ver = torch.zeros(1, P, V, dtype=torch.bfloat16, device="cuda")
+    places = [V - 5 if r == P - 1 else V * (r + 1) // P - 1 for r in range(P)]
+    ver[0, torch.arange(P), torch.tensor(places)] = 8.0
+    tok, fl = torch.zeros(1, P, dtype=torch.int32, device="cuda"), torch.ones(1, P, dtype=torch.uint8, device="cuda")
+    # (KL: of the constant distribution from this one)
+    dra = torch.zeros_like(ver) if mode == KL else None
+    got = dd.verify(dra, ver, tok, fl, mode, 100.0 if mode == KL else 0.0, 0, 0)
+    assert got[0].cpu().tolist() == [places] and not got[1].any()
+    total = np.exp(8.0) + V - 1
+    want = -8.0 / V - np.log(V) + np.log(total) if mode == KL else np.exp(8.0) / total
+    # KL is a difference of numbers of the size of log V, which come from fp32 sums
+    assert np.abs(got[2].cpu().numpy() - want).max() <= (1e-5 * np.log(V) if mode == KL else 1e-4 * want)
+    assert dd.verify_status() == 0
+
+
 @pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 100, 299, 300, 301])
 def test_minimum_keep_with_many_equal_scores(dd, oracle_mod, k):
     """300 rows of which many are the same: ties at every place of the order, kept lowest index first."""
