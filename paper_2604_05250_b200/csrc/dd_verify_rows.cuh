@@ -49,8 +49,12 @@ constexpr float kLowestLogit = -3.38e38f;        // (bf16's lowest finite is -3.
 // A piece: lane_pass1 and lane_pass2 in one, for registers that are all filled.  Logits are not raised to finite ones beforehand, which
 // only excluded tokens (-inf) need: their terms of T come out as NaN or infinity, and then the lane computes the piece's
 // terms again that way.
+// A warp's share of a row is up to kLongShare pieces, twice a chunk of the streaming kernel and more, and its sums must not be less
+// exact for that.  KL: a piece is summed by itself and added to the lane's sums.  Else the chains are sum_v, which the pieces use in turn: half of
+// them go through the caller's second one (adding each piece's sum cost 3 to 14 % there).  256 rows of 126464, mean error of KL relative
+// to 64 bits 5.6e-8 as one chain, 4.3e-8 so and in the streaming kernel; no difference in time.
 template <bool KL>
-__device__ __forceinline__ void lane_piece(LaneState &L, const uint4 (&rv)[kVecPerThread], const uint4 (&rd)[kVecPerThread], int ordinal, bool first)
+__device__ __forceinline__ void lane_piece(LaneState &L, float2 &sum_v, const uint4 (&rv)[kVecPerThread], const uint4 (&rd)[kVecPerThread], int ordinal, bool first)
 {
     lane_pass1<KL>(L, rv, rd, ordinal, first);
     if (first) {
@@ -60,7 +64,8 @@ __device__ __forceinline__ void lane_piece(LaneState &L, const uint4 (&rv)[kVecP
     }
     const float2 log2e2 = make_float2(kLog2e, kLog2e), neg1 = make_float2(-1.f, -1.f);
     const float2 nMv2 = make_float2(-L.M_v, -L.M_v), nMd2 = make_float2(-L.M_d, -L.M_d);
-    float2 s_v = L.s_v, s_d = L.s_d, t = L.t;
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 s_v = KL ? zero : sum_v, s_d = zero, t = zero;
 #pragma unroll
     for (int j = 0; j < (KL ? 1 : 2) * kVecPerThread; ++j) {
         const uint4 &x = j < kVecPerThread ? rv[j] : rd[j - kVecPerThread];
@@ -83,7 +88,7 @@ __device__ __forceinline__ void lane_piece(LaneState &L, const uint4 (&rv)[kVecP
     if (KL && !isfinite(t.x + t.y)) {
         // Both logits raised to the lowest finite one: a token that the drafter excludes adds an exact 0, one that only the verifier
         // excludes e * 3.4e38 (kExcludedExcess).
-        t = L.t;
+        t = zero;
 #pragma unroll 1
         for (int j = 0; j < kVecPerThread; ++j) {
             uint4 v = rv[0], d = rd[0];
@@ -100,7 +105,13 @@ __device__ __forceinline__ void lane_piece(LaneState &L, const uint4 (&rv)[kVecP
             }
         }
     }
-    L.s_v = s_v; L.s_d = s_d; L.t = t;
+    if (KL) {
+        L.s_v = __fadd2_rn(L.s_v, s_v);
+        L.s_d = __fadd2_rn(L.s_d, s_d);
+        L.t = __fadd2_rn(L.t, t);
+    } else {
+        sum_v = s_v;
+    }
 }
 
 // The part of a row that one warp takes: the pieces at x0, x0 + stride, ... (logits, counted from the row's first vector), from
@@ -244,13 +255,14 @@ __device__ __forceinline__ Partial row_part_deep(const VerifyParams &p, int row,
             trim(rd[j], dra, lane + 32 * (KL ? j : kVecPerThread + j));
         }
     };
+    float2 second = make_float2(0.f, 0.f);               // the other chain (lane_piece)
     uint4 av[kVecPerThread], ad[kVecPerThread];
 #pragma unroll
     for (int j = 0; j < kVecPerThread; ++j) av[j] = ad[j] = make_uint4(0u, 0u, 0u, 0u);
     int x = x0, ordinal = 0;
     auto edge = [&] {
         load_edge(av, ad, x);
-        lane_piece<KL>(L, av, ad, ordinal, ordinal == 0);
+        lane_piece<KL>(L, L.s_v, av, ad, ordinal, ordinal == 0);
         x += stride;
         ++ordinal;
     };
@@ -265,17 +277,18 @@ __device__ __forceinline__ Partial row_part_deep(const VerifyParams &p, int row,
         for (;;) {
             x += stride;
             load_full(bv, bd, x, full(x));
-            lane_piece<KL>(L, av, ad, ordinal, ordinal == 0);
+            lane_piece<KL>(L, L.s_v, av, ad, ordinal, ordinal == 0);
             ++ordinal;
             if (!full(x)) break;
             x += stride;
             load_full(av, ad, x, full(x));
-            lane_piece<KL>(L, bv, bd, ordinal, false);
+            lane_piece<KL>(L, second, bv, bd, ordinal, false);
             ++ordinal;
             if (!full(x)) break;
         }
     }
     if (x < extent) edge();
+    if (!KL) L.s_v = __fadd2_rn(L.s_v, second);
     Partial part = lanes_to_partial<KL>(L, x0 - head, lane, stride);
     if (x0 < extent &&
         (!(isfinite(part.s_v) && isfinite(part.s_d) && isfinite(part.t) && part.m_v > kLowestLogit) ||

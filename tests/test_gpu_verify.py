@@ -408,6 +408,29 @@ def test_mask_in_place_of_the_flags(dd, B, P, V, flagged, mode):
     assert dd.verify_status() == 0
 
 
+@pytest.mark.parametrize("B,P,V,mode", [(1, 256, 126464, KL), (1, 256, 126464, CONF), (2, 200, 126464, KL), (2, 200, 126464, CONF),
+                                        (4, 200, 126464, KL), (4, 200, 126464, CONF)])
+def test_long_sums_are_as_exact_as_short_ones(dd, B, P, V, mode):
+    """Terms of 2^-8.8 added to sums that begin at 1: every addition rounds down.  A chain of 128 additions (a lane's half of a chunk of 8192
+    logits) is out by no more than 128 * 2^-24; one over a warp's share of a row in the row kernel would be out by 9.6e-6."""
+    import torch
+    row = torch.full((V,), -6.09375, dtype=torch.float64)
+    step = 1024 if mode == KL else 2048
+    for piece in range(8):                       # each lane's first word, in each warp's first piece of the row kernel
+        first = piece * step + 8 * torch.arange(32)
+        row[first] = row[first + 1] = 0.0
+    ver = row.to(torch.bfloat16).cuda().expand(B, P, V).contiguous()
+    dra = torch.zeros_like(ver) if mode == KL else None          # all terms of its sums are exact
+    tok, fl = torch.zeros(B, P, dtype=torch.int32, device="cuda"), torch.ones(B, P, dtype=torch.uint8, device="cuda")
+    got = dd.verify(dra, ver, tok, fl, mode, 0.5, 0, 0)[2].double()
+    bound = 128 * 2.0 ** -24
+    lse = torch.logsumexp(row, 0).item()
+    # the logarithm of the sum has the sum's relative error as its absolute one
+    want, tol = (lse - np.log(V) - row.mean().item(), bound) if mode == KL else (np.exp(-lse), bound * np.exp(-lse))
+    assert (got - want).abs().max().item() <= tol
+    assert dd.verify_status() == 0
+
+
 # lengths at the lines between the row kernel and the streaming kernel on 148 SMs (one row: 23680 pieces; 150 and 40 rows: 20 pieces for each of
 # eight and thirty-two warps), and far beyond what a warp of the row kernel could count
 @pytest.mark.parametrize("P,V,mode", [
