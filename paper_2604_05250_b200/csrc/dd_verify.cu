@@ -356,7 +356,12 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     // with more rows a third CTA per SM is worth more than deep loads.  us, three CTAs : deep (B x P, V): 1 x 256, 126464, KL 36.8 : 29.9; 1 x 128
     // 23.9 : 20.4; 1 x 32 14.1 : 12.8; 1 x 200, 50000, KL 19.9 : 18.2; but 1 x 256, 16000, KL 11.8 : 12.0, 1 x 256, 16001, CONF 8.8 : 9.6; 2 x 300,
     // 32001, KL 50 % 19.9 : 22.0; 4 x 256, 8000, KL 50 % 13.4 : 16.8; 16 x 512, 1000, CONF 17.8 : 22.4.
-    const bool deep = (groups * shape.cluster <= 2L * sms && (shape.cluster > 1 || pieces >= 3 * shape.wpr)) || rows * pieces > 160L * sms;
+    // Not with too few pieces a warp for its start to be earned back (pieces a warp, us three CTAs : deep): where every CTA has an SM, CONF: 3.1,
+    // 1 x 36, 49203 11.8 : 12.7, 4 x 37 13.4 : 14.7 (KL 4 x 25, 24576 the same); clusters of four, two CTAs on an SM: 2.0, 4 x 18, 64000, KL
+    // 15.3 : 17.0, 2.5, 80000 16.8 : 18.4, 3.1, 100001 18.8 : 20.9, 3.9, 126464 20.8 : 20.9 (of two: 2.8, 4 x 37, 45000 16.0 : 15.0).
+    const long ctas = groups * shape.cluster;
+    const int least2 = shape.cluster == 1 ? (KL || ctas > sms ? 6 : 7) : shape.cluster >= 4 && ctas > sms ? 7 : 0;
+    const bool deep = (ctas <= 2L * sms && 2 * pieces >= least2 * shape.wpr * shape.cluster) || rows * pieces > 160L * sms;
     // flagged rows first (mapped_row): a row per CTA, and long ones (all flagged: 1 x 512, 32000, CONF 16.9 : 18.5, 3 x 200, 60000, CONF 23.8 :
     // 24.9, 2 x 300, 32001, KL 28.5 : 28.1)
     // Not where the mask is written over the flags: every CTA derives its row from all of them, and would see those of sequences already
@@ -368,8 +373,8 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     // round take up the room of the first one's last.  us, early : ordinary, after attention of 32 heads of 1024: 256 rows of 126464, KL
     // 55.5 : 53.0, 2 x 300 of 32001 42.7 : 39.3, 1 x 100 of 50000, CONF 35.1 : 33.1, 1 x 512 of 32000, CONF 39.2 : 38.3; but 128 of
     // 1024, KL 27.1 : 28.4, 64 of 1000 27.9 : 28.5.  One after the other, 1024 of 4000, KL 19.4 : 18.7.
-    const bool early = !deep && groups * shape.cluster <= sms;
-    DD_CUDA_TRY(dd::launch_as(early, deep ? verify_rows_kernel<KL, true> : verify_rows_kernel<KL, false>, (unsigned)(groups * shape.cluster),
+    const bool early = !deep && ctas <= sms;
+    DD_CUDA_TRY(dd::launch_as(early, deep ? verify_rows_kernel<KL, true> : verify_rows_kernel<KL, false>, (unsigned)ctas,
                               32 * kRWarps, 0, stream, shape.cluster, p, shape));
     dd::count_launch();
     return DD_OK;
