@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kFoldThreads) lm_head_fold_kernel(const __grid
         float score;
         int argmax;
         const int n_tiles = q.plan ? q.plan->n_tiles : q.all_rows.n_tiles;
-        ddv::fold_partials<KL>(p.partials + ddv::checked_run(p, (long)w * n_tiles, n_tiles, (long)rows * n_tiles, ddv::kSitePartial),
+        ddv::fold_partials<KL, true>(p.partials + ddv::checked_run(p, (long)w * n_tiles, n_tiles, (long)rows * n_tiles, ddv::kSitePartial),
                                n_tiles, score, argmax);
         if ((threadIdx.x & 31) == 0) {
             const size_t row_at = ddv::checked(p, w, (long)p.B * p.P, ddv::kSiteRow);

@@ -274,15 +274,17 @@ __device__ __forceinline__ float4 ld_volatile16(const void *ptr)
 
 // Folds n chunk partials of one row, in chunk order, in fp64 (warp-level; src may point to
 // shared or global memory).  Every lane returns the row's score (KL_i of Eq. 5, or c_i of
-// Eq. 7) and the lowest index of the verifier's maximum.
-template <bool KL>
+// Eq. 7) and the lowest index of the verifier's maximum.  kNarrow: the row kernel's and the fused head's form, cold at the end of
+// a call and often of a few partials: little code, and an exchange among as many lanes as there are partials.  The streaming kernel has
+// rehearsed it and folds rows while it streams: unrolled (of some 900 drawn shapes the slowest twentieth lost 2.6 % to the short form, 2.0 % so).
+template <bool KL, bool kNarrow = false>
 __device__ __noinline__ void fold_partials(const Partial *src, int n, float &score, int &argmax)
 {
     const int lane = threadIdx.x & 31;
     float bm_v = -INFINITY, bm_d = -INFINITY;
     int bidx = 0x7FFFFFFF;
     // up to 16 partials: every `width` lanes take all of them, and as many steps of the exchange are left out
-    const int width = n > 16 ? 32 : n <= 1 ? 1 : 2 << (31 - __clz(n - 1)), ch0 = lane & (width - 1);
+    const int width = !kNarrow || n > 16 ? 32 : n <= 1 ? 1 : 2 << (31 - __clz(n - 1)), ch0 = lane & (width - 1);
     for (int ch = ch0; ch < n; ch += width) {
         const float4 a = ld_volatile16(src + ch);
         const float mv = a.x, md = a.w;
@@ -290,7 +292,7 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
         if (mv > bm_v || (mv == bm_v && ix < bidx)) { bm_v = mv; bidx = ix; }
         bm_d = fmaxf(bm_d, md);
     }
-#pragma unroll 1
+#pragma unroll (kNarrow ? 1 : 5)
     for (int o = width >> 1; o > 0; o >>= 1) {
         const float om = __shfl_xor_sync(0xFFFFFFFFu, bm_v, o);
         const int oi = __shfl_xor_sync(0xFFFFFFFFu, bidx, o);
@@ -314,7 +316,7 @@ __device__ __noinline__ void fold_partials(const Partial *src, int n, float &sco
             tt += (double)bq.y * f;
         }
     }
-#pragma unroll 1
+#pragma unroll (kNarrow ? 1 : 5)
     for (int o = width >> 1; o > 0; o >>= 1) {
         sv += __shfl_xor_sync(0xFFFFFFFFu, sv, o);
         if (KL) {

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(32 * kRWarps, kDeep ? 2 : 3) verify_rows_kerne
     if (mine && warp % wpr == 0) {
         float score;
         int argmax;
-        fold_partials<KL>(parts, min(cluster * wpr, pieces), score, argmax);
+        fold_partials<KL, true>(parts, min(cluster * wpr, pieces), score, argmax);
         if (lane == 0) {
             __stcg(p.row_score + row, score);
             __stcg(p.row_argmax + row, argmax);
