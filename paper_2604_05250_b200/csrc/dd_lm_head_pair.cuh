@@ -44,24 +44,21 @@ struct PairWalk {
     {
         n_tiles = plan.n_tiles;
         blocks = KL ? (plan.n_rows + kRowsPerItem - 1) / kRowsPerItem : (plan.n_rows + kRowsPerItem - 1) / (2 * kRowsPerItem);
-        per_group = KL ? blocks : 2 * blocks + (plan.n_rows > blocks * 2 * kRowsPerItem);
-        n_items = (n_tiles + 1) / 2 * per_group;
+        const int rest = !KL && plan.n_rows > blocks * 2 * kRowsPerItem;
+        per_group = KL ? blocks : 2 * blocks + rest;
+        // (KL: an item with the last of an odd number of tiles has one to reduce; else the last tile alone has an item per block)
+        n_items = KL ? (n_tiles + 1) / 2 * blocks : n_tiles / 2 * per_group + (n_tiles & 1) * (blocks + rest);
         item = (int)blockIdx.x >> 1;
         step = (int)gridDim.x >> 1;
         set();
     }
     __device__ __forceinline__ void set()
     {
-#pragma unroll 1
-        for (; item < n_items; item += step) {
-            const int group = item / per_group;
-            int k = item - group * per_group;
-            tile = 2 * group;
-            wide = KL || k == 2 * blocks;
-            row0 = (wide && !KL ? blocks : k >= blocks ? k - blocks : k) * (KL ? 1 : 2) * kRowsPerItem;
-            if (!wide && k >= blocks) ++tile;
-            if (tile < n_tiles) break;             // an odd number of tiles: the last group has one
-        }
+        const int group = item / max(per_group, 1), k = item - group * per_group;
+        const int tiles = KL ? 2 : min(2, n_tiles - 2 * group);        // in this group
+        wide = KL || k == tiles * blocks;
+        tile = 2 * group + (!wide && k >= blocks);
+        row0 = (wide && !KL ? blocks : k >= blocks ? k - blocks : k) * (KL ? 1 : 2) * kRowsPerItem;
     }
     __device__ __forceinline__ bool valid() const { return item < n_items; }
     __device__ __forceinline__ void next() { item += step; set(); }
