@@ -156,11 +156,12 @@ int dd_unmask(const void *logits, const int32_t *tokens, const uint8_t *mask_fla
  * output embedding of token x); all contiguous, K innermost, 16-byte aligned, the same K for both
  * models.  The other arguments, outputs, scratch and errors are dd_verify's.  The hidden states of
  * positions with mask_flags == 0 may be read (they share tiles with their neighbours) but nothing is
- * computed from them.  Three kernels per call, in stream order: a small one that gathers the flagged
- * rows where that saves products, the products with their per-tile reductions, and a small one that
+ * computed from them.  Two to four kernels per call, in stream order: a small one that gathers the flagged
+ * rows where that saves products, the products with their per-tile reductions (two kernels of which the number
+ * of flagged rows lets one work, where that pays), and a small one that
  * combines the tiles of every row and decides the sequences.  Scratch: 32 bytes for each row and vocabulary
- * tile, of 128 entries (KL: 64) at the narrowest; where that is more than a quarter of the free memory, for the tiles picked where
- * every row is multiplied, of 128 to 256 (64 to 128).  And a copy of the hidden states as large as they are (KL: both
+ * tile, of 128 entries (KL: 64) at the narrowest, or down to 32 where wider ones leave SMs idle; where that is more than a
+ * quarter of the free memory, for the tiles picked where every row is multiplied.  And a copy of the hidden states as large as they are (KL: both
  * models'), without which every row is multiplied; it is not allocated beyond a quarter of the free memory, nor while
  * `stream` is captured.
  * Supported: K a multiple of 64; any V >= 1; P <= 8192.

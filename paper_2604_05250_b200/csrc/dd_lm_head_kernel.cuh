@@ -74,18 +74,19 @@ struct Widths {
     static constexpr int count = max_n / 32;
 };
 
-// What the first kernel finds out, for the two behind it.
+// What the first kernel finds out, for those behind it.
 struct LmPlan {
     int n_rows;                // rows to multiply: the flagged ones, or all of them where that costs no more
     int gathered;              // 1: their hidden states stand one after the other in the scratch
     int N;                     // vocabulary entries per work item
     int n_tiles;               // ceil(V / N): the "chunks" of a row
+    int pairs;                 // 1: lm_head_pair_kernel multiplies, 0: lm_head_kernel
 };
 
 struct LmParams {
     int rows, K, V;            // rows = B * P
     int ctas;                  // CTAs the tile width is chosen for
-    int pairs;                 // 1: the products are lm_head_pair_kernel's
+    int pairs;                 // 0: the products are lm_head_kernel's, 2: lm_head_pair_kernel's, 1: of more than 128 rows
     int min_n;                 // the narrowest width the scratch has partials for
     int rows_per_block;        // rows that a block of the first kernel copies: a multiple of kRowsWarps
     LmPlan *plan;              // null: nothing is gathered, the plan is all_rows and the first kernel is not launched
@@ -133,7 +134,8 @@ __host__ __device__ inline LmPlan plan_for(const LmParams &q, int n_rows, bool g
     LmPlan plan;
     plan.n_rows = n_rows;
     plan.gathered = gathered;
-    plan.N = pick_tile_n<KL>(q.V, n_rows, q.ctas, q.min_n, q.pairs != 0);
+    plan.pairs = q.pairs == 2 || (q.pairs == 1 && n_rows > kTileRows);
+    plan.N = pick_tile_n<KL>(q.V, n_rows, q.ctas, q.min_n, plan.pairs != 0);
     plan.n_tiles = (q.V + plan.N - 1) / plan.N;
     return plan;
 }
@@ -177,7 +179,7 @@ lm_head_rows_kernel(const LmParams q, const ddv::VerifyParams p, const uint4 *hi
     if (lane == 0) { atomicAdd(&s_before, before); atomicAdd(&s_all, all); }
     __syncthreads();
     all = s_all;
-    const int unit = q.pairs ? kRowsPerItem : kTileRows;           // rows that cost as much as one
+    const int unit = q.pairs == 2 || (q.pairs == 1 && all > kTileRows) ? kRowsPerItem : kTileRows;           // rows that cost as much as one
     const bool gather = (all + unit - 1) / unit < (q.rows + unit - 1) / unit &&
                         (q.all_rows.n_tiles > 2 || 3L * all < (long)q.rows * q.all_rows.n_tiles);
     if (blockIdx.x == 0 && tid == 0) *q.plan = plan_for<KL>(q, gather ? all : q.rows, gather);
@@ -404,6 +406,11 @@ template <bool KL>
 __global__ void __launch_bounds__(kThreads, 1)
 lm_head_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const ddv::VerifyParams p)
 {
+    // the rows' kernel may have left the products to lm_head_pair_kernel
+    if (q.pairs == 1) {
+        grid_wait();
+        if (q.plan->pairs) return;
+    }
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;     // swizzled tiles: 1024-byte aligned
     unsigned char *smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));

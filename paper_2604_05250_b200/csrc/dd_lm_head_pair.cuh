@@ -68,6 +68,11 @@ template <bool KL>
 __global__ void __launch_bounds__(kThreads, 1)
 lm_head_pair_kernel(const __grid_constant__ LmMaps<KL> maps, const LmParams q, const ddv::VerifyParams p)
 {
+    // ... or to lm_head_kernel (the same answer in both CTAs)
+    if (q.pairs == 1) {
+        grid_wait();
+        if (!q.plan->pairs) return;
+    }
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;     // the same in both CTAs
     unsigned char *smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));

@@ -593,13 +593,21 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
         if ((rc = make_matrix_tmap(&m.hd, dh, q.rows, q.K, kTileRows)) != DD_OK) return rc;
         if ((rc = make_matrix_tmap(&m.hd_gathered, gathered + gathered_bytes, q.rows, q.K, kTileRows)) != DD_OK) return rc;
     }
-    // a map per width that the device may choose; one where the host has chosen
-    for (int i = 0; i < Widths<KL>::count; ++i) {
-        if (q.plan ? Widths<KL>::max_n - 32 * i < q.min_n : Widths<KL>::max_n - 32 * i != q.all_rows.N) continue;
-        const int width = Widths<KL>::max_n - 32 * i, box = q.pairs && !KL ? width / 2 : width;      // what one CTA loads at a time
-        if ((rc = make_matrix_tmap(&m.w[i], vw, q.V, q.K, box)) != DD_OK) return rc;
-        if (KL && (rc = make_matrix_tmap(&m.wd[i], dw, q.V, q.K, box)) != DD_OK) return rc;
-    }
+    // a map per width that the device may choose; one where the host has chosen.  `part`: what one CTA loads at a time is N / part
+    auto weight_maps = [&](LmMaps<KL> &to, int part) {
+        for (int i = 0; i < Widths<KL>::count; ++i) {
+            const int width = Widths<KL>::max_n - 32 * i;
+            if (q.plan ? width < q.min_n : width != q.all_rows.N) continue;
+            if ((rc = make_matrix_tmap(&to.w[i], vw, q.V, q.K, width / part)) != DD_OK) return rc;
+            if (KL && (rc = make_matrix_tmap(&to.wd[i], dw, q.V, q.K, width / part)) != DD_OK) return rc;
+        }
+        return (int)DD_OK;
+    };
+    const bool single = q.pairs < 2, pairs = q.pairs > 0;          // both: the number of rows to be multiplied decides which of them works
+    LmMaps<KL> m2 = m;                                 // lm_head_pair_kernel's
+    if (single && (rc = weight_maps(m, 1)) != DD_OK) return rc;
+    if (pairs && KL && single) m2 = m;
+    else if (pairs && (rc = weight_maps(m2, KL ? 1 : 2)) != DD_OK) return rc;
     // One CTA per SM, fewer if even the narrowest tiles of all rows do not make that many items.
     const long items = (long)((q.V + q.min_n - 1) / q.min_n) * ((q.rows + kRowsPerItem - 1) / kRowsPerItem);
     const unsigned grid = (unsigned)(items < ctas ? items : ctas);
@@ -609,12 +617,12 @@ int launch_lm_head(ddlm::LmParams q, VerifyParams p, const void *dh, const void 
                                q, p, static_cast<const uint4 *>(vh), reinterpret_cast<uint4 *>(gathered),
                                static_cast<const uint4 *>(dh), reinterpret_cast<uint4 *>(gathered + gathered_bytes)));
     }
-    if (q.pairs) DD_CUDA_TRY(dd::launch(lm_head_pair_kernel<KL>, grid + (grid & 1), ddlm::kThreads, kSmemBytes, stream, 2, m, q, p));
-    else DD_CUDA_TRY(dd::launch(lm_head_kernel<KL>, grid, ddlm::kThreads, kSmemBytes, stream, 1, m, q, p));
+    if (pairs) DD_CUDA_TRY(dd::launch(lm_head_pair_kernel<KL>, grid + (grid & 1), ddlm::kThreads, kSmemBytes, stream, 2, m2, q, p));
+    if (single) DD_CUDA_TRY(dd::launch(lm_head_kernel<KL>, grid, ddlm::kThreads, kSmemBytes, stream, 1, m, q, p));
     // one warp per row
     const unsigned fold_grid = (unsigned)(((long)q.rows + kFoldThreads / 32 - 1) / (kFoldThreads / 32));
     DD_CUDA_TRY(dd::launch(lm_head_fold_kernel<KL>, fold_grid, kFoldThreads, 0, stream, 1, p, q));
-    dd::count_launch(q.plan ? 3 : 2);
+    dd::count_launch(1 + (q.plan ? 1 : 0) + (pairs ? 1 : 0) + (single ? 1 : 0));
     return DD_OK;
 }
 
@@ -696,7 +704,7 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     ddlm::LmParams q;
     q.rows = (int)rows; q.K = K; q.V = V;
     q.min_n = min_n;
-    q.pairs = pairs;
+    q.pairs = pairs ? 2 : 0;
     q.ctas = sms;
     q.plan = nullptr;
     q.all_rows = kl ? ddlm::plan_for<true>(q, q.rows, false) : ddlm::plan_for<false>(q, q.rows, false);
@@ -707,6 +715,12 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     if (gathering_can_pay(q, kl) &&
         dd::try_bytes(&ctx->head_ws, &ctx->head_ws_bytes, (kl ? 2 : 1) * gathered_bytes, (cudaStream_t)stream) == DD_OK)
         q.plan = (ddlm::LmPlan *)(control + kPlanOffset);
+    // Of more rows than one tile the flagged ones may fit one, and half of a pair's products are then with padding: with more than two rounds of tiles (KL)
+    // the device chooses the kernel, and the other one finds nothing to do (1.6 us).  us, pairs : single CTAs (flagged of rows, K, V): KL,
+    // 107 of 180, 576, 79839 74.0 : 58.0, 76 of 324, 512, 46208 51.1 : 38.9, 100 of 1060, 2560, 91072 218 : 180; others 42 of 266, 3648, 107112
+    // 165 : 143, 45 of 513, 3520, 54830 95.4 : 85.2.  With less to read pairs are the faster ones all the same (KL, 54 of 216, 2880, 16960 53.7 : 62.9, 118 of
+    // 189, 2624, 13376 43.9 : 53.9; others 115 of 184, 3008, 31232 50.7 : 53.5), or the second launch costs as much as it gains.
+    if (q.pairs && q.plan && (long)V > 256L * sms) q.pairs = 1;
     q.row_map = p.row_argmax;
     char *gathered = (char *)ctx->head_ws;
     return kl ? launch_lm_head<true>(q, p, drafter_hidden, drafter_weight, verifier_hidden, verifier_weight, gathered,

@@ -108,6 +108,37 @@ def test_pairs_of_ctas_verifier_only(dd, oracle_mod, P, K, V, flagged):
     compare(dd, oracle_mod, hidden, weight, tokens, flags, CONF | PROB, 0.05, 9, 11)
 
 
+@pytest.mark.parametrize("mode,K", [(KL, 64), (CONF, 2048)])
+@pytest.mark.parametrize("P,flagged", [(300, [128]), (300, [129]), (129, [0, 1, 129]), (520, [520, 1])])
+def test_kernel_chosen_on_the_device(dd, mode, K, P, flagged):
+    """Vocabularies of more than 37888 entries (148 SMs): up to 128 flagged rows by single CTAs, more in pairs, one call after the other.  A row's result does
+    not depend on the other rows' flags, nor on which kernel multiplied it."""
+    import torch
+    V = 38000
+    gen = torch.Generator(device="cuda").manual_seed(P)
+    vh, vw, dh, dw = (torch.randn(n, K, device="cuda", generator=gen).mul_(s).to(torch.bfloat16)
+                      for n, s in ((P, 1.0), (V, 2.0 / K ** 0.5), (P, 1.0), (V, 2.0 / K ** 0.5)))
+    vh, dh = vh[None], dh[None]
+    d = (dh, dw) if mode == KL else (None, None)
+    tok = torch.zeros(1, P, dtype=torch.int32, device="cuda")
+    logits = vh[0].double() @ vw.double().T
+    lv = torch.log_softmax(logits, -1)
+    if mode == KL:
+        ld = torch.log_softmax(dh[0].double() @ dw.double().T, -1)
+        want = (ld.exp() * (ld - lv)).sum(-1)
+    else:
+        want = lv.max(-1).values.exp()
+    top = logits.topk(2, -1)
+    clear = top.values[:, 0] - top.values[:, 1] > TOP2_GAP
+    for n in flagged:
+        on = torch.randperm(P, device="cuda", generator=gen) < n
+        got = dd.lm_head_verify(*d, vh, vw, tok, on[None].to(torch.uint8), mode, 1e9 if mode == KL else 0.0, 0, 0)
+        assert dd.verify_status() == 0
+        tol = KL_SCORE_ABS if mode == KL else 1e-4 * want.max().item()
+        assert (got[2][0].double() - want)[on].abs().max().item() <= tol if n else not got[2].any()
+        assert torch.equal(got[0][0][on & clear], top.indices[:, 0].int()[on & clear]) and not got[0][0][~on].any() and not got[1].any()
+
+
 @pytest.mark.parametrize("P", [700, 1100, 2100])
 def test_long_sequences(dd, oracle_mod, P):
     """Sequences longer than the register-resident decision stage holds (512 positions), longer
