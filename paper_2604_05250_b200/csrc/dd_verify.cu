@@ -680,7 +680,9 @@ extern "C" int dd_lm_head_verify(const void *drafter_hidden, const void *drafter
     if ((rc = dd::ensure_mirror(ctx)) != DD_OK) return rc;
     if ((rc = dd::check_mirror(ctx, 1)) != DD_OK) return rc;
     if (dd::try_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)), (cudaStream_t)stream) != DD_OK) {
-        // no room for the narrowest: no narrower than what is picked where every row is multiplied
+        // no room for the narrowest, or none may be made: of half the widest at least, and no narrower than what is picked where every row is
+        // multiplied
+        min_n = std::max(min_n, max_n / 2);
         min_n = kl ? ddlm::pick_tile_n<true>(V, rows, sms, min_n, pairs) : ddlm::pick_tile_n<false>(V, rows, sms, min_n, pairs);
         rc = dd::ensure_bytes(&ctx->verify_ws, &ctx->verify_ws_bytes, workspace_bytes(B, P, tiles_of(min_n)));
         if (rc != DD_OK) return rc;

@@ -310,6 +310,34 @@ def test_without_room_for_the_gathered_rows(dd):
     assert dd.verify_status() == 0
 
 
+def test_captured_with_the_scratch_of_a_smaller_call(dd):
+    """A call whose narrowest tiles need more scratch than there is, first seen under capture: wider tiles, as nothing may be allocated."""
+    import torch
+    P, V = 100, 2000
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    tok, fl = torch.zeros(1, P, dtype=torch.int32, device="cuda"), torch.ones(1, P, dtype=torch.uint8, device="cuda")
+
+    def arguments(K):
+        h, w = (torch.randn(n, K, device="cuda", generator=gen).mul_(s).to(torch.bfloat16) for n, s in ((P, 1.0), (V, 2.0 / K ** 0.5)))
+        return None, None, h[None], w, tok, fl, CONF, 0.0, 0, 0
+    small, large = arguments(128), arguments(1024)
+    outs = dict(out_tokens=torch.empty_like(tok), out_mask=torch.empty_like(fl), out_score=torch.empty(1, P, device="cuda"))
+    dd.release()
+    dd.lm_head_verify(*small)                    # 32 tiles of 64 entries; the larger one would like 63 of 32
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dd.lm_head_verify(*large, **outs)
+    graph.replay()
+    torch.cuda.synchronize()
+    got = [outs[x].clone() for x in ("out_tokens", "out_mask", "out_score")]
+    del graph
+    want = dd.lm_head_verify(*large)             # now there is room
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    torch.testing.assert_close(got[2], want[2], rtol=1e-5, atol=0)
+    assert dd.verify_status() == 0
+
+
 # Rows gathered or not: nothing flagged where rows are not listed; many rows (more than one for a warp of the listing
 # kernel) with two tiles of the vocabulary, where few and where most of them are flagged, and with three.
 @pytest.mark.parametrize("B,P,K,V,share", [(1, 20, 128, 1000, 0.0), (2, 500, 64, 300, 0.0), (3, 8000, 64, 300, 0.15),
