@@ -905,19 +905,20 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
         return D == 64 ? launch_split<64, 1>(tq, tk, tv, p, q_rows, parts, s) : launch_split<128, 1>(tq, tk, tv, p, q_rows, parts, s);
     }
     if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
-    if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
     p.longest_first = longest_first(BH * m_blocks, sms);
-    if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
     // More items than SMs: persistent CTAs, whose rounds run across items.  us, a CTA per item : persistent: D = 128, 16 x 32 heads of
     // 512 tokens 101 : 76, 40 x 32 of 330 (a short kernel with rounds of its own, until then) 164 : 134, 64 x 32 of 256 148 : 91, 4 x
     // 32 of 4096 936 : 875, 32 of 8192 955 : 921, 3 x 24 of 1357 73.3 : 66.6; D = 64, 3 x 24 of 1357 61.5 : 56.8, 16 x 32 of 512 60.0 :
     // 54.8, 32 x 32 of 384 105 : 78.  With one round of items the one-item kernel's shorter start counts: 32 x 300 11.1 : 11.2, 16
     // x 512 at D = 128 11.65 : 11.8, 2 x 16 of 640 at D = 64 12.2 : 12.4.
-    if (nkv >= 2 && BH * m_blocks > sms) {
+    if (!general && nkv >= 2 && BH * m_blocks > sms) {
         static bool attr_done[2][64] = {};
         if (D == 64) return launch_persistent(attention_persistent_kernel<64>, SmemL<64>::kTotal + 1024, attr_done[0], p, sms, s, tq, tk, tv);
         return launch_persistent(attention_persistent_kernel<128>, SmemL<128>::kTotal + 1024, attr_done[1], p, sms, s, tq, tk, tv);
     }
+    // (only this kernel stores through a map)
+    if ((rc = make_tmap(&to, out, B, H, Nq, D, head_major)) != DD_OK) return rc;
+    if (general) return D == 64 ? launch<64, true>(tq, tk, tv, to, p, s) : launch<128, true>(tq, tk, tv, to, p, s);
     return D == 64 ? launch<64, false>(tq, tk, tv, to, p, s) : launch<128, false>(tq, tk, tv, to, p, s);
 }
 
