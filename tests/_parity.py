@@ -34,6 +34,15 @@ def off_vector_boundary(bits):
     return view
 
 
+def takes_the_streaming_kernel(B, P, V, kl):
+    """Whether dd_verify's rule on sizes gives (aligned) logits of this shape to the streaming kernel on this GPU: more than 160 pieces
+    of 4 KB per SM, and more than four rows per SM (of no more than 150000 logits)."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    pieces = (V + 7) // (1024 if kl else 2048) + 1
+    return B * P > 32768 or (B * P * pieces > 160 * sms and B * P > 4 * sms)
+
+
 def bf16_tensor_to_f64(t):
     import torch
     return t.detach().to("cpu").to(torch.float64).numpy()

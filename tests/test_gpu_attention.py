@@ -217,6 +217,16 @@ def test_kernel_choice(dd, oracle_mod, B, H, N, D):
     check_attention(got[:, :, rows], ref)
 
 
+@pytest.mark.parametrize("more", [0, 1])
+@pytest.mark.parametrize("N,D", [(129, 128), (200, 64), (256, 128)])
+def test_as_many_items_as_SMs_and_one_more(dd, oracle_mod, N, D, more):
+    """The line between the kernel with a CTA per item and the persistent one."""
+    import torch
+    H = torch.cuda.get_device_properties(0).multi_processor_count + more
+    q, k, v = synth.attention_inputs(1, H, N, D, seed=N)
+    check_attention(run_gpu(dd, q, k, v, D ** -0.5), oracle_mod.attention(q, k, v, D ** -0.5))
+
+
 @pytest.mark.parametrize("B,H,N", [(1, 2, 512), (1, 80, 500)])
 def test_peaked_rows_with_the_polynomial(dd, oracle_mod, B, H, N):
     q, k, v = synth.attention_inputs(B, H, N, 64, seed=8, planted=True, strength=6.0)

@@ -56,9 +56,12 @@ def both_builds(binding, check_path, call):
     (15, 700, 64, 380, CONF | PROB),             # many short rows, sequences beyond the short decision
     (1, 1500, 4104, 900, TRUST | EMIT),          # a sequence beyond the short decision
     (4, 8, 8, 0, KL),                            # nothing flagged: every sequence passes through
-    # the streaming kernel: rows cut by range boundaries, on and off vector boundaries; short rows, several rounds
+    # its deep form, flagged rows first
     (2, 200, 65000, 150, KL | PROB),
     (2, 200, 65003, 150, KL),
+    # the streaming kernel: rows cut by range boundaries, on and off vector boundaries; short rows, several rounds
+    (4, 200, 65000, 150, KL | PROB),
+    (4, 200, 65003, 150, KL),
     (4, 256, 65003, 40, CONF),
     (60, 700, 64, 500, KL),
     (24, 1500, 37, 900, CONF | PROB),
@@ -88,7 +91,7 @@ def test_element_wise_kernel(libs, B, P, V, flagged, mode, static):
                                                             **(fresh_outputs(B, P) if static else {})))
 
 
-@pytest.mark.parametrize("B,P,V,flagged", [(2, 96, 20000, 61), (2, 200, 65003, 150)])      # row and streaming kernel
+@pytest.mark.parametrize("B,P,V,flagged", [(2, 96, 20000, 61), (2, 200, 65003, 150), (4, 200, 65003, 150)])      # row kernel, its deep form, streaming kernel
 def test_static_scratch_and_unmask(libs, B, P, V, flagged):
     import torch
     binding, check_path = libs
@@ -99,7 +102,7 @@ def test_static_scratch_and_unmask(libs, B, P, V, flagged):
     both_builds(binding, check_path, lambda: binding.unmask(t[1], t[2], t[3], 0.3, 2))
 
 
-@pytest.mark.parametrize("B,P,K,V", [(2, 300, 128, 4100), (3, 700, 64, 20000)])        # every row; flagged rows only
+@pytest.mark.parametrize("B,P,K,V", [(2, 300, 128, 4100), (3, 700, 64, 20000), (1, 300, 64, 40000)])        # every row; flagged rows only; kernel chosen on the device
 @pytest.mark.parametrize("mode", [CONF | PROB, KL])
 def test_fused_heads(libs, mode, B, P, K, V):
     import torch

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2604_05250_b200 import synth
-from tests._parity import Guarded, check_verify, off_vector_boundary, to_torch_bf16
+from tests._parity import Guarded, check_verify, off_vector_boundary, takes_the_streaming_kernel, to_torch_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -248,18 +248,23 @@ def test_results_do_not_depend_on_the_grid(dd, oracle_mod, cta_cap):
     """Same inputs on 1, 7, 37 CTAs and on every SM: tokens, masks and scores bit-identical (which
     warp computes a unit, and in which order units finish, must not matter)."""
     cases = [
-        # the streaming kernel: rows on and off vector boundaries, long and short
+        # the row kernel's deep form, whose grid the cap leaves alone
         (synth.verify_inputs(2, 200, 65000, 150, 0.2, seed=43), KL | PROB, 0.5, 8, 0),
         (synth.verify_inputs(2, 200, 65003, 150, 0.2, seed=44), KL, 0.5, 4, 1),
+        # the streaming kernel: rows on and off vector boundaries, long and short
+        (synth.verify_inputs(4, 200, 65000, 150, 0.2, seed=47), KL | PROB, 0.5, 8, 0),
+        (synth.verify_inputs(4, 200, 65003, 150, 0.2, seed=48), KL, 0.5, 4, 1),
         (synth.verify_inputs(4, 256, 65003, 40, 0.2, seed=45), CONF | PROB, 0.5, 4, 2),
         (synth.verify_inputs(6, 6000, 41, 3000, 0.2, seed=46), KL, 0.5, 40, 3),
-        # the row kernel, whose grid the cap leaves alone
+        # the row kernel
         (synth.verify_config_inputs(0), KL | PROB, 0.5, 8, 0),
         (synth.verify_inputs(2, 40, 20000 + 8 * 37, 29, 0.2, seed=41), KL, 0.5, 4, 1),       # ragged last chunk
         (synth.verify_inputs(2, 40, 20000 + 8 * 37, 29, 0.2, seed=41), CONF | PROB, 0.5, 4, 2),
-        (synth.verify_inputs(15, 8192, 64, 5700, 0.2, seed=31), KL, 0.5, 40, 3),              # many short rows
+        (synth.verify_inputs(15, 8192, 64, 5700, 0.2, seed=31), KL, 0.5, 40, 3),              # many short rows: streamed
         (synth.verify_inputs(3, 96, 32000, 80, 0.3, seed=42), TRUST, 0.5, 0, 0),
     ]
+    streamed = [takes_the_streaming_kernel(*c[0][1].shape, (c[1] & 0xFF) == KL) for c in cases]
+    assert streamed == 2 * [False] + 4 * [True] + 3 * [False] + [True, False]
     for (dra, ver, tokens, flags), mode, tau, k, seed in cases:
         d_in = dra if (mode & 0xFF) == KL else None
         cta_cap(0)
@@ -292,6 +297,29 @@ def test_token_excluded_by_the_verifier_alone(dd, oracle_mod, V):
         inf_at[0, 2] = inf_at[1, 3] = True
         assert np.isposinf(ref["out_score"][inf_at]).all() and np.isposinf(got[2][inf_at]).all()
         assert np.isfinite(ref["out_score"][~inf_at]).all() and np.isfinite(got[2][~inf_at]).all()
+
+
+@pytest.mark.parametrize("V", [41000, 41003])
+def test_excluded_tokens_in_the_streaming_kernel(dd, oracle_mod, V):
+    """The same in rows of several chunks, cut by the ends of ranges."""
+    assert takes_the_streaming_kernel(5, 130, V, True)
+    ninf = np.uint16(0xFF80)
+    dra, ver, tokens, flags = synth.verify_inputs(5, 130, V, 20, 0.25, seed=V)
+    rng = np.random.default_rng(V)
+    rows = np.argwhere(flags)
+    alone, both, drafter, run = rows[3::7], rows[4::7], rows[5::7], rows[6::7]
+    for b, i in alone:
+        ver[b, i, int(np.argmax(synth.bf16_bits_to_f32(dra[b, i])))] = ninf
+    for b, i in both:
+        at = rng.choice(V, size=V // 16, replace=False)
+        dra[b, i, at] = ninf; ver[b, i, at] = ninf
+    for b, i in drafter:
+        dra[b, i, rng.choice(V, size=50, replace=False)] = ninf
+    for b, i in run:                                          # a chunk and more, and all but the last logits
+        dra[b, i, 8:30000] = ninf; ver[b, i, 8:30000] = ninf
+    tokens[:] = np.argmax(synth.bf16_bits_to_f32(dra), axis=2)
+    _, ref, got = compare(dd, oracle_mod, dra, ver, tokens, flags, KL, 0.5, 3, 7)
+    assert sorted(map(tuple, np.argwhere(np.isposinf(got[2])))) == sorted(map(tuple, alone))
 
 
 @pytest.mark.parametrize("V", [4096, 20000, 1003])
@@ -348,12 +376,14 @@ def test_logits_off_16_byte_boundaries(dd, oracle_mod, V, mode):
 # both tensors or 2048 of one on 148 SMs), rows on and off vector boundaries; in the streaming kernel rows cut
 # by range boundaries and grids of any size; in the row kernel clusters, CTAs, warps per row
 @pytest.mark.parametrize("B,P,V,flagged,mode", [
-    (2, 200, 65000, 150, KL), (2, 200, 65003, 150, KL),              # streaming
+    (2, 200, 65000, 150, KL), (2, 200, 65003, 150, KL),              # the deep form of the row kernel
+    (4, 200, 65000, 150, KL | PROB), (4, 200, 65003, 150, KL),       # streaming
     (4, 256, 65000, 40, CONF), (4, 256, 65003, 40, CONF | PROB),     # streaming
     (1, 20, 126464, 20, KL | PROB), (1, 40, 65003, 33, KL), (2, 70, 40003, 60, CONF),   # clusters of eight, four and two
     (1, 300, 20003, 77, KL), (4, 200, 9001, 150, KL), (6, 512, 4100, 100, KL), (24, 300, 1001, 100, CONF),   # 8, 4, 2 and 1 warps
 ])
 def test_row_and_streaming_kernels(dd, oracle_mod, B, P, V, flagged, mode):
+    assert takes_the_streaming_kernel(B, P, V, (mode & 0xFF) == KL) == (B * P > 592 and V > 60000)
     dra, ver, tokens, flags = synth.verify_inputs(B, P, V, flagged, 0.2, seed=V + P)
     hot = np.argmax(synth.bf16_bits_to_f32(ver[0, :1]), axis=1)
     flags[0, 0] = 1

@@ -62,10 +62,12 @@ def test_static_scratch_matches_dd_verify_on_two_calls_in_a_row(oracle_mod):
     both_entry_points(dd, oracle_mod, (2, 96, 20000, 61), KL | PROB, seed=21)
     frees = [both_entry_points(dd, oracle_mod, (3, 40, 126464, 33), KL, seed=22),
              both_entry_points(dd, oracle_mod, (1, 128, 1024, 32), CONF, seed=23),
-             # rows off vector boundaries; tensors off them, which take the element-wise kernel; the streaming kernel
+             # rows off vector boundaries; tensors off them, which take the element-wise kernel; the streaming kernel; the row
+             # kernel with long rows
              both_entry_points(dd, oracle_mod, (2, 50, 1003, 31), KL, seed=24),
              both_entry_points(dd, oracle_mod, (2, 50, 1003, 31), KL, seed=25, off=True),
-             both_entry_points(dd, oracle_mod, (2, 200, 65003, 150), KL, seed=26)]
+             both_entry_points(dd, oracle_mod, (4, 200, 65003, 150), KL, seed=26),
+             both_entry_points(dd, oracle_mod, (2, 200, 65003, 150), KL, seed=27)]
     # once the first call on the device has looked up the array, a call takes no device memory
     for before, after in frees:
         assert after == before
