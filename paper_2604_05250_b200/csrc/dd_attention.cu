@@ -907,8 +907,8 @@ int attention_impl(const void *q, const void *k, const void *v, void *out, int B
     if ((rc = make_tmap(&tq, q, B, H, Nq, D, head_major)) != DD_OK) return rc;
     p.longest_first = longest_first(BH * m_blocks, sms);
     // More items than SMs: persistent CTAs, whose rounds run across items.  us, a CTA per item : persistent: D = 128, 16 x 32 heads of
-    // 512 tokens 101 : 76, 40 x 32 of 330 (a short kernel with rounds of its own, until then) 164 : 134, 64 x 32 of 256 148 : 91, 4 x
-    // 32 of 4096 936 : 875, 32 of 8192 955 : 921, 3 x 24 of 1357 73.3 : 66.6; D = 64, 3 x 24 of 1357 61.5 : 56.8, 16 x 32 of 512 60.0 :
+    // 512 tokens 101 : 78, 40 x 32 of 330 (a short kernel with rounds of its own, until then) 164 : 134, 64 x 32 of 256 148 : 91, 4 x
+    // 32 of 4096 936 : 875, 32 of 8192 954 : 937, 3 x 24 of 1357 73.3 : 66.6; D = 64, 3 x 24 of 1357 61.5 : 56.8, 16 x 32 of 512 60.0 :
     // 54.8, 32 x 32 of 384 105 : 78.  With one round of items the one-item kernel's shorter start counts: 32 x 300 11.1 : 11.2, 16
     // x 512 at D = 128 11.65 : 11.8, 2 x 16 of 640 at D = 64 12.2 : 12.4.
     if (!general && nkv >= 2 && BH * m_blocks > sms) {

@@ -23,7 +23,7 @@
 //   * Every lane storing its own row, 32 bytes at a time, took 2500 to 2900 cycles per item and group; four lanes
 //     now exchange pieces first and store 128 bytes of a row together: 2000 (16 x 32 of 512 71.3 -> 68.5 us in short bursts).
 //   * A group writes an item's result behind the weights of the next item's first tile, whose products the stores then overlap: 68.5
-//     -> 67.2 in bursts; both, under the power cap, 85.3 -> 76.0.
+//     -> 67.2 in bursts; both, under the power cap, 84.7 -> 78.0.
 //   * o_free: the group has read the finished accumulator out of tensor memory; the next item's
 //     first P V may overwrite it.
 // Every wait is bounded and reports to the attention health word.  Included by dd_attention.cu

@@ -22,7 +22,7 @@
 // 16 sequences of 256 positions, 62 % of them flagged, K = 4096, V = 126464: 3024 us
 // with every row multiplied, 1961 us so.
 //
-// More than 128 rows are multiplied by pairs of CTAs where that is faster, always in the KL mode (dd_lm_head_pair.cuh).
+// More than 128 rows are multiplied by pairs of CTAs where that is faster (dd_lm_head_pair.cuh; the rule is dd_lm_head_verify's).
 //
 // Tensor memory (512 columns): TRUST/CONF, N <= 256: the verifier's two accumulators at columns 0
 // and 256.  KL, N <= 128: the drafter's at 0 and 128, the verifier's at 256 and 384; a work item

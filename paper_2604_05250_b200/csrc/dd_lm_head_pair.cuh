@@ -1,5 +1,6 @@
-// The products of dd_lm_head_verify by pairs of CTAs (tcgen05 cta_group::2), for more than 128 rows: always in the KL mode (Eq. 4-5 from
-// both models' hidden states: two products per vocabulary tile), in the others where dd_lm_head_verify says so.
+// The products of dd_lm_head_verify by pairs of CTAs (tcgen05 cta_group::2), for more than 128 rows, in the KL mode (Eq. 4-5 from
+// both models' hidden states: two products per vocabulary tile) and in the others where dd_lm_head_verify says so, or the kernel that lists the
+// flagged rows (LmParams::pairs).
 //
 // What bounds lm_head_kernel is neither the tensor core nor memory but the operands' way from L2 into the SMs, some 45 bytes
 // per clock and SM (10-11 TB/s over the chip): 64 KB a k-step for 256 x 256 x 64 products, 48 KB for 256 x 128 x 64 in the KL

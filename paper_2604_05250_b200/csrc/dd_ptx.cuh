@@ -46,8 +46,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 }
 // Bounded wait: false if the phase did not complete within `limit` polls.  Left to itself the compiler peels the first 64 polls,
 // a kilobyte or two of code at each of some thirty waits of a kernel; a warp that polls then reads code all the time that the other warps of its
-// scheduler, with some 12 KB of softmax a key tile, need the instruction caches for.  As a loop: attention_kernel<128>
-// 107 -> 78 KB of code, 16 x 32 heads of 512 tokens 88.6 -> 86.9 us, 64 x 32 heads of 32 queries over 256-1024 keys 135 -> 131.
+// scheduler, with some 12 KB of softmax a key tile, need the instruction caches for.  As a loop:
+// 16 x 32 heads of 512 tokens 88.6 -> 86.9 us, 64 x 32 heads of 32 queries over 256-1024 keys 135 -> 131.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t limit = (1u << 22))
 {
 #pragma unroll 1

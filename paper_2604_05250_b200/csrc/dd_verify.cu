@@ -370,7 +370,7 @@ int launch_rows(const VerifyParams &p, cudaStream_t stream)
     const uintptr_t flags = (uintptr_t)p.flags, mask = (uintptr_t)p.out_mask;
     const bool in_place = flags < mask + (size_t)rows && mask < flags + (size_t)rows;
     shape.mapped = shape.wpr == kRWarps && shape.cluster == 1 && rows <= kMappedRows && (deep || (KL && pieces >= 24)) && !in_place;
-    // Early only where every CTA has an SM to itself: CTAs that arrive early pile up on the SMs that are free first, and waiting ones of a second
+    // Early only in the short form and where every CTA has an SM to itself (the deep one reads for longer than the gap between two kernels): CTAs that arrive early pile up on the SMs that are free first, and waiting ones of a second
     // round take up the room of the first one's last.  us, early : ordinary, after attention of 32 heads of 1024: 256 rows of 126464, KL
     // 55.5 : 53.0, 2 x 300 of 32001 42.7 : 39.3, 1 x 100 of 50000, CONF 35.1 : 33.1, 1 x 512 of 32000, CONF 39.2 : 38.3; but 128 of
     // 1024, KL 27.1 : 28.4, 64 of 1000 27.9 : 28.5.  One after the other, 1024 of 4000, KL 19.4 : 18.7.

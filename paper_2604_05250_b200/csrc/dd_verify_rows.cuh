@@ -193,7 +193,7 @@ __device__ __forceinline__ Partial row_part(const VerifyParams &p, int row, int 
 
 // The same with more than a few pieces to a warp: the next one is on its way while one is worked on, pieces that are all there are loaded
 // without a comparison per vector, and -inf is dealt with where it occurs (lane_piece).  The pieces' loop holds no branch around a
-// load.  1 x 256 positions, V = 126464, KL (357 instructions a piece; in the short form 470, one piece at a time): 36.8 -> 29.9 us; 1 x 128
+// load.  1 x 256 positions, V = 126464, KL (363 instructions a piece; in the short form 470, one piece at a time): 36.8 -> 29.9 us; 1 x 128
 // 23.9 -> 20.4; 1 x 400, half flagged, CONF 25.4 -> 19.9.
 template <bool KL>
 __device__ __forceinline__ Partial row_part_deep(const VerifyParams &p, int row, int x0, int stride)
